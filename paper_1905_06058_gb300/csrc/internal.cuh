@@ -25,6 +25,11 @@ struct StoltConst {
   int I0;
   int K, logK, nx, ny, nk, nz, J;
   int focus;      // z0 != 0
+  // no column is evanescent and samples lie less than 2.3 bins apart: the
+  // axial kernels may share bin windows between a thread's samples (WINDOW in
+  // k_axial.cuh)
+  int window;
+  int past;       // then: bins a column's windows may reach past one period of K
 };
 
 // Stolt position and spectral phase of one (|q|, k_j) sample (mfl == INT_MIN:
@@ -118,6 +123,7 @@ template <typename T> struct AxArgs {
   // FP32, K = 2048 or 4096: 1 runs the column-split radix-16 transforms, 0 the
   // radix-8 column-pair ones (the plan's tuned choice); ignored elsewhere
   int radix16;
+  unsigned past_offset;  // shared-memory offset of window_past's bins (set at launch)
   // fused kernel in a solve with the device-side stop rule: as LatArgs::stop
   const int* stop;
 };

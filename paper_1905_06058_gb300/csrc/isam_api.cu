@@ -843,6 +843,20 @@ void make_stolt(isam_plan* P) {
   c.K = P->K; c.logK = ilog2(P->K);
   c.nx = P->nx; c.ny = P->ny; c.nk = P->nk; c.nz = P->nz; c.J = P->J;
   c.focus = c.zeta != 0.0;
+  // the largest step between samples, dp/dj = 4 kappa / p at the lowest kappa
+  // and the largest |q|, for the window form of the axial kernels
+  const double a_max = c.Qx * pow(P->nx / 2, 2.0) + c.Qy * pow(P->ny / 2, 2.0);
+  const double x = 4.0 * c.kap * c.kap - a_max;
+  c.window = x > 0.0 && 4.0 * c.kap <= 2.3 * sqrt(x);
+  if (c.window) {
+    // the longest span of positions, one bin for each end's rounding, J + 7 bins
+    // of the last window (window_slots)
+    const double k1 = c.kap + (P->nk - 1);
+    const double span = sqrt(4.0 * k1 * k1 - a_max) - sqrt(x);
+    c.past = std::max(0, int(ceil(span)) + 2 + P->J + 7 - P->K);
+  } else {
+    c.past = 0;
+  }
 }
 
 // Least squares min ||V a - v|| for the Vandermonde V_ik = y_i^k (k <= deg),

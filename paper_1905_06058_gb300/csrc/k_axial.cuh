@@ -117,6 +117,29 @@ __device__ __forceinline__ int stolt_class(const StoltConst& sc, int mx, int my)
   return abs(my) * (sc.nx / 2 + 1) + abs(mx);
 }
 
+// consecutive samples a thread of the adjoint interpolation owns (see
+// scatter_samples)
+constexpr int NRES = 4;
+
+template <typename T> struct Sample {
+  cpair<T> val;   // conj(phase) R of both columns
+  T frac;         // fractional Stolt offset
+  int mfl;        // unwrapped floor of the Stolt position; INT_MIN: no contribution
+                  // (evanescent, or past nk)
+};
+
+// the position half of a table entry
+__device__ __forceinline__ void stolt_position(const StoltEntry<float>* e, int& mfl, float& frac) {
+  const int2 v = __ldg(reinterpret_cast<const int2*>(e));
+  mfl = v.x;
+  frac = __int_as_float(v.y);
+}
+__device__ __forceinline__ void stolt_position(const StoltEntry<double>* e, int& mfl,
+                                               double& frac) {
+  mfl = e->mfl;
+  frac = e->frac;
+}
+
 // Stolt position and spectral phase of sample j of one column pair, from the
 // plan's table when present, else evaluated (float-float / double).
 template <typename T> struct Positions {
@@ -127,6 +150,33 @@ template <typename T> struct Positions {
     const size_t cls = size_t(stolt_class(A.sc, mx, my)) * A.sc.nk;
     row = A.tab.stab ? A.tab.stab + cls : nullptr;
     frow = A.tab.filt ? A.tab.filt + cls : nullptr;
+  }
+  // floor and fraction of samples j0 .. j0 + NRES - 1 (mfl INT_MIN: evanescent
+  // or past nk), and their phases one by one: a thread's positions and phases
+  // are used apart, and the table's two halves read apart keep registers free
+  __device__ __forceinline__ void quad(const AxArgs<T>& A, int j0, Sample<T>* sm) const {
+#pragma unroll
+    for (int rho = 0; rho < NRES; ++rho) {
+      const int j = j0 + rho;
+      sm[rho].mfl = INT_MIN;
+      if (j >= A.sc.nk) continue;
+      if (row) {
+        stolt_position(row + j, sm[rho].mfl, sm[rho].frac);
+      } else {
+        T turn;
+        if (!sp.at(A.sc, j, sm[rho].mfl, sm[rho].frac, turn)) sm[rho].mfl = INT_MIN;
+      }
+    }
+  }
+  __device__ __forceinline__ cplx<T> phase(const AxArgs<T>& A, int j, bool prop) const {
+    if (row) return row[j].ph;
+    if (!prop) return mk<T>(0, 0);
+    int mfl;
+    T frac, turn;
+    sp.at(A.sc, j, mfl, frac, turn);
+    cplx<T> ph = spectral_phase<T>(A.sc, A.tab.disp, j, turn);
+    if (frow) ph = cmul(ph, __ldg(frow + j));
+    return ph;
   }
   __device__ __forceinline__ bool at(const AxArgs<T>& A, int j, int& mfl, T& frac,
                                      cplx<T>& ph) const {
@@ -256,15 +306,6 @@ __device__ __forceinline__ void interp_pair(const cpair<T>* Y, int K, int mfl, c
 // that the wrap mod K never folds two neighbourhoods of one phase together.
 // Each bin receives at most ceil(J/2) + 1 contributions per chunk, summed in
 // a fixed order with fused multiply-adds.
-constexpr int NRES = 4;
-
-template <typename T> struct Sample {
-  cpair<T> val;   // conj(phase) R of both columns
-  T frac;         // fractional Stolt offset
-  int mfl;        // unwrapped floor of the Stolt position
-  int chunk;      // INT_MIN: evanescent (no contribution)
-};
-
 // Zero Y, find the block's range of Stolt positions (shared atomics on
 // *lo, *hi, initialised by the caller before an earlier barrier) and assign
 // every sample to a chunk of width K - J of unwrapped positions: within a
@@ -279,14 +320,15 @@ template <typename T> struct Sample {
 // and is in chunk 0 or evanescent.  Its position goes through *tail
 // (INT_MAX: j* >= nk, INT_MIN: evanescent).
 template <typename T, int J>
-__device__ __forceinline__ int prepare_scatter(cpair<T>* Y, int K, int nt, int nk, Sample<T>* sm,
-                                               int* lo, int* hi, int* tail, bool& warp_tail) {
+__device__ __forceinline__ int prepare_scatter(cpair<T>* Y, int K, int nt, int nk,
+                                               const Sample<T>* sm, int* chunk, int* lo, int* hi,
+                                               int* tail, bool& warp_tail) {
   const cpair<T> zero = {mk<T>(0, 0), mk<T>(0, 0)};
   for (int i = threadIdx.x; i < K; i += nt) Y[prow(i)] = zero;
   int l = INT_MAX, h = INT_MIN;
 #pragma unroll
   for (int rho = 0; rho < NRES; ++rho)
-    if (sm[rho].chunk != INT_MIN) {
+    if (sm[rho].mfl != INT_MIN) {
       l = min(l, sm[rho].mfl);
       h = max(h, sm[rho].mfl);
     }
@@ -296,18 +338,20 @@ __device__ __forceinline__ int prepare_scatter(cpair<T>* Y, int K, int nt, int n
   }
   if (int(threadIdx.x) == nt - 33)
     *tail = NRES * (nt - 32) - 1 >= nk ? INT_MAX
-            : (sm[NRES - 1].chunk != INT_MIN ? sm[NRES - 1].mfl : INT_MIN);
+            : sm[NRES - 1].mfl;
   __syncthreads();
   const int base = *lo, width = K - J;
   warp_tail = false;
   if (base == INT_MAX) return 0;
 #pragma unroll
-  for (int rho = 0; rho < NRES; ++rho)
-    if (sm[rho].chunk != INT_MIN) {
+  for (int rho = 0; rho < NRES; ++rho) {
+    chunk[rho] = INT_MIN;
+    if (sm[rho].mfl != INT_MIN) {
       int c = 0, d = sm[rho].mfl - base;
       while (d >= width) { d -= width; ++c; }
-      sm[rho].chunk = c;
+      chunk[rho] = c;
     }
+  }
   int n = 1;
   for (int d = *hi - base; d >= width; d -= width) ++n;
   const int t = *tail;
@@ -341,12 +385,13 @@ __device__ __forceinline__ void add_sample(const AxArgs<T>& A, cpair<T>* Y, int 
 // block barrier: the same phases in the same order, so the same sums.
 template <typename T, int J>
 __device__ __forceinline__ void scatter_samples(const AxArgs<T>& A, cpair<T>* Y, int K, int nt,
-                                                const Sample<T>* sm, int nchunks, bool warp_tail) {
+                                                const Sample<T>* sm, const int* chunk, int nchunks,
+                                                bool warp_tail) {
   const int block_chunks = warp_tail ? 1 : nchunks;
   for (int ch = 0; ch < block_chunks; ++ch) {
 #pragma unroll
     for (int rho = 0; rho < NRES; ++rho) {
-      if (sm[rho].chunk == ch) add_sample<T, J>(A, Y, K, sm[rho]);
+      if (chunk[rho] == ch) add_sample<T, J>(A, Y, K, sm[rho]);
       __syncthreads();
     }
   }
@@ -354,11 +399,210 @@ __device__ __forceinline__ void scatter_samples(const AxArgs<T>& A, cpair<T>* Y,
     if ((int(threadIdx.x) >> 5) == (nt >> 5) - 1) {
 #pragma unroll
       for (int rho = 0; rho < NRES; ++rho) {
-        if (sm[rho].chunk == 1) add_sample<T, J>(A, Y, K, sm[rho]);
+        if (chunk[rho] == 1) add_sample<T, J>(A, Y, K, sm[rho]);
         __syncwarp();
       }
     }
     __syncthreads();
+  }
+}
+
+// WINDOW form of the interpolation's and the scatter's shared-memory traffic.
+//
+// A thread's four samples lie 2 to 2.3 bins apart (StoltConst::window), so
+// their J-bin neighbourhoods overlap: together they touch WS = J + 7 bins, not
+// 4 J.  Sample rho sits at cumulative offset 2 rho or 2 rho + 1 from the
+// thread's first sample; with its J coefficients shifted by that 0 or 1 into
+// J + 1 taps (window_taps) every register index is a constant.  The gather
+// reads each of the WS bins once.  The scatter sums the four samples in
+// registers and touches shared memory once per bin: the bins before the next
+// thread's window belong to this thread alone and are stored (no zeroing pass,
+// no read), the J - 1 or so after it are added after a barrier, where they are
+// disjoint again (at least seven bins separate the windows of neighbours).
+// Bins a window reaches past one period of K are added in a second pass of the
+// same two phases, taken only by the last warps' threads and only when a column
+// spans more than K.
+//
+// What bounded the kernels was the load/store data path: the residue-class
+// scatter took 56 shared-memory accesses a thread (8 to zero, 24 reads, 24
+// writes) in 8 barrier phases, the per-sample gather 24; the windows take 23
+// and 13 (J = 6).  k_ax_fused, 1024 x 2048 B-scan: 51.5 -> 47.6 us, 256 x 256 x
+// 2048 volume: 2,414 -> 2,117 us; k_ax_adj 36.8 -> 30.7 us and 1,598 -> 1,300 us.
+//
+// The bound of 2.3 bins keeps four samples and the next thread's first within
+// the offsets the kernels hold as constants (three steps below 7 bins, four
+// below 10); the acquisitions in use reach 2.06 (B-scan, NA 0.15) to 2.23
+// (volume corner, NA 0.2).
+//
+// Positions of q = 0 columns can round to an offset outside {0, 1} when their
+// common fraction is within rounding of an integer; then the block takes the
+// residue-class scatter, as do all blocks of evanescent or steeper geometries.
+template <int J> __host__ __device__ constexpr int window_slots() { return J + 2 * NRES - 1; }
+
+// sample rho's offset from bin 2 rho of the thread's window (0 or 1 where it fits)
+template <typename T> __device__ __forceinline__ unsigned window_offset(const Sample<T>* sm, int rho) {
+  return unsigned(sm[rho].mfl) - unsigned(sm[0].mfl) - 2u * unsigned(rho);
+}
+
+// J coefficients as J + 1 taps, shifted up by one when `shift`
+template <typename T, int J>
+__device__ __forceinline__ void window_taps(const Poly<T>& P, T frac, bool shift, T* e) {
+  T c[J];
+  coefficients<T, J>(P, frac, c);
+  e[0] = shift ? T(0) : c[0];
+#pragma unroll
+  for (int l = 1; l < J; ++l) e[l] = shift ? c[l - 1] : c[l];
+  e[J] = shift ? c[J - 1] : T(0);
+}
+
+// Per block: the first sample's floor of every thread that has samples.
+struct WindowHeads { int mfl[512]; };
+
+// One thread's window: sums its samples slot by slot and hands each finished
+// slot (l, value) to put.
+template <typename T, int J, typename Put>
+__device__ __forceinline__ void window_sums(const AxArgs<T>& A, const Sample<T>* sm, Put put) {
+  using V = cpair<T>;
+  constexpr int WS = window_slots<J>();
+  V w[WS];
+#pragma unroll
+  for (int rho = 0; rho < NRES; ++rho) {
+    T e[J + 1];
+    window_taps<T, J>(A.poly, sm[rho].frac, window_offset(sm, rho) != 0, e);
+#pragma unroll
+    for (int l = 0; l <= J; ++l) {
+      V& x = w[2 * rho + l];
+      if (rho == 0 || l > J - 2) x = escale(sm[rho].val, e[l]);
+      else {
+        x.a = cfma_r(e[l], sm[rho].val.a, x.a);
+        x.b = cfma_r(e[l], sm[rho].val.b, x.b);
+      }
+    }
+    if (rho < NRES - 1) {
+      put(2 * rho, w[2 * rho]);
+      put(2 * rho + 1, w[2 * rho + 1]);
+    }
+  }
+#pragma unroll
+  for (int l = 2 * (NRES - 1); l < WS; ++l) put(l, w[l]);
+}
+
+// Y = the scatter of all samples (every bin written; ends with a barrier).
+// Every read of Y must be done and heads complete (a barrier before).
+template <typename T, int J>
+__device__ __forceinline__ void window_scatter(const AxArgs<T>& A, cpair<T>* Y, int K, int nt,
+                                               int nk, const Sample<T>* sm, cpair<T>* past,
+                                               const WindowHeads& heads) {
+  using V = cpair<T>;
+  constexpr int WS = window_slots<J>(), W_MIN = 2 * NRES - 1, W_MAX = 2 * NRES + 2;
+  const int tid = threadIdx.x, nact = nk / NRES;
+  const bool active = tid < nact;
+  const int off = 1 - J / 2;                          // first bin of a window - its head
+  const int base = heads.mfl[0] + off, end = heads.mfl[nact - 1] + off + WS;
+  const int m0 = active ? heads.mfl[tid] + off : 0;
+  // bins before the next thread's window (all of them for the last thread)
+  const int own = tid < nact - 1 ? heads.mfl[tid + 1] + off - m0 : WS;
+  const int limit = base + K - m0;                    // slots from here on lie past one period
+  for (int i = end + tid; i < base + K; i += nt)
+    Y[prow(i & (K - 1))] = {mk<T>(0, 0), mk<T>(0, 0)};
+  auto row = [&](int l) -> V& {
+    return l < limit ? Y[prow((m0 + l) & (K - 1))] : past[l - limit];
+  };
+  V tail[WS - W_MIN];
+  if (active)
+    window_sums<T, J>(A, sm, [&](int l, const V& v) {
+      if (l >= W_MIN) tail[l - W_MIN] = v;
+      if (l < W_MIN || l < own) row(l) = v;
+    });
+  __syncthreads();
+  if (active)
+#pragma unroll
+    for (int l = W_MIN; l < WS; ++l)
+      if (l >= own) {
+        V& y = row(l);
+        y = eadd(y, tail[l - W_MIN]);
+      }
+  __syncthreads();
+  if (end > base + K) {                               // the same for the whole block
+    for (int i = tid; i < end - base - K; i += nt) {
+      V& y = Y[prow((base + i) & (K - 1))];
+      y = eadd(y, past[i]);
+    }
+    __syncthreads();
+  }
+}
+
+// The bins past one period: A.sc.window_past elements after the twiddles.
+template <typename T>
+__device__ __forceinline__ cpair<T>* window_past(const AxArgs<T>& A, cpair<T>* Y) {
+  return reinterpret_cast<cpair<T>*>(reinterpret_cast<unsigned char*>(Y) + A.past_offset);
+}
+
+// Y = the scatter of the block's samples, in the window form where every
+// thread's samples fit one.  Starts with a barrier (all reads of Y are done)
+// and ends with one.
+template <typename T, int J>
+__device__ __forceinline__ void scatter(const AxArgs<T>& A, cpair<T>* Y, int K, int nt, int nk,
+                                        Sample<T>* sm, int* lo, int* hi, int* ch_tail,
+                                        WindowHeads& heads) {
+  bool ok = A.sc.window != 0;
+  if (NRES * int(threadIdx.x) < nk) {
+    heads.mfl[threadIdx.x] = sm[0].mfl;
+#pragma unroll
+    for (int rho = 0; rho < NRES; ++rho)
+      ok &= window_offset(sm, rho) <= 1u;
+  }
+  if (__syncthreads_and(ok)) {
+    window_scatter<T, J>(A, Y, K, nt, nk, sm, window_past<T>(A, Y), heads);
+    return;
+  }
+  bool warp_tail;
+  int chunk[NRES];
+  const int nch = prepare_scatter<T, J>(Y, K, nt, nk, sm, chunk, lo, hi, ch_tail, warp_tail);
+  scatter_samples<T, J>(A, Y, K, nt, sm, chunk, nch, warp_tail);
+}
+
+// The forward interpolation of a thread's samples (before the phase): hands
+// (rho, N(x1), N(x2)) to put, in order; evanescent samples give 0.
+template <typename T, int J, typename Put>
+__device__ __forceinline__ void interp_quad(const AxArgs<T>& A, const cpair<T>* Y, int K,
+                                            const Sample<T>* sm, Put put) {
+  using C = cplx<T>;
+  bool fits = A.sc.window != 0;
+#pragma unroll
+  for (int rho = 0; rho < NRES; ++rho) fits &= window_offset(sm, rho) <= 1u;
+  if (fits) {
+    constexpr int WS = window_slots<J>();
+    const int m0 = sm[0].mfl - J / 2 + 1;
+    cpair<T> y[WS];
+#pragma unroll
+    for (int l = 0; l < J - 1; ++l) y[l] = Y[prow((m0 + l) & (K - 1))];
+#pragma unroll
+    for (int rho = 0; rho < NRES; ++rho) {
+#pragma unroll
+      for (int l = J - 1; l <= J; ++l)
+        y[2 * rho + l] = Y[prow((m0 + 2 * rho + l) & (K - 1))];
+      T e[J + 1];
+      window_taps<T, J>(A.poly, sm[rho].frac, window_offset(sm, rho) != 0, e);
+      C s1 = cscale(y[2 * rho].a, e[0]), s2 = cscale(y[2 * rho].b, e[0]);
+#pragma unroll
+      for (int l = 1; l <= J; ++l) {
+        s1 = cfma_r(e[l], y[2 * rho + l].a, s1);
+        s2 = cfma_r(e[l], y[2 * rho + l].b, s2);
+      }
+      put(rho, s1, s2);
+    }
+    return;
+  }
+#pragma unroll
+  for (int rho = 0; rho < NRES; ++rho) {
+    C s1 = mk<T>(0, 0), s2 = mk<T>(0, 0);
+    if (sm[rho].mfl != INT_MIN) {
+      T c[J];
+      coefficients<T, J>(A.poly, sm[rho].frac, c);
+      interp_pair<T, J>(Y, K, sm[rho].mfl, c, s1, s2);
+    }
+    put(rho, s1, s2);
   }
 }
 
@@ -493,6 +737,13 @@ __device__ __forceinline__ void ax_inverse(const AxArgs<T>& A, cpair<T>* Y, cons
   }
 }
 
+// FP32: two blocks of 512 threads on an SM (64 registers).  FP64: the pair at
+// K = 4096 fills an SM's shared memory by itself, so one (128 registers; at 64
+// the adjoint half spilled 0.5 to 2 KB a thread).
+template <typename T> __host__ __device__ constexpr int ax_min_blocks() {
+  return std::is_same<T, float>::value ? 2 : 1;
+}
+
 template <typename T, int J, int LOGK, bool C16>
 __global__ void __launch_bounds__(512) k_ax_fwd(const __grid_constant__ AxArgs<T> A) {
   using C = cplx<T>;
@@ -532,7 +783,7 @@ __global__ void __launch_bounds__(512) k_ax_fwd(const __grid_constant__ AxArgs<T
 }
 
 template <typename T, int J, int LOGK, bool C16>
-__global__ void __launch_bounds__(512, 2) k_ax_adj(const __grid_constant__ AxArgs<T> A) {
+__global__ void __launch_bounds__(512, ax_min_blocks<T>()) k_ax_adj(const __grid_constant__ AxArgs<T> A) {
   using C = cplx<T>;
   using V = cpair<T>;
   extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -541,6 +792,7 @@ __global__ void __launch_bounds__(512, 2) k_ax_adj(const __grid_constant__ AxArg
   V* Y = reinterpret_cast<V*>(smem_raw);
   cplx<T>* tw = twiddle_table<T>(smem_raw, K);
   __shared__ int ch_lo, ch_hi, ch_tail;
+  __shared__ WindowHeads heads;
   const int tid = threadIdx.x, nt = axial_threads<LOGK>();
   int c1, c2, mx, my;
   pair_columns(A, c1, c2, mx, my);
@@ -557,7 +809,7 @@ __global__ void __launch_bounds__(512, 2) k_ax_adj(const __grid_constant__ AxArg
 #pragma unroll
   for (int rho = 0; rho < NRES; ++rho) {
     const int j = NRES * tid + rho;
-    sm[rho].chunk = INT_MIN;
+    sm[rho].mfl = INT_MIN;
     int mfl;
     T frac;
     C ph;
@@ -566,12 +818,9 @@ __global__ void __launch_bounds__(512, 2) k_ax_adj(const __grid_constant__ AxArg
       sm[rho].val.b = two ? cmulc(r2[j], ph) : mk<T>(0, 0);
       sm[rho].frac = frac;
       sm[rho].mfl = mfl;
-      sm[rho].chunk = 0;
     }
   }
-  bool warp_tail;
-  const int nch = prepare_scatter<T, J>(Y, K, nt, nk, sm, &ch_lo, &ch_hi, &ch_tail, warp_tail);
-  scatter_samples<T, J>(A, Y, K, nt, sm, nch, warp_tail);
+  scatter<T, J>(A, Y, K, nt, nk, sm, &ch_lo, &ch_hi, &ch_tail, heads);
   ax_inverse<T, LOGK, C16>(A, Y, tw, c1, c2, two);
 }
 
@@ -585,7 +834,7 @@ __global__ void __launch_bounds__(512, 2) k_ax_adj(const __grid_constant__ AxArg
 // Hermitian, so only its c1 column is read.
 // WS: also write the model spectra S to A.s_out.
 template <typename T, int J, int LOGK, bool WS, bool C16>
-__global__ void __launch_bounds__(512, 2) k_ax_fused(const __grid_constant__ AxArgs<T> A) {
+__global__ void __launch_bounds__(512, ax_min_blocks<T>()) k_ax_fused(const __grid_constant__ AxArgs<T> A) {
   using C = cplx<T>;
   using V = cpair<T>;
   extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -594,6 +843,7 @@ __global__ void __launch_bounds__(512, 2) k_ax_fused(const __grid_constant__ AxA
   V* Y = reinterpret_cast<V*>(smem_raw);
   cplx<T>* tw = twiddle_table<T>(smem_raw, K);
   __shared__ int ch_lo, ch_hi, ch_tail;
+  __shared__ WindowHeads heads;
   const int tid = threadIdx.x, nt = axial_threads<LOGK>();
   int c1, c2, mx, my;
   pair_columns(A, c1, c2, mx, my);
@@ -624,51 +874,26 @@ __global__ void __launch_bounds__(512, 2) k_ax_fused(const __grid_constant__ AxA
   }
   ax_forward<T, LOGK, C16>(A, Y, tw, c1, c2, two);
   if (stopped) return;   // an earlier check stopped the solve: write nothing
-  if constexpr (COL16) {
-#pragma unroll
-    for (int rho = 0; rho < NRES; ++rho) {
-      const int j = NRES * tid + rho;
-      dqv[rho] = j < nk ? d1[j] : mk<T>(0, 0);
-    }
-  }
-
   const Positions<T> pos(A, mx, my);
   Sample<T> sm[NRES];
-#pragma unroll
-  for (int rho = 0; rho < NRES; ++rho) {
-    const int j = NRES * tid + rho;
-    sm[rho].chunk = INT_MIN;
-    if (j >= nk) continue;
-    const C dq = dqv[rho];
-    int mfl;
-    T frac;
-    C s1 = mk<T>(0, 0), s2 = mk<T>(0, 0), ph = mk<T>(0, 0);
-    const bool prop = pos.at(A, j, mfl, frac, ph);
-    if (prop) {
-      T c[J];
-      coefficients<T, J>(A.poly, frac, c);
-      interp_pair<T, J>(Y, K, mfl, c, s1, s2);
+  pos.quad(A, NRES * tid, sm);
+  if (NRES * tid < nk) {
+    interp_quad<T, J>(A, Y, K, sm, [&](int rho, C s1, C s2) {
+      const int j = NRES * tid + rho;
+      const C ph = pos.phase(A, j, sm[rho].mfl != INT_MIN);
       s1 = cmul(s1, ph);
       s2 = two ? cmul(s2, ph) : s1;
-    }
-    if (WS) {
-      A.s_out[size_t(c1) * nk + j] = s1;
-      if (two) A.s_out[size_t(c2) * nk + j] = s2;
-    }
-    const C R1 = csub(cscale(cadd(s1, cconj(s2)), T(0.5)), dq);
-    const C R2 = csub(cscale(cadd(s2, cconj(s1)), T(0.5)), cconj(dq));   // F s_d(-q)
-    if (prop) {
-      sm[rho].val.a = cmulc(R1, ph);
-      sm[rho].val.b = two ? cmulc(R2, ph) : mk<T>(0, 0);
-      sm[rho].frac = frac;
-      sm[rho].mfl = mfl;
-      sm[rho].chunk = 0;
-    }
+      if (WS) {
+        A.s_out[size_t(c1) * nk + j] = s1;
+        if (two) A.s_out[size_t(c2) * nk + j] = s2;
+      }
+      // R(-q) = conj R(q): the residual is real
+      const C R = csub(cscale(cadd(s1, cconj(s2)), T(0.5)), COL16 ? d1[j] : dqv[rho]);
+      sm[rho].val.a = cmulc(R, ph);
+      sm[rho].val.b = two ? cmulc(cconj(R), ph) : mk<T>(0, 0);
+    });
   }
-  __syncthreads();                       // all reads of Y are done
-  bool warp_tail;
-  const int nch = prepare_scatter<T, J>(Y, K, nt, nk, sm, &ch_lo, &ch_hi, &ch_tail, warp_tail);
-  scatter_samples<T, J>(A, Y, K, nt, sm, nch, warp_tail);
+  scatter<T, J>(A, Y, K, nt, nk, sm, &ch_lo, &ch_hi, &ch_tail, heads);
   ax_inverse<T, LOGK, C16>(A, Y, tw, c1, c2, two);
 }
 
@@ -707,8 +932,9 @@ template <typename T> cudaError_t launch_stolt_table(const AxArgs<T>& a, StoltEn
 template <typename T> size_t ax_smem_bytes(int K, int nk, bool adj) {
   (void)nk;
   (void)adj;
-  return size_t(padded_rows(K)) * sizeof(cpair<T>) +
-         size_t(twiddle_entries(K, ilog2_dev(K))) * sizeof(cplx<T>);
+  const size_t b = size_t(padded_rows(K)) * sizeof(cpair<T>) +
+                   size_t(twiddle_entries(K, ilog2_dev(K))) * sizeof(cplx<T>);
+  return (b + sizeof(cpair<T>) - 1) / sizeof(cpair<T>) * sizeof(cpair<T>);
 }
 
 enum { AX_FWD = 0, AX_ADJ = 1, AX_FUSED = 2 };
@@ -717,7 +943,10 @@ template <typename T, int J, int LOGK, bool C16>
 static cudaError_t launch_ax_JKC(const AxArgs<T>& a, int npairs, cudaStream_t s, int kind) {
   const int K = a.sc.K;
   const int threads = K / 8;
-  const size_t sm = ax_smem_bytes<T>(K, a.sc.nk, kind != AX_FWD);
+  size_t sm = ax_smem_bytes<T>(K, a.sc.nk, kind != AX_FWD);
+  AxArgs<T> b = a;
+  b.past_offset = unsigned(sm);
+  if (kind != AX_FWD) sm += size_t(a.sc.past) * sizeof(cpair<T>);
   void (*kern)(AxArgs<T>);
   if (kind == AX_ADJ) kern = k_ax_adj<T, J, LOGK, C16>;
   else if (kind == AX_FWD) kern = k_ax_fwd<T, J, LOGK, C16>;
@@ -735,7 +964,7 @@ static cudaError_t launch_ax_JKC(const AxArgs<T>& a, int npairs, cudaStream_t s,
   at[0].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = at;
   cfg.numAttrs = 1;
-  return cudaLaunchKernelEx(&cfg, kern, a);
+  return cudaLaunchKernelEx(&cfg, kern, b);
 }
 
 // the plan's radix choice (a.radix16) where both forms exist
