@@ -32,16 +32,23 @@ struct StoltConst {
   int past;       // then: bins a column's windows may reach past one period of K
 };
 
-// Stolt position and spectral phase of one (|q|, k_j) sample (mfl == INT_MIN:
-// evanescent).  Tabulated per plan when the table is small (B-scans).
-template <typename T> struct StoltEntry;
-template <> struct alignas(16) StoltEntry<float> { int mfl; float frac; float2 ph; };
-template <> struct alignas(16) StoltEntry<double> { int mfl; int pad; double frac; double2 ph; };
+// Stolt positions and spectral phases of one |q| class, tabulated per plan when
+// the table is small (B-scans) or at most one image.  The axial kernels' threads
+// take four consecutive samples each (a quad), so a class is kept as planes of
+// one 16-byte vector per quad, and a warp's load of a plane is contiguous: plane
+// 0 the floors (int4; INT_MIN: evanescent), then the fractions and the phases.
+// FP32: [floors][fractions][phases 0, 1][phases 2, 3], 16 B a sample; FP64:
+// [floors][2 x fractions][4 x phases] and one unused plane, 32 B a sample.
+template <typename T> struct StoltTable {
+  static constexpr int planes = sizeof(T) == 4 ? 4 : 8;        // of nk / 4 vectors each
+  static constexpr size_t sample_bytes = 4 * planes;
+};
 
 template <typename T> struct Tables {
   T* scale = nullptr;        // [nz]  s(n - nz/2) / sqrt(nz)
   cplx<T>* disp = nullptr;   // [nk]  e^{j phi(k_j)}
-  StoltEntry<T>* stab = nullptr;  // [(ny/2+1)(nx/2+1)][nk] or null (computed on the fly)
+  int4* stab = nullptr;      // [(ny/2+1)(nx/2+1)][planes][nk/4] (StoltTable) or null
+                             // (computed on the fly)
   cplx<T>* filt = nullptr;   // [(ny/2+1)(nx/2+1)][nk] filter B of Eq. 3, or null (B = 1);
                              // folded into stab's phases when stab exists
 };
@@ -135,8 +142,8 @@ template <typename T> cudaError_t launch_ax_adj(const AxArgs<T>& a, int npairs, 
 template <typename T> cudaError_t launch_ax_fused(const AxArgs<T>& a, int npairs, cudaStream_t s);
 template <typename T> size_t ax_smem_bytes(int K, int nk, bool adj);
 
-// Stolt table: entry [(|my| (nx/2+1) + |mx|) nk + j] for every |q| class
-template <typename T> cudaError_t launch_stolt_table(const AxArgs<T>& a, StoltEntry<T>* out,
+// Stolt table: class |my| (nx/2+1) + |mx| of every |q|
+template <typename T> cudaError_t launch_stolt_table(const AxArgs<T>& a, int4* out,
                                                      cudaStream_t s);
 
 // FP64 exact min-max coefficients at offsets f[0..n) (device), out[i*J + l]

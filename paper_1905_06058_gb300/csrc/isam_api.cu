@@ -279,10 +279,10 @@ template <typename T> isam_status phase_tables(isam_plan* P, Impl<T>& im) {
     CUDA_TRY(cudaMemcpy(im.tab.disp, h.data(), sizeof(cplx<T>) * P->nk, cudaMemcpyHostToDevice));
   }
   {
-    const size_t bytes = rows * P->nk * sizeof(StoltEntry<T>);
+    const size_t bytes = rows * P->nk * StoltTable<T>::sample_bytes;
     const size_t cap = std::max(kStoltTableMaxBytes, P->n_img * sizeof(cplx<T>));
     if (bytes <= cap && !(p.flags & ISAM_FLAG_NO_STOLT_TABLE)) {
-      if (!im.tab.stab) ISAM_TRY(dalloc(&im.tab.stab, rows * P->nk));
+      if (!im.tab.stab) ISAM_TRY(dalloc(&im.tab.stab, bytes / sizeof(int4)));
       AxArgs<T> a{};
       a.sc = P->sc;
       a.tab = im.tab;

@@ -4,7 +4,7 @@
 
 namespace isam {
 
-template cudaError_t launch_stolt_table<float>(const AxArgs<float>&, StoltEntry<float>*, cudaStream_t);
+template cudaError_t launch_stolt_table<float>(const AxArgs<float>&, int4*, cudaStream_t);
 template size_t ax_smem_bytes<float>(int, int, bool);
 template cudaError_t launch_ax_fwd<float>(const AxArgs<float>&, int, cudaStream_t);
 template cudaError_t launch_ax_adj<float>(const AxArgs<float>&, int, cudaStream_t);

@@ -128,70 +128,76 @@ template <typename T> struct Sample {
                   // (evanescent, or past nk)
 };
 
-// the position half of a table entry
-__device__ __forceinline__ void stolt_position(const StoltEntry<float>* e, int& mfl, float& frac) {
-  const int2 v = __ldg(reinterpret_cast<const int2*>(e));
-  mfl = v.x;
-  frac = __int_as_float(v.y);
+// Two complex numbers next to each other in memory, one 16-byte (32-byte) load
+// or store; p is a multiple of that.
+template <typename T> __device__ __forceinline__ cpair<T> load_two(const cplx<T>* p) {
+  return *reinterpret_cast<const cpair<T>*>(p);
 }
-__device__ __forceinline__ void stolt_position(const StoltEntry<double>* e, int& mfl,
-                                               double& frac) {
-  mfl = e->mfl;
-  frac = e->frac;
+template <typename T> __device__ __forceinline__ void store_two(cplx<T>* p, cplx<T> a, cplx<T> b) {
+  *reinterpret_cast<cpair<T>*>(p) = {a, b};
 }
 
-// Stolt position and spectral phase of sample j of one column pair, from the
-// plan's table when present, else evaluated (float-float / double).
+// Stolt positions and spectral phases of a quad of samples 4 q .. 4 q + 3 of one
+// column pair, from the plan's table when present, else evaluated (float-float /
+// double).
 template <typename T> struct Positions {
   StoltPos<T> sp;
-  const StoltEntry<T>* row;
+  const int4* row;           // the class's planes, nq vectors each
   const cplx<T>* frow;       // filter B of this column's |q| class (evaluated path)
+  int nq;
   __device__ Positions(const AxArgs<T>& A, int mx, int my) : sp(A.sc, mx, my) {
-    const size_t cls = size_t(stolt_class(A.sc, mx, my)) * A.sc.nk;
-    row = A.tab.stab ? A.tab.stab + cls : nullptr;
-    frow = A.tab.filt ? A.tab.filt + cls : nullptr;
+    const size_t cls = size_t(stolt_class(A.sc, mx, my));
+    nq = A.sc.nk / NRES;
+    row = A.tab.stab ? A.tab.stab + cls * (size_t(StoltTable<T>::planes) * nq) : nullptr;
+    frow = A.tab.filt ? A.tab.filt + cls * A.sc.nk : nullptr;
   }
-  // floor and fraction of samples j0 .. j0 + NRES - 1 (mfl INT_MIN: evanescent
-  // or past nk), and their phases one by one: a thread's positions and phases
-  // are used apart, and the table's two halves read apart keep registers free
-  __device__ __forceinline__ void quad(const AxArgs<T>& A, int j0, Sample<T>* sm) const {
+  // floors and fractions of the quad; an evaluated position also leaves its focus
+  // turn in val.a.x, for phases()
+  __device__ __forceinline__ void quad(const AxArgs<T>& A, int q, Sample<T>* sm) const {
+    if (row) {
+      const int4 m = __ldg(row + q);
+      sm[0].mfl = m.x; sm[1].mfl = m.y; sm[2].mfl = m.z; sm[3].mfl = m.w;
+      if constexpr (sizeof(T) == 4) {
+        const float4 f = __ldg(reinterpret_cast<const float4*>(row + nq + q));
+        sm[0].frac = f.x; sm[1].frac = f.y; sm[2].frac = f.z; sm[3].frac = f.w;
+      } else {
+        const double2 f0 = __ldg(reinterpret_cast<const double2*>(row + nq + q));
+        const double2 f1 = __ldg(reinterpret_cast<const double2*>(row + 2 * nq + q));
+        sm[0].frac = f0.x; sm[1].frac = f0.y; sm[2].frac = f1.x; sm[3].frac = f1.y;
+      }
+      return;
+    }
 #pragma unroll
     for (int rho = 0; rho < NRES; ++rho) {
-      const int j = j0 + rho;
-      sm[rho].mfl = INT_MIN;
-      if (j >= A.sc.nk) continue;
-      if (row) {
-        stolt_position(row + j, sm[rho].mfl, sm[rho].frac);
-      } else {
-        T turn;
-        if (!sp.at(A.sc, j, sm[rho].mfl, sm[rho].frac, turn)) sm[rho].mfl = INT_MIN;
-      }
+      sm[rho].frac = T(0);
+      if (!sp.at(A.sc, NRES * q + rho, sm[rho].mfl, sm[rho].frac, sm[rho].val.a.x))
+        sm[rho].mfl = INT_MIN;
     }
   }
-  __device__ __forceinline__ cplx<T> phase(const AxArgs<T>& A, int j, bool prop) const {
-    if (row) return row[j].ph;
-    if (!prop) return mk<T>(0, 0);
-    int mfl;
-    T frac, turn;
-    sp.at(A.sc, j, mfl, frac, turn);
-    cplx<T> ph = spectral_phase<T>(A.sc, A.tab.disp, j, turn);
+  // phases of samples 2 h and 2 h + 1 of the quad (0 where evanescent)
+  __device__ __forceinline__ cpair<T> phases(const AxArgs<T>& A, int q, int h,
+                                             const Sample<T>* sm) const {
+    cpair<T> p;
+    if (row) {
+      if constexpr (sizeof(T) == 4) {
+        const float4 v = __ldg(reinterpret_cast<const float4*>(row + (2 + h) * nq + q));
+        p.a = make_float2(v.x, v.y);
+        p.b = make_float2(v.z, v.w);
+      } else {
+        p.a = __ldg(reinterpret_cast<const double2*>(row + (3 + 2 * h) * nq + q));
+        p.b = __ldg(reinterpret_cast<const double2*>(row + (4 + 2 * h) * nq + q));
+      }
+      return p;
+    }
+    p.a = evaluated(A, NRES * q + 2 * h, sm[2 * h]);
+    p.b = evaluated(A, NRES * q + 2 * h + 1, sm[2 * h + 1]);
+    return p;
+  }
+  __device__ __forceinline__ cplx<T> evaluated(const AxArgs<T>& A, int j, const Sample<T>& s) const {
+    if (s.mfl == INT_MIN) return mk<T>(0, 0);
+    cplx<T> ph = spectral_phase<T>(A.sc, A.tab.disp, j, s.val.a.x);
     if (frow) ph = cmul(ph, __ldg(frow + j));
     return ph;
-  }
-  __device__ __forceinline__ bool at(const AxArgs<T>& A, int j, int& mfl, T& frac,
-                                     cplx<T>& ph) const {
-    if (row) {
-      const StoltEntry<T> e = row[j];
-      mfl = e.mfl;
-      frac = e.frac;
-      ph = e.ph;
-      return e.mfl != INT_MIN;
-    }
-    T turn;
-    if (!sp.at(A.sc, j, mfl, frac, turn)) return false;
-    ph = spectral_phase<T>(A.sc, A.tab.disp, j, turn);
-    if (frow) ph = cmul(ph, __ldg(frow + j));
-    return true;
   }
 };
 
@@ -745,7 +751,7 @@ template <typename T> __host__ __device__ constexpr int ax_min_blocks() {
 }
 
 template <typename T, int J, int LOGK, bool C16>
-__global__ void __launch_bounds__(512) k_ax_fwd(const __grid_constant__ AxArgs<T> A) {
+__global__ void __launch_bounds__(512, ax_min_blocks<T>()) k_ax_fwd(const __grid_constant__ AxArgs<T> A) {
   using C = cplx<T>;
   using V = cpair<T>;
   extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -765,21 +771,24 @@ __global__ void __launch_bounds__(512) k_ax_fwd(const __grid_constant__ AxArgs<T
   const Positions<T> pos(A, mx, my);
   C* o1 = A.out + size_t(c1) * nk;
   C* o2 = A.out + size_t(c2) * nk;
-  for (int j = threadIdx.x; j < nk; j += axial_threads<LOGK>()) {
-    int mfl;
-    T frac;
-    C ph;
-    C a1 = mk<T>(0, 0), a2 = mk<T>(0, 0);
-    if (pos.at(A, j, mfl, frac, ph)) {
-      T c[J];
-      coefficients<T, J>(A.poly, frac, c);
-      interp_pair<T, J>(Y, K, mfl, c, a1, a2);
-      a1 = cmul(a1, ph);
-      a2 = cmul(a2, ph);
+  // nk <= K/2 = NRES blockDim: a quad of samples per thread
+  const int q = threadIdx.x;
+  if (NRES * q >= nk) return;
+  Sample<T> sm[NRES];
+  pos.quad(A, q, sm);
+  cpair<T> ph;
+  C a1, a2;
+  interp_quad<T, J>(A, Y, K, sm, [&](int rho, C s1, C s2) {
+    if (rho % 2 == 0) {
+      ph = pos.phases(A, q, rho / 2, sm);
+      a1 = cmul(s1, ph.a);
+      a2 = cmul(s2, ph.a);
+      return;
     }
-    o1[j] = a1;
-    if (two) o2[j] = a2;
-  }
+    const int j = NRES * q + rho - 1;
+    store_two<T>(o1 + j, a1, cmul(s1, ph.b));
+    if (two) store_two<T>(o2 + j, a2, cmul(s2, ph.b));
+  });
 }
 
 template <typename T, int J, int LOGK, bool C16>
@@ -807,17 +816,16 @@ __global__ void __launch_bounds__(512, ax_min_blocks<T>()) k_ax_adj(const __grid
   const C* r2 = A.in + size_t(c2) * nk;
   Sample<T> sm[NRES];
 #pragma unroll
-  for (int rho = 0; rho < NRES; ++rho) {
-    const int j = NRES * tid + rho;
-    sm[rho].mfl = INT_MIN;
-    int mfl;
-    T frac;
-    C ph;
-    if (j < nk && pos.at(A, j, mfl, frac, ph)) {
-      sm[rho].val.a = cmulc(r1[j], ph);
-      sm[rho].val.b = two ? cmulc(r2[j], ph) : mk<T>(0, 0);
-      sm[rho].frac = frac;
-      sm[rho].mfl = mfl;
+  for (int rho = 0; rho < NRES; ++rho) sm[rho].mfl = INT_MIN;
+  if (NRES * tid < nk) {
+    pos.quad(A, tid, sm);
+#pragma unroll
+    for (int h = 0; h < NRES / 2; ++h) {
+      const int j = NRES * tid + 2 * h;
+      const V ph = pos.phases(A, tid, h, sm);
+      const V x = load_two<T>(r1 + j), y = two ? load_two<T>(r2 + j) : V{};
+      sm[2 * h].val = {cmulc(x.a, ph.a), cmulc(y.a, ph.a)};
+      sm[2 * h + 1].val = {cmulc(x.b, ph.b), cmulc(y.b, ph.b)};
     }
   }
   scatter<T, J>(A, Y, K, nt, nk, sm, &ch_lo, &ch_hi, &ch_tail, heads);
@@ -849,7 +857,6 @@ __global__ void __launch_bounds__(512, ax_min_blocks<T>()) k_ax_fused(const __gr
   pair_columns(A, c1, c2, mx, my);
   const bool two = c2 != c1;
   if (tid == 0) { ch_lo = INT_MAX; ch_hi = INT_MIN; }
-  constexpr bool COL16 = ax_col16<T, LOGK, C16>();
   // Programmatic dependent launch: the next kernel in the stream may start its
   // own prologue on SMs this grid leaves idle; this grid builds its twiddles,
   // then waits for the previous kernel before touching global data.
@@ -860,35 +867,36 @@ __global__ void __launch_bounds__(512, ax_min_blocks<T>()) k_ax_fused(const __gr
   // wait): loaded here, tested after the forward transform (before the first
   // global write), so its latency overlaps the transform
   const bool stopped = A.stop != nullptr && __ldcg(A.stop) != 0;
-  // F s_d at this pair's samples, fetched before the transforms need them (the
-  // column-split transforms take them after the forward transform: their
-  // registers are needed there)
   const C* d1 = A.sdh + size_t(c1) * nk;
-  C dqv[NRES];
-  if constexpr (!COL16) {
-#pragma unroll
-    for (int rho = 0; rho < NRES; ++rho) {
-      const int j = NRES * tid + rho;
-      dqv[rho] = j < nk ? d1[j] : mk<T>(0, 0);
-    }
-  }
   ax_forward<T, LOGK, C16>(A, Y, tw, c1, c2, two);
   if (stopped) return;   // an earlier check stopped the solve: write nothing
   const Positions<T> pos(A, mx, my);
   Sample<T> sm[NRES];
-  pos.quad(A, NRES * tid, sm);
+#pragma unroll
+  for (int rho = 0; rho < NRES; ++rho) sm[rho].mfl = INT_MIN;
   if (NRES * tid < nk) {
+    pos.quad(A, tid, sm);
+    V php, dq, w1, w2;                   // of two samples: phases, F s_d, model spectra
     interp_quad<T, J>(A, Y, K, sm, [&](int rho, C s1, C s2) {
       const int j = NRES * tid + rho;
-      const C ph = pos.phase(A, j, sm[rho].mfl != INT_MIN);
+      if (rho % 2 == 0) {
+        php = pos.phases(A, tid, rho / 2, sm);
+        dq = load_two<T>(d1 + j);
+      }
+      const C ph = rho % 2 == 0 ? php.a : php.b;
       s1 = cmul(s1, ph);
       s2 = two ? cmul(s2, ph) : s1;
       if (WS) {
-        A.s_out[size_t(c1) * nk + j] = s1;
-        if (two) A.s_out[size_t(c2) * nk + j] = s2;
+        if (rho % 2 == 0) {
+          w1.a = s1;
+          w2.a = s2;
+        } else {
+          store_two<T>(A.s_out + size_t(c1) * nk + j - 1, w1.a, s1);
+          if (two) store_two<T>(A.s_out + size_t(c2) * nk + j - 1, w2.a, s2);
+        }
       }
       // R(-q) = conj R(q): the residual is real
-      const C R = csub(cscale(cadd(s1, cconj(s2)), T(0.5)), COL16 ? d1[j] : dqv[rho]);
+      const C R = csub(cscale(cadd(s1, cconj(s2)), T(0.5)), rho % 2 == 0 ? dq.a : dq.b);
       sm[rho].val.a = cmulc(R, ph);
       sm[rho].val.b = two ? cmulc(cconj(R), ph) : mk<T>(0, 0);
     });
@@ -897,35 +905,44 @@ __global__ void __launch_bounds__(512, ax_min_blocks<T>()) k_ax_fused(const __gr
   ax_inverse<T, LOGK, C16>(A, Y, tw, c1, c2, two);
 }
 
-// One thread per (|q| class, k_j): the same evaluation the kernels do on the fly.
+// One thread per (|q| class, quad): the same evaluation the kernels do on the fly.
 template <typename T>
-__global__ void k_stolt_table(const __grid_constant__ AxArgs<T> A, StoltEntry<T>* out) {
-  const int j = blockIdx.x * blockDim.x + threadIdx.x;
+__global__ void k_stolt_table(const __grid_constant__ AxArgs<T> A, int4* out) {
+  const int q = blockIdx.x * blockDim.x + threadIdx.x;
   const int cls = blockIdx.y;
-  if (j >= A.sc.nk) return;
+  const int nq = A.sc.nk / NRES;
+  if (q >= nq) return;
   const int ncx = A.sc.nx / 2 + 1;
   const int mx = cls % ncx, my = cls / ncx;
-  const StoltPos<T> sp(A.sc, mx, my);
-  StoltEntry<T> e{};
-  T turn;
-  if (sp.at(A.sc, j, e.mfl, e.frac, turn)) {
-    e.ph = spectral_phase<T>(A.sc, A.tab.disp, j, turn);
-    if (A.tab.filt) e.ph = cmul(e.ph, A.tab.filt[size_t(cls) * A.sc.nk + j]);
+  const Positions<T> pos(A, mx, my);
+  Sample<T> sm[NRES];
+  pos.quad(A, q, sm);
+  const cpair<T> p0 = pos.phases(A, q, 0, sm), p1 = pos.phases(A, q, 1, sm);
+  int4* row = out + size_t(cls) * (size_t(StoltTable<T>::planes) * nq) + q;
+  row[0] = make_int4(sm[0].mfl, sm[1].mfl, sm[2].mfl, sm[3].mfl);
+  if constexpr (sizeof(T) == 4) {
+    float4* f = reinterpret_cast<float4*>(row);
+    f[nq] = make_float4(sm[0].frac, sm[1].frac, sm[2].frac, sm[3].frac);
+    f[2 * nq] = make_float4(p0.a.x, p0.a.y, p0.b.x, p0.b.y);
+    f[3 * nq] = make_float4(p1.a.x, p1.a.y, p1.b.x, p1.b.y);
   } else {
-    e.mfl = INT_MIN;
-    e.frac = T(0);
-    e.ph = mk<T>(0, 0);
+    double2* f = reinterpret_cast<double2*>(row);
+    f[nq] = make_double2(sm[0].frac, sm[1].frac);
+    f[2 * nq] = make_double2(sm[2].frac, sm[3].frac);
+    f[3 * nq] = p0.a;
+    f[4 * nq] = p0.b;
+    f[5 * nq] = p1.a;
+    f[6 * nq] = p1.b;
   }
-  out[size_t(cls) * A.sc.nk + j] = e;
 }
 
-template <typename T> cudaError_t launch_stolt_table(const AxArgs<T>& a, StoltEntry<T>* out,
+template <typename T> cudaError_t launch_stolt_table(const AxArgs<T>& a, int4* out,
                                                      cudaStream_t s) {
   const int rows = (a.sc.ny / 2 + 1) * (a.sc.nx / 2 + 1);
-  dim3 grid((a.sc.nk + 255) / 256, rows);
+  dim3 grid((a.sc.nk / NRES + 127) / 128, rows);
   AxArgs<T> b = a;
   b.tab.stab = nullptr;
-  k_stolt_table<T><<<grid, 256, 0, s>>>(b, out);
+  k_stolt_table<T><<<grid, 128, 0, s>>>(b, out);
   return cudaGetLastError();
 }
 
