@@ -340,8 +340,10 @@ void isam_batch_destroy(isam_batch* batch);
  *                  transforms at K = 2048 and 4096 (three shared-memory passes);
  *                  8: radix-8 passes on column pairs (four); other plans run
  *                  radix 8 whatever the value
- *   lateral_radix  the same choice for the FP32 lateral tiles of L = 1024 (4
- *                  pairs) and L = 256 (8 pairs) */
+ *   lateral_radix  16: FP32 lateral passes of lengths 64 to 1024 (2^p, 3 * 2^p
+ *                  from 192) at the built-in tile keep it in registers; 8: radix-8
+ *                  passes on column pairs in shared memory; other plans and
+ *                  tiles run the latter whatever the value */
 typedef struct {
   int32_t lateral_tile;
   int32_t stolt_table;

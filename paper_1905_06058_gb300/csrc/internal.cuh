@@ -100,8 +100,8 @@ template <typename T> struct LatArgs {
   cplx<T>* uout;         // optional: u^k = eta^k - g^k before the threshold
   const double* lam_dev; // optional: lambda / L = lam_scale * (*lam_dev), read on the device
   double lam_scale;
-  // FP32 compile-time tiles at L = 1024 and 256: 1 runs the column-split
-  // radix-16 transforms, 0 the radix-8 column-pair ones; ignored elsewhere
+  // FP32 tiles that have a register form (lat_reg_takes): 1 runs it, 0 the
+  // radix-8 column-pair transforms in shared memory; ignored elsewhere
   int radix16;
   // solve with the device-side stop rule (see StopRule): a nonzero *stop, read
   // after the wait for the previous kernel, makes the launch return at once;
@@ -137,6 +137,10 @@ template <typename T> struct AxArgs {
 
 // launchers (return cudaGetLastError())
 template <typename T> cudaError_t launch_lat(int mode, const LatArgs<T>& a, cudaStream_t s);
+// the FP32 passes with the tile in registers, for lengths L at TZ pair-columns
+// that lat_reg_takes
+bool lat_reg_takes(int L, int TZ);
+cudaError_t launch_lat_reg(int mode, const LatArgs<float>& a, cudaStream_t s);
 template <typename T> cudaError_t launch_ax_fwd(const AxArgs<T>& a, int npairs, cudaStream_t s);
 template <typename T> cudaError_t launch_ax_adj(const AxArgs<T>& a, int npairs, cudaStream_t s);
 template <typename T> cudaError_t launch_ax_fused(const AxArgs<T>& a, int npairs, cudaStream_t s);

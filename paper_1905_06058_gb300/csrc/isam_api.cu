@@ -81,8 +81,8 @@ struct isam_plan {
   int tune_tp = 0;
   int tune_table = 0;
   // FFT radix of the FP32 axial transforms at K = 2048 / 4096 and of the
-  // compile-time lateral tiles at L = 1024 / 256: 16 (column-split radix-16
-  // passes, the default) or 8 (radix-8 column-pair passes)
+  // lateral tiles with a register form: 16 (column-split radix-16 passes, tiles
+  // in registers, the default) or 8 (radix-8 column-pair passes)
   int tune_radix_ax = 16;
   int tune_radix_lat = 16;
   int batch_refs = 0;           // batches whose graph records this plan's kernels
@@ -1990,8 +1990,8 @@ template <typename T> isam_status autotune_impl(isam_plan* P, isam_tuning* out) 
   update_geometry(P, &L, &M);
   const int threads_per_tp = L >= 8 ? L / 8 : 1;
   const bool fp32 = P->p.precision == ISAM_FP32;
-  // radix-16 forms exist for FP32 axial transforms at K = 2048, 4096 and FP32
-  // lateral tiles (L, tile) = (1024, 4) and (256, 8) of lengths 2^p
+  // both radices exist for FP32 axial transforms at K = 2048, 4096 and the FP32
+  // lateral tiles with a register form
   const bool ax_both = fp32 && (P->K == 2048 || P->K == 4096);
   const bool prof = P->prof;
   P->prof = false;
@@ -2005,7 +2005,7 @@ template <typename T> isam_status autotune_impl(isam_plan* P, isam_tuning* out) 
   for (int it = 0; it < ntab && st == ISAM_OK; ++it) {
     for (int tp = 1; tp <= 8 && st == ISAM_OK; tp *= 2) {
       if (tp > M / 2 || threads_per_tp * tp > 512) continue;
-      const bool lat_both = fp32 && ((L == 1024 && tp == 4) || (L == 256 && tp == 8));
+      const bool lat_both = fp32 && lat_reg_takes(L, tp);
       for (int ra = ax_both ? 8 : 16; ra <= 16 && st == ISAM_OK; ra += 8) {
         for (int rl = lat_both ? 8 : 16; rl <= 16 && st == ISAM_OK; rl += 8) {
           Tuning t;

@@ -17,9 +17,9 @@
 
 #include <type_traits>
 
-#include "fft_col16.cuh"
 #include "fft_smem.cuh"
 #include "internal.cuh"
+#include "lat_point.cuh"
 
 namespace isam {
 
@@ -45,35 +45,6 @@ bool fft_length(int L, int* log2, int* r3) {
   return true;
 }
 
-// T_tau(u) = u max(|u| - tau, 0) / (max(|u| - tau, 0) + tau)  (Eq. 14),
-// evaluated as u max(1 - tau / |u|, 0); 0 where |u| = 0.
-__device__ __forceinline__ float2 soft_threshold(float2 u, float tau) {
-  const float m2 = fmaf(u.x, u.x, u.y * u.y);
-  const float f = m2 > 0.0f ? fmaxf(1.0f - tau * rsqrtf(m2), 0.0f) : 0.0f;
-  return cscale(u, f);
-}
-__device__ __forceinline__ double2 soft_threshold(double2 u, double tau) {
-  const double m2 = fma(u.x, u.x, u.y * u.y);
-  const double f = m2 > 0.0 ? fmax(1.0 - tau / sqrt(m2), 0.0) : 0.0;
-  return cscale(u, f);
-}
-
-// Sum of v over the threads of one warp that exist: a block of nt threads
-// (any count, e.g. 8, 24 or 48 for short or 3 * 2^p lateral lengths) has a
-// last warp of n = nt - 32 w lanes, and a shuffle may only name lanes that
-// exist, so the mask holds lanes [0, n) and a lane adds a partner's value only
-// when that partner exists.  The sum lands in lane 0.
-__device__ __forceinline__ double warp_sum_lanes(double v, int n) {
-  const unsigned mask = n >= 32 ? 0xffffffffu : ((1u << n) - 1u);
-  const int lane = threadIdx.x & 31;
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) {
-    const double t = __shfl_down_sync(mask, v, o);
-    if (lane + o < n) v += t;
-  }
-  return v;
-}
-
 template <typename T> struct rpair_t;
 template <> struct rpair_t<float> { using type = float2; };
 template <> struct rpair_t<double> { using type = double2; };
@@ -81,7 +52,7 @@ template <> struct rpair_t<double> { using type = double2; };
 // LOGL > 0: the transforms are the compile-time-length ones for L = 2^LOGL at
 // the stride 2^LOGTP = TP (no radix-3 pass), with constant row offsets;
 // LOGL = 0: runtime-length transforms.  The tile indexing is the same.
-template <typename T, int MODE, int LOGL, int LOGTP, bool C16>
+template <typename T, int MODE, int LOGL, int LOGTP>
 __global__ void __launch_bounds__(512, 2) k_lat(const __grid_constant__ LatArgs<T> a) {
   using C = cplx<T>;
   using V = cpair<T>;
@@ -92,14 +63,10 @@ __global__ void __launch_bounds__(512, 2) k_lat(const __grid_constant__ LatArgs<
   constexpr bool CT = LOGL > 0;
   const int TP = a.TZ, L = CT ? (1 << LOGL) : a.L, logTP = a.logTZ;
   cplx<T>* tw = reinterpret_cast<cplx<T>*>(buf + size_t(padded_rows(L)) * TP);
-  // FP32 at L = 1024 and 256: column-split radix-16 transforms (fft_col16.cuh)
-  // when the plan chose them (C16)
-  constexpr bool COL16 = C16 && CT && std::is_same<T, float>::value && (LOGL == 10 || LOGL == 8);
   // programmatic dependent launch: let the next kernel start its prologue,
   // build the twiddles, then wait for the previous kernel's results
   cudaTriggerProgrammaticLaunchCompletion();
-  if constexpr (COL16) c16::build_lat_twiddles<LOGL>(reinterpret_cast<float4*>(tw));
-  else build_twiddles<T>(tw, L, CT ? LOGL : a.logL, CT ? 0 : a.r3);
+  build_twiddles<T>(tw, L, CT ? LOGL : a.logL, CT ? 0 : a.r3);
   cudaGridDependencySynchronize();
   // the solve's stop flag (written by an earlier kernel, so visible after the
   // wait): loaded here, tested before the first global write (after the first
@@ -118,10 +85,7 @@ __global__ void __launch_bounds__(512, 2) k_lat(const __grid_constant__ LatArgs<
   auto sidx = [&](int e) { return prow(e >> logTP) * TP + (e & (TP - 1)); };
   auto lat_fft = [&](auto sign) {
     constexpr int SIGN = decltype(sign)::value;
-    if constexpr (COL16)
-      c16::lat_transform<SIGN, LOGL, 2 * (1 << LOGTP)>(reinterpret_cast<float2*>(buf),
-                                                        reinterpret_cast<const float4*>(tw));
-    else if constexpr (CT) fft_cols_ct<SIGN, false, LOGL, (1 << LOGTP), T>(buf, col, b, tw);
+    if constexpr (CT) fft_cols_ct<SIGN, false, LOGL, (1 << LOGTP), T>(buf, col, b, tw);
     else fft_smem<SIGN, false, T>(buf, TP, col, b, L, a.logL, tw, true, a.r3);
   };
   using FWD = std::integral_constant<int, -1>;
@@ -355,11 +319,11 @@ template <typename T> size_t lat_smem_bytes(int L, int TP) {
          size_t(twiddle_entries(L, lg, r3)) * sizeof(cplx<T>);
 }
 
-template <typename T, int MODE, int LOGL, int LOGTP, bool C16 = false>
+template <typename T, int MODE, int LOGL, int LOGTP>
 static cudaError_t launch_lat_tile(const LatArgs<T>& a, cudaStream_t s) {
   const int threads = (a.L >= 8 ? a.L / 8 : 1) * a.TZ;
   const size_t sm = lat_smem_bytes<T>(a.L, a.TZ);
-  auto* kern = k_lat<T, MODE, LOGL, LOGTP, C16>;
+  auto* kern = k_lat<T, MODE, LOGL, LOGTP>;
   cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, int(sm));
   dim3 grid(a.M / (2 * a.TZ), a.B);
   cudaLaunchConfig_t cfg = {};
@@ -375,24 +339,22 @@ static cudaError_t launch_lat_tile(const LatArgs<T>& a, cudaStream_t s) {
   return cudaLaunchKernelEx(&cfg, kern, a);
 }
 
-// The FP32 solve passes at the tiles of the 1024-wide B-scans (L = 1024, 4
-// pair-columns), the 512-wide ones and the 256 x 256 volumes (L = 512 or 256, 8
-// pair-columns) run compile-time-length transforms, at L = 1024 and 256 in the
-// column-split radix-16 form when the plan chose it (a.radix16); every other
-// case the runtime-length ones.
+// FP32 passes at the built-in tile of the lengths that have a register form take
+// it (k_lateral_reg.cu) unless the plan chose radix 8 (a.radix16 = 0).  That form
+// of the solve's passes runs compile-time-length transforms at (L, pair-columns) =
+// (1024, 4), (512, 8) and (256, 8); every other case the runtime-length ones.
 template <typename T, int MODE>
 static cudaError_t launch_lat_mode(const LatArgs<T>& a, cudaStream_t s) {
   constexpr bool hot = std::is_same<T, float>::value &&
                        (MODE == LAT_UPDATE || MODE == LAT_UPDATE_U || MODE == LAT_C2C_FWD ||
                         MODE == LAT_C2C_INV);
+  if constexpr (std::is_same<T, float>::value) {
+    if (a.radix16 && lat_reg_takes(a.L, a.TZ)) return launch_lat_reg(MODE, a, s);
+  }
   if constexpr (hot) {
-    if (!a.r3 && a.L == 1024 && a.TZ == 4)
-      return a.radix16 ? launch_lat_tile<T, MODE, 10, 2, true>(a, s)
-                       : launch_lat_tile<T, MODE, 10, 2>(a, s);
+    if (!a.r3 && a.L == 1024 && a.TZ == 4) return launch_lat_tile<T, MODE, 10, 2>(a, s);
     if (!a.r3 && a.L == 512 && a.TZ == 8) return launch_lat_tile<T, MODE, 9, 3>(a, s);
-    if (!a.r3 && a.L == 256 && a.TZ == 8)
-      return a.radix16 ? launch_lat_tile<T, MODE, 8, 3, true>(a, s)
-                       : launch_lat_tile<T, MODE, 8, 3>(a, s);
+    if (!a.r3 && a.L == 256 && a.TZ == 8) return launch_lat_tile<T, MODE, 8, 3>(a, s);
   }
   return launch_lat_tile<T, MODE, 0, 0>(a, s);
 }

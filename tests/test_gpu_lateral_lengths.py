@@ -1,0 +1,75 @@
+"""The FP32 lateral passes that keep their tile in registers, at every length
+they take (64 to 1024, 2^p and 3 * 2^p), along x and along y of a volume.
+
+A and A^H go through the complex, real-input and real-output passes and are
+compared with the oracle (1e-5 relative L2, the bar of test_gpu_operator.py).
+The passes of the solve (update from u_hat with depth weights, update with the
+norm partials of the stop rule, gradient step and extrapolation of the other
+priors) are compared with the radix-8 shared-memory form of the same plan, which
+is the same arithmetic in another order: 1e-5 on the image as in
+test_gpu_autotune.py, and 1e-3 on r_r, the bar of test_gpu_stop_rule.py."""
+import numpy as np
+import pytest
+
+from oracle import isam_oracle as O
+from paper_1905_06058_gb300 import inputs as I
+
+pytestmark = pytest.mark.gpu
+
+LENGTHS = [64, 128, 192, 256, 384, 512, 768, 1024]
+
+
+@pytest.fixture(scope="module")
+def torch():
+    import torch as T
+    if not T.cuda.is_available():
+        pytest.skip("no CUDA device")
+    import __graft_entry__ as g
+    g.build()
+    return T
+
+
+def rel(a, b):
+    return float(np.linalg.norm(a - b) / np.linalg.norm(b))
+
+
+def shape(L, along_y):
+    # 16 depth samples: one tile of 16 columns or two of 8; y: 2 x 16 columns
+    return dict(nx=2, ny=L, nk=16, nz=16) if along_y else dict(nx=L, nk=16, nz=32)
+
+
+@pytest.mark.parametrize("along_y", [False, True], ids=["x", "y"])
+@pytest.mark.parametrize("L", LENGTHS)
+def test_operators(torch, L, along_y):
+    from paper_1905_06058_gb300.isam import Plan
+    g = I.small_bscan(seed=60, **shape(L, along_y)).geom
+    ref = O.IsamOracle(g, "nufft")
+    eta = I.random_image(ref.image_shape, 61).astype(np.complex64)
+    y = I.random_spectra(ref.spec_shape, 62).astype(np.float32)
+    plan = Plan(g)
+    a = plan.forward(torch.from_numpy(eta).cuda()).cpu().numpy()
+    b = plan.adjoint(torch.from_numpy(y).cuda()).cpu().numpy()
+    plan.close()
+    assert rel(a, ref.forward(eta.astype(np.complex128))) < 1e-5
+    assert rel(b, ref.adjoint(y.astype(np.float64))) < 1e-5
+
+
+@pytest.mark.parametrize("along_y", [False, True], ids=["x", "y"])
+@pytest.mark.parametrize("L", LENGTHS)
+def test_solve_passes_match_radix8(torch, L, along_y):
+    from paper_1905_06058_gb300.isam import Plan
+    g = I.small_bscan(seed=63, **shape(L, along_y)).geom
+    plan = Plan(g)
+    s = plan.forward(torch.from_numpy(I.random_image(plan.image_shape, 64).astype(np.complex64)).cuda())
+    w = torch.from_numpy(I.depth_weights(plan.image_shape[2]).astype(np.float32)).cuda()
+    kws = [dict(max_iter=6, w=w), dict(max_iter=6, w=w, tol=1e-300, check_every=3),
+           dict(max_iter=3, prior="haar_depth")]
+    for kw in kws:
+        got = []
+        for r in (16, 8):
+            plan.set_tuning(lateral_radix=r)
+            out, info = plan.solve(s, lambda_rel=0.02, L=4.0, **kw)
+            got.append((out.cpu().numpy(), info["rr"]))
+        assert rel(got[0][0], got[1][0]) < 1e-5
+        assert got[0][1] == pytest.approx(got[1][1], rel=1e-3)
+    plan.close()
