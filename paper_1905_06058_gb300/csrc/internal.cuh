@@ -221,6 +221,24 @@ template <typename T> cudaError_t launch_haar_prox(const cplx<T>* u, cplx<T>* z,
                                                    size_t n_ascans, T tau, const double* lam_dev,
                                                    double lam_scale, cudaStream_t s);
 
+// FP32 total-variation prox, up to TV_STEPS dual steps of every B-scan slice in one
+// launch (k_prior.cu): in -> out = (p_x, p_z, r_x, r_z), different images; in[2]
+// null: r = p.  z not null: the last launch, which forms z = u - tau grad^H p and
+// leaves r out.  tau as below.
+constexpr int TV_STEPS = 8;
+struct TvLaunch {
+  const float2* u;
+  const float2* in[4];
+  float2* out[4];
+  float2* z;
+  float tau;
+  const double* lam_dev;
+  double lam_scale;
+  int nx, ny, nz, steps;
+  float beta[TV_STEPS];
+};
+cudaError_t launch_tv_tile(const TvLaunch& l, cudaStream_t s);
+
 // total-variation prox pieces (k_prior.cu); tau = lam_scale * (*lam_dev) when lam_dev
 template <typename T> cudaError_t launch_tv_primal(const cplx<T>* u, const cplx<T>* rx,
                                                    const cplx<T>* rz, T tau, const double* lam_dev,

@@ -46,7 +46,10 @@ template <typename T> struct Impl {
   int seg_cap = 0;
   cplx<T>* cal = nullptr;       // [5][n_img]: zbar x 3, ubar, b
   cplx<T>* dc_post = nullptr;   // [nz] output phase of the Eq. 9 reconstruction
-  cplx<T>* tv = nullptr;        // [5][n_img]: TV dual p_x, p_z, momentum r_x, r_z, primal w
+  // [tv_images][n_img]; FP32: TV duals p (x, z) of two launches in turn and a
+  // momentum r; FP64: p_x, p_z, r_x, r_z and the primal w
+  cplx<T>* tv = nullptr;
+  int tv_cur = 0;               // FP32: which p the next prox starts from
   bool ready = false;
 };
 
@@ -478,6 +481,91 @@ template <typename T> isam_status power_iteration(isam_plan* P, int iters, doubl
 // ----------------------------------------------------------------------------
 // FISTA (Alg. 1)
 // ----------------------------------------------------------------------------
+// Images of the TV workspace.  FP32 launches read (p, r) and write the next ones,
+// so each exists twice; of the two r pairs one is lent by eta_hat and z^k, which
+// are free during the prox, and half of the other by the spectra when they are as
+// large as an image (nk = nz).
+template <typename T> int tv_images(const isam_plan* P) {
+  return sizeof(T) == 8 || P->n_spec == P->n_img ? 5 : 6;
+}
+
+// TV prox of u = im.grad into zout: the dual p carries over from the previous
+// iteration; r starts at p; fast gradient projection; z = u - tau grad^H p
+template <typename T> isam_status tv_prox(isam_plan* P, Impl<T>& im, cplx<T>* zout, double lam,
+                                          double L, const double* lam_dev, double lam_scale,
+                                          int iters) {
+  cudaStream_t s = P->stream;
+  if constexpr (sizeof(T) == 4) {
+    // five steps a launch: 20 in four launches of tiles whose inner 54 x 54 pixels
+    // are 71% of what they compute
+    constexpr int kSteps = 5;
+    static_assert(kSteps <= TV_STEPS, "TvLaunch holds the momentum of a launch");
+    const size_t n = P->n_img;
+    const int nl = (iters + kSteps - 1) / kSteps;
+    float2* p[2][2] = {{im.tv, im.tv + n}, {im.tv + 2 * n, im.tv + 3 * n}};
+    float2* lent[2] = {im.eta_hat, zout};
+    float2* kept[2] = {im.tv + 4 * n, P->n_spec == n ? im.spec : im.tv + 5 * n};
+    TvLaunch l{};
+    l.u = im.grad;
+    l.tau = float(lam / L); l.lam_dev = lam_dev; l.lam_scale = lam_scale;
+    l.nx = P->nx; l.ny = P->ny; l.nz = P->nz;
+    double t = 1.0;
+    float2** r_in = nullptr;
+    for (int i = 0; i < nl; ++i) {
+      // the last launch writes z^k, so the r it reads is not the lent pair
+      float2** r_out = (nl - i) % 2 ? lent : kept;
+      float2** p_in = p[im.tv_cur];
+      float2** p_out = p[im.tv_cur ^ 1];
+      im.tv_cur ^= 1;
+      const bool last = i == nl - 1;
+      for (int k = 0; k < 2; ++k) {
+        l.in[k] = p_in[k];
+        l.in[2 + k] = r_in ? r_in[k] : nullptr;
+        l.out[k] = p_out[k];
+        l.out[2 + k] = last ? nullptr : r_out[k];
+      }
+      l.z = last ? zout : nullptr;
+      l.steps = iters / nl + (i < iters % nl ? 1 : 0);
+      for (int k = 0; k < l.steps; ++k) {
+        const double t_next = 0.5 * (1.0 + sqrt(1.0 + 4.0 * t * t));
+        l.beta[k] = float((t - 1.0) / t_next);
+        t = t_next;
+      }
+      ISAM_TRY(launch(P, ISAM_KCLASS_MISC, [&] { return launch_tv_tile(l, s); }));
+      r_in = r_out;
+    }
+    return ISAM_OK;
+  } else {
+    const size_t n = P->n_img;
+    cplx<T>* px = im.tv;
+    cplx<T>* pz = im.tv + n;
+    cplx<T>* rx = im.tv + 2 * n;
+    cplx<T>* rz = im.tv + 3 * n;
+    cplx<T>* w = im.tv + 4 * n;
+    const T tau = T(lam / L);
+    CUDA_TRY(cudaMemcpyAsync(rx, px, 2 * n * sizeof(cplx<T>), cudaMemcpyDeviceToDevice, s));
+    double t = 1.0;
+    for (int i = 0; i < iters; ++i) {
+      const double t_next = 0.5 * (1.0 + sqrt(1.0 + 4.0 * t * t));
+      const T beta = T((t - 1.0) / t_next);
+      t = t_next;
+      ISAM_TRY(launch(P, ISAM_KCLASS_MISC, [&] {
+        return launch_tv_primal<T>(im.grad, rx, rz, tau, lam_dev, lam_scale, w, P->nx, P->nz, n,
+                                   s);
+      }));
+      ISAM_TRY(launch(P, ISAM_KCLASS_MISC, [&] {
+        return launch_tv_dual<T>(w, px, pz, rx, rz, tau, lam_dev, lam_scale, beta, P->nx, P->nz,
+                                 n, s);
+      }));
+    }
+    ISAM_TRY(launch(P, ISAM_KCLASS_MISC, [&] {
+      return launch_tv_primal<T>(im.grad, px, pz, tau, lam_dev, lam_scale, zout, P->nx, P->nz,
+                                 n, s);
+    }));
+    return ISAM_OK;
+  }
+}
+
 // One iteration of Alg. 1: the fused gradient kernel on eta_hat^k (ehat_in,
 // default the plan's buffer), then the lateral update, which writes z^k to
 // zout, eta_hat^{k+1} to ehat_out (default the plan's buffer) and, when
@@ -531,35 +619,8 @@ template <typename T> isam_status fista_iteration(isam_plan* P, Impl<T>& im,
                                    lam_dev, lam_scale, s);
       }));
     } else {
-      // TV prox of u = im.grad: the dual (p) carries over from the previous
-      // iteration; r starts at p; fast gradient projection; z = u - tau grad^H p
-      const size_t n = P->n_img;
-      cplx<T>* px = im.tv;
-      cplx<T>* pz = im.tv + n;
-      cplx<T>* rx = im.tv + 2 * n;
-      cplx<T>* rz = im.tv + 3 * n;
-      cplx<T>* w = im.tv + 4 * n;
-      const T tau = T(lam / L);
-      CUDA_TRY(cudaMemcpyAsync(rx, px, 2 * n * sizeof(cplx<T>), cudaMemcpyDeviceToDevice, s));
-      double t = 1.0;
-      const int iters = prior_iters > 0 ? prior_iters : 20;
-      for (int i = 0; i < iters; ++i) {
-        const double t_next = 0.5 * (1.0 + sqrt(1.0 + 4.0 * t * t));
-        const T beta = T((t - 1.0) / t_next);
-        t = t_next;
-        ISAM_TRY(launch(P, ISAM_KCLASS_MISC, [&] {
-          return launch_tv_primal<T>(im.grad, rx, rz, tau, lam_dev, lam_scale, w, P->nx, P->nz, n,
-                                     s);
-        }));
-        ISAM_TRY(launch(P, ISAM_KCLASS_MISC, [&] {
-          return launch_tv_dual<T>(w, px, pz, rx, rz, tau, lam_dev, lam_scale, beta, P->nx, P->nz,
-                                   n, s);
-        }));
-      }
-      ISAM_TRY(launch(P, ISAM_KCLASS_MISC, [&] {
-        return launch_tv_primal<T>(im.grad, px, pz, tau, lam_dev, lam_scale, zout, P->nx, P->nz,
-                                   n, s);
-      }));
+      ISAM_TRY(tv_prox<T>(P, im, zout, lam, L, lam_dev, lam_scale,
+                          prior_iters > 0 ? prior_iters : 20));
     }
     LatArgs<T> e = lat_args<T>(P->ny, P->nx, P->nz, nullptr, ehat_out);
     e.z1 = zout; e.z2 = z1; e.mu = T(mu);
@@ -663,8 +724,9 @@ template <typename T> isam_status solve_impl(isam_plan* P, const T* s_d, const i
     CUDA_TRY(cudaMemsetAsync(im.eta_hat, 0, sizeof(cplx<T>) * P->n_img, s));
   }
   if (o->prior == ISAM_PRIOR_TV) {                 // TV dual starts at 0 for every solve
-    if (!im.tv) ISAM_TRY(dalloc(&im.tv, 5 * P->n_img));
+    if (!im.tv) ISAM_TRY(dalloc(&im.tv, tv_images<T>(P) * P->n_img));
     CUDA_TRY(cudaMemsetAsync(im.tv, 0, 2 * sizeof(cplx<T>) * P->n_img, s));
+    im.tv_cur = 0;
   }
   // lateral spectrum of the data, used by every iteration's residual
   if (!im.sdh) ISAM_TRY(dalloc(&im.sdh, P->n_spec));
@@ -1586,7 +1648,7 @@ template <typename T> isam_status batch_prepare(isam_plan* P, const isam_solve_o
   if (!im.zB) ISAM_TRY(dalloc(&im.zB, P->n_img));
   if (!im.sdh) ISAM_TRY(dalloc(&im.sdh, P->n_spec));
   if (!im.s_tmp) ISAM_TRY(dalloc(&im.s_tmp, P->n_spec));
-  if (o->prior == ISAM_PRIOR_TV && !im.tv) ISAM_TRY(dalloc(&im.tv, 5 * P->n_img));
+  if (o->prior == ISAM_PRIOR_TV && !im.tv) ISAM_TRY(dalloc(&im.tv, tv_images<T>(P) * P->n_img));
   double L = o->L;
   if (!(L > 0)) {
     if (!(P->L_cache > 0)) {
@@ -1632,7 +1694,10 @@ template <typename T> isam_status batch_enqueue(isam_plan* P, const T* s_d,
   CUDA_TRY(cudaMemsetAsync(im.zA, 0, bytes, s));
   CUDA_TRY(cudaMemsetAsync(im.zB, 0, bytes, s));
   CUDA_TRY(cudaMemsetAsync(im.eta_hat, 0, bytes, s));
-  if (o->prior == ISAM_PRIOR_TV) CUDA_TRY(cudaMemsetAsync(im.tv, 0, 2 * bytes, s));
+  if (o->prior == ISAM_PRIOR_TV) {
+    CUDA_TRY(cudaMemsetAsync(im.tv, 0, 2 * bytes, s));
+    im.tv_cur = 0;
+  }
   std::vector<double> mu;
   momentum(o->max_iter + 1, mu);
   cplx<T>* zP = im.zA;
