@@ -11,8 +11,13 @@
 // 16- or 32-byte shared-memory access per point).
 //
 // Direction SIGN = -1 computes X_m = sum_p x_p e^{-2 pi i m p / L},
-// SIGN = +1 the same with e^{+...}; no normalisation.  Twiddles come from a
-// per-block shared-memory table (build_twiddles).
+// SIGN = +1 the same with e^{+...}; no normalisation.
+//
+// Twiddles.  FP32: a per-block shared-memory table of one factor per butterfly
+// (build_twiddles), raised to its powers in registers.  FP64: the L roots of unity
+// in global memory (the plan's table, read through L1), every factor loaded: the
+// FP64 pipe, two lanes a cycle on an SM, bounds these kernels, and building a
+// table per block and multiplying powers took a quarter of its instructions.
 #pragma once
 
 #include "common.cuh"
@@ -20,6 +25,8 @@
 namespace isam {
 
 template <typename T> struct alignas(2 * sizeof(cplx<T>)) cpair { cplx<T> a, b; };
+// one column where the axial kernels otherwise take a pair
+template <typename T> struct alignas(sizeof(cplx<T>)) cone { cplx<T> a; };
 
 // arithmetic on complex numbers and complex pairs
 template <typename C> __device__ __forceinline__ C eadd(C a, C b) { return cadd(a, b); }
@@ -30,6 +37,19 @@ template <typename T> __device__ __forceinline__ cpair<T> eadd(cpair<T> a, cpair
 template <typename T> __device__ __forceinline__ cpair<T> esub(cpair<T> a, cpair<T> b) {
   return {csub(a.a, b.a), csub(a.b, b.b)};
 }
+template <typename T> __device__ __forceinline__ cone<T> eadd(cone<T> a, cone<T> b) {
+  return {cadd(a.a, b.a)};
+}
+template <typename T> __device__ __forceinline__ cone<T> esub(cone<T> a, cone<T> b) {
+  return {csub(a.a, b.a)};
+}
+// acc + c y for a real c
+template <typename T> __device__ __forceinline__ cpair<T> efma_r(T c, cpair<T> y, cpair<T> acc) {
+  return {cfma_r(c, y.a, acc.a), cfma_r(c, y.b, acc.b)};
+}
+template <typename T> __device__ __forceinline__ cone<T> efma_r(T c, cone<T> y, cone<T> acc) {
+  return {cfma_r(c, y.a, acc.a)};
+}
 template <int SIGN, typename C> __device__ __forceinline__ C emul_i(C a) { return cmul_i<SIGN>(a); }
 template <int SIGN, typename T> __device__ __forceinline__ cpair<T> emul_i(cpair<T> a) {
   return {cmul_i<SIGN>(a.a), cmul_i<SIGN>(a.b)};
@@ -37,6 +57,15 @@ template <int SIGN, typename T> __device__ __forceinline__ cpair<T> emul_i(cpair
 template <typename C> __device__ __forceinline__ C emul(C a, C w) { return cmul(a, w); }
 template <typename T> __device__ __forceinline__ cpair<T> emul(cpair<T> a, cplx<T> w) {
   return {cmul(a.a, w), cmul(a.b, w)};
+}
+template <typename T> __device__ __forceinline__ cone<T> emul(cone<T> a, cplx<T> w) {
+  return {cmul(a.a, w)};
+}
+template <typename T> __device__ __forceinline__ cone<T> escale(cone<T> a, T s) {
+  return {cscale(a.a, s)};
+}
+template <int SIGN, typename T> __device__ __forceinline__ cone<T> emul_i(cone<T> a) {
+  return {cmul_i<SIGN>(a.a)};
 }
 template <typename C, typename T> __device__ __forceinline__ C escale(C a, T s) { return cscale(a, s); }
 template <typename T> __device__ __forceinline__ cpair<T> escale(cpair<T> a, T s) {
@@ -60,6 +89,13 @@ template <int SIGN, typename T> __device__ __forceinline__ cpair<T> ew8_3(cpair<
   return {ew8_3<SIGN>(o.a), ew8_3<SIGN>(o.b)};
 }
 
+template <int SIGN, typename T> __device__ __forceinline__ cone<T> ew8_1(cone<T> o) {
+  return {ew8_1<SIGN>(o.a)};
+}
+template <int SIGN, typename T> __device__ __forceinline__ cone<T> ew8_3(cone<T> o) {
+  return {ew8_3<SIGN>(o.a)};
+}
+
 // t + SIGN i s and t - SIGN i s, lane by lane (no operand swap for the
 // packed two-lane adds of the FP32 forms)
 template <int SIGN, typename C> __device__ __forceinline__ C add_rot(C t, C s) {
@@ -73,6 +109,13 @@ template <int SIGN, typename T> __device__ __forceinline__ cpair<T> add_rot(cpai
 }
 template <int SIGN, typename T> __device__ __forceinline__ cpair<T> sub_rot(cpair<T> t, cpair<T> s) {
   return {sub_rot<SIGN>(t.a, s.a), sub_rot<SIGN>(t.b, s.b)};
+}
+
+template <int SIGN, typename T> __device__ __forceinline__ cone<T> add_rot(cone<T> t, cone<T> s) {
+  return {add_rot<SIGN>(t.a, s.a)};
+}
+template <int SIGN, typename T> __device__ __forceinline__ cone<T> sub_rot(cone<T> t, cone<T> s) {
+  return {sub_rot<SIGN>(t.a, s.a)};
 }
 
 template <int SIGN, typename E>
@@ -126,13 +169,14 @@ __host__ __device__ __forceinline__ int padded_rows(int L) { return L + (L >> 3)
 __device__ __forceinline__ void sincospi_(float x, float* s, float* c) { sincospif(x, s, c); }
 __device__ __forceinline__ void sincospi_(double x, double* s, double* c) { sincospi(x, s, c); }
 
-// Twiddle table of an L-point transform, in shared memory: for every pass
+// FP32 twiddle table of an L-point transform, in shared memory: for every pass
 // with span Ns > 1 and radix R, entry k of that pass's segment holds
 // w_k = e^{-2 pi i k / (Ns R)}, k < Ns.  A butterfly raises w_k to the powers
 // r = 2 .. R-1 itself by repeated complex multiplication, so each pass reads
 // one table entry per butterfly instead of R - 1.
+template <typename T>
 __host__ __device__ __forceinline__ int twiddle_entries(int L, int logL, int r3 = 0) {
-  if (L < 8) return 0;
+  if (L < 8 || sizeof(T) == 8) return 0;
   int n = 0, Ns = 1;
   const int n8 = logL / 3;
   for (int p = 0; p < n8; ++p) {
@@ -146,10 +190,13 @@ __host__ __device__ __forceinline__ int twiddle_entries(int L, int logL, int r3 
   return n;
 }
 
-// All threads of the block fill the table (ends with a barrier).  logL is
+// The transform's twiddles: FP32: all threads of the block fill the table at tab
+// (ends with a barrier); FP64: the plan's roots e^{-2 pi i m / L}, m < L.  logL is
 // log2 of the power-of-two factor; r3 = 1 for L = 3 * 2^logL.
 template <typename T>
-__device__ __forceinline__ void build_twiddles(cplx<T>* tab, int L, int logL, int r3 = 0) {
+__device__ __forceinline__ const cplx<T>* build_twiddles(cplx<T>* tab, const cplx<T>* roots, int L,
+                                                         int logL, int r3 = 0) {
+  if constexpr (sizeof(T) == 8) return roots;
   if (L >= 8) {
     const int n8 = logL / 3, rem = logL - 3 * n8;
     const int npass = n8 + (rem ? 1 : 0) + r3;
@@ -168,6 +215,38 @@ __device__ __forceinline__ void build_twiddles(cplx<T>* tab, int L, int logL, in
     }
   }
   __syncthreads();
+  return tab;
+}
+
+// the twiddles of the passes after one of span Ns
+template <typename T> __device__ __forceinline__ const cplx<T>* next_twiddles(const cplx<T>* tw,
+                                                                            int Ns) {
+  return sizeof(T) == 8 || Ns == 1 ? tw : tw + Ns;
+}
+
+// a[r] *= w^r, r = 1 .. R-1, w = e^{-2 pi i k / (Ns R)} (conjugated for SIGN > 0);
+// stride = L / (Ns R)
+template <int SIGN, int R, typename T, typename E>
+__device__ __forceinline__ void twiddle_powers(E* a, const cplx<T>* tw, int k, int stride) {
+  if constexpr (sizeof(T) == 8) {
+    const cplx<T>* p = tw + k * stride;
+#pragma unroll
+    for (int r = 1; r < R; ++r) {
+      cplx<T> w = __ldg(p + (r - 1) * (k * stride));
+      if (SIGN > 0) w.y = -w.y;
+      a[r] = emul(a[r], w);
+    }
+  } else {
+    cplx<T> w1 = tw[k];
+    if (SIGN > 0) w1.y = -w1.y;
+    cplx<T> w = w1;
+    a[1] = emul(a[1], w);
+#pragma unroll
+    for (int r = 2; r < R; ++r) {
+      w = cmul(w, w1);
+      a[r] = emul(a[r], w);
+    }
+  }
 }
 
 // One Stockham pass of radix R on column `col` (logical row r at
@@ -203,17 +282,7 @@ __device__ __forceinline__ void stockham_pass(E* buf, int stride, int col, int b
       const int j = b + u * L8;
       const int k = j & (Ns - 1);
       E* a = v + u * R;
-      if (Ns > 1) {
-        cplx<T> w1 = tw[k];
-        if (SIGN > 0) w1.y = -w1.y;
-        cplx<T> w = w1;
-        a[1] = emul(a[1], w);
-#pragma unroll
-        for (int r = 2; r < R; ++r) {
-          w = cmul(w, w1);
-          a[r] = emul(a[r], w);
-        }
-      }
+      if (Ns > 1) twiddle_powers<SIGN, R, T>(a, tw, k, L / (Ns * R));
       if (R == 8) dft8<SIGN, HALF_ZERO>(a);
       else if (R == 4) dft4<SIGN>(a[0], a[1], a[2], a[3]);
       else dft2<SIGN>(a[0], a[1]);
@@ -249,11 +318,8 @@ __device__ __forceinline__ void stockham_pass3(E* buf, int stride, int col, int 
   for (int u = 0; u < 3; ++u) {
     const int j = b + u * L8;
     if (active && j < Ns) {
-      cplx<T> w1 = tw[j];
-      if (SIGN > 0) w1.y = -w1.y;
       E* a = v + 3 * u;
-      a[1] = emul(a[1], w1);
-      a[2] = emul(a[2], cmul(w1, w1));
+      twiddle_powers<SIGN, 3, T>(a, tw, j, 1);
       const E t1 = eadd(a[1], a[2]);
       const E t2 = esub(a[0], escale(t1, T(0.5)));
       const E t3 = escale(emul_i<SIGN>(esub(a[1], a[2])), h);
@@ -266,7 +332,7 @@ __device__ __forceinline__ void stockham_pass3(E* buf, int stride, int col, int 
 }
 
 // Length-L transform (L = 2^logL, or 3 * 2^logL when r3, L <= 8192) of column
-// `col`, using the twiddle table built by build_twiddles.  For L >= 8 the
+// `col`, with the twiddles of build_twiddles.  For L >= 8 the
 // active threads own butterfly b < L/8; for L < 8 the thread with b == 0
 // transforms the column directly.  HALF_ZERO: rows [L/4, 3L/4) of the input
 // are zero (and need not be stored; powers of two only).  Every thread of the
@@ -282,14 +348,14 @@ __device__ __forceinline__ void fft_smem(E* buf, int stride, int col, int b, int
         stockham_pass<SIGN, 8, true, T>(buf, stride, col, b, L, Ns, tw, active);
       else
         stockham_pass<SIGN, 8, false, T>(buf, stride, col, b, L, Ns, tw, active);
-      if (Ns > 1) tw += Ns;
+      tw = next_twiddles<T>(tw, Ns);
       Ns *= 8;
     }
     const int rem = logL - 3 * n8;
     if (rem == 2) stockham_pass<SIGN, 4, false, T>(buf, stride, col, b, L, Ns, tw, active);
     else if (rem == 1) stockham_pass<SIGN, 2, false, T>(buf, stride, col, b, L, Ns, tw, active);
     if (rem) {
-      if (Ns > 1) tw += Ns;
+      tw = next_twiddles<T>(tw, Ns);
       Ns <<= rem;
     }
     if (r3) stockham_pass3<SIGN, T>(buf, stride, col, b, L, Ns, tw, active);
@@ -329,18 +395,6 @@ __device__ __forceinline__ int prow_at(int r0, int p0, int r) {
   else return prow(r0 + r * STEP);
 }
 
-template <int SIGN, int R, typename T, typename E>
-__device__ __forceinline__ void twiddle_powers(E* a, cplx<T> w1) {
-  if (SIGN > 0) w1.y = -w1.y;
-  cplx<T> w = w1;
-  a[1] = emul(a[1], w);
-#pragma unroll
-  for (int r = 2; r < R; ++r) {
-    w = cmul(w, w1);
-    a[r] = emul(a[r], w);
-  }
-}
-
 template <int SIGN, int R, int L, int NS, bool HALF_ZERO, int STRIDE, typename T, typename E>
 __device__ __forceinline__ void stockham_pass_ct(E* buf, int col, int b, const cplx<T>* tw) {
   constexpr int NB = 8 / R;          // butterflies per thread
@@ -363,7 +417,7 @@ __device__ __forceinline__ void stockham_pass_ct(E* buf, int col, int b, const c
     const int j = b + u * L8;
     const int k = j & (NS - 1);
     E* a = v + u * R;
-    if (NS > 1) twiddle_powers<SIGN, R, T>(a, tw[k]);
+    if (NS > 1) twiddle_powers<SIGN, R, T>(a, tw, k, L / (NS * R));
     if (R == 8) dft8<SIGN, HALF_ZERO>(a);
     else if (R == 4) dft4<SIGN>(a[0], a[1], a[2], a[3]);
     else dft2<SIGN>(a[0], a[1]);
@@ -385,7 +439,7 @@ __device__ __forceinline__ void fft_passes_ct(E* buf, int col, int b, const cplx
     if constexpr (!(last && SKIP_LAST))
       stockham_pass_ct<SIGN, 8, L, NS, HALF_ZERO && NS == 1, STRIDE, T>(buf, col, b, tw);
     fft_passes_ct<SIGN, HALF_ZERO, L, NS * 8, STRIDE, T, SKIP_LAST>(buf, col, b,
-                                                                    tw + (NS > 1 ? NS : 0));
+                                                                    next_twiddles<T>(tw, NS));
   } else if constexpr (NS * 4 == L && !SKIP_LAST) {
     stockham_pass_ct<SIGN, 4, L, NS, false, STRIDE, T>(buf, col, b, tw);
   } else if constexpr (NS * 2 == L && !SKIP_LAST) {
@@ -395,8 +449,9 @@ __device__ __forceinline__ void fft_passes_ct(E* buf, int col, int b, const cplx
 
 // Offset in the twiddle table of the segment of the pass with span ns (a
 // power of 8): the segments of the spans 8, 64, ... below it come first.
-__host__ __device__ constexpr int tw_offset(int ns) {
+template <typename T> __host__ __device__ constexpr int tw_offset(int ns) {
   int o = 0;
+  if (sizeof(T) == 8) return o;
   for (int s = 8; s < ns; s *= 8) o += s;
   return o;
 }
@@ -416,14 +471,14 @@ __device__ __forceinline__ void last_pass_regs_ct(const E* buf, int col, int b,
   constexpr int L = 1 << LOGL, n8 = LOGL / 3, rem = LOGL - 3 * (LOGL / 3);
   constexpr int R = rem == 0 ? 8 : (1 << rem);
   constexpr int NS = L / R, NB = 8 / R, L8 = L / 8;
-  const cplx<T>* tw = tw_table + tw_offset(rem == 0 ? (1 << (3 * (n8 - 1))) : (1 << (3 * n8)));
+  const cplx<T>* tw = tw_table + tw_offset<T>(rem == 0 ? (1 << (3 * (n8 - 1))) : (1 << (3 * n8)));
   const int p0 = prow(b);
 #pragma unroll
   for (int u = 0; u < NB; ++u) {
     E a[R];
 #pragma unroll
     for (int r = 0; r < R; ++r) a[r] = buf[prow_at<L8>(b, p0, u + r * NB) * STRIDE + col];
-    if (NS > 1) twiddle_powers<SIGN, R, T>(a, tw[(b + u * L8) & (NS - 1)]);
+    if (NS > 1) twiddle_powers<SIGN, R, T>(a, tw, (b + u * L8) & (NS - 1), L / (NS * R));
     if (R == 8) dft8<SIGN>(a);
     else if (R == 4) dft4<SIGN>(a[0], a[1], a[2], a[3]);
     else dft2<SIGN>(a[0], a[1]);

@@ -51,6 +51,9 @@ template <typename T> struct Tables {
                              // (computed on the fly)
   cplx<T>* filt = nullptr;   // [(ny/2+1)(nx/2+1)][nk] filter B of Eq. 3, or null (B = 1);
                              // folded into stab's phases when stab exists
+  cplx<T>* coef = nullptr;   // FP64: [(ny/2+1)(nx/2+1)][2 J][nk/4] interpolation
+                             // coefficients (k_axial.cuh), or null (evaluated)
+  cplx<T>* roots = nullptr;  // FP64: e^{-2 pi i m / K}, m < K (see fft_smem.cuh)
 };
 
 // Min-max coefficients as polynomials in the fractional offset f.  With
@@ -88,6 +91,7 @@ template <typename T> struct LatArgs {
   int r3;                // L = 3 * 2^logL (else L = 2^logL)
   int TZ, logTZ;         // pair-columns (2 columns each) per block
   T norm;                // 1/sqrt(L)
+  const cplx<T>* roots;  // FP64: e^{-2 pi i m / L}, m < L
   // LAT_UPDATE
   const cplx<T>* z1;     // z^{k-1}
   const cplx<T>* z2;     // z^{k-2}
@@ -100,7 +104,7 @@ template <typename T> struct LatArgs {
   cplx<T>* uout;         // optional: u^k = eta^k - g^k before the threshold
   const double* lam_dev; // optional: lambda / L = lam_scale * (*lam_dev), read on the device
   double lam_scale;
-  // FP32 tiles that have a register form (lat_reg_takes): 1 runs it, 0 the
+  // tiles that have a register form (lat_reg_takes): 1 runs it, 0 the
   // radix-8 column-pair transforms in shared memory; ignored elsewhere
   int radix16;
   // solve with the device-side stop rule (see StopRule): a nonzero *stop, read
@@ -114,6 +118,8 @@ template <typename T> struct LatArgs {
 template <typename T> struct AxArgs {
   const cplx<T>* in;
   cplx<T>* out;
+  const cplx<T>* eta;        // gradient kernels: eta_hat (for u_hat)
+  cplx<T>* spec;             // FP64 gradient: workspace for the model spectra
   StoltConst sc;
   Tables<T> tab;
   Poly<T> poly;
@@ -121,7 +127,7 @@ template <typename T> struct AxArgs {
   // fused kernel only: lateral spectrum of the data, F s_d ([ny][nx][nk]; the
   // first column of each pair is read)
   const cplx<T>* sdh;
-  // fused kernel: 0 writes G; else writes u_hat = in - u_hat_scale * G (the
+  // fused kernel: 0 writes G; else writes u_hat = eta - u_hat_scale * G (the
   // lateral spectrum of eta^k - g/L, u_hat_scale = 1/L)
   T u_hat_scale;
   // fused kernel, optional: the model spectra S = phase . N(eta_hat)
@@ -137,10 +143,14 @@ template <typename T> struct AxArgs {
 
 // launchers (return cudaGetLastError())
 template <typename T> cudaError_t launch_lat(int mode, const LatArgs<T>& a, cudaStream_t s);
-// the FP32 passes with the tile in registers, for lengths L at TZ pair-columns
-// that lat_reg_takes
-bool lat_reg_takes(int L, int TZ);
-cudaError_t launch_lat_reg(int mode, const LatArgs<float>& a, cudaStream_t s);
+// the passes with the tile in registers, for lengths L at TZ pair-columns that
+// lat_reg_takes
+template <typename T> bool lat_reg_takes(int L, int TZ);
+template <> bool lat_reg_takes<float>(int L, int TZ);
+template <> bool lat_reg_takes<double>(int L, int TZ);
+template <typename T> cudaError_t launch_lat_reg(int mode, const LatArgs<T>& a, cudaStream_t s);
+template <> cudaError_t launch_lat_reg<float>(int mode, const LatArgs<float>& a, cudaStream_t s);
+template <> cudaError_t launch_lat_reg<double>(int mode, const LatArgs<double>& a, cudaStream_t s);
 template <typename T> cudaError_t launch_ax_fwd(const AxArgs<T>& a, int npairs, cudaStream_t s);
 template <typename T> cudaError_t launch_ax_adj(const AxArgs<T>& a, int npairs, cudaStream_t s);
 template <typename T> cudaError_t launch_ax_fused(const AxArgs<T>& a, int npairs, cudaStream_t s);
@@ -149,6 +159,9 @@ template <typename T> size_t ax_smem_bytes(int K, int nk, bool adj);
 // Stolt table: class |my| (nx/2+1) + |mx| of every |q|
 template <typename T> cudaError_t launch_stolt_table(const AxArgs<T>& a, int4* out,
                                                      cudaStream_t s);
+
+// FP64 coefficients of every quad (Tables::coef), from a.tab.stab
+cudaError_t launch_coef_table(const AxArgs<double>& a, double2* out, cudaStream_t s);
 
 // FP64 exact min-max coefficients at offsets f[0..n) (device), out[i*J + l]
 cudaError_t minmax_nodes(int nz, int K, int J, const double* f, int n, double* out,
@@ -251,10 +264,13 @@ template <typename T> cudaError_t launch_tv_dual(const cplx<T>* w, cplx<T>* px, 
 
 // Eq. 9 direct reconstruction (k_direct.cu)
 template <typename T> cudaError_t launch_dc_ifft(const T* s, cplx<T>* out, const cplx<T>* disp,
-                                                 const cplx<T>* post, int nk, int nz, int lognz,
-                                                 int n_ascans, cudaStream_t st);
+                                                 const cplx<T>* post, const cplx<T>* roots, int nk,
+                                                 int nz, int lognz, int n_ascans, cudaStream_t st);
 
-int lat_tile(int L, int M);   // pair-columns per block of a lateral pass
+// out[m] = e^{-2 pi i m / n}, m < n (k_misc.cu)
+cudaError_t launch_roots(double2* out, int n, cudaStream_t s);
+
+template <typename T> int lat_tile(int L, int M);   // pair-columns per block of a lateral pass
 template <typename T> size_t lat_smem_bytes(int L, int TP);
 // L = 2^log2 or 3 * 2^log2 (log2 >= 3): *log2, *r3; false for other lengths
 bool fft_length(int L, int* log2, int* r3);

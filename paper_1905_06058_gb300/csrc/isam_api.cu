@@ -45,6 +45,7 @@ template <typename T> struct Impl {
   cplx<T>* seg = nullptr;
   int seg_cap = 0;
   cplx<T>* cal = nullptr;       // [5][n_img]: zbar x 3, ubar, b
+  cplx<T>* roots = nullptr;     // FP64: roots of unity of K, nx, ny and nz, one after another
   cplx<T>* dc_post = nullptr;   // [nz] output phase of the Eq. 9 reconstruction
   // [tv_images][n_img]; FP32: TV duals p (x, z) of two launches in turn and a
   // momentum r; FP64: p_x, p_z, r_x, r_z and the primal w
@@ -232,10 +233,12 @@ template <typename T> isam_status dalloc(T** p, size_t n) {
 
 template <typename T> void impl_free(Impl<T>& im) {
   dfree(im.tab.scale); dfree(im.tab.disp); dfree(im.tab.stab); dfree(im.tab.filt);
+  dfree(im.tab.coef);
   dfree(im.eta_hat); dfree(im.spec); dfree(im.grad); dfree(im.sdh);
   dfree(im.zA); dfree(im.zB); dfree(im.s_tmp);
   dfree(im.s_host_stage); dfree(im.out_stage);
   dfree(im.spec2); dfree(im.seg); dfree(im.cal); dfree(im.dc_post); dfree(im.tv);
+  dfree(im.roots);
   im = Impl<T>();
 }
 
@@ -290,6 +293,17 @@ template <typename T> isam_status phase_tables(isam_plan* P, Impl<T>& im) {
       a.sc = P->sc;
       a.tab = im.tab;
       CUDA_TRY(launch_stolt_table<T>(a, im.tab.stab, P->stream));
+      // FP64: the coefficients too, under the same cap (they depend on the
+      // positions only, so once)
+      if constexpr (sizeof(T) == 8) {
+        const size_t n = rows * P->nk * size_t(P->J) / 2;
+        if (!im.tab.coef && n * sizeof(double2) <= cap) {
+          ISAM_TRY(dalloc(&im.tab.coef, n));
+          a.tab = im.tab;
+          a.poly = P->poly64;
+          CUDA_TRY(launch_coef_table(a, im.tab.coef, P->stream));
+        }
+      }
     }
   }
   return ISAM_OK;
@@ -305,6 +319,16 @@ template <typename T> isam_status impl_init(isam_plan* P, Impl<T>& im) {
       h[n] = T(host_kb_scale(n - P->nz / 2, P->K, P->J) / sqrt(double(P->nz)));
     ISAM_TRY(dalloc(&im.tab.scale, P->nz));
     CUDA_TRY(cudaMemcpy(im.tab.scale, h.data(), sizeof(T) * P->nz, cudaMemcpyHostToDevice));
+  }
+  if constexpr (sizeof(T) == 8) {
+    const int len[4] = {P->K, P->nx, P->ny, P->nz};
+    ISAM_TRY(dalloc(&im.roots, size_t(len[0]) + len[1] + len[2] + len[3]));
+    double2* r = im.roots;
+    for (int n : len) {
+      CUDA_TRY(launch_roots(r, n, P->stream));
+      r += n;
+    }
+    im.tab.roots = im.roots;
   }
   ISAM_TRY(phase_tables<T>(P, im));
   ISAM_TRY(dalloc(&im.eta_hat, P->n_img));
@@ -329,7 +353,7 @@ LatArgs<T> lat_args(int B, int L, int M, const void* in, void* out) {
   a.in = in; a.out = out;
   a.B = B; a.L = L; a.M = M;
   fft_length(L, &a.logL, &a.r3);
-  a.TZ = lat_tile(L, M); a.logTZ = ilog2(a.TZ);
+  a.TZ = lat_tile<T>(L, M); a.logTZ = ilog2(a.TZ);
   a.norm = T(1.0 / sqrt(double(L)));
   return a;
 }
@@ -339,6 +363,8 @@ template <typename T> isam_status lat(isam_plan* P, int mode, const LatArgs<T>& 
                                                              : ISAM_KCLASS_LAT_FFT;
   LatArgs<T> b = a;
   b.radix16 = P->tune_radix_lat == 16 ? 1 : 0;
+  if constexpr (sizeof(T) == 8)
+    b.roots = impl_of<T>(P).roots + P->K + (b.L == P->nx ? 0 : P->nx);
   return launch(P, cls, [&] { return launch_lat<T>(mode, b, P->stream); });
 }
 
@@ -352,7 +378,10 @@ template <typename T> AxArgs<T> ax_args(isam_plan* P, const Impl<T>& im, const c
   a.in = in; a.out = out; a.sc = P->sc; a.tab = im.tab;
   a.poly = poly_of<T>(P);
   a.pairs = P->pairs;
-  if (P->tune_table == 2) a.tab.stab = nullptr;
+  if (P->tune_table == 2) {
+    a.tab.stab = nullptr;
+    a.tab.coef = nullptr;
+  }
   a.radix16 = P->tune_radix_ax == 16 ? 1 : 0;
   return a;
 }
@@ -591,6 +620,9 @@ template <typename T> isam_status fista_iteration(isam_plan* P, Impl<T>& im,
   // iteration writes nothing when an earlier check has stopped the solve;
   // stop_rule: the check iteration's reduction evaluates Eq. 15 (StopRule)
   AxArgs<T> ax = ax_args<T>(P, im, ehat_in, im.grad);
+  ax.eta = ehat_in;
+  ax.spec = im.spec;
+  if (sizeof(T) == 8) P->launches += 1;   // FP64: two kernels
   ax.sdh = im.sdh;
   ax.s_out = s_out;
   ax.stop = stop;
@@ -1592,7 +1624,8 @@ template <typename T> isam_status dc_ifft_impl(isam_plan* P, const T* s, cplx<T>
     CUDA_TRY(cudaMemcpy(im.dc_post, h.data(), sizeof(cplx<T>) * P->nz, cudaMemcpyHostToDevice));
   }
   return launch(P, ISAM_KCLASS_MISC, [&] {
-    return launch_dc_ifft<T>(s, out, im.tab.disp, im.dc_post, P->nk, P->nz, ilog2(P->nz),
+    return launch_dc_ifft<T>(s, out, im.tab.disp, im.dc_post,
+                             im.roots ? im.roots + P->K + P->nx + P->ny : nullptr, P->nk, P->nz, ilog2(P->nz),
                              P->nx * P->ny, P->stream);
   });
 }
@@ -2030,7 +2063,7 @@ template <typename T> void report_tuning(const isam_plan* P, isam_tuning* out) {
   const Impl<T>& im = impl_of<T>(const_cast<isam_plan*>(P));
   int L, M;
   update_geometry(P, &L, &M);
-  out->lateral_tile = P->tune_tp ? P->tune_tp : lat_tile(L, M);
+  out->lateral_tile = P->tune_tp ? P->tune_tp : lat_tile<T>(L, M);
   out->stolt_table = P->tune_table == 2 ? 0 : (im.tab.stab ? 1 : 0);
   out->axial_radix = P->tune_radix_ax;
   out->lateral_radix = P->tune_radix_lat;
@@ -2055,8 +2088,8 @@ template <typename T> isam_status autotune_impl(isam_plan* P, isam_tuning* out) 
   update_geometry(P, &L, &M);
   const int threads_per_tp = L >= 8 ? L / 8 : 1;
   const bool fp32 = P->p.precision == ISAM_FP32;
-  // both radices exist for FP32 axial transforms at K = 2048, 4096 and the FP32
-  // lateral tiles with a register form
+  // both radices exist for FP32 axial transforms at K = 2048, 4096 and the lateral
+  // tiles with a register form
   const bool ax_both = fp32 && (P->K == 2048 || P->K == 4096);
   const bool prof = P->prof;
   P->prof = false;
@@ -2070,7 +2103,7 @@ template <typename T> isam_status autotune_impl(isam_plan* P, isam_tuning* out) 
   for (int it = 0; it < ntab && st == ISAM_OK; ++it) {
     for (int tp = 1; tp <= 8 && st == ISAM_OK; tp *= 2) {
       if (tp > M / 2 || threads_per_tp * tp > 512) continue;
-      const bool lat_both = fp32 && lat_reg_takes(L, tp);
+      const bool lat_both = lat_reg_takes<T>(L, tp);
       for (int ra = ax_both ? 8 : 16; ra <= 16 && st == ISAM_OK; ra += 8) {
         for (int rl = lat_both ? 8 : 16; rl <= 16 && st == ISAM_OK; rl += 8) {
           Tuning t;

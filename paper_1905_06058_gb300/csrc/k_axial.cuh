@@ -121,8 +121,8 @@ __device__ __forceinline__ int stolt_class(const StoltConst& sc, int mx, int my)
 // scatter_samples)
 constexpr int NRES = 4;
 
-template <typename T> struct Sample {
-  cpair<T> val;   // conj(phase) R of both columns
+template <typename T, typename V> struct Sample {
+  V val;          // conj(phase) R of the block's column or columns
   T frac;         // fractional Stolt offset
   int mfl;        // unwrapped floor of the Stolt position; INT_MIN: no contribution
                   // (evanescent, or past nk)
@@ -144,16 +144,17 @@ template <typename T> struct Positions {
   StoltPos<T> sp;
   const int4* row;           // the class's planes, nq vectors each
   const cplx<T>* frow;       // filter B of this column's |q| class (evaluated path)
-  int nq;
+  int nq, cls;
   __device__ Positions(const AxArgs<T>& A, int mx, int my) : sp(A.sc, mx, my) {
-    const size_t cls = size_t(stolt_class(A.sc, mx, my));
+    cls = stolt_class(A.sc, mx, my);
     nq = A.sc.nk / NRES;
-    row = A.tab.stab ? A.tab.stab + cls * (size_t(StoltTable<T>::planes) * nq) : nullptr;
-    frow = A.tab.filt ? A.tab.filt + cls * A.sc.nk : nullptr;
+    row = A.tab.stab ? A.tab.stab + size_t(cls) * (size_t(StoltTable<T>::planes) * nq) : nullptr;
+    frow = A.tab.filt ? A.tab.filt + size_t(cls) * A.sc.nk : nullptr;
   }
   // floors and fractions of the quad; an evaluated position also leaves its focus
   // turn in val.a.x, for phases()
-  __device__ __forceinline__ void quad(const AxArgs<T>& A, int q, Sample<T>* sm) const {
+  template <typename V>
+  __device__ __forceinline__ void quad(const AxArgs<T>& A, int q, Sample<T, V>* sm) const {
     if (row) {
       const int4 m = __ldg(row + q);
       sm[0].mfl = m.x; sm[1].mfl = m.y; sm[2].mfl = m.z; sm[3].mfl = m.w;
@@ -175,8 +176,9 @@ template <typename T> struct Positions {
     }
   }
   // phases of samples 2 h and 2 h + 1 of the quad (0 where evanescent)
+  template <typename V>
   __device__ __forceinline__ cpair<T> phases(const AxArgs<T>& A, int q, int h,
-                                             const Sample<T>* sm) const {
+                                             const Sample<T, V>* sm) const {
     cpair<T> p;
     if (row) {
       if constexpr (sizeof(T) == 4) {
@@ -189,13 +191,13 @@ template <typename T> struct Positions {
       }
       return p;
     }
-    p.a = evaluated(A, NRES * q + 2 * h, sm[2 * h]);
-    p.b = evaluated(A, NRES * q + 2 * h + 1, sm[2 * h + 1]);
+    p.a = evaluated(A, NRES * q + 2 * h, sm[2 * h].mfl, sm[2 * h].val.a.x);
+    p.b = evaluated(A, NRES * q + 2 * h + 1, sm[2 * h + 1].mfl, sm[2 * h + 1].val.a.x);
     return p;
   }
-  __device__ __forceinline__ cplx<T> evaluated(const AxArgs<T>& A, int j, const Sample<T>& s) const {
-    if (s.mfl == INT_MIN) return mk<T>(0, 0);
-    cplx<T> ph = spectral_phase<T>(A.sc, A.tab.disp, j, s.val.a.x);
+  __device__ __forceinline__ cplx<T> evaluated(const AxArgs<T>& A, int j, int mfl, T turn) const {
+    if (mfl == INT_MIN) return mk<T>(0, 0);
+    cplx<T> ph = spectral_phase<T>(A.sc, A.tab.disp, j, turn);
     if (frow) ph = cmul(ph, __ldg(frow + j));
     return ph;
   }
@@ -220,12 +222,48 @@ __device__ __forceinline__ void coefficients(const Poly<T>& P, T frac, T* c) {
   }
 }
 
-template <typename T>
+// The coefficients of a quad's samples.  FP64 plans tabulate them next to the Stolt
+// table (the polynomials took 42 of an FP64 sample's 56 FMAs): 2 J planes of one
+// double2 per quad of the class, (c_{2i}, c_{2i+1}) of sample rho in plane
+// rho J/2 + i.
+template <typename T, int J> struct Coefficients {
+  const Poly<T>& poly;
+  const cplx<T>* tab;        // the quad's first plane, or null: evaluate
+  int nq;
+  __device__ __forceinline__ Coefficients(const AxArgs<T>& A, const Positions<T>& pos, int q)
+      : poly(A.poly), tab(nullptr), nq(pos.nq) {
+    if (sizeof(T) == 8 && A.tab.coef) tab = A.tab.coef + size_t(pos.cls) * (2 * J) * nq + q;
+  }
+  __device__ __forceinline__ void operator()(int rho, T frac, T* c) const {
+    if constexpr (sizeof(T) == 8) {
+      if (tab) {
+#pragma unroll
+        for (int i = 0; i < J / 2; ++i) {
+          const cplx<T> v = __ldg(tab + (rho * (J / 2) + i) * nq);
+          c[2 * i] = v.x;
+          c[2 * i + 1] = v.y;
+        }
+        return;
+      }
+    }
+    coefficients<T, J>(poly, frac, c);
+  }
+};
+
+// The block's columns: a pair (q, -q), or with ONE the column blockIdx.x (c1; c2 is
+// the column of -q).
+template <typename T, bool ONE = false>
 __device__ __forceinline__ void pair_columns(const AxArgs<T>& A, int& c1, int& c2, int& mx,
                                              int& my) {
-  const int2 pr = A.pairs[blockIdx.x];
-  c1 = pr.x;
-  c2 = pr.y;
+  if (ONE) {
+    const int nx = A.sc.nx, ny = A.sc.ny, ix = blockIdx.x % nx, iy = blockIdx.x / nx;
+    c1 = blockIdx.x;
+    c2 = (iy ? ny - iy : 0) * nx + (ix ? nx - ix : 0);
+  } else {
+    const int2 pr = A.pairs[blockIdx.x];
+    c1 = pr.x;
+    c2 = pr.y;
+  }
   mx = signed_freq(c1 % A.sc.nx, A.sc.nx);
   my = signed_freq(c1 / A.sc.nx, A.sc.ny);
 }
@@ -236,13 +274,15 @@ template <typename T>
 __device__ __forceinline__ cplx<T>* twiddle_table(unsigned char* raw, int K) {
   return reinterpret_cast<cplx<T>*>(raw + size_t(padded_rows(K)) * sizeof(cpair<T>));
 }
+// the element of Y: a pair's two columns, or one column
+template <typename T, bool ONE> using column_t = std::conditional_t<ONE, cone<T>, cpair<T>>;
 
 // The forward K-point transform of the block's column pair: the
 // compile-time-length Stockham form when LOGK > 0 (K = 2^LOGK, the sizes the
 // kernels are instantiated for), else the runtime-length one.  Ends with a
 // barrier.  (The inverse is in inverse_and_store.)
-template <int LOGK, typename T>
-__device__ __forceinline__ void axial_fft_fwd(cpair<T>* Y, int K, int logK, const cplx<T>* tw) {
+template <int LOGK, typename T, typename V>
+__device__ __forceinline__ void axial_fft_fwd(V* Y, int K, int logK, const cplx<T>* tw) {
   if constexpr (LOGK > 0) fft_smem_ct<+1, true, LOGK, T>(Y, threadIdx.x, tw);
   else fft_smem<+1, true, T>(Y, 1, 0, threadIdx.x, K, logK, tw, true);
 }
@@ -258,11 +298,11 @@ template <int LOGK> __device__ __forceinline__ int axial_threads() {
 // Y (padded rows) = scaled columns c1 (a) and c2 (b), zero-padded to K, then
 // the K-point e^{+} DFT.  The padding rows [nz/2, K - nz/2) are never stored:
 // the first FFT pass knows them to be zero.  Ends with a barrier.
-template <typename T, int LOGK>
-__device__ __forceinline__ void load_and_fft(const AxArgs<T>& A, cpair<T>* Y, const cplx<T>* tw,
+template <typename T, int LOGK, typename V>
+__device__ __forceinline__ void load_and_fft(const AxArgs<T>& A, V* Y, const cplx<T>* tw,
                                              int c1, int c2, bool two) {
   using C = cplx<T>;
-  using V = cpair<T>;
+  constexpr bool ONE = sizeof(V) == sizeof(C);
   const StoltConst& sc = A.sc;
   const int K = axial_K<LOGK>(sc), nz = K / 2;
   const int tid = threadIdx.x, nt = axial_threads<LOGK>();
@@ -274,7 +314,7 @@ __device__ __forceinline__ void load_and_fft(const AxArgs<T>& A, cpair<T>* Y, co
   for (int i = 0; i < 4; ++i) {
     const int n = tid + i * nt;
     v[i].a = x1[n];
-    v[i].b = two ? x2[n] : mk<T>(0, 0);
+    if constexpr (!ONE) v[i].b = two ? x2[n] : mk<T>(0, 0);
   }
 #pragma unroll
   for (int i = 0; i < 4; ++i) {
@@ -284,22 +324,17 @@ __device__ __forceinline__ void load_and_fft(const AxArgs<T>& A, cpair<T>* Y, co
     Y[prow(p)] = escale(v[i], __ldg(A.tab.scale + n));
   }
   __syncthreads();
-  axial_fft_fwd<LOGK, T>(Y, K, sc.logK, tw);
+  axial_fft_fwd<LOGK, T, V>(Y, K, sc.logK, tw);
 }
 
-// forward interpolation of both columns at sample j (before the phase)
-template <typename T, int J>
-__device__ __forceinline__ void interp_pair(const cpair<T>* Y, int K, int mfl, const T* c,
-                                            cplx<T>& a1, cplx<T>& a2) {
+// forward interpolation of the columns at one sample (before the phase)
+template <typename T, int J, typename V>
+__device__ __forceinline__ V interp_sample(const V* Y, int K, int mfl, const T* c) {
   const int m0 = mfl - J / 2 + 1;
-  a1 = mk<T>(0, 0);
-  a2 = mk<T>(0, 0);
+  V s{};
 #pragma unroll
-  for (int l = 0; l < J; ++l) {
-    const cpair<T> y = Y[prow((m0 + l) & (K - 1))];
-    a1 = cfma_r(c[l], y.a, a1);
-    a2 = cfma_r(c[l], y.b, a2);
-  }
+  for (int l = 0; l < J; ++l) s = efma_r(c[l], Y[prow((m0 + l) & (K - 1))], s);
+  return s;
 }
 
 // Adjoint interpolation in scatter form.  Thread t owns samples
@@ -325,11 +360,11 @@ __device__ __forceinline__ void interp_pair(const cpair<T>* Y, int K, int mfl, c
 // warp before it, j* = NRES (nt - 32) - 1 (thread nt - 33), exists (j* < nk)
 // and is in chunk 0 or evanescent.  Its position goes through *tail
 // (INT_MAX: j* >= nk, INT_MIN: evanescent).
-template <typename T, int J>
-__device__ __forceinline__ int prepare_scatter(cpair<T>* Y, int K, int nt, int nk,
-                                               const Sample<T>* sm, int* chunk, int* lo, int* hi,
-                                               int* tail, bool& warp_tail) {
-  const cpair<T> zero = {mk<T>(0, 0), mk<T>(0, 0)};
+template <typename T, int J, typename V>
+__device__ __forceinline__ int prepare_scatter(V* Y, int K, int nt, int nk,
+                                               const Sample<T, V>* sm, int* chunk, int* lo,
+                                               int* hi, int* tail, bool& warp_tail) {
+  const V zero{};
   for (int i = threadIdx.x; i < K; i += nt) Y[prow(i)] = zero;
   int l = INT_MAX, h = INT_MIN;
 #pragma unroll
@@ -366,21 +401,16 @@ __device__ __forceinline__ int prepare_scatter(cpair<T>* Y, int K, int nt, int n
 }
 
 // the J contributions of one sample
-template <typename T, int J>
-__device__ __forceinline__ void add_sample(const AxArgs<T>& A, cpair<T>* Y, int K,
-                                           const Sample<T>& sm) {
-  using V = cpair<T>;
+template <typename T, int J, typename V>
+__device__ __forceinline__ void add_sample(const Coefficients<T, J>& co, V* Y, int K, int rho,
+                                           const Sample<T, V>& sm) {
   T c[J];
-  coefficients<T, J>(A.poly, sm.frac, c);
+  co(rho, sm.frac, c);
   const int m0 = sm.mfl - J / 2 + 1;
-  const V v = sm.val;
 #pragma unroll
   for (int l = 0; l < J; ++l) {
     const int bi = prow((m0 + l) & (K - 1));
-    V y = Y[bi];
-    y.a = cfma_r(c[l], v.a, y.a);
-    y.b = cfma_r(c[l], v.b, y.b);
-    Y[bi] = y;
+    Y[bi] = efma_r(c[l], sm.val, Y[bi]);
   }
 }
 
@@ -389,15 +419,15 @@ __device__ __forceinline__ void add_sample(const AxArgs<T>& A, cpair<T>* Y, int 
 // each phase closed by a block barrier.  With warp_tail the last chunk's
 // phases involve the last warp only and are closed by warp barriers, then one
 // block barrier: the same phases in the same order, so the same sums.
-template <typename T, int J>
-__device__ __forceinline__ void scatter_samples(const AxArgs<T>& A, cpair<T>* Y, int K, int nt,
-                                                const Sample<T>* sm, const int* chunk, int nchunks,
-                                                bool warp_tail) {
+template <typename T, int J, typename V>
+__device__ __forceinline__ void scatter_samples(const Coefficients<T, J>& co, V* Y, int K, int nt,
+                                                const Sample<T, V>* sm, const int* chunk,
+                                                int nchunks, bool warp_tail) {
   const int block_chunks = warp_tail ? 1 : nchunks;
   for (int ch = 0; ch < block_chunks; ++ch) {
 #pragma unroll
     for (int rho = 0; rho < NRES; ++rho) {
-      if (chunk[rho] == ch) add_sample<T, J>(A, Y, K, sm[rho]);
+      if (chunk[rho] == ch) add_sample<T, J, V>(co, Y, K, rho, sm[rho]);
       __syncthreads();
     }
   }
@@ -405,7 +435,7 @@ __device__ __forceinline__ void scatter_samples(const AxArgs<T>& A, cpair<T>* Y,
     if ((int(threadIdx.x) >> 5) == (nt >> 5) - 1) {
 #pragma unroll
       for (int rho = 0; rho < NRES; ++rho) {
-        if (chunk[rho] == 1) add_sample<T, J>(A, Y, K, sm[rho]);
+        if (chunk[rho] == 1) add_sample<T, J, V>(co, Y, K, rho, sm[rho]);
         __syncwarp();
       }
     }
@@ -446,15 +476,16 @@ __device__ __forceinline__ void scatter_samples(const AxArgs<T>& A, cpair<T>* Y,
 template <int J> __host__ __device__ constexpr int window_slots() { return J + 2 * NRES - 1; }
 
 // sample rho's offset from bin 2 rho of the thread's window (0 or 1 where it fits)
-template <typename T> __device__ __forceinline__ unsigned window_offset(const Sample<T>* sm, int rho) {
+template <typename S> __device__ __forceinline__ unsigned window_offset(const S* sm, int rho) {
   return unsigned(sm[rho].mfl) - unsigned(sm[0].mfl) - 2u * unsigned(rho);
 }
 
 // J coefficients as J + 1 taps, shifted up by one when `shift`
 template <typename T, int J>
-__device__ __forceinline__ void window_taps(const Poly<T>& P, T frac, bool shift, T* e) {
+__device__ __forceinline__ void window_taps(const Coefficients<T, J>& co, int rho, T frac,
+                                            bool shift, T* e) {
   T c[J];
-  coefficients<T, J>(P, frac, c);
+  co(rho, frac, c);
   e[0] = shift ? T(0) : c[0];
 #pragma unroll
   for (int l = 1; l < J; ++l) e[l] = shift ? c[l - 1] : c[l];
@@ -466,23 +497,20 @@ struct WindowHeads { int mfl[512]; };
 
 // One thread's window: sums its samples slot by slot and hands each finished
 // slot (l, value) to put.
-template <typename T, int J, typename Put>
-__device__ __forceinline__ void window_sums(const AxArgs<T>& A, const Sample<T>* sm, Put put) {
-  using V = cpair<T>;
+template <typename T, int J, typename V, typename Put>
+__device__ __forceinline__ void window_sums(const Coefficients<T, J>& co, const Sample<T, V>* sm,
+                                            Put put) {
   constexpr int WS = window_slots<J>();
   V w[WS];
 #pragma unroll
   for (int rho = 0; rho < NRES; ++rho) {
     T e[J + 1];
-    window_taps<T, J>(A.poly, sm[rho].frac, window_offset(sm, rho) != 0, e);
+    window_taps<T, J>(co, rho, sm[rho].frac, window_offset(sm, rho) != 0, e);
 #pragma unroll
     for (int l = 0; l <= J; ++l) {
       V& x = w[2 * rho + l];
       if (rho == 0 || l > J - 2) x = escale(sm[rho].val, e[l]);
-      else {
-        x.a = cfma_r(e[l], sm[rho].val.a, x.a);
-        x.b = cfma_r(e[l], sm[rho].val.b, x.b);
-      }
+      else x = efma_r(e[l], sm[rho].val, x);
     }
     if (rho < NRES - 1) {
       put(2 * rho, w[2 * rho]);
@@ -495,11 +523,10 @@ __device__ __forceinline__ void window_sums(const AxArgs<T>& A, const Sample<T>*
 
 // Y = the scatter of all samples (every bin written; ends with a barrier).
 // Every read of Y must be done and heads complete (a barrier before).
-template <typename T, int J>
-__device__ __forceinline__ void window_scatter(const AxArgs<T>& A, cpair<T>* Y, int K, int nt,
-                                               int nk, const Sample<T>* sm, cpair<T>* past,
+template <typename T, int J, typename V>
+__device__ __forceinline__ void window_scatter(const Coefficients<T, J>& co, V* Y, int K, int nt,
+                                               int nk, const Sample<T, V>* sm, V* past,
                                                const WindowHeads& heads) {
-  using V = cpair<T>;
   constexpr int WS = window_slots<J>(), W_MIN = 2 * NRES - 1, W_MAX = 2 * NRES + 2;
   const int tid = threadIdx.x, nact = nk / NRES;
   const bool active = tid < nact;
@@ -510,13 +537,13 @@ __device__ __forceinline__ void window_scatter(const AxArgs<T>& A, cpair<T>* Y, 
   const int own = tid < nact - 1 ? heads.mfl[tid + 1] + off - m0 : WS;
   const int limit = base + K - m0;                    // slots from here on lie past one period
   for (int i = end + tid; i < base + K; i += nt)
-    Y[prow(i & (K - 1))] = {mk<T>(0, 0), mk<T>(0, 0)};
+    Y[prow(i & (K - 1))] = V{};
   auto row = [&](int l) -> V& {
     return l < limit ? Y[prow((m0 + l) & (K - 1))] : past[l - limit];
   };
   V tail[WS - W_MIN];
   if (active)
-    window_sums<T, J>(A, sm, [&](int l, const V& v) {
+    window_sums<T, J, V>(co, sm, [&](int l, const V& v) {
       if (l >= W_MIN) tail[l - W_MIN] = v;
       if (l < W_MIN || l < own) row(l) = v;
     });
@@ -539,17 +566,17 @@ __device__ __forceinline__ void window_scatter(const AxArgs<T>& A, cpair<T>* Y, 
 }
 
 // The bins past one period: A.sc.window_past elements after the twiddles.
-template <typename T>
-__device__ __forceinline__ cpair<T>* window_past(const AxArgs<T>& A, cpair<T>* Y) {
-  return reinterpret_cast<cpair<T>*>(reinterpret_cast<unsigned char*>(Y) + A.past_offset);
+template <typename T, typename V>
+__device__ __forceinline__ V* window_past(const AxArgs<T>& A, V* Y) {
+  return reinterpret_cast<V*>(reinterpret_cast<unsigned char*>(Y) + A.past_offset);
 }
 
 // Y = the scatter of the block's samples, in the window form where every
 // thread's samples fit one.  Starts with a barrier (all reads of Y are done)
 // and ends with one.
-template <typename T, int J>
-__device__ __forceinline__ void scatter(const AxArgs<T>& A, cpair<T>* Y, int K, int nt, int nk,
-                                        Sample<T>* sm, int* lo, int* hi, int* ch_tail,
+template <typename T, int J, typename V>
+__device__ __forceinline__ void scatter(const AxArgs<T>& A, const Coefficients<T, J>& co, V* Y,
+                                        int K, int nt, int nk, const Sample<T, V>* sm, int* lo, int* hi, int* ch_tail,
                                         WindowHeads& heads) {
   bool ok = A.sc.window != 0;
   if (NRES * int(threadIdx.x) < nk) {
@@ -559,28 +586,27 @@ __device__ __forceinline__ void scatter(const AxArgs<T>& A, cpair<T>* Y, int K, 
       ok &= window_offset(sm, rho) <= 1u;
   }
   if (__syncthreads_and(ok)) {
-    window_scatter<T, J>(A, Y, K, nt, nk, sm, window_past<T>(A, Y), heads);
+    window_scatter<T, J, V>(co, Y, K, nt, nk, sm, window_past<T, V>(A, Y), heads);
     return;
   }
   bool warp_tail;
   int chunk[NRES];
-  const int nch = prepare_scatter<T, J>(Y, K, nt, nk, sm, chunk, lo, hi, ch_tail, warp_tail);
-  scatter_samples<T, J>(A, Y, K, nt, sm, chunk, nch, warp_tail);
+  const int nch = prepare_scatter<T, J, V>(Y, K, nt, nk, sm, chunk, lo, hi, ch_tail, warp_tail);
+  scatter_samples<T, J, V>(co, Y, K, nt, sm, chunk, nch, warp_tail);
 }
 
 // The forward interpolation of a thread's samples (before the phase): hands
-// (rho, N(x1), N(x2)) to put, in order; evanescent samples give 0.
-template <typename T, int J, typename Put>
-__device__ __forceinline__ void interp_quad(const AxArgs<T>& A, const cpair<T>* Y, int K,
-                                            const Sample<T>* sm, Put put) {
-  using C = cplx<T>;
+// (rho, N(x) of the columns) to put, in order; evanescent samples give 0.
+template <typename T, int J, typename V, typename Put>
+__device__ __forceinline__ void interp_quad(const AxArgs<T>& A, const Coefficients<T, J>& co,
+                                            const V* Y, int K, const Sample<T, V>* sm, Put put) {
   bool fits = A.sc.window != 0;
 #pragma unroll
   for (int rho = 0; rho < NRES; ++rho) fits &= window_offset(sm, rho) <= 1u;
   if (fits) {
     constexpr int WS = window_slots<J>();
     const int m0 = sm[0].mfl - J / 2 + 1;
-    cpair<T> y[WS];
+    V y[WS];
 #pragma unroll
     for (int l = 0; l < J - 1; ++l) y[l] = Y[prow((m0 + l) & (K - 1))];
 #pragma unroll
@@ -589,40 +615,37 @@ __device__ __forceinline__ void interp_quad(const AxArgs<T>& A, const cpair<T>* 
       for (int l = J - 1; l <= J; ++l)
         y[2 * rho + l] = Y[prow((m0 + 2 * rho + l) & (K - 1))];
       T e[J + 1];
-      window_taps<T, J>(A.poly, sm[rho].frac, window_offset(sm, rho) != 0, e);
-      C s1 = cscale(y[2 * rho].a, e[0]), s2 = cscale(y[2 * rho].b, e[0]);
+      window_taps<T, J>(co, rho, sm[rho].frac, window_offset(sm, rho) != 0, e);
+      V s = escale(y[2 * rho], e[0]);
 #pragma unroll
-      for (int l = 1; l <= J; ++l) {
-        s1 = cfma_r(e[l], y[2 * rho + l].a, s1);
-        s2 = cfma_r(e[l], y[2 * rho + l].b, s2);
-      }
-      put(rho, s1, s2);
+      for (int l = 1; l <= J; ++l) s = efma_r(e[l], y[2 * rho + l], s);
+      put(rho, s);
     }
     return;
   }
 #pragma unroll
   for (int rho = 0; rho < NRES; ++rho) {
-    C s1 = mk<T>(0, 0), s2 = mk<T>(0, 0);
+    V s{};
     if (sm[rho].mfl != INT_MIN) {
       T c[J];
-      coefficients<T, J>(A.poly, sm[rho].frac, c);
-      interp_pair<T, J>(Y, K, sm[rho].mfl, c, s1, s2);
+      co(rho, sm[rho].frac, c);
+      s = interp_sample<T, J, V>(Y, K, sm[rho].mfl, c);
     }
-    put(rho, s1, s2);
+    put(rho, s);
   }
 }
 
 // Sample n of both output columns: G = s y, or, when the kernel writes the
-// lateral spectrum of u = eta^k - g/L, u_hat = eta_hat - G/L with eta_hat the
-// kernel's own input (A.in, re-read here: the same samples the block loaded).
+// lateral spectrum of u = eta^k - g/L, u_hat = eta_hat - G/L with eta_hat = A.eta
+// (the fused kernel's own input, re-read here).
 template <typename T>
 __device__ __forceinline__ void put_output(const AxArgs<T>& A, cplx<T>* o1, cplx<T>* o2, int n,
                                            const cpair<T>& y, T s, int c1, int c2, bool two) {
   const int nz = A.sc.nz;
   if (A.u_hat_scale != T(0)) {
     const T f = s * A.u_hat_scale;
-    o1[n] = csub(A.in[size_t(c1) * nz + n], cscale(y.a, f));
-    if (two) o2[n] = csub(A.in[size_t(c2) * nz + n], cscale(y.b, f));
+    o1[n] = csub(A.eta[size_t(c1) * nz + n], cscale(y.a, f));
+    if (two) o2[n] = csub(A.eta[size_t(c2) * nz + n], cscale(y.b, f));
   } else {
     o1[n] = cscale(y.a, s);
     if (two) o2[n] = cscale(y.b, s);
@@ -635,15 +658,21 @@ template <typename T>
 __device__ __forceinline__ void put_output1(const AxArgs<T>& A, cplx<T>* o, int col, int n,
                                             const cplx<T>& y, T s) {
   if (A.u_hat_scale != T(0))
-    o[n] = csub(A.in[size_t(col) * A.sc.nz + n], cscale(y, s * A.u_hat_scale));
+    o[n] = csub(A.eta[size_t(col) * A.sc.nz + n], cscale(y, s * A.u_hat_scale));
   else
     o[n] = cscale(y, s);
 }
 
+template <typename T>
+__device__ __forceinline__ void put_output(const AxArgs<T>& A, cplx<T>* o1, cplx<T>* o2, int n,
+                                           const cone<T>& y, T s, int c1, int c2, bool two) {
+  put_output1(A, o1, c1, n, y.a, s);
+}
+
 // Y (after the e^{-} DFT): truncate to the nz samples, scale, store columns.
-template <typename T, int LOGK>
-__device__ __forceinline__ void store_columns(const AxArgs<T>& A, const cpair<T>* Y, int c1,
-                                              int c2, bool two) {
+template <typename T, int LOGK, typename V>
+__device__ __forceinline__ void store_columns(const AxArgs<T>& A, const V* Y, int c1, int c2,
+                                              bool two) {
   using C = cplx<T>;
   const int K = axial_K<LOGK>(A.sc), nz = K / 2, nt = axial_threads<LOGK>();
   C* o1 = A.out + size_t(c1) * nz;
@@ -652,7 +681,7 @@ __device__ __forceinline__ void store_columns(const AxArgs<T>& A, const cpair<T>
     int p = n - nz / 2;
     if (p < 0) p += K;
     const T s = __ldg(A.tab.scale + n);
-    const cpair<T> y = Y[prow(p)];
+    const V y = Y[prow(p)];
     put_output(A, o1, o2, n, y, s, c1, c2, two);
   }
 }
@@ -662,9 +691,9 @@ __device__ __forceinline__ void store_columns(const AxArgs<T>& A, const cpair<T>
 // (the rows thread b's last-pass butterfly produces, b + i K/8, are rows it
 // stores: natural row p goes to sample n = p + nz/2 for p < nz/2 and
 // p - (K - nz/2) for p >= K - nz/2, nz = K/2; the others are dropped).
-template <typename T, int LOGK>
-__device__ __forceinline__ void inverse_and_store(const AxArgs<T>& A, cpair<T>* Y,
-                                                  const cplx<T>* tw, int c1, int c2, bool two) {
+template <typename T, int LOGK, typename V>
+__device__ __forceinline__ void inverse_and_store(const AxArgs<T>& A, V* Y, const cplx<T>* tw,
+                                                  int c1, int c2, bool two) {
   if constexpr (LOGK > 0) {
     using C = cplx<T>;
     constexpr int K = 1 << LOGK, nz = K / 2, K8 = K / 8;
@@ -672,7 +701,7 @@ __device__ __forceinline__ void inverse_and_store(const AxArgs<T>& A, cpair<T>* 
     fft_passes_ct<-1, false, K, 1, 1, T, true>(Y, 0, b, tw);
     C* o1 = A.out + size_t(c1) * nz;
     C* o2 = A.out + size_t(c2) * nz;
-    last_pass_regs_ct<-1, LOGK, 1, T>(Y, 0, b, tw, [&](int i, const cpair<T>& y) {
+    last_pass_regs_ct<-1, LOGK, 1, T>(Y, 0, b, tw, [&](int i, const V& y) {
       const int p = b + i * K8;
       if (i * K8 >= K / 4 && (i + 1) * K8 <= 3 * K / 4) return;   // rows [K/4, 3K/4)
       const int n = p < K / 4 ? p + nz / 2 : p - (K - nz / 2);
@@ -680,7 +709,7 @@ __device__ __forceinline__ void inverse_and_store(const AxArgs<T>& A, cpair<T>* 
     });
   } else {
     fft_smem<-1, false, T>(Y, 1, 0, threadIdx.x, A.sc.K, A.sc.logK, tw, true);
-    store_columns<T, LOGK>(A, Y, c1, c2, two);
+    store_columns<T, LOGK, V>(A, Y, c1, c2, two);
   }
 }
 
@@ -697,14 +726,20 @@ template <typename T, int LOGK, bool C16> __host__ __device__ constexpr bool ax_
 }
 
 template <typename T, int LOGK, bool C16>
-__device__ __forceinline__ void ax_twiddles(cplx<T>* tw, const StoltConst& sc) {
-  if constexpr (ax_col16<T, LOGK, C16>()) c16::build_twiddles<LOGK>(reinterpret_cast<float4*>(tw));
-  else build_twiddles<T>(tw, axial_K<LOGK>(sc), sc.logK);
+__device__ __forceinline__ const cplx<T>* ax_twiddles(const AxArgs<T>& A, unsigned char* smem) {
+  const int K = axial_K<LOGK>(A.sc);
+  cplx<T>* tw = twiddle_table<T>(smem, K);
+  if constexpr (ax_col16<T, LOGK, C16>()) {
+    c16::build_twiddles<LOGK>(reinterpret_cast<float4*>(tw));
+    return tw;
+  } else {
+    return build_twiddles<T>(tw, A.tab.roots, K, A.sc.logK);
+  }
 }
 
 // Y = the K-point e^{+} DFT of the pair's scaled, zero-padded columns
-template <typename T, int LOGK, bool C16>
-__device__ __forceinline__ void ax_forward(const AxArgs<T>& A, cpair<T>* Y, const cplx<T>* tw,
+template <typename T, int LOGK, bool C16, typename V>
+__device__ __forceinline__ void ax_forward(const AxArgs<T>& A, V* Y, const cplx<T>* tw,
                                            int c1, int c2, bool two) {
   if constexpr (ax_col16<T, LOGK, C16>()) {
     constexpr int nz = (1 << LOGK) / 2;
@@ -714,14 +749,14 @@ __device__ __forceinline__ void ax_forward(const AxArgs<T>& A, cpair<T>* Y, cons
                        reinterpret_cast<const float*>(A.tab.scale),
                        reinterpret_cast<const float4*>(tw));
   } else {
-    load_and_fft<T, LOGK>(A, Y, tw, c1, c2, two);
+    load_and_fft<T, LOGK, V>(A, Y, tw, c1, c2, two);
   }
 }
 
 // The e^{-} DFT of Y, truncation to the nz kept rows, scaling, the columns'
 // output (G, or u_hat = eta_hat - G/L)
-template <typename T, int LOGK, bool C16>
-__device__ __forceinline__ void ax_inverse(const AxArgs<T>& A, cpair<T>* Y, const cplx<T>* tw,
+template <typename T, int LOGK, bool C16, typename V>
+__device__ __forceinline__ void ax_inverse(const AxArgs<T>& A, V* Y, const cplx<T>* tw,
                                            int c1, int c2, bool two) {
   if constexpr (ax_col16<T, LOGK, C16>()) {
     // rows j + i K/16 of this thread's column; rows [K/4, 3K/4) are dropped
@@ -739,7 +774,7 @@ __device__ __forceinline__ void ax_inverse(const AxArgs<T>& A, cpair<T>* Y, cons
                                      __ldg(A.tab.scale + n));
                        });
   } else {
-    inverse_and_store<T, LOGK>(A, Y, tw, c1, c2, two);
+    inverse_and_store<T, LOGK, V>(A, Y, tw, c1, c2, two);
   }
 }
 
@@ -750,23 +785,24 @@ template <typename T> __host__ __device__ constexpr int ax_min_blocks() {
   return std::is_same<T, float>::value ? 2 : 1;
 }
 
-template <typename T, int J, int LOGK, bool C16>
+// ONE: a block per column instead of per pair (FP64, see
+// launch_ax_JKC).
+template <typename T, int J, int LOGK, bool C16, bool ONE>
 __global__ void __launch_bounds__(512, ax_min_blocks<T>()) k_ax_fwd(const __grid_constant__ AxArgs<T> A) {
   using C = cplx<T>;
-  using V = cpair<T>;
+  using V = column_t<T, ONE>;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   const StoltConst& sc = A.sc;
   const int K = axial_K<LOGK>(sc), nk = sc.nk;
   V* Y = reinterpret_cast<V*>(smem_raw);
-  cplx<T>* tw = twiddle_table<T>(smem_raw, K);
   int c1, c2, mx, my;
-  pair_columns(A, c1, c2, mx, my);
-  const bool two = c2 != c1;
+  pair_columns<T, ONE>(A, c1, c2, mx, my);
+  const bool two = !ONE && c2 != c1;
   // programmatic dependent launch (as k_ax_fused): twiddles before the wait
   cudaTriggerProgrammaticLaunchCompletion();
-  ax_twiddles<T, LOGK, C16>(tw, sc);
+  const C* tw = ax_twiddles<T, LOGK, C16>(A, smem_raw);
   cudaGridDependencySynchronize();
-  ax_forward<T, LOGK, C16>(A, Y, tw, c1, c2, two);
+  ax_forward<T, LOGK, C16, V>(A, Y, tw, c1, c2, two);
 
   const Positions<T> pos(A, mx, my);
   C* o1 = A.out + size_t(c1) * nk;
@@ -774,47 +810,51 @@ __global__ void __launch_bounds__(512, ax_min_blocks<T>()) k_ax_fwd(const __grid
   // nk <= K/2 = NRES blockDim: a quad of samples per thread
   const int q = threadIdx.x;
   if (NRES * q >= nk) return;
-  Sample<T> sm[NRES];
+  Sample<T, V> sm[NRES];
   pos.quad(A, q, sm);
   cpair<T> ph;
   C a1, a2;
-  interp_quad<T, J>(A, Y, K, sm, [&](int rho, C s1, C s2) {
+  interp_quad<T, J, V>(A, Coefficients<T, J>(A, pos, q), Y, K, sm, [&](int rho, V s) {
+    const int j = NRES * q + rho;
     if (rho % 2 == 0) {
       ph = pos.phases(A, q, rho / 2, sm);
-      a1 = cmul(s1, ph.a);
-      a2 = cmul(s2, ph.a);
-      return;
+      a1 = cmul(s.a, ph.a);
+      if constexpr (!ONE) a2 = cmul(s.b, ph.a);
+    } else {
+      store_two<T>(o1 + j - 1, a1, cmul(s.a, ph.b));
+      if constexpr (!ONE)
+        if (two) store_two<T>(o2 + j - 1, a2, cmul(s.b, ph.b));
     }
-    const int j = NRES * q + rho - 1;
-    store_two<T>(o1 + j, a1, cmul(s1, ph.b));
-    if (two) store_two<T>(o2 + j, a2, cmul(s2, ph.b));
   });
 }
 
-template <typename T, int J, int LOGK, bool C16>
+// RES: the input holds the model spectra S and the kernel forms the residual
+// spectrum R(q) = (S(q) + conj S(-q)) / 2 - F s_d(q) on load (ONE only; see
+// k_ax_fused).
+template <typename T, int J, int LOGK, bool C16, bool ONE, bool RES>
 __global__ void __launch_bounds__(512, ax_min_blocks<T>()) k_ax_adj(const __grid_constant__ AxArgs<T> A) {
+  static_assert(ONE || !RES, "the pair kernel with a residual is k_ax_fused");
   using C = cplx<T>;
-  using V = cpair<T>;
+  using V = column_t<T, ONE>;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   const StoltConst& sc = A.sc;
   const int K = axial_K<LOGK>(sc), nk = sc.nk;
   V* Y = reinterpret_cast<V*>(smem_raw);
-  cplx<T>* tw = twiddle_table<T>(smem_raw, K);
   __shared__ int ch_lo, ch_hi, ch_tail;
   __shared__ WindowHeads heads;
   const int tid = threadIdx.x, nt = axial_threads<LOGK>();
   int c1, c2, mx, my;
-  pair_columns(A, c1, c2, mx, my);
-  const bool two = c2 != c1;
+  pair_columns<T, ONE>(A, c1, c2, mx, my);
+  const bool two = !ONE && c2 != c1;
   if (tid == 0) { ch_lo = INT_MAX; ch_hi = INT_MIN; }
   // programmatic dependent launch (as k_ax_fused): twiddles before the wait
-  cudaTriggerProgrammaticLaunchCompletion();
-  ax_twiddles<T, LOGK, C16>(tw, sc);
+  const C* tw = ax_twiddles<T, LOGK, C16>(A, smem_raw);
   cudaGridDependencySynchronize();
+  const bool stopped = RES && A.stop != nullptr && __ldcg(A.stop) != 0;
   const Positions<T> pos(A, mx, my);
   const C* r1 = A.in + size_t(c1) * nk;
   const C* r2 = A.in + size_t(c2) * nk;
-  Sample<T> sm[NRES];
+  Sample<T, V> sm[NRES];
 #pragma unroll
   for (int rho = 0; rho < NRES; ++rho) sm[rho].mfl = INT_MIN;
   if (NRES * tid < nk) {
@@ -822,14 +862,27 @@ __global__ void __launch_bounds__(512, ax_min_blocks<T>()) k_ax_adj(const __grid
 #pragma unroll
     for (int h = 0; h < NRES / 2; ++h) {
       const int j = NRES * tid + 2 * h;
-      const V ph = pos.phases(A, tid, h, sm);
-      const V x = load_two<T>(r1 + j), y = two ? load_two<T>(r2 + j) : V{};
-      sm[2 * h].val = {cmulc(x.a, ph.a), cmulc(y.a, ph.a)};
-      sm[2 * h + 1].val = {cmulc(x.b, ph.b), cmulc(y.b, ph.b)};
+      const cpair<T> ph = pos.phases(A, tid, h, sm);
+      cpair<T> x = load_two<T>(r1 + j);
+      if constexpr (RES) {
+        const cpair<T> y = load_two<T>(r2 + j), d = load_two<T>(A.sdh + size_t(c1) * nk + j);
+        x.a = csub(cscale(cadd(x.a, cconj(y.a)), T(0.5)), d.a);
+        x.b = csub(cscale(cadd(x.b, cconj(y.b)), T(0.5)), d.b);
+      }
+      sm[2 * h].val.a = cmulc(x.a, ph.a);
+      sm[2 * h + 1].val.a = cmulc(x.b, ph.b);
+      if constexpr (!ONE) {
+        const cpair<T> y = two ? load_two<T>(r2 + j) : cpair<T>{};
+        sm[2 * h].val.b = cmulc(y.a, ph.a);
+        sm[2 * h + 1].val.b = cmulc(y.b, ph.b);
+      }
     }
   }
-  scatter<T, J>(A, Y, K, nt, nk, sm, &ch_lo, &ch_hi, &ch_tail, heads);
-  ax_inverse<T, LOGK, C16>(A, Y, tw, c1, c2, two);
+  if (stopped) return;   // an earlier check stopped the solve: write nothing
+  scatter<T, J, V>(A, Coefficients<T, J>(A, pos, tid), Y, K, nt, nk, sm, &ch_lo, &ch_hi, &ch_tail,
+                   heads);
+  cudaTriggerProgrammaticLaunchCompletion();
+  ax_inverse<T, LOGK, C16, V>(A, Y, tw, c1, c2, two);
 }
 
 // Forward model, data residual and adjoint of one column pair in one pass
@@ -849,7 +902,6 @@ __global__ void __launch_bounds__(512, ax_min_blocks<T>()) k_ax_fused(const __gr
   const StoltConst& sc = A.sc;
   const int K = axial_K<LOGK>(sc), nk = sc.nk;
   V* Y = reinterpret_cast<V*>(smem_raw);
-  cplx<T>* tw = twiddle_table<T>(smem_raw, K);
   __shared__ int ch_lo, ch_hi, ch_tail;
   __shared__ WindowHeads heads;
   const int tid = threadIdx.x, nt = axial_threads<LOGK>();
@@ -857,35 +909,33 @@ __global__ void __launch_bounds__(512, ax_min_blocks<T>()) k_ax_fused(const __gr
   pair_columns(A, c1, c2, mx, my);
   const bool two = c2 != c1;
   if (tid == 0) { ch_lo = INT_MAX; ch_hi = INT_MIN; }
-  // Programmatic dependent launch: the next kernel in the stream may start its
-  // own prologue on SMs this grid leaves idle; this grid builds its twiddles,
-  // then waits for the previous kernel before touching global data.
-  cudaTriggerProgrammaticLaunchCompletion();
-  ax_twiddles<T, LOGK, C16>(tw, sc);
+  // Programmatic dependent launch: this grid builds its twiddles, then waits for
+  // the previous kernel before touching global data; the next kernel may start
+  // once every block here is in its inverse transform (below).
+  const C* tw = ax_twiddles<T, LOGK, C16>(A, smem_raw);
   cudaGridDependencySynchronize();
   // the solve's stop flag (written by an earlier kernel, so visible after the
   // wait): loaded here, tested after the forward transform (before the first
   // global write), so its latency overlaps the transform
   const bool stopped = A.stop != nullptr && __ldcg(A.stop) != 0;
   const C* d1 = A.sdh + size_t(c1) * nk;
-  ax_forward<T, LOGK, C16>(A, Y, tw, c1, c2, two);
+  ax_forward<T, LOGK, C16, V>(A, Y, tw, c1, c2, two);
   if (stopped) return;   // an earlier check stopped the solve: write nothing
   const Positions<T> pos(A, mx, my);
-  Sample<T> sm[NRES];
+  Sample<T, V> sm[NRES];
 #pragma unroll
   for (int rho = 0; rho < NRES; ++rho) sm[rho].mfl = INT_MIN;
   if (NRES * tid < nk) {
     pos.quad(A, tid, sm);
     V php, dq, w1, w2;                   // of two samples: phases, F s_d, model spectra
-    interp_quad<T, J>(A, Y, K, sm, [&](int rho, C s1, C s2) {
+    interp_quad<T, J, V>(A, Coefficients<T, J>(A, pos, tid), Y, K, sm, [&](int rho, V n) {
       const int j = NRES * tid + rho;
       if (rho % 2 == 0) {
         php = pos.phases(A, tid, rho / 2, sm);
         dq = load_two<T>(d1 + j);
       }
       const C ph = rho % 2 == 0 ? php.a : php.b;
-      s1 = cmul(s1, ph);
-      s2 = two ? cmul(s2, ph) : s1;
+      const C s1 = cmul(n.a, ph), s2 = two ? cmul(n.b, ph) : s1;
       if (WS) {
         if (rho % 2 == 0) {
           w1.a = s1;
@@ -901,8 +951,13 @@ __global__ void __launch_bounds__(512, ax_min_blocks<T>()) k_ax_fused(const __gr
       sm[rho].val.b = two ? cmulc(cconj(R), ph) : mk<T>(0, 0);
     });
   }
-  scatter<T, J>(A, Y, K, nt, nk, sm, &ch_lo, &ch_hi, &ch_tail, heads);
-  ax_inverse<T, LOGK, C16>(A, Y, tw, c1, c2, two);
+  scatter<T, J, V>(A, Coefficients<T, J>(A, pos, tid), Y, K, nt, nk, sm, &ch_lo, &ch_hi, &ch_tail,
+                   heads);
+  // Not earlier: the next kernel's waiting blocks take the first slots that fall
+  // free, several to a multiprocessor, and stay there (1024 x 2048 solve 11.4 ms
+  // with the trigger at the start of this kernel and of the update, 10.9 ms so)
+  cudaTriggerProgrammaticLaunchCompletion();
+  ax_inverse<T, LOGK, C16, V>(A, Y, tw, c1, c2, two);
 }
 
 // One thread per (|q| class, quad): the same evaluation the kernels do on the fly.
@@ -915,7 +970,7 @@ __global__ void k_stolt_table(const __grid_constant__ AxArgs<T> A, int4* out) {
   const int ncx = A.sc.nx / 2 + 1;
   const int mx = cls % ncx, my = cls / ncx;
   const Positions<T> pos(A, mx, my);
-  Sample<T> sm[NRES];
+  Sample<T, cone<T>> sm[NRES];
   pos.quad(A, q, sm);
   const cpair<T> p0 = pos.phases(A, q, 0, sm), p1 = pos.phases(A, q, 1, sm);
   int4* row = out + size_t(cls) * (size_t(StoltTable<T>::planes) * nq) + q;
@@ -936,6 +991,24 @@ __global__ void k_stolt_table(const __grid_constant__ AxArgs<T> A, int4* out) {
   }
 }
 
+// The FP64 coefficient table, from the Stolt table's fractions.
+template <int J>
+__global__ void k_coef_table(const __grid_constant__ AxArgs<double> A, double2* out) {
+  const int q = blockIdx.x * blockDim.x + threadIdx.x, nq = A.sc.nk / NRES;
+  if (q >= nq) return;
+  const int ncx = A.sc.nx / 2 + 1, cls = blockIdx.y;
+  const Positions<double> pos(A, cls % ncx, cls / ncx);
+  Sample<double, cone<double>> sm[NRES];
+  pos.quad(A, q, sm);
+  double2* o = out + size_t(cls) * (2 * J) * nq + q;
+  for (int rho = 0; rho < NRES; ++rho) {
+    double c[J];
+    coefficients<double, J>(A.poly, sm[rho].mfl == INT_MIN ? 0.0 : sm[rho].frac, c);
+    for (int i = 0; i < J / 2; ++i)
+      o[(rho * (J / 2) + i) * nq] = make_double2(c[2 * i], c[2 * i + 1]);
+  }
+}
+
 template <typename T> cudaError_t launch_stolt_table(const AxArgs<T>& a, int4* out,
                                                      cudaStream_t s) {
   const int rows = (a.sc.ny / 2 + 1) * (a.sc.nx / 2 + 1);
@@ -946,39 +1019,54 @@ template <typename T> cudaError_t launch_stolt_table(const AxArgs<T>& a, int4* o
   return cudaGetLastError();
 }
 
+// shared memory of a pair's block (ONE: of a column's): Y and the twiddles
+template <typename T, bool ONE> static size_t ax_smem(int K) {
+  using V = column_t<T, ONE>;
+  const size_t b = size_t(padded_rows(K)) * sizeof(V) +
+                   size_t(twiddle_entries<T>(K, ilog2_dev(K))) * sizeof(cplx<T>);
+  return (b + sizeof(V) - 1) / sizeof(V) * sizeof(V);
+}
 template <typename T> size_t ax_smem_bytes(int K, int nk, bool adj) {
   (void)nk;
   (void)adj;
-  const size_t b = size_t(padded_rows(K)) * sizeof(cpair<T>) +
-                   size_t(twiddle_entries(K, ilog2_dev(K))) * sizeof(cplx<T>);
-  return (b + sizeof(cpair<T>) - 1) / sizeof(cpair<T>) * sizeof(cpair<T>);
+  return ax_smem<T, false>(K);
 }
 
-enum { AX_FWD = 0, AX_ADJ = 1, AX_FUSED = 2 };
+// AX_ADJ_RES: the adjoint of the residual of model spectra (one column a block)
+enum { AX_FWD = 0, AX_ADJ = 1, AX_FUSED = 2, AX_ADJ_RES = 3 };
+
+// FP64 runs one column per block: no shared kernel, so the pair's fused form is
+// compiled for FP32 only
+template <typename T> constexpr bool ax_one() { return sizeof(T) == 8; }
 
 template <typename T, int J, int LOGK, bool C16>
 static cudaError_t launch_ax_JKC(const AxArgs<T>& a, int npairs, cudaStream_t s, int kind) {
+  constexpr bool ONE = ax_one<T>();
+  using V = column_t<T, ONE>;
   const int K = a.sc.K;
   const int threads = K / 8;
-  size_t sm = ax_smem_bytes<T>(K, a.sc.nk, kind != AX_FWD);
+  size_t sm = ax_smem<T, ONE>(K);
   AxArgs<T> b = a;
   b.past_offset = unsigned(sm);
-  if (kind != AX_FWD) sm += size_t(a.sc.past) * sizeof(cpair<T>);
-  void (*kern)(AxArgs<T>);
-  if (kind == AX_ADJ) kern = k_ax_adj<T, J, LOGK, C16>;
-  else if (kind == AX_FWD) kern = k_ax_fwd<T, J, LOGK, C16>;
+  if (kind != AX_FWD) sm += size_t(a.sc.past) * sizeof(V);
+  void (*kern)(AxArgs<T>) = nullptr;
+  if (kind == AX_ADJ) kern = k_ax_adj<T, J, LOGK, C16, ONE, false>;
+  else if (kind == AX_FWD) kern = k_ax_fwd<T, J, LOGK, C16, ONE>;
+  else if constexpr (ONE) kern = k_ax_adj<T, J, LOGK, C16, ONE, true>;
   else kern = a.s_out ? k_ax_fused<T, J, LOGK, true, C16> : k_ax_fused<T, J, LOGK, false, C16>;
   cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, int(sm));
   // programmatic dependent launch: each axial kernel builds its twiddles while
   // the previous kernel finishes, then waits for it (cudaGridDependencySynchronize)
   cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3(npairs);
+  cfg.gridDim = dim3(ONE ? a.sc.nx * a.sc.ny : npairs);
   cfg.blockDim = dim3(threads);
   cfg.dynamicSmemBytes = sm;
   cfg.stream = s;
   cudaLaunchAttribute at[1];
   at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  at[0].val.programmaticStreamSerializationAllowed = 1;
+  // not FP64: its blocks' time is the FP64 pipe's, so two of the next grid waiting
+  // on one multiprocessor double that grid's time (128 x 512 solve: 28 ms against 10)
+  at[0].val.programmaticStreamSerializationAllowed = sizeof(T) == 4;
   cfg.attrs = at;
   cfg.numAttrs = 1;
   return cudaLaunchKernelEx(&cfg, kern, b);
@@ -1021,7 +1109,18 @@ template <typename T> cudaError_t launch_ax_adj(const AxArgs<T>& a, int npairs, 
 }
 template <typename T> cudaError_t launch_ax_fused(const AxArgs<T>& a, int npairs,
                                                   cudaStream_t s) {
-  return launch_ax<T>(a, npairs, s, AX_FUSED);
+  if constexpr (ax_one<T>()) {
+    // forward into the spectra workspace (or s_out), then the residual's adjoint
+    AxArgs<T> f = a;
+    f.out = a.s_out ? a.s_out : a.spec;
+    const cudaError_t e = launch_ax<T>(f, npairs, s, AX_FWD);
+    if (e != cudaSuccess) return e;
+    f.in = f.out;
+    f.out = a.out;
+    return launch_ax<T>(f, npairs, s, AX_ADJ_RES);
+  } else {
+    return launch_ax<T>(a, npairs, s, AX_FUSED);
+  }
 }
 
 }  // namespace isam

@@ -13,13 +13,12 @@ namespace isam {
 
 template <typename T>
 __global__ void k_dc_ifft(const T* s, cplx<T>* out, const cplx<T>* disp, const cplx<T>* post,
-                          int nk, int nz, int lognz) {
+                          const cplx<T>* roots, int nk, int nz, int lognz) {
   extern __shared__ __align__(16) unsigned char raw[];
   cplx<T>* buf = reinterpret_cast<cplx<T>*>(raw);
-  cplx<T>* tw = buf + padded_rows(nz);
   const size_t a = blockIdx.x;
   const T* x = s + a * nk;
-  build_twiddles<T>(tw, nz, lognz);
+  const cplx<T>* tw = build_twiddles<T>(buf + padded_rows(nz), roots, nz, lognz);
   for (int j = threadIdx.x; j < nz; j += blockDim.x) {
     cplx<T> v = mk<T>(0, 0);
     if (j < nk) {
@@ -37,17 +36,18 @@ __global__ void k_dc_ifft(const T* s, cplx<T>* out, const cplx<T>* disp, const c
 }
 
 template <typename T> cudaError_t launch_dc_ifft(const T* s, cplx<T>* out, const cplx<T>* disp,
-                                                 const cplx<T>* post, int nk, int nz, int lognz,
-                                                 int n_ascans, cudaStream_t st) {
+                                                 const cplx<T>* post, const cplx<T>* roots, int nk,
+                                                 int nz, int lognz, int n_ascans, cudaStream_t st) {
   const int threads = nz / 8 > 32 ? nz / 8 : 32;
-  const size_t sm = size_t(padded_rows(nz) + twiddle_entries(nz, lognz)) * sizeof(cplx<T>);
+  const size_t sm = size_t(padded_rows(nz) + twiddle_entries<T>(nz, lognz)) * sizeof(cplx<T>);
   cudaFuncSetAttribute(k_dc_ifft<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, int(sm));
-  k_dc_ifft<T><<<n_ascans, threads, sm, st>>>(s, out, disp, post, nk, nz, lognz);
+  k_dc_ifft<T><<<n_ascans, threads, sm, st>>>(s, out, disp, post, roots, nk, nz, lognz);
   return cudaGetLastError();
 }
 template cudaError_t launch_dc_ifft<float>(const float*, float2*, const float2*, const float2*,
-                                           int, int, int, int, cudaStream_t);
+                                           const float2*, int, int, int, int, cudaStream_t);
 template cudaError_t launch_dc_ifft<double>(const double*, double2*, const double2*,
-                                            const double2*, int, int, int, int, cudaStream_t);
+                                            const double2*, const double2*, int, int, int, int,
+                                            cudaStream_t);
 
 }  // namespace isam

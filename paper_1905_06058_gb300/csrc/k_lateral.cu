@@ -23,7 +23,15 @@
 
 namespace isam {
 
-int lat_tile(int L, int M) {   // pair-columns per block (a power of two)
+template <typename T> int lat_tile(int L, int M) {   // pair-columns per block (a power of two)
+  if (sizeof(T) == 8 && lat_reg_takes<T>(L, 2)) return 2;
+  // FP64 in shared memory: the smallest tile that fills a warp, for the most blocks
+  // to spread over the SMs (1024 x 2048 update: 398 us, 467 at four)
+  if (sizeof(T) == 8) {
+    int t = 1;
+    while (t < 8 && t < M / 2 && t * (L / 8) < 32) t *= 2;
+    return t;
+  }
   int tp = L >= 8 ? 4096 / L : 8;
   if (tp > 8) tp = 8;
   if (tp > M / 2) tp = M / 2;
@@ -31,6 +39,9 @@ int lat_tile(int L, int M) {   // pair-columns per block (a power of two)
   while (tp & (tp - 1)) tp &= tp - 1;
   return tp;
 }
+
+template int lat_tile<float>(int, int);
+template int lat_tile<double>(int, int);
 
 bool fft_length(int L, int* log2, int* r3) {
   if (L < 1) return false;
@@ -53,7 +64,7 @@ template <> struct rpair_t<double> { using type = double2; };
 // the stride 2^LOGTP = TP (no radix-3 pass), with constant row offsets;
 // LOGL = 0: runtime-length transforms.  The tile indexing is the same.
 template <typename T, int MODE, int LOGL, int LOGTP>
-__global__ void __launch_bounds__(512, 2) k_lat(const __grid_constant__ LatArgs<T> a) {
+__global__ void __launch_bounds__(512, std::is_same<T, float>::value ? 2 : 1) k_lat(const __grid_constant__ LatArgs<T> a) {
   using C = cplx<T>;
   using V = cpair<T>;
   using RP = typename rpair_t<T>::type;   // two adjacent reals
@@ -62,11 +73,11 @@ __global__ void __launch_bounds__(512, 2) k_lat(const __grid_constant__ LatArgs<
   const int tid = threadIdx.x, nt = blockDim.x;
   constexpr bool CT = LOGL > 0;
   const int TP = a.TZ, L = CT ? (1 << LOGL) : a.L, logTP = a.logTZ;
-  cplx<T>* tw = reinterpret_cast<cplx<T>*>(buf + size_t(padded_rows(L)) * TP);
   // programmatic dependent launch: let the next kernel start its prologue,
   // build the twiddles, then wait for the previous kernel's results
   cudaTriggerProgrammaticLaunchCompletion();
-  build_twiddles<T>(tw, L, CT ? LOGL : a.logL, CT ? 0 : a.r3);
+  const C* tw = build_twiddles<T>(reinterpret_cast<C*>(buf + size_t(padded_rows(L)) * TP), a.roots,
+                                  L, CT ? LOGL : a.logL, CT ? 0 : a.r3);
   cudaGridDependencySynchronize();
   // the solve's stop flag (written by an earlier kernel, so visible after the
   // wait): loaded here, tested before the first global write (after the first
@@ -316,7 +327,7 @@ template <typename T> size_t lat_smem_bytes(int L, int TP) {
   int lg = 0, r3 = 0;
   fft_length(L, &lg, &r3);
   return size_t(padded_rows(L)) * TP * sizeof(cpair<T>) +
-         size_t(twiddle_entries(L, lg, r3)) * sizeof(cplx<T>);
+         size_t(twiddle_entries<T>(L, lg, r3)) * sizeof(cplx<T>);
 }
 
 template <typename T, int MODE, int LOGL, int LOGTP>
@@ -333,24 +344,22 @@ static cudaError_t launch_lat_tile(const LatArgs<T>& a, cudaStream_t s) {
   cfg.stream = s;
   cudaLaunchAttribute at[1];
   at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  at[0].val.programmaticStreamSerializationAllowed = 1;
+  at[0].val.programmaticStreamSerializationAllowed = sizeof(T) == 4;   // as the axial kernels
   cfg.attrs = at;
   cfg.numAttrs = 1;
   return cudaLaunchKernelEx(&cfg, kern, a);
 }
 
-// FP32 passes at the built-in tile of the lengths that have a register form take
-// it (k_lateral_reg.cu) unless the plan chose radix 8 (a.radix16 = 0).  That form
-// of the solve's passes runs compile-time-length transforms at (L, pair-columns) =
+// Passes at the built-in tile of the lengths that have a register form take it
+// (k_lateral_reg.cuh) unless the plan chose radix 8 (a.radix16 = 0).  That form of
+// the FP32 solve's passes runs compile-time-length transforms at (L, pair-columns) =
 // (1024, 4), (512, 8) and (256, 8); every other case the runtime-length ones.
 template <typename T, int MODE>
 static cudaError_t launch_lat_mode(const LatArgs<T>& a, cudaStream_t s) {
   constexpr bool hot = std::is_same<T, float>::value &&
                        (MODE == LAT_UPDATE || MODE == LAT_UPDATE_U || MODE == LAT_C2C_FWD ||
                         MODE == LAT_C2C_INV);
-  if constexpr (std::is_same<T, float>::value) {
-    if (a.radix16 && lat_reg_takes(a.L, a.TZ)) return launch_lat_reg(MODE, a, s);
-  }
+  if (a.radix16 && lat_reg_takes<T>(a.L, a.TZ)) return launch_lat_reg<T>(MODE, a, s);
   if constexpr (hot) {
     if (!a.r3 && a.L == 1024 && a.TZ == 4) return launch_lat_tile<T, MODE, 10, 2>(a, s);
     if (!a.r3 && a.L == 512 && a.TZ == 8) return launch_lat_tile<T, MODE, 9, 3>(a, s);

@@ -1,203 +1,9 @@
-// k_lat's modes for FP32 with the tile in registers (lat_reg.cuh).
-//
-// What bounds it: the update's four global streams (u_hat, z^{k-1} in; z^k,
-// eta_hat^{k+1} out), 67 MB at 1024 x 2048 out of the L2.  256 blocks of 256
-// threads, two on a multiprocessor (128 registers: 32 points of data, 8 of
-// z^{k-1} in flight).  The iterates are loaded in batches of eight, the first
-// before the last exchange's barrier so that its latency covers the exchange.
-#include <type_traits>
-
-#include "lat_point.cuh"
-#include "lat_reg.cuh"
+// FP32 instances of the lateral passes with the tile in registers.
+#include "k_lateral_reg.cuh"
 
 namespace isam {
 
-template <int L, int W> __host__ __device__ constexpr int lat_reg_threads() {
-  return lreg::threads_per_column<L>() * W;
-}
-template <int L, int W> __host__ __device__ constexpr int lat_reg_min_blocks() {
-  constexpr int regs = lreg::Plan<L>::P == 32 ? 128 : lreg::Plan<L>::P == 24 ? 112 : 80;
-  constexpr int n = 65536 / (regs * lat_reg_threads<L, W>());
-  return n > 16 ? 16 : n;
-}
-
-template <int MODE, int L, int W>
-__global__ void __launch_bounds__(lat_reg_threads<L, W>(), lat_reg_min_blocks<L, W>())
-    k_lat_reg(const __grid_constant__ LatArgs<float> a) {
-  constexpr int P = lreg::Plan<L>::P, T = L / P, NT = lat_reg_threads<L, W>();
-  // iterates in flight: eight points of z^{k-1}, or four of z^{k-1} and z^{k-2}
-  constexpr int BATCH = MODE == LAT_UPDATE ? 4 : 8;
-  static_assert(P % BATCH == 0, "the iterates are loaded in whole batches");
-  extern __shared__ __align__(16) unsigned char smem_raw[];
-  float2* S = reinterpret_cast<float2*>(smem_raw);
-  const int tid = threadIdx.x, c = tid % W, b = tid / W;
-  // programmatic dependent launch: let the next kernel start its prologue,
-  // build the twiddles, then wait for the previous kernel's results
-  cudaTriggerProgrammaticLaunchCompletion();
-  const lreg::Twiddles<L> tw(b);
-  cudaGridDependencySynchronize();
-  // the solve's stop flag (written by an earlier kernel, so visible after the
-  // wait): loaded here, tested before the first global write
-  const bool stopped = a.stop != nullptr && __ldcg(a.stop) != 0;
-  const size_t M = size_t(a.M), step = M * T;          // rows b + i T of the thread
-  const size_t g0 = size_t(blockIdx.y) * L * M + size_t(b) * M + size_t(blockIdx.x) * W + c;
-  const float nrm = a.norm;
-  auto nothing = [] {};
-
-  float2 v[P];
-#pragma unroll
-  for (int i = 0; i < P; ++i) {
-    const size_t g = g0 + i * step;
-    if constexpr (MODE == LAT_R2C_FWD) {
-      v[i] = make_float2(static_cast<const float*>(a.in)[g], 0.0f);
-    } else if constexpr (MODE == LAT_EXTRAP_FWD) {
-      const float2 z1 = a.z1[g];
-      v[i] = cadd(z1, cscale(csub(z1, a.z2[g]), a.mu));
-    } else {
-      v[i] = static_cast<const float2*>(a.in)[g];
-    }
-  }
-  constexpr bool UPDATE = MODE == LAT_UPDATE || MODE == LAT_UPDATE_U;
-  constexpr bool FROM_U = MODE == LAT_UPDATE_U;
-  constexpr bool EARLY = FROM_U || MODE == LAT_GRAD_STEP;   // first batch before the barrier
-  float2 z1v[BATCH], z2v[BATCH];
-  auto load_iterates = [&](int h) {
-#pragma unroll
-    for (int i = 0; i < BATCH; ++i) {
-      z1v[i] = a.z1[g0 + (h + i) * step];
-      if constexpr (!FROM_U) z2v[i] = a.z2[g0 + (h + i) * step];
-    }
-  };
-  if constexpr (MODE == LAT_C2C_FWD || MODE == LAT_R2C_FWD || MODE == LAT_EXTRAP_FWD)
-    lreg::transform<-1, L, W>(v, S, tw, b, c, true, nothing);
-  else if constexpr (EARLY)
-    lreg::transform<+1, L, W>(v, S, tw, b, c, true, [&] { load_iterates(0); });
-  else
-    lreg::transform<+1, L, W>(v, S, tw, b, c, true, nothing);
-  if (stopped) return;   // an earlier check stopped the solve: write nothing
-
-  if constexpr (MODE == LAT_INV_REAL) {
-    float* out = static_cast<float*>(a.out);
-#pragma unroll
-    for (int i = 0; i < P; ++i) out[g0 + i * step] = v[i].x * nrm;
-  }
-  float2* out = static_cast<float2*>(a.out);
-  if constexpr (MODE == LAT_GRAD_STEP) {
-    // u = eta^k - g/L with eta^k = z1 + mu_prev (z1 - z2), written to out
-    const float sg = nrm * a.inv_L;
-    bool bad = false;
-#pragma unroll
-    for (int h = 0; h < P; h += BATCH) {
-      if (h || !EARLY) load_iterates(h);
-#pragma unroll
-      for (int i = 0; i < BATCH; ++i) {
-        const float2 eta = cadd(z1v[i], cscale(csub(z1v[i], z2v[i]), a.mu_prev));
-        const float2 u = csub(eta, cscale(v[h + i], sg));
-        out[g0 + (h + i) * step] = u;
-        bad |= !(isfinite(u.x) && isfinite(u.y));
-      }
-    }
-    if (bad) atomicOr(a.flag, 1);
-  }
-  if constexpr (UPDATE) {
-    // the FISTA step of k_lat: LAT_UPDATE forms u = eta^k - g/L from the gradient,
-    // LAT_UPDATE_U transformed u itself; norm partials as there (a thread's points
-    // in float, the block's threads in double)
-    float acc0 = 0.0f, acc1 = 0.0f, acc2 = 0.0f;
-    bool bad = false;
-    const float sg = nrm * a.inv_L;
-    float tau = a.lam_dev ? float(a.lam_scale * *a.lam_dev) : a.lam_over_L;
-    if (a.w) tau *= a.w[(size_t(blockIdx.x) * W + c) & size_t(a.nz - 1)];
-#pragma unroll
-    for (int h = 0; h < P; h += BATCH) {
-      if (h || !EARLY) load_iterates(h);
-#pragma unroll
-      for (int i = 0; i < BATCH; ++i) {
-        const size_t g = g0 + (h + i) * step;
-        const float2 z1 = z1v[i];
-        float2 gr, eta, u;
-        if constexpr (FROM_U) {
-          u = cscale(v[h + i], nrm);
-        } else {
-          gr = cscale(v[h + i], sg);                       // g^k = (1/L) A^H(A eta - s)
-          eta = cadd(z1, cscale(csub(z1, z2v[i]), a.mu_prev));
-          u = csub(eta, gr);
-        }
-        if (a.uout) a.uout[g] = u;
-        const float2 z = soft_threshold(u, tau);
-        a.zout[g] = z;
-        v[h + i] = cadd(z, cscale(csub(z, z1), a.mu));
-        if constexpr (!FROM_U) {
-          if (a.partial) {
-            const float2 d = csub(z, eta);
-            const float2 dg = cadd(d, gr);
-            acc0 += d.x * d.x + d.y * d.y;
-            acc1 += gr.x * gr.x + gr.y * gr.y;
-            acc2 += dg.x * dg.x + dg.y * dg.y;
-          }
-        }
-        bad |= !(isfinite(z.x) && isfinite(z.y));
-      }
-    }
-    if (bad) atomicOr(a.flag, 1);
-    lreg::transform<-1, L, W>(v, S, tw, b, c, false, nothing);
-    if constexpr (!FROM_U) {
-      if (a.partial != nullptr) {
-        __shared__ double red[3][NT / 32];
-        const int wid = tid >> 5, lane = tid & 31;
-        const double w0 = warp_sum_lanes(double(acc0), 32);
-        const double w1 = warp_sum_lanes(double(acc1), 32);
-        const double w2 = warp_sum_lanes(double(acc2), 32);
-        if (lane == 0) { red[0][wid] = w0; red[1][wid] = w1; red[2][wid] = w2; }
-        __syncthreads();
-        if (tid < 3) {
-          double s = 0.0;
-          for (int w = 0; w < NT / 32; ++w) s += red[tid][w];
-          a.partial[3 * (size_t(blockIdx.y) * gridDim.x + blockIdx.x) + tid] = s;
-        }
-      }
-    }
-  }
-  if constexpr (MODE != LAT_INV_REAL && MODE != LAT_GRAD_STEP) {
-#pragma unroll
-    for (int i = 0; i < P; ++i) out[g0 + i * step] = cscale(v[i], nrm);
-  }
-}
-
-template <int MODE, int L, int W>
-static cudaError_t launch_one(const LatArgs<float>& a, cudaStream_t s) {
-  auto* kern = k_lat_reg<MODE, L, W>;
-  constexpr size_t sm = lreg::smem_bytes<L, W>();
-  cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, int(sm));
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3(a.M / W, a.B);
-  cfg.blockDim = dim3(lat_reg_threads<L, W>());
-  cfg.dynamicSmemBytes = sm;
-  cfg.stream = s;
-  cudaLaunchAttribute at[1];
-  at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  at[0].val.programmaticStreamSerializationAllowed = 1;
-  cfg.attrs = at;
-  cfg.numAttrs = 1;
-  return cudaLaunchKernelEx(&cfg, kern, a);
-}
-
-template <int L, int W>
-static cudaError_t launch_modes(int mode, const LatArgs<float>& a, cudaStream_t s) {
-  switch (mode) {
-    case LAT_C2C_FWD: return launch_one<LAT_C2C_FWD, L, W>(a, s);
-    case LAT_C2C_INV: return launch_one<LAT_C2C_INV, L, W>(a, s);
-    case LAT_R2C_FWD: return launch_one<LAT_R2C_FWD, L, W>(a, s);
-    case LAT_INV_REAL: return launch_one<LAT_INV_REAL, L, W>(a, s);
-    case LAT_UPDATE: return launch_one<LAT_UPDATE, L, W>(a, s);
-    case LAT_GRAD_STEP: return launch_one<LAT_GRAD_STEP, L, W>(a, s);
-    case LAT_EXTRAP_FWD: return launch_one<LAT_EXTRAP_FWD, L, W>(a, s);
-    case LAT_UPDATE_U: return launch_one<LAT_UPDATE_U, L, W>(a, s);
-  }
-  return cudaErrorInvalidValue;
-}
-
-bool lat_reg_takes(int L, int TZ) {
+template <> bool lat_reg_takes<float>(int L, int TZ) {
   switch (L) {
     case 1024: case 768: return TZ == 4;
     case 512: case 384: case 256: case 192: case 128: case 64: return TZ == 8;
@@ -205,16 +11,16 @@ bool lat_reg_takes(int L, int TZ) {
   return false;
 }
 
-cudaError_t launch_lat_reg(int mode, const LatArgs<float>& a, cudaStream_t s) {
+template <> cudaError_t launch_lat_reg<float>(int mode, const LatArgs<float>& a, cudaStream_t s) {
   switch (a.L) {
-    case 1024: return launch_modes<1024, 8>(mode, a, s);
-    case 768: return launch_modes<768, 8>(mode, a, s);
-    case 512: return launch_modes<512, 16>(mode, a, s);
-    case 384: return launch_modes<384, 16>(mode, a, s);
-    case 256: return launch_modes<256, 16>(mode, a, s);
-    case 192: return launch_modes<192, 16>(mode, a, s);
-    case 128: return launch_modes<128, 16>(mode, a, s);
-    case 64: return launch_modes<64, 16>(mode, a, s);
+    case 1024: return launch_lat_reg_length<float, 1024>(mode, a, s);
+    case 768: return launch_lat_reg_length<float, 768>(mode, a, s);
+    case 512: return launch_lat_reg_length<float, 512>(mode, a, s);
+    case 384: return launch_lat_reg_length<float, 384>(mode, a, s);
+    case 256: return launch_lat_reg_length<float, 256>(mode, a, s);
+    case 192: return launch_lat_reg_length<float, 192>(mode, a, s);
+    case 128: return launch_lat_reg_length<float, 128>(mode, a, s);
+    case 64: return launch_lat_reg_length<float, 64>(mode, a, s);
   }
   return cudaErrorInvalidValue;
 }

@@ -1,0 +1,212 @@
+// k_lat's modes with the tile in registers (lat_reg.cuh); instances in
+// k_lateral_reg.cu (FP32) and k_lateral_reg_f64.cu.
+//
+// What bounds the FP32 form: the update's four global streams (u_hat, z^{k-1} in; z^k,
+// eta_hat^{k+1} out), 67 MB at 1024 x 2048 out of the L2.  256 blocks of 256
+// threads, two on a multiprocessor (128 registers: 32 points of data, 8 of
+// z^{k-1} in flight).  The iterates are loaded in batches of eight, the first
+// before the last exchange's barrier so that its latency covers the exchange.
+#pragma once
+
+#include <type_traits>
+
+#include "lat_point.cuh"
+#include "lat_reg.cuh"
+
+namespace isam {
+
+template <typename T, int L> __host__ __device__ constexpr int lat_reg_threads() {
+  return lreg::threads_per_column<T, L>() * lreg::columns<T, L>();
+}
+template <typename T, int L> __host__ __device__ constexpr int lat_reg_min_blocks() {
+  constexpr int P = lreg::Plan<T, L>::P;
+  constexpr int regs = sizeof(T) == 8 ? 128 : P == 32 ? 128 : P == 24 ? 112 : 80;
+  constexpr int n = 65536 / (regs * lat_reg_threads<T, L>());
+  return n > 16 ? 16 : n;
+}
+
+template <typename T, int MODE, int L>
+__global__ void __launch_bounds__(lat_reg_threads<T, L>(), lat_reg_min_blocks<T, L>())
+    k_lat_reg(const __grid_constant__ LatArgs<T> a) {
+  using C = cplx<T>;
+  constexpr int P = lreg::Plan<T, L>::P, TH = L / P, NT = lat_reg_threads<T, L>();
+  constexpr int W = lreg::columns<T, L>();
+  // iterates in flight: eight points of z^{k-1}, or four of z^{k-1} and z^{k-2}
+  constexpr int BATCH = MODE == LAT_UPDATE ? 4 : 8;
+  static_assert(P % BATCH == 0, "the iterates are loaded in whole batches");
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  C* S = reinterpret_cast<C*>(smem_raw);
+  const int tid = threadIdx.x, c = tid % W, b = tid / W;
+  // programmatic dependent launch: build the twiddles, then wait for the previous
+  // kernel's results.  The plain transforms let the next kernel start its prologue
+  // at once (A + A^H at 1024 x 2048: 72 us against 75), the solve's passes only
+  // before their last transform or stores (see k_ax_fused).
+  constexpr bool PLAIN = MODE == LAT_C2C_FWD || MODE == LAT_C2C_INV || MODE == LAT_R2C_FWD ||
+                         MODE == LAT_INV_REAL;
+  if constexpr (PLAIN) cudaTriggerProgrammaticLaunchCompletion();
+  const lreg::Twiddles<T, L> tw(b, a.roots);
+  cudaGridDependencySynchronize();
+  // the solve's stop flag (written by an earlier kernel, so visible after the
+  // wait): loaded here, tested before the first global write
+  const bool stopped = a.stop != nullptr && __ldcg(a.stop) != 0;
+  const size_t M = size_t(a.M), step = M * TH;         // rows b + i TH of the thread
+  const size_t g0 = size_t(blockIdx.y) * L * M + size_t(b) * M + size_t(blockIdx.x) * W + c;
+  const T nrm = a.norm;
+  auto nothing = [] {};
+
+  C v[P];
+#pragma unroll
+  for (int i = 0; i < P; ++i) {
+    const size_t g = g0 + i * step;
+    if constexpr (MODE == LAT_R2C_FWD) {
+      v[i] = mk<T>(static_cast<const T*>(a.in)[g], T(0));
+    } else if constexpr (MODE == LAT_EXTRAP_FWD) {
+      const C z1 = a.z1[g];
+      v[i] = cadd(z1, cscale(csub(z1, a.z2[g]), a.mu));
+    } else {
+      v[i] = static_cast<const C*>(a.in)[g];
+    }
+  }
+  constexpr bool UPDATE = MODE == LAT_UPDATE || MODE == LAT_UPDATE_U;
+  constexpr bool FROM_U = MODE == LAT_UPDATE_U;
+  constexpr bool EARLY = FROM_U || MODE == LAT_GRAD_STEP;   // first batch before the barrier
+  C z1v[BATCH], z2v[BATCH];
+  auto load_iterates = [&](int h) {
+#pragma unroll
+    for (int i = 0; i < BATCH; ++i) {
+      z1v[i] = a.z1[g0 + (h + i) * step];
+      if constexpr (!FROM_U) z2v[i] = a.z2[g0 + (h + i) * step];
+    }
+  };
+  if constexpr (MODE == LAT_C2C_FWD || MODE == LAT_R2C_FWD || MODE == LAT_EXTRAP_FWD)
+    lreg::transform<-1, L, 0, T>(v, S, tw, b, c, true, nothing);
+  else if constexpr (EARLY)
+    lreg::transform<+1, L, 0, T>(v, S, tw, b, c, true, [&] { load_iterates(0); });
+  else
+    lreg::transform<+1, L, 0, T>(v, S, tw, b, c, true, nothing);
+  if constexpr (!PLAIN && !UPDATE) cudaTriggerProgrammaticLaunchCompletion();
+  if (stopped) return;   // an earlier check stopped the solve: write nothing
+
+  if constexpr (MODE == LAT_INV_REAL) {
+    T* out = static_cast<T*>(a.out);
+#pragma unroll
+    for (int i = 0; i < P; ++i) out[g0 + i * step] = v[i].x * nrm;
+  }
+  C* out = static_cast<C*>(a.out);
+  if constexpr (MODE == LAT_GRAD_STEP) {
+    // u = eta^k - g/L with eta^k = z1 + mu_prev (z1 - z2), written to out
+    const T sg = nrm * a.inv_L;
+    bool bad = false;
+#pragma unroll
+    for (int h = 0; h < P; h += BATCH) {
+      if (h || !EARLY) load_iterates(h);
+#pragma unroll
+      for (int i = 0; i < BATCH; ++i) {
+        const C eta = cadd(z1v[i], cscale(csub(z1v[i], z2v[i]), a.mu_prev));
+        const C u = csub(eta, cscale(v[h + i], sg));
+        out[g0 + (h + i) * step] = u;
+        bad |= !(isfinite(u.x) && isfinite(u.y));
+      }
+    }
+    if (bad) atomicOr(a.flag, 1);
+  }
+  if constexpr (UPDATE) {
+    // the FISTA step of k_lat: LAT_UPDATE forms u = eta^k - g/L from the gradient,
+    // LAT_UPDATE_U transformed u itself; norm partials as there (a thread's points
+    // in the plan's precision, the block's threads in double)
+    T acc0 = T(0), acc1 = T(0), acc2 = T(0);
+    bool bad = false;
+    const T sg = nrm * a.inv_L;
+    T tau = a.lam_dev ? T(a.lam_scale * *a.lam_dev) : a.lam_over_L;
+    if (a.w) tau *= a.w[(size_t(blockIdx.x) * W + c) & size_t(a.nz - 1)];
+#pragma unroll
+    for (int h = 0; h < P; h += BATCH) {
+      if (h || !EARLY) load_iterates(h);
+#pragma unroll
+      for (int i = 0; i < BATCH; ++i) {
+        const size_t g = g0 + (h + i) * step;
+        const C z1 = z1v[i];
+        C gr, eta, u;
+        if constexpr (FROM_U) {
+          u = cscale(v[h + i], nrm);
+        } else {
+          gr = cscale(v[h + i], sg);                       // g^k = (1/L) A^H(A eta - s)
+          eta = cadd(z1, cscale(csub(z1, z2v[i]), a.mu_prev));
+          u = csub(eta, gr);
+        }
+        if (a.uout) a.uout[g] = u;
+        const C z = soft_threshold(u, tau);
+        a.zout[g] = z;
+        v[h + i] = cadd(z, cscale(csub(z, z1), a.mu));
+        if constexpr (!FROM_U) {
+          if (a.partial) {
+            const C d = csub(z, eta);
+            const C dg = cadd(d, gr);
+            acc0 += d.x * d.x + d.y * d.y;
+            acc1 += gr.x * gr.x + gr.y * gr.y;
+            acc2 += dg.x * dg.x + dg.y * dg.y;
+          }
+        }
+        bad |= !(isfinite(z.x) && isfinite(z.y));
+      }
+    }
+    if (bad) atomicOr(a.flag, 1);
+    cudaTriggerProgrammaticLaunchCompletion();
+    lreg::transform<-1, L, 0, T>(v, S, tw, b, c, false, nothing);
+    if constexpr (!FROM_U) {
+      if (a.partial != nullptr) {
+        __shared__ double red[3][NT / 32];
+        const int wid = tid >> 5, lane = tid & 31;
+        const double w0 = warp_sum_lanes(double(acc0), 32);
+        const double w1 = warp_sum_lanes(double(acc1), 32);
+        const double w2 = warp_sum_lanes(double(acc2), 32);
+        if (lane == 0) { red[0][wid] = w0; red[1][wid] = w1; red[2][wid] = w2; }
+        __syncthreads();
+        if (tid < 3) {
+          double s = 0.0;
+          for (int w = 0; w < NT / 32; ++w) s += red[tid][w];
+          a.partial[3 * (size_t(blockIdx.y) * gridDim.x + blockIdx.x) + tid] = s;
+        }
+      }
+    }
+  }
+  if constexpr (MODE != LAT_INV_REAL && MODE != LAT_GRAD_STEP) {
+#pragma unroll
+    for (int i = 0; i < P; ++i) out[g0 + i * step] = cscale(v[i], nrm);
+  }
+}
+
+template <typename T, int MODE, int L>
+static cudaError_t launch_lat_reg_mode(const LatArgs<T>& a, cudaStream_t s) {
+  auto* kern = k_lat_reg<T, MODE, L>;
+  constexpr size_t sm = lreg::smem_bytes<T, L>();
+  cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, int(sm));
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(a.M / lreg::columns<T, L>(), a.B);
+  cfg.blockDim = dim3(lat_reg_threads<T, L>());
+  cfg.dynamicSmemBytes = sm;
+  cfg.stream = s;
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at[0].val.programmaticStreamSerializationAllowed = sizeof(T) == 4;   // as the axial kernels
+  cfg.attrs = at;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, kern, a);
+}
+
+template <typename T, int L>
+static cudaError_t launch_lat_reg_length(int mode, const LatArgs<T>& a, cudaStream_t s) {
+  switch (mode) {
+    case LAT_C2C_FWD: return launch_lat_reg_mode<T, LAT_C2C_FWD, L>(a, s);
+    case LAT_C2C_INV: return launch_lat_reg_mode<T, LAT_C2C_INV, L>(a, s);
+    case LAT_R2C_FWD: return launch_lat_reg_mode<T, LAT_R2C_FWD, L>(a, s);
+    case LAT_INV_REAL: return launch_lat_reg_mode<T, LAT_INV_REAL, L>(a, s);
+    case LAT_UPDATE: return launch_lat_reg_mode<T, LAT_UPDATE, L>(a, s);
+    case LAT_GRAD_STEP: return launch_lat_reg_mode<T, LAT_GRAD_STEP, L>(a, s);
+    case LAT_EXTRAP_FWD: return launch_lat_reg_mode<T, LAT_EXTRAP_FWD, L>(a, s);
+    case LAT_UPDATE_U: return launch_lat_reg_mode<T, LAT_UPDATE_U, L>(a, s);
+  }
+  return cudaErrorInvalidValue;
+}
+
+}  // namespace isam

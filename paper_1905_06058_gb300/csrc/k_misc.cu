@@ -307,6 +307,18 @@ template <typename Tsrc, typename Tdst> cudaError_t launch_convert(const cplx<Ts
 template cudaError_t launch_convert<float, double>(const float2*, double2*, size_t, cudaStream_t);
 template cudaError_t launch_convert<double, float>(const double2*, float2*, size_t, cudaStream_t);
 
+__global__ void k_roots(double2* out, int n) {
+  const int m = blockIdx.x * blockDim.x + threadIdx.x;
+  if (m >= n) return;
+  double s, c;
+  sincospi(2.0 * double(m) / double(n), &s, &c);
+  out[m] = make_double2(c, -s);
+}
+cudaError_t launch_roots(double2* out, int n, cudaStream_t s) {
+  k_roots<<<(n + 127) / 128, 128, 0, s>>>(out, n);
+  return cudaGetLastError();
+}
+
 // deterministic start vector: splitmix64 of the index, uniform in [-0.5, 0.5)
 __device__ __forceinline__ double hash01(uint64_t x) {
   x += 0x9E3779B97F4A7C15ull;

@@ -1,5 +1,6 @@
-"""The FP32 lateral passes that keep their tile in registers, at every length
-they take (64 to 1024, 2^p and 3 * 2^p), along x and along y of a volume.
+"""The lateral passes that keep their tile in registers, at every length they take
+(FP32: 64 to 1024, 2^p and 3 * 2^p; FP64: 64 to 512, 2^p), along x and along y of a
+volume.
 
 A and A^H go through the complex, real-input and real-output passes and are
 compared with the oracle (1e-5 relative L2, the bar of test_gpu_operator.py).
@@ -7,7 +8,8 @@ The passes of the solve (update from u_hat with depth weights, update with the
 norm partials of the stop rule, gradient step and extrapolation of the other
 priors) are compared with the radix-8 shared-memory form of the same plan, which
 is the same arithmetic in another order: 1e-5 on the image as in
-test_gpu_autotune.py, and 1e-3 on r_r, the bar of test_gpu_stop_rule.py."""
+test_gpu_autotune.py, and 1e-3 on r_r, the bar of test_gpu_stop_rule.py.  FP64:
+1e-10 (test_gpu_operator.py) for all of them."""
 import numpy as np
 import pytest
 
@@ -72,4 +74,29 @@ def test_solve_passes_match_radix8(torch, L, along_y):
             got.append((out.cpu().numpy(), info["rr"]))
         assert rel(got[0][0], got[1][0]) < 1e-5
         assert got[0][1] == pytest.approx(got[1][1], rel=1e-3)
+    plan.close()
+
+
+@pytest.mark.parametrize("along_y", [False, True], ids=["x", "y"])
+@pytest.mark.parametrize("L", [64, 128, 256, 512])
+def test_fp64(torch, L, along_y):
+    from paper_1905_06058_gb300.isam import Plan
+    g = I.small_bscan(seed=65, **shape(L, along_y)).geom
+    ref = O.IsamOracle(g, "nufft")
+    eta = I.random_image(ref.image_shape, 66)
+    y = I.random_spectra(ref.spec_shape, 67)
+    plan = Plan(g, precision="fp64")
+    s = plan.forward(torch.from_numpy(eta).cuda())
+    assert rel(s.cpu().numpy(), ref.forward(eta)) < 1e-10
+    assert rel(plan.adjoint(torch.from_numpy(y).cuda()).cpu().numpy(), ref.adjoint(y)) < 1e-10
+    w = torch.from_numpy(I.depth_weights(plan.image_shape[2])).cuda()
+    for kw in (dict(max_iter=5, w=w), dict(max_iter=5, w=w, tol=1e-300, check_every=2),
+               dict(max_iter=3, prior="haar_depth")):
+        got = []
+        for r in (16, 8):
+            plan.set_tuning(lateral_radix=r)
+            out, info = plan.solve(s, lambda_rel=0.02, L=4.0, **kw)
+            got.append((out.cpu().numpy(), info["rr"]))
+        assert rel(got[0][0], got[1][0]) < 1e-10
+        assert got[0][1] == pytest.approx(got[1][1], rel=1e-10)
     plan.close()
