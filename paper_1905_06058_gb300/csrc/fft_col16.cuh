@@ -29,6 +29,15 @@ enum { P8 = 8, P16 = 16 };
 template <int PAD> __device__ __forceinline__ int el(int row, int c) {
   return 2 * (PAD == P8 ? row + (row >> 3) : row + (row >> 4)) + c;
 }
+// ... of (row + STEP r, c), given e = el(row, c): a constant distance, which the
+// compiler does not find through the shift (left to it, the index arithmetic of the
+// passes was a tenth of k_ax_fused's instructions).  STEP is a multiple of the
+// padding period, or the rows row .. row + STEP r stay within one (row a multiple
+// of 16, STEP 1, r < 16 in P16).
+template <int PAD, int STEP> __device__ __forceinline__ constexpr int el_step(int r) {
+  static_assert(STEP % PAD == 0 || (STEP == 1 && PAD == P16), "a constant distance in the layout");
+  return STEP % PAD == 0 ? 2 * r * (STEP + STEP / PAD) : 2 * r;
+}
 
 // multiply by W16^1 = e^{SIGN 2 pi i / 16} and W16^3
 template <int SIGN> __device__ __forceinline__ float2 w16_1(float2 o) {
@@ -149,9 +158,9 @@ __device__ __forceinline__ void pass(float2* Y, int b, int c, const float4* tw) 
   float2 v[16];
 #pragma unroll
   for (int u = 0; u < NB; ++u) {
-    const int j = b + u * L16;
+    const float2* in = Y + el<IN>(b + u * L16, c);
 #pragma unroll
-    for (int r = 0; r < R; ++r) v[u * R + r] = Y[el<IN>(j + r * LR, c)];
+    for (int r = 0; r < R; ++r) v[u * R + r] = in[el_step<IN, LR>(r)];
   }
   __syncthreads();
 #pragma unroll
@@ -161,9 +170,9 @@ __device__ __forceinline__ void pass(float2* Y, int b, int c, const float4* tw) 
     float2* a = v + u * R;
     if (NS > 1) twiddle<SIGN, R>(a, tw[k]);
     dft_r<SIGN, R>(a);
-    const int base = (j - k) * R + k;
+    float2* out = Y + el<OUT>((j - k) * R + k, c);
 #pragma unroll
-    for (int r = 0; r < R; ++r) Y[el<OUT>(base + r * NS, c)] = a[r];
+    for (int r = 0; r < R; ++r) out[el_step<OUT, NS>(r)] = a[r];
   }
   __syncthreads();
 }
@@ -186,8 +195,9 @@ __device__ __forceinline__ void forward(float2* Y, const float2* x, const float*
     a[i < 4 ? i + 12 : i - 4] = x ? cscale(x[n], __ldg(scale + n)) : make_float2(0.0f, 0.0f);
   }
   dft16<+1, true>(a);
+  float2* out = Y + el<P16>(16 * j, c);
 #pragma unroll
-  for (int r = 0; r < 16; ++r) Y[el<P16>(16 * j + r, c)] = a[r];
+  for (int r = 0; r < 16; ++r) out[el_step<P16, 1>(r)] = a[r];
   __syncthreads();
   pass<+1, 16, K, 16, P16, P16>(Y, j, c, tw);
   pass<+1, Passes<LOGK>::R3, K, 256, P16, P8>(Y, j, c, tw + 16);
@@ -205,9 +215,10 @@ __device__ __forceinline__ void inverse(float2* Y, const float4* tw, Emit emit) 
 #pragma unroll
   for (int u = 0; u < NB; ++u) {
     const int jj = j + u * K16;          // jj < 256 = NS: k = jj, output rows jj + 256 r
+    const float2* in = Y + el<P16>(jj, c);
     float2 a[R];
 #pragma unroll
-    for (int r = 0; r < R; ++r) a[r] = Y[el<P16>(jj + r * LR, c)];
+    for (int r = 0; r < R; ++r) a[r] = in[el_step<P16, LR>(r)];
     twiddle<-1, R>(a, tw[16 + jj]);
     dft_r<-1, R>(a);
 #pragma unroll

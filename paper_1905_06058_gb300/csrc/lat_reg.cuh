@@ -173,6 +173,13 @@ template <typename T, int L> __device__ __forceinline__ int slot(int row, int c)
   if constexpr (padded<T, L>()) return (row + row / Plan<T, L>::R0) * W + c;
   else return row * W + c;
 }
+// ... of (row + STEP r, c) less that of (row, c), for a STEP that is a multiple of
+// the padding period or r < R0 rows from a multiple of it: a constant
+template <typename T, int L, int STEP> __device__ __forceinline__ constexpr int slot_step(int r) {
+  constexpr int W = columns<T, L>(), R0 = Plan<T, L>::R0;
+  static_assert(!padded<T, L>() || STEP == 1 || STEP % R0 == 0, "a constant distance");
+  return (padded<T, L>() && STEP % R0 == 0 ? r * (STEP + STEP / R0) : r * STEP) * W;
+}
 template <typename T, int L> __host__ __device__ constexpr size_t smem_bytes() {
   return size_t(padded<T, L>() ? L + L / Plan<T, L>::R0 : L) * columns<T, L>() * sizeof(cplx<T>);
 }
@@ -253,14 +260,15 @@ __device__ __forceinline__ void transform(cplx<T>* v, cplx<T>* S, const Twiddles
     const int k = b % NS;
 #pragma unroll
     for (int u = 0; u < NB; ++u) {
-      const int base = (b + u * TH - k) * R + k;
+      cplx<T>* out = S + slot<T, L>((b + u * TH - k) * R + k, c);
 #pragma unroll
-      for (int r = 0; r < R; ++r) S[slot<T, L>(base + r * NS, c)] = a[u][r];
+      for (int r = 0; r < R; ++r) out[slot_step<T, L, NS>(r)] = a[u][r];
     }
     if constexpr (PASS == Pl::N - 2) before();
     __syncthreads();
+    const cplx<T>* in = S + slot<T, L>(b, c);
 #pragma unroll
-    for (int i = 0; i < P; ++i) v[i] = S[slot<T, L>(b + i * TH, c)];
+    for (int i = 0; i < P; ++i) v[i] = in[slot_step<T, L, TH>(i)];
     transform<SIGN, L, PASS + 1, T>(v, S, tw, b, c, false, before);
   }
 }
