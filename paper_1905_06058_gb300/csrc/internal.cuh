@@ -229,7 +229,7 @@ template <typename T> cudaError_t launch_bwd_combine(const cplx<T>* ubar, const 
                                                      size_t n, cudaStream_t s);
 
 // prox of tau ||details(W u)||_1, W the orthonormal Haar transform along depth
-// of each A-scan (k_lateral.cu); tau = lam_scale * (*lam_dev) when lam_dev
+// of each A-scan (k_prior.cu); tau = lam_scale * (*lam_dev) when lam_dev
 template <typename T> cudaError_t launch_haar_prox(const cplx<T>* u, cplx<T>* z, int nz,
                                                    size_t n_ascans, T tau, const double* lam_dev,
                                                    double lam_scale, cudaStream_t s);

@@ -268,61 +268,6 @@ __global__ void __launch_bounds__(512, std::is_same<T, float>::value ? 2 : 1) k_
   }
 }
 
-// prox of tau ||details(W u)||_1 per A-scan (nz contiguous samples), W the
-// orthonormal Haar transform along depth: in-place lifting levels with
-// stride h = 1, 2, .., nz/2 (pair (i, i + h), i a multiple of 2h, becomes
-// ((x_i + x_{i+h})/sqrt 2, (x_i - x_{i+h})/sqrt 2)), the complex soft
-// threshold on every coefficient but the approximation (index 0), and the
-// same butterflies in reverse order, which invert them.
-template <typename T>
-__global__ void k_haar_prox(const cplx<T>* u, cplx<T>* z, int nz, T tau, const double* lam_dev,
-                            double lam_scale) {
-  extern __shared__ __align__(16) unsigned char raw[];
-  cplx<T>* x = reinterpret_cast<cplx<T>*>(raw);
-  const size_t col = blockIdx.x;
-  const int tid = threadIdx.x, nt = blockDim.x;
-  for (int i = tid; i < nz; i += nt) x[i] = u[col * nz + i];
-  __syncthreads();
-  const T r = T(0.70710678118654752440);
-  for (int h = 1; h < nz; h <<= 1) {
-    for (int p = tid; p < nz / (2 * h); p += nt) {
-      const int i = p * 2 * h;
-      const cplx<T> a0 = x[i], a1 = x[i + h];
-      x[i] = cscale(cadd(a0, a1), r);
-      x[i + h] = cscale(csub(a0, a1), r);
-    }
-    __syncthreads();
-  }
-  const T t = lam_dev ? T(lam_scale * *lam_dev) : tau;
-  for (int i = tid; i < nz; i += nt)
-    if (i) x[i] = soft_threshold(x[i], t);
-  __syncthreads();
-  for (int h = nz >> 1; h >= 1; h >>= 1) {
-    for (int p = tid; p < nz / (2 * h); p += nt) {
-      const int i = p * 2 * h;
-      const cplx<T> a0 = x[i], a1 = x[i + h];
-      x[i] = cscale(cadd(a0, a1), r);
-      x[i + h] = cscale(csub(a0, a1), r);
-    }
-    __syncthreads();
-  }
-  for (int i = tid; i < nz; i += nt) z[col * nz + i] = x[i];
-}
-
-template <typename T> cudaError_t launch_haar_prox(const cplx<T>* u, cplx<T>* z, int nz,
-                                                   size_t n_ascans, T tau, const double* lam_dev,
-                                                   double lam_scale, cudaStream_t s) {
-  const int threads = nz / 2 >= 256 ? 256 : (nz / 2 >= 32 ? nz / 2 : 32);
-  const size_t sm = size_t(nz) * sizeof(cplx<T>);
-  cudaFuncSetAttribute(k_haar_prox<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, int(sm));
-  k_haar_prox<T><<<unsigned(n_ascans), threads, sm, s>>>(u, z, nz, tau, lam_dev, lam_scale);
-  return cudaGetLastError();
-}
-template cudaError_t launch_haar_prox<float>(const float2*, float2*, int, size_t, float,
-                                             const double*, double, cudaStream_t);
-template cudaError_t launch_haar_prox<double>(const double2*, double2*, int, size_t, double,
-                                              const double*, double, cudaStream_t);
-
 template <typename T> size_t lat_smem_bytes(int L, int TP) {
   int lg = 0, r3 = 0;
   fft_length(L, &lg, &r3);

@@ -1,3 +1,5 @@
+// The other priors' proxes.
+//
 // Total-variation prior (§3.1 names TV among the convex priors Eq. 12 extends
 // to): isotropic TV over (x, z) of each B-scan slice of the image
 // [ny][nx][nz], with forward differences that are zero at the far edge.  Its
@@ -12,6 +14,7 @@
 #include <math.h>
 
 #include "internal.cuh"
+#include "lat_point.cuh"
 
 namespace isam {
 
@@ -247,5 +250,160 @@ template cudaError_t launch_tv_primal<double>(const double2*, const double2*, co
 template cudaError_t launch_tv_dual<double>(const double2*, double2*, double2*, double2*, double2*,
                                             double, const double*, double, double, int, int, size_t,
                                             cudaStream_t);
+
+// ---------------------------------------------------------------------------
+// Haar prior
+// ---------------------------------------------------------------------------
+// prox of tau ||details(W u)||_1 per A-scan (nz contiguous samples), W the
+// orthonormal Haar transform along depth: in-place lifting levels with
+// stride h = 1, 2, .., nz/2 (pair (i, i + h), i a multiple of 2h, becomes
+// ((x_i + x_{i+h})/sqrt 2, (x_i - x_{i+h})/sqrt 2)), the complex soft
+// threshold on every coefficient but the approximation (index 0), and the
+// same butterflies in reverse order, which invert them.
+template <typename T>
+__global__ void k_haar_prox(const cplx<T>* u, cplx<T>* z, int nz, T tau, const double* lam_dev,
+                            double lam_scale) {
+  extern __shared__ __align__(16) unsigned char raw[];
+  cplx<T>* x = reinterpret_cast<cplx<T>*>(raw);
+  const size_t col = blockIdx.x;
+  const int tid = threadIdx.x, nt = blockDim.x;
+  for (int i = tid; i < nz; i += nt) x[i] = u[col * nz + i];
+  __syncthreads();
+  const T r = T(0.70710678118654752440);
+  for (int h = 1; h < nz; h <<= 1) {
+    for (int p = tid; p < nz / (2 * h); p += nt) {
+      const int i = p * 2 * h;
+      const cplx<T> a0 = x[i], a1 = x[i + h];
+      x[i] = cscale(cadd(a0, a1), r);
+      x[i + h] = cscale(csub(a0, a1), r);
+    }
+    __syncthreads();
+  }
+  const T t = lam_dev ? T(lam_scale * *lam_dev) : tau;
+  for (int i = tid; i < nz; i += nt)
+    if (i) x[i] = soft_threshold(x[i], t);
+  __syncthreads();
+  for (int h = nz >> 1; h >= 1; h >>= 1) {
+    for (int p = tid; p < nz / (2 * h); p += nt) {
+      const int i = p * 2 * h;
+      const cplx<T> a0 = x[i], a1 = x[i + h];
+      x[i] = cscale(cadd(a0, a1), r);
+      x[i + h] = cscale(csub(a0, a1), r);
+    }
+    __syncthreads();
+  }
+  for (int i = tid; i < nz; i += nt) z[col * nz + i] = x[i];
+}
+
+// The same for nz = 256 .. 2048, with the A-scan in registers: a lane holds 8
+// consecutive samples (three levels), a warp 256 (five more by shuffles), and the
+// A-scan's nz / 256 warps combine their approximations through shared memory; 8
+// warps, so 2048 / nz A-scans, a block.  Loads and stores are transposed within
+// the warp so that global rows stay contiguous.  The levels through shared memory
+// took 22 barriers, the last of them for one pair: 17.5 us at 512 x 2048, whose
+// 16.8 MB it now moves at the L2's rate.
+template <typename T> __device__ __forceinline__ cplx<T> shfl_xor_c(cplx<T> a, int m) {
+  return mk<T>(__shfl_xor_sync(0xffffffffu, a.x, m), __shfl_xor_sync(0xffffffffu, a.y, m));
+}
+template <typename T>
+__global__ void __launch_bounds__(256) k_haar_regs(const cplx<T>* u, cplx<T>* z, int nz, size_t n,
+                                                   T tau, const double* lam_dev,
+                                                   double lam_scale) {
+  using C = cplx<T>;
+  __shared__ C buf[8][288];                            // a warp's 256 samples, padded
+  __shared__ C approx[8];
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int G = nz / 256, first = warp / G * G, part = warp - first;
+  const size_t scan = size_t(blockIdx.x) * (8 / G) + warp / G;
+  const bool in = scan < n;
+  const size_t base = scan * nz + size_t(part) * 256;
+  const T r = T(0.70710678118654752440);
+  cudaTriggerProgrammaticLaunchCompletion();
+  cudaGridDependencySynchronize();
+  const T t = lam_dev ? T(lam_scale * *lam_dev) : tau;
+  C x[8];
+#pragma unroll
+  for (int k = 0; k < 8; ++k) {
+    const int e = 32 * k + lane;
+    buf[warp][e + (e >> 3)] = in ? u[base + e] : mk<T>(0, 0);
+  }
+  __syncwarp();
+#pragma unroll
+  for (int k = 0; k < 8; ++k) x[k] = buf[warp][9 * lane + k];
+#pragma unroll
+  for (int h = 1; h < 8; h <<= 1)
+#pragma unroll
+    for (int i = 0; i < 8; i += 2 * h) {
+      const C a0 = x[i], a1 = x[i + h];
+      x[i] = cscale(cadd(a0, a1), r);
+      x[i + h] = soft_threshold(cscale(csub(a0, a1), r), t);
+    }
+  // one level between lanes h apart: sums on the lanes of even multiples of h, and
+  // on those of odd ones the differences, thresholded on the way up
+  auto level = [&](C a, int h, bool up) {
+    const C v = shfl_xor_c<T>(a, h);
+    const int m = lane & (2 * h - 1);
+    if (m == 0) return cscale(cadd(a, v), r);
+    if (m != h) return a;
+    const C d = cscale(csub(v, a), r);
+    return up ? soft_threshold(d, t) : d;
+  };
+  C a = x[0];
+#pragma unroll
+  for (int h = 1; h < 32; h <<= 1) a = level(a, h, true);
+  if (lane == 0) approx[warp] = a;
+  __syncthreads();
+  C y = approx[first + (lane & (G - 1))];
+  for (int h = 1; h < G; h <<= 1) y = level(y, h, true);
+  for (int h = G >> 1; h >= 1; h >>= 1) y = level(y, h, false);
+  y = mk<T>(__shfl_sync(0xffffffffu, y.x, part), __shfl_sync(0xffffffffu, y.y, part));
+  if (lane == 0) a = y;
+#pragma unroll
+  for (int h = 16; h >= 1; h >>= 1) a = level(a, h, false);
+  x[0] = a;
+#pragma unroll
+  for (int h = 4; h >= 1; h >>= 1)
+#pragma unroll
+    for (int i = 0; i < 8; i += 2 * h) {
+      const C a0 = x[i], a1 = x[i + h];
+      x[i] = cscale(cadd(a0, a1), r);
+      x[i + h] = cscale(csub(a0, a1), r);
+    }
+#pragma unroll
+  for (int k = 0; k < 8; ++k) buf[warp][9 * lane + k] = x[k];
+  __syncwarp();
+  if (!in) return;
+#pragma unroll
+  for (int k = 0; k < 8; ++k) {
+    const int e = 32 * k + lane;
+    z[base + e] = buf[warp][e + (e >> 3)];
+  }
+}
+
+template <typename T> cudaError_t launch_haar_prox(const cplx<T>* u, cplx<T>* z, int nz,
+                                                   size_t n_ascans, T tau, const double* lam_dev,
+                                                   double lam_scale, cudaStream_t s) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.stream = s;
+  if (nz >= 256) {
+    const size_t per_block = 2048 / nz;
+    cfg.gridDim = dim3(unsigned((n_ascans + per_block - 1) / per_block));
+    cfg.blockDim = dim3(256);
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[0].val.programmaticStreamSerializationAllowed = sizeof(T) == 4;
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, k_haar_regs<T>, u, z, nz, n_ascans, tau, lam_dev, lam_scale);
+  }
+  cfg.gridDim = dim3(unsigned(n_ascans));
+  cfg.blockDim = dim3(nz / 2 >= 32 ? nz / 2 : 32);
+  cfg.dynamicSmemBytes = size_t(nz) * sizeof(cplx<T>);
+  return cudaLaunchKernelEx(&cfg, k_haar_prox<T>, u, z, nz, tau, lam_dev, lam_scale);
+}
+template cudaError_t launch_haar_prox<float>(const float2*, float2*, int, size_t, float,
+                                             const double*, double, cudaStream_t);
+template cudaError_t launch_haar_prox<double>(const double2*, double2*, int, size_t, double,
+                                              const double*, double, cudaStream_t);
 
 }  // namespace isam
