@@ -8,6 +8,7 @@
 // an nz-point DFT of the zero-padded, modulated samples (nk <= nz).
 #include "fft_smem.cuh"
 #include "internal.cuh"
+#include "lat_reg.cuh"
 
 namespace isam {
 
@@ -35,9 +36,70 @@ __global__ void k_dc_ifft(const T* s, cplx<T>* out, const cplx<T>* disp, const c
   for (int n = threadIdx.x; n < nz; n += blockDim.x) o[n] = cmul(buf[prow(n)], __ldg(post + n));
 }
 
+// FP32, nz = 256 .. 2048: the register transform of lat_reg.cuh on A-scans (columns
+// of contiguous rows, so W = 1), 128 threads a block.  The shared-memory form's 256
+// threads an A-scan moved it ten times through shared memory between barriers that
+// left 1,024 blocks' loads and stores uncovered; here 512 blocks of two A-scans are
+// resident at once.
+template <int L>
+__global__ void __launch_bounds__(128, lreg::Plan<float, L>::P == 32 ? 4 : 6)
+    k_dc_ifft_regs(const float* s, float2* out, const float2* disp, const float2* post, int nk,
+                   int n_ascans) {
+  constexpr int P = lreg::Plan<float, L>::P, TH = L / P, PER = 128 / TH;
+  __shared__ float2 S[PER][lreg::smem_elements<float, L, 1>()];
+  const int b = threadIdx.x % TH, sl = threadIdx.x / TH;
+  const int scan = blockIdx.x * PER + sl;
+  const bool in = scan < n_ascans;
+  const lreg::Twiddles<float, L> tw(b, nullptr);
+  cudaGridDependencySynchronize();
+  const float* x = s + size_t(scan) * nk;
+  float2 v[P];
+#pragma unroll
+  for (int i = 0; i < P; ++i) {
+    const int j = b + i * TH;                          // parity of j: that of b
+    float2 w = make_float2(0.0f, 0.0f);
+    if (in && j < nk) {
+      const float sj = (b & 1) ? -x[j] : x[j];
+      const float2 d = __ldg(disp + j);
+      w = make_float2(sj * d.x, -sj * d.y);
+    }
+    v[i] = w;
+  }
+  lreg::transform<-1, L, 1, 0, float>(v, S[sl], tw, b, 0, true, [] {});
+  cudaTriggerProgrammaticLaunchCompletion();
+  if (!in) return;
+  float2* o = out + size_t(scan) * L;
+#pragma unroll
+  for (int i = 0; i < P; ++i) o[b + i * TH] = cmul(v[i], __ldg(post + b + i * TH));
+}
+
+template <int L>
+static cudaError_t launch_dc_regs(const float* s, float2* out, const float2* disp,
+                                  const float2* post, int nk, int n, cudaStream_t st) {
+  constexpr int PER = 128 / (L / lreg::Plan<float, L>::P);
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3((n + PER - 1) / PER);
+  cfg.blockDim = dim3(128);
+  cfg.stream = st;
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = at;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, k_dc_ifft_regs<L>, s, out, disp, post, nk, n);
+}
+
 template <typename T> cudaError_t launch_dc_ifft(const T* s, cplx<T>* out, const cplx<T>* disp,
                                                  const cplx<T>* post, const cplx<T>* roots, int nk,
                                                  int nz, int lognz, int n_ascans, cudaStream_t st) {
+  if constexpr (sizeof(T) == 4) {
+    switch (nz) {
+      case 2048: return launch_dc_regs<2048>(s, out, disp, post, nk, n_ascans, st);
+      case 1024: return launch_dc_regs<1024>(s, out, disp, post, nk, n_ascans, st);
+      case 512: return launch_dc_regs<512>(s, out, disp, post, nk, n_ascans, st);
+      case 256: return launch_dc_regs<256>(s, out, disp, post, nk, n_ascans, st);
+    }
+  }
   const int threads = nz / 8 > 32 ? nz / 8 : 32;
   const size_t sm = size_t(padded_rows(nz) + twiddle_entries<T>(nz, lognz)) * sizeof(cplx<T>);
   cudaFuncSetAttribute(k_dc_ifft<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, int(sm));

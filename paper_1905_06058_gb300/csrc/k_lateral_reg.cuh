@@ -79,11 +79,11 @@ __global__ void __launch_bounds__(lat_reg_threads<T, L>(), lat_reg_min_blocks<T,
     }
   };
   if constexpr (MODE == LAT_C2C_FWD || MODE == LAT_R2C_FWD || MODE == LAT_EXTRAP_FWD)
-    lreg::transform<-1, L, 0, T>(v, S, tw, b, c, true, nothing);
+    lreg::transform<-1, L, W, 0, T>(v, S, tw, b, c, true, nothing);
   else if constexpr (EARLY)
-    lreg::transform<+1, L, 0, T>(v, S, tw, b, c, true, [&] { load_iterates(0); });
+    lreg::transform<+1, L, W, 0, T>(v, S, tw, b, c, true, [&] { load_iterates(0); });
   else
-    lreg::transform<+1, L, 0, T>(v, S, tw, b, c, true, nothing);
+    lreg::transform<+1, L, W, 0, T>(v, S, tw, b, c, true, nothing);
   if constexpr (!PLAIN && !UPDATE) cudaTriggerProgrammaticLaunchCompletion();
   if (stopped) return;   // an earlier check stopped the solve: write nothing
 
@@ -152,7 +152,7 @@ __global__ void __launch_bounds__(lat_reg_threads<T, L>(), lat_reg_min_blocks<T,
     }
     if (bad) atomicOr(a.flag, 1);
     cudaTriggerProgrammaticLaunchCompletion();
-    lreg::transform<-1, L, 0, T>(v, S, tw, b, c, false, nothing);
+    lreg::transform<-1, L, W, 0, T>(v, S, tw, b, c, false, nothing);
     if constexpr (!FROM_U) {
       if (a.partial != nullptr) {
         __shared__ double red[3][NT / 32];
@@ -179,7 +179,7 @@ __global__ void __launch_bounds__(lat_reg_threads<T, L>(), lat_reg_min_blocks<T,
 template <typename T, int MODE, int L>
 static cudaError_t launch_lat_reg_mode(const LatArgs<T>& a, cudaStream_t s) {
   auto* kern = k_lat_reg<T, MODE, L>;
-  constexpr size_t sm = lreg::smem_bytes<T, L>();
+  constexpr size_t sm = lreg::smem_elements<T, L, lreg::columns<T, L>()>() * sizeof(cplx<T>);
   cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, int(sm));
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(a.M / lreg::columns<T, L>(), a.B);

@@ -134,6 +134,7 @@ template <int SIGN, int R, typename C> __device__ __forceinline__ void dft(C* a)
 // the span of those before it.  Every span divides T = L / P, so a thread's butterflies of a
 // pass share one twiddle base.
 template <typename T, int L> struct Plan;
+template <> struct Plan<float, 2048> { static constexpr int P = 32, N = 3, R0 = 8, R1 = 8, R2 = 32; };
 template <> struct Plan<float, 1024> { static constexpr int P = 32, N = 2, R0 = 32, R1 = 32, R2 = 1; };
 template <> struct Plan<float, 512> { static constexpr int P = 32, N = 2, R0 = 16, R1 = 32, R2 = 1; };
 template <> struct Plan<float, 256> { static constexpr int P = 16, N = 2, R0 = 16, R1 = 16, R2 = 1; };
@@ -162,26 +163,26 @@ template <typename T, int L> __host__ __device__ constexpr int span(int pass) {
 template <typename T, int L> __host__ __device__ constexpr int columns() {
   return sizeof(T) == 8 ? 4 : L >= 768 ? 8 : 16;
 }
-// Rows of 64 bytes get a padding row after every R0: the first pass's writes to
-// rows R0 b + r of neighbouring b then fall in different halves of the banks.
-// Rows of 128 bytes need none.
-template <typename T, int L> __host__ __device__ constexpr bool padded() {
-  return columns<T, L>() * sizeof(cplx<T>) < 128;
+// Rows of W columns.  Rows shorter than 128 bytes get a padding row after every R0:
+// the first pass's writes to rows R0 b + r of neighbouring b then fall in different
+// banks.  Rows of 128 bytes need none.
+template <typename T, int W> __host__ __device__ constexpr bool padded() {
+  return W * sizeof(cplx<T>) < 128;
 }
-template <typename T, int L> __device__ __forceinline__ int slot(int row, int c) {
-  constexpr int W = columns<T, L>();
-  if constexpr (padded<T, L>()) return (row + row / Plan<T, L>::R0) * W + c;
+template <typename T, int L, int W> __device__ __forceinline__ int slot(int row, int c) {
+  if constexpr (padded<T, W>()) return (row + row / Plan<T, L>::R0) * W + c;
   else return row * W + c;
 }
 // ... of (row + STEP r, c) less that of (row, c), for a STEP that is a multiple of
 // the padding period or r < R0 rows from a multiple of it: a constant
-template <typename T, int L, int STEP> __device__ __forceinline__ constexpr int slot_step(int r) {
-  constexpr int W = columns<T, L>(), R0 = Plan<T, L>::R0;
-  static_assert(!padded<T, L>() || STEP == 1 || STEP % R0 == 0, "a constant distance");
-  return (padded<T, L>() && STEP % R0 == 0 ? r * (STEP + STEP / R0) : r * STEP) * W;
+template <typename T, int L, int W, int STEP>
+__device__ __forceinline__ constexpr int slot_step(int r) {
+  constexpr int R0 = Plan<T, L>::R0;
+  static_assert(!padded<T, W>() || STEP == 1 || STEP % R0 == 0, "a constant distance");
+  return (padded<T, W>() && STEP % R0 == 0 ? r * (STEP + STEP / R0) : r * STEP) * W;
 }
-template <typename T, int L> __host__ __device__ constexpr size_t smem_bytes() {
-  return size_t(padded<T, L>() ? L + L / Plan<T, L>::R0 : L) * columns<T, L>() * sizeof(cplx<T>);
+template <typename T, int L, int W> __host__ __device__ constexpr size_t smem_elements() {
+  return size_t(padded<T, W>() ? L + L / Plan<T, L>::R0 : L) * W;
 }
 
 // w^1, w^4, w^16 of a pass, w = e^{-2 pi i k / (span R)}, k = b mod span
@@ -235,7 +236,7 @@ template <int L> struct Twiddles<double, L> {
 // Unnormalised transform of the thread's column in registers (SIGN -1: e^{-}).
 // `first`: no thread of the block may still be reading S.  before(): called once,
 // after the last exchange's writes, before its barrier.
-template <int SIGN, int L, int PASS = 0, typename T, typename Before>
+template <int SIGN, int L, int W, int PASS = 0, typename T, typename Before>
 __device__ __forceinline__ void transform(cplx<T>* v, cplx<T>* S, const Twiddles<T, L>& tw, int b,
                                           int c, bool first, Before before) {
   using Pl = Plan<T, L>;
@@ -260,16 +261,16 @@ __device__ __forceinline__ void transform(cplx<T>* v, cplx<T>* S, const Twiddles
     const int k = b % NS;
 #pragma unroll
     for (int u = 0; u < NB; ++u) {
-      cplx<T>* out = S + slot<T, L>((b + u * TH - k) * R + k, c);
+      cplx<T>* out = S + slot<T, L, W>((b + u * TH - k) * R + k, c);
 #pragma unroll
-      for (int r = 0; r < R; ++r) out[slot_step<T, L, NS>(r)] = a[u][r];
+      for (int r = 0; r < R; ++r) out[slot_step<T, L, W, NS>(r)] = a[u][r];
     }
     if constexpr (PASS == Pl::N - 2) before();
     __syncthreads();
-    const cplx<T>* in = S + slot<T, L>(b, c);
+    const cplx<T>* in = S + slot<T, L, W>(b, c);
 #pragma unroll
-    for (int i = 0; i < P; ++i) v[i] = in[slot_step<T, L, TH>(i)];
-    transform<SIGN, L, PASS + 1, T>(v, S, tw, b, c, false, before);
+    for (int i = 0; i < P; ++i) v[i] = in[slot_step<T, L, W, TH>(i)];
+    transform<SIGN, L, W, PASS + 1, T>(v, S, tw, b, c, false, before);
   }
 }
 
