@@ -141,6 +141,14 @@ template <typename T> struct AxArgs {
   const int* stop;
 };
 
+// Lets a kernel take `bytes` of dynamic shared memory; up to 44 KB (48 with the
+// kernels' static arrays) it may without being told, which saves small plans' launches
+// the call.
+template <typename F> void allow_smem(F* kern, size_t bytes) {
+  if (bytes > 44 * 1024)
+    cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, int(bytes));
+}
+
 // launchers (return cudaGetLastError())
 template <typename T> cudaError_t launch_lat(int mode, const LatArgs<T>& a, cudaStream_t s);
 // the passes with the tile in registers, for lengths L at TZ pair-columns that

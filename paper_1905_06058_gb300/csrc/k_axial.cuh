@@ -1054,7 +1054,7 @@ static cudaError_t launch_ax_JKC(const AxArgs<T>& a, int npairs, cudaStream_t s,
   else if (kind == AX_FWD) kern = k_ax_fwd<T, J, LOGK, C16, ONE>;
   else if constexpr (ONE) kern = k_ax_adj<T, J, LOGK, C16, ONE, true>;
   else kern = a.s_out ? k_ax_fused<T, J, LOGK, true, C16> : k_ax_fused<T, J, LOGK, false, C16>;
-  cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, int(sm));
+  allow_smem(kern, sm);
   // programmatic dependent launch: each axial kernel builds its twiddles while
   // the previous kernel finishes, then waits for it (cudaGridDependencySynchronize)
   cudaLaunchConfig_t cfg = {};

@@ -102,7 +102,7 @@ template <typename T> cudaError_t launch_dc_ifft(const T* s, cplx<T>* out, const
   }
   const int threads = nz / 8 > 32 ? nz / 8 : 32;
   const size_t sm = size_t(padded_rows(nz) + twiddle_entries<T>(nz, lognz)) * sizeof(cplx<T>);
-  cudaFuncSetAttribute(k_dc_ifft<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, int(sm));
+  allow_smem(k_dc_ifft<T>, sm);
   k_dc_ifft<T><<<n_ascans, threads, sm, st>>>(s, out, disp, post, roots, nk, nz, lognz);
   return cudaGetLastError();
 }

@@ -280,7 +280,7 @@ static cudaError_t launch_lat_tile(const LatArgs<T>& a, cudaStream_t s) {
   const int threads = (a.L >= 8 ? a.L / 8 : 1) * a.TZ;
   const size_t sm = lat_smem_bytes<T>(a.L, a.TZ);
   auto* kern = k_lat<T, MODE, LOGL, LOGTP>;
-  cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, int(sm));
+  allow_smem(kern, sm);
   dim3 grid(a.M / (2 * a.TZ), a.B);
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = grid;

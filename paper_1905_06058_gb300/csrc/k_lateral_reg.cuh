@@ -180,7 +180,7 @@ template <typename T, int MODE, int L>
 static cudaError_t launch_lat_reg_mode(const LatArgs<T>& a, cudaStream_t s) {
   auto* kern = k_lat_reg<T, MODE, L>;
   constexpr size_t sm = lreg::smem_elements<T, L, lreg::columns<T, L>()>() * sizeof(cplx<T>);
-  cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, int(sm));
+  allow_smem(kern, sm);
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(a.M / lreg::columns<T, L>(), a.B);
   cfg.blockDim = dim3(lat_reg_threads<T, L>());

@@ -216,7 +216,7 @@ cudaError_t launch_tv_tile(const TvLaunch& l, cudaStream_t s) {
   const int inner = TV_TILE - 2 * a.halo;
   const dim3 grid((l.nz + inner - 1) / inner, (l.nx + inner - 1) / inner, l.ny);
   const size_t sm = (2 * TV_TILE + TV_TILE / TV_ROWS) * TV_TILE * sizeof(float2);
-  cudaFuncSetAttribute(k_tv_tile, cudaFuncAttributeMaxDynamicSharedMemorySize, int(sm));
+  allow_smem(k_tv_tile, sm);
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = grid;
   cfg.blockDim = dim3(512);

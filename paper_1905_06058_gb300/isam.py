@@ -161,6 +161,17 @@ def _stream_handle(stream) -> int:
     return int(s.cuda_stream)
 
 
+def _current_stream() -> int:
+    """Handle of the current stream of the current device: what
+    torch.cuda.current_stream().cuda_stream gives, without the Stream object it
+    builds (2.9 us of a 19 us call at 128 x 256)."""
+    import torch
+    try:
+        return torch._C._cuda_getCurrentRawStream(torch._C._cuda_getDevice())
+    except AttributeError:
+        return _stream_handle(None)
+
+
 # Every callback pair ever installed stays referenced: blocks are returned to
 # the allocator that made them, possibly after another one was installed.
 _ALLOCATORS = []
@@ -220,13 +231,13 @@ class Plan:
         import torch
         if not isinstance(t, torch.Tensor) or not t.is_cuda:
             raise TypeError(f"{name} must be a CUDA tensor")
-        if t.dtype != dtype or tuple(t.shape) != tuple(shape) or not t.is_contiguous():
+        if t.dtype != dtype or t.shape != shape or not t.is_contiguous():
             raise ValueError(f"{name}: need contiguous {dtype} {shape}, got {t.dtype} "
                              f"{tuple(t.shape)}")
-        return _P(t.data_ptr())
+        return t.data_ptr()
 
     def _sync_stream(self):
-        _check(_lib.isam_set_stream(self._h, _P(_stream_handle(None))), "isam_set_stream")
+        _check(_lib.isam_set_stream(self._h, _current_stream()), "isam_set_stream")
 
     @property
     def handle(self):
