@@ -799,11 +799,11 @@ __global__ void __launch_bounds__(512, ax_min_blocks<T>()) k_ax_fwd(const __grid
   pair_columns<T, ONE>(A, c1, c2, mx, my);
   const bool two = !ONE && c2 != c1;
   // programmatic dependent launch (as k_ax_fused): twiddles before the wait
-  cudaTriggerProgrammaticLaunchCompletion();
   const C* tw = ax_twiddles<T, LOGK, C16>(A, smem_raw);
   cudaGridDependencySynchronize();
   ax_forward<T, LOGK, C16, V>(A, Y, tw, c1, c2, two);
 
+  cudaTriggerProgrammaticLaunchCompletion();   // as late as k_ax_fused, for its reason
   const Positions<T> pos(A, mx, my);
   C* o1 = A.out + size_t(c1) * nk;
   C* o2 = A.out + size_t(c2) * nk;

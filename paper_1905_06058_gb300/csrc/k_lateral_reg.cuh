@@ -38,12 +38,16 @@ __global__ void __launch_bounds__(lat_reg_threads<T, L>(), lat_reg_min_blocks<T,
   C* S = reinterpret_cast<C*>(smem_raw);
   const int tid = threadIdx.x, c = tid % W, b = tid / W;
   // programmatic dependent launch: build the twiddles, then wait for the previous
-  // kernel's results.  The plain transforms let the next kernel start its prologue
-  // at once (A + A^H at 1024 x 2048: 72 us against 75), the solve's passes only
-  // before their last transform or stores (see k_ax_fused).
+  // kernel's results.  The next kernel may start its prologue before the last
+  // transform or stores of a solve's pass (see k_ax_fused).  The plain transforms of
+  // 33 to 152 blocks, which leave multiprocessors free for the next grid's blocks to
+  // crowd, allow it before their stores (A^H at 512 x 1024: 15.1 us, 17.5 if at
+  // once), the others at once (A + A^H at 1024 x 2048: 69 us, 71 if late).
   constexpr bool PLAIN = MODE == LAT_C2C_FWD || MODE == LAT_C2C_INV || MODE == LAT_R2C_FWD ||
                          MODE == LAT_INV_REAL;
-  if constexpr (PLAIN) cudaTriggerProgrammaticLaunchCompletion();
+  const unsigned blocks = gridDim.x * gridDim.y;
+  const bool early = PLAIN && (blocks <= 32 || blocks > 152);
+  if (early) cudaTriggerProgrammaticLaunchCompletion();
   const lreg::Twiddles<T, L> tw(b, a.roots);
   cudaGridDependencySynchronize();
   // the solve's stop flag (written by an earlier kernel, so visible after the
@@ -84,7 +88,7 @@ __global__ void __launch_bounds__(lat_reg_threads<T, L>(), lat_reg_min_blocks<T,
     lreg::transform<+1, L, W, 0, T>(v, S, tw, b, c, true, [&] { load_iterates(0); });
   else
     lreg::transform<+1, L, W, 0, T>(v, S, tw, b, c, true, nothing);
-  if constexpr (!PLAIN && !UPDATE) cudaTriggerProgrammaticLaunchCompletion();
+  if (!UPDATE && !early) cudaTriggerProgrammaticLaunchCompletion();
   if (stopped) return;   // an earlier check stopped the solve: write nothing
 
   if constexpr (MODE == LAT_INV_REAL) {
