@@ -337,7 +337,7 @@ void isam_batch_destroy(isam_batch* batch);
  *   stolt_table    1: read the plan's table of Stolt positions and phases; 0:
  *                  evaluate them in the kernels (the only mode without a table)
  *   axial_radix    16: column-split radix-16 passes for the FP32 axial
- *                  transforms at K = 2048 and 4096 (three shared-memory passes);
+ *                  transforms at K = 1024 to 4096 (three shared-memory passes);
  *                  8: radix-8 passes on column pairs (four); other plans run
  *                  radix 8 whatever the value
  *   lateral_radix  16: FP32 lateral passes of lengths 64 to 1024 (2^p, 3 * 2^p

@@ -1,5 +1,5 @@
 // Column-split radix-16 transforms of the axial kernels' column pair, for
-// FP32 and K = 2^LOGK, LOGK = 11 or 12 (K = 16 * 16 * 8 or 16 * 16 * 16).
+// FP32 and K = 2^LOGK, LOGK = 10 .. 12 (K = 16 * 16 * 4 .. 16 * 16 * 16).
 //
 // The pair's FFT buffer holds rows of two complex columns (cpair).  Here each
 // of the K/8 threads owns one column of one radix-16 butterfly per pass
@@ -102,7 +102,7 @@ template <int SIGN, int R> __device__ __forceinline__ void dft_r(float2* a) {
 // the span-256 one (256 entries).
 template <int LOGK> struct Passes {
   static constexpr int K = 1 << LOGK;
-  static constexpr int R3 = LOGK == 12 ? 16 : 8;   // radix of the span-256 pass
+  static constexpr int R3 = K / 256;               // radix of the span-256 pass
   static constexpr int entries = 16 + 256;
 };
 

@@ -133,7 +133,7 @@ template <typename T> struct AxArgs {
   // fused kernel, optional: the model spectra S = phase . N(eta_hat)
   // ([ny][nx][nk], as k_ax_fwd writes them)
   cplx<T>* s_out;
-  // FP32, K = 2048 or 4096: 1 runs the column-split radix-16 transforms, 0 the
+  // FP32, K = 1024 to 4096: 1 runs the column-split radix-16 transforms, 0 the
   // radix-8 column-pair ones (the plan's tuned choice); ignored elsewhere
   int radix16;
   unsigned past_offset;  // shared-memory offset of window_past's bins (set at launch)

@@ -84,7 +84,7 @@ struct isam_plan {
   // and whether the fused kernel reads the Stolt table (1) or evaluates (2)
   int tune_tp = 0;
   int tune_table = 0;
-  // FFT radix of the FP32 axial transforms at K = 2048 / 4096 and of the
+  // FFT radix of the FP32 axial transforms at K = 1024 to 4096 and of the
   // lateral tiles with a register form: 16 (column-split radix-16 passes, tiles
   // in registers, the default) or 8 (radix-8 column-pair passes)
   int tune_radix_ax = 16;
@@ -2088,9 +2088,9 @@ template <typename T> isam_status autotune_impl(isam_plan* P, isam_tuning* out) 
   update_geometry(P, &L, &M);
   const int threads_per_tp = L >= 8 ? L / 8 : 1;
   const bool fp32 = P->p.precision == ISAM_FP32;
-  // both radices exist for FP32 axial transforms at K = 2048, 4096 and the lateral
+  // both radices exist for FP32 axial transforms at K = 1024 to 4096 and the lateral
   // tiles with a register form
-  const bool ax_both = fp32 && (P->K == 2048 || P->K == 4096);
+  const bool ax_both = fp32 && P->K >= 1024;
   const bool prof = P->prof;
   P->prof = false;
   const int reps = 10;

@@ -713,13 +713,13 @@ __device__ __forceinline__ void inverse_and_store(const AxArgs<T>& A, V* Y, cons
   }
 }
 
-// FP32 plans at K = 2048 and 4096 can take the column-split radix-16
+// FP32 plans at K = 1024 to 4096 can take the column-split radix-16
 // transforms (fft_col16.cuh): three shared-memory passes per transform instead
 // of four, the same threads and registers; the forward ends, and the inverse
 // starts, in the layout of the interpolation and the scatter.  C16 selects
 // them (the plan's choice, AxArgs::radix16); other instances ignore it.
 template <typename T, int LOGK> __host__ __device__ constexpr bool ax_col16_exists() {
-  return std::is_same<T, float>::value && LOGK >= 11;
+  return std::is_same<T, float>::value && LOGK >= 10;
 }
 template <typename T, int LOGK, bool C16> __host__ __device__ constexpr bool ax_col16() {
   return C16 && ax_col16_exists<T, LOGK>();
@@ -1081,12 +1081,18 @@ static cudaError_t launch_ax_JK(const AxArgs<T>& a, int npairs, cudaStream_t s, 
   return launch_ax_JKC<T, J, LOGK, false>(a, npairs, s, kind);
 }
 
-// K = 4096 and 2048 (nz = 2048, 1024) run the compile-time-length instances
+// K = 4096 and 2048 (nz = 2048, 1024) run the compile-time-length instances, and
+// K = 1024 the FP32 column-split form (A + A^H at 128 x 256 -> 512: 14.4 us, 16.1 in
+// runtime-length radix-8 passes; at K = 512, where it saves no pass, those stay
+// ahead: a 128 x 128 x 256 volume's iteration takes 98 us, 102 split)
 template <typename T, int J>
-static cudaError_t launch_ax_J(const AxArgs<T>& a, int npairs, cudaStream_t s, int kind) {
+cudaError_t launch_ax_J(const AxArgs<T>& a, int npairs, cudaStream_t s, int kind) {
   switch (a.sc.K) {
     case 4096: return launch_ax_JK<T, J, 12>(a, npairs, s, kind);
     case 2048: return launch_ax_JK<T, J, 11>(a, npairs, s, kind);
+  }
+  if constexpr (sizeof(T) == 4) {
+    if (a.radix16 && a.sc.K == 1024) return launch_ax_JKC<T, J, 10, true>(a, npairs, s, kind);
   }
   return launch_ax_JK<T, J, 0>(a, npairs, s, kind);
 }

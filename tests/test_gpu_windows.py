@@ -79,7 +79,8 @@ def check(torch, g, prec, J, table, more=0.0):
 
 @pytest.mark.parametrize("step", [2.0, 2.2, 2.299, 2.301, None], ids=str)
 @pytest.mark.parametrize("nk,nz,J", [(16, 16, 4), (16, 16, 8), (64, 128, 6), (256, 256, 6),
-                                     (512, 512, 8), (1024, 1024, 4), (512, 1024, 6),
+                                     (512, 512, 8), (512, 512, 6), (256, 512, 4), (256, 256, 8),
+                                     (1024, 1024, 4), (512, 1024, 6),
                                      (2048, 2048, 8)])
 def test_steps_fp32(torch, nk, nz, J, step):
     check(torch, geometry(8, nk, nz, step), "fp32", J, True)
