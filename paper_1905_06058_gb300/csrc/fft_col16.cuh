@@ -182,18 +182,20 @@ __device__ __forceinline__ void pass(float2* Y, int b, int c, const float4* tw) 
 // The span-1 pass runs on the loaded samples: butterfly j reads rows
 // j + r K/16; rows [K/4, 3K/4) are zero and row j + r K/16 holds sample
 // n = j + i K/16 with i = r - 12 (r >= 12) or r + 4 (r < 4).  x: this thread's
-// column (NULL: a zero column).  Ends with a barrier.
-template <int LOGK>
+// column (NULL: a zero column); loaded(v): given its eight samples as loaded, x[j +
+// i K/16].  Ends with a barrier.
+template <int LOGK, typename Loaded>
 __device__ __forceinline__ void forward(float2* Y, const float2* x, const float* scale,
-                                        const float4* tw) {
+                                        const float4* tw, Loaded loaded) {
   constexpr int K = 1 << LOGK, K16 = K / 16;
   const int c = threadIdx.x & 1, j = threadIdx.x >> 1;
-  float2 a[16];
+  float2 v[8], a[16];
 #pragma unroll
-  for (int i = 0; i < 8; ++i) {
-    const int n = j + i * K16;
-    a[i < 4 ? i + 12 : i - 4] = x ? cscale(x[n], __ldg(scale + n)) : make_float2(0.0f, 0.0f);
-  }
+  for (int i = 0; i < 8; ++i) v[i] = x ? x[j + i * K16] : make_float2(0.0f, 0.0f);
+  loaded(v);
+#pragma unroll
+  for (int i = 0; i < 8; ++i)
+    a[i < 4 ? i + 12 : i - 4] = cscale(v[i], __ldg(scale + j + i * K16));
   dft16<+1, true>(a);
   float2* out = Y + el<P16>(16 * j, c);
 #pragma unroll
@@ -205,9 +207,10 @@ __device__ __forceinline__ void forward(float2* Y, const float2* x, const float*
 
 // Inverse transform of the pair from layout P8 (e^{-} DFT): two passes in
 // shared memory, the last in registers, handing output row j + i K/16 of this
-// thread's column to emit(i, value), i < 16.
-template <int LOGK, typename Emit>
-__device__ __forceinline__ void inverse(float2* Y, const float4* tw, Emit emit) {
+// thread's column to emit(i, value), i < 16; before(): called once, ahead of the
+// first emit.
+template <int LOGK, typename Before, typename Emit>
+__device__ __forceinline__ void inverse(float2* Y, const float4* tw, Before before, Emit emit) {
   constexpr int K = 1 << LOGK, K16 = K / 16, R = Passes<LOGK>::R3, NB = 16 / R, LR = K / R;
   const int c = threadIdx.x & 1, j = threadIdx.x >> 1;
   pass<-1, 16, K, 1, P8, P16>(Y, j, c, tw);
@@ -221,6 +224,7 @@ __device__ __forceinline__ void inverse(float2* Y, const float4* tw, Emit emit) 
     for (int r = 0; r < R; ++r) a[r] = in[el_step<P16, LR>(r)];
     twiddle<-1, R>(a, tw[16 + jj]);
     dft_r<-1, R>(a);
+    if (u == 0) before();
 #pragma unroll
     for (int r = 0; r < R; ++r) emit(u + r * NB, a[r]);   // row jj + 256 r = j + (u + r NB) K/16
   }

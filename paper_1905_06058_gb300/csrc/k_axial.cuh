@@ -27,6 +27,7 @@
 #include "fft_col16.cuh"
 #include "fft_smem.cuh"
 #include "internal.cuh"
+#include "tmem.cuh"
 
 namespace isam {
 
@@ -495,17 +496,16 @@ __device__ __forceinline__ void window_taps(const Coefficients<T, J>& co, int rh
 // Per block: the first sample's floor of every thread that has samples.
 struct WindowHeads { int mfl[512]; };
 
-// One thread's window: sums its samples slot by slot and hands each finished
-// slot (l, value) to put.
-template <typename T, int J, typename V, typename Put>
-__device__ __forceinline__ void window_sums(const Coefficients<T, J>& co, const Sample<T, V>* sm,
-                                            Put put) {
+// One thread's window: sums its samples, of taps (rho, e), slot by slot and hands
+// each finished slot (l, value) to put.
+template <typename T, int J, typename V, typename Taps, typename Put>
+__device__ __forceinline__ void window_sums(const Sample<T, V>* sm, Taps taps, Put put) {
   constexpr int WS = window_slots<J>();
   V w[WS];
 #pragma unroll
   for (int rho = 0; rho < NRES; ++rho) {
     T e[J + 1];
-    window_taps<T, J>(co, rho, sm[rho].frac, window_offset(sm, rho) != 0, e);
+    taps(rho, e);
 #pragma unroll
     for (int l = 0; l <= J; ++l) {
       V& x = w[2 * rho + l];
@@ -522,11 +522,12 @@ __device__ __forceinline__ void window_sums(const Coefficients<T, J>& co, const 
 }
 
 // Y = the scatter of all samples (every bin written; ends with a barrier).
-// Every read of Y must be done and heads complete (a barrier before).
-template <typename T, int J, typename V>
-__device__ __forceinline__ void window_scatter(const Coefficients<T, J>& co, V* Y, int K, int nt,
-                                               int nk, const Sample<T, V>* sm, V* past,
-                                               const WindowHeads& heads) {
+// Every read of Y must be done and heads complete (a barrier before).  WARP: taps is
+// called by whole warps.
+template <typename T, int J, bool WARP, typename V, typename Taps>
+__device__ __forceinline__ void window_scatter(V* Y, int K, int nt, int nk,
+                                               const Sample<T, V>* sm, V* past,
+                                               const WindowHeads& heads, Taps taps) {
   constexpr int WS = window_slots<J>(), W_MIN = 2 * NRES - 1, W_MAX = 2 * NRES + 2;
   const int tid = threadIdx.x, nact = nk / NRES;
   const bool active = tid < nact;
@@ -542,10 +543,10 @@ __device__ __forceinline__ void window_scatter(const Coefficients<T, J>& co, V* 
     return l < limit ? Y[prow((m0 + l) & (K - 1))] : past[l - limit];
   };
   V tail[WS - W_MIN];
-  if (active)
-    window_sums<T, J, V>(co, sm, [&](int l, const V& v) {
+  if (WARP ? (tid & ~31) < nact : active)
+    window_sums<T, J, V>(sm, taps, [&](int l, const V& v) {
       if (l >= W_MIN) tail[l - W_MIN] = v;
-      if (l < W_MIN || l < own) row(l) = v;
+      if ((!WARP || active) && (l < W_MIN || l < own)) row(l) = v;
     });
   __syncthreads();
   if (active)
@@ -571,24 +572,30 @@ __device__ __forceinline__ V* window_past(const AxArgs<T>& A, V* Y) {
   return reinterpret_cast<V*>(reinterpret_cast<unsigned char*>(Y) + A.past_offset);
 }
 
-// Y = the scatter of the block's samples, in the window form where every
-// thread's samples fit one.  Starts with a barrier (all reads of Y are done)
-// and ends with one.
-template <typename T, int J, typename V>
-__device__ __forceinline__ void scatter(const AxArgs<T>& A, const Coefficients<T, J>& co, V* Y,
-                                        int K, int nt, int nk, const Sample<T, V>* sm, int* lo, int* hi, int* ch_tail,
-                                        WindowHeads& heads) {
+// the thread's samples fit one window
+template <typename T, typename V>
+__device__ __forceinline__ bool quad_fits(const AxArgs<T>& A, const Sample<T, V>* sm) {
   bool ok = A.sc.window != 0;
-  if (NRES * int(threadIdx.x) < nk) {
-    heads.mfl[threadIdx.x] = sm[0].mfl;
 #pragma unroll
-    for (int rho = 0; rho < NRES; ++rho)
-      ok &= window_offset(sm, rho) <= 1u;
-  }
-  if (__syncthreads_and(ok)) {
-    window_scatter<T, J, V>(co, Y, K, nt, nk, sm, window_past<T, V>(A, Y), heads);
+  for (int rho = 0; rho < NRES; ++rho) ok &= window_offset(sm, rho) <= 1u;
+  return ok;
+}
+
+// Y = the scatter of the block's samples, in the window form where every thread's
+// samples fit one (fits; true where a thread has none).  heads holds every such
+// thread's first floor; taps gives the window's taps (see window_scatter), reload the
+// samples' positions again for the residue-class form.  Starts with a barrier (all
+// reads of Y are done) and ends with one.
+template <typename T, int J, bool WARP, typename V, typename Taps, typename Reload>
+__device__ __forceinline__ void scatter(const AxArgs<T>& A, const Coefficients<T, J>& co, V* Y,
+                                        int K, int nt, int nk, Sample<T, V>* sm, bool fits,
+                                        int* lo, int* hi, int* ch_tail, WindowHeads& heads,
+                                        Taps taps, Reload reload) {
+  if (__syncthreads_and(fits)) {
+    window_scatter<T, J, WARP, V>(Y, K, nt, nk, sm, window_past<T, V>(A, Y), heads, taps);
     return;
   }
+  reload();
   bool warp_tail;
   int chunk[NRES];
   const int nch = prepare_scatter<T, J, V>(Y, K, nt, nk, sm, chunk, lo, hi, ch_tail, warp_tail);
@@ -596,13 +603,11 @@ __device__ __forceinline__ void scatter(const AxArgs<T>& A, const Coefficients<T
 }
 
 // The forward interpolation of a thread's samples (before the phase): hands
-// (rho, N(x) of the columns) to put, in order; evanescent samples give 0.
-template <typename T, int J, typename V, typename Put>
-__device__ __forceinline__ void interp_quad(const AxArgs<T>& A, const Coefficients<T, J>& co,
-                                            const V* Y, int K, const Sample<T, V>* sm, Put put) {
-  bool fits = A.sc.window != 0;
-#pragma unroll
-  for (int rho = 0; rho < NRES; ++rho) fits &= window_offset(sm, rho) <= 1u;
+// (rho, N(x) of the columns) to put, in order; evanescent samples give 0.  Where they
+// fit a window, keep is given its taps (rho, e) too.
+template <typename T, int J, typename V, typename Keep, typename Put>
+__device__ __forceinline__ void interp_quad(const Coefficients<T, J>& co, const V* Y, int K,
+                                            const Sample<T, V>* sm, bool fits, Keep keep, Put put) {
   if (fits) {
     constexpr int WS = window_slots<J>();
     const int m0 = sm[0].mfl - J / 2 + 1;
@@ -616,6 +621,7 @@ __device__ __forceinline__ void interp_quad(const AxArgs<T>& A, const Coefficien
         y[2 * rho + l] = Y[prow((m0 + 2 * rho + l) & (K - 1))];
       T e[J + 1];
       window_taps<T, J>(co, rho, sm[rho].frac, window_offset(sm, rho) != 0, e);
+      keep(rho, e);
       V s = escale(y[2 * rho], e[0]);
 #pragma unroll
       for (int l = 1; l <= J; ++l) s = efma_r(e[l], y[2 * rho + l], s);
@@ -738,26 +744,28 @@ __device__ __forceinline__ const cplx<T>* ax_twiddles(const AxArgs<T>& A, unsign
 }
 
 // Y = the K-point e^{+} DFT of the pair's scaled, zero-padded columns
-template <typename T, int LOGK, bool C16, typename V>
+// (column-split form: loaded(v) as c16::forward)
+template <typename T, int LOGK, bool C16, typename V, typename Loaded>
 __device__ __forceinline__ void ax_forward(const AxArgs<T>& A, V* Y, const cplx<T>* tw,
-                                           int c1, int c2, bool two) {
+                                           int c1, int c2, bool two, Loaded loaded) {
   if constexpr (ax_col16<T, LOGK, C16>()) {
     constexpr int nz = (1 << LOGK) / 2;
     const int c = threadIdx.x & 1;
     const cplx<T>* x = c == 0 ? A.in + size_t(c1) * nz : (two ? A.in + size_t(c2) * nz : nullptr);
     c16::forward<LOGK>(reinterpret_cast<float2*>(Y), reinterpret_cast<const float2*>(x),
                        reinterpret_cast<const float*>(A.tab.scale),
-                       reinterpret_cast<const float4*>(tw));
+                       reinterpret_cast<const float4*>(tw), loaded);
   } else {
     load_and_fft<T, LOGK, V>(A, Y, tw, c1, c2, two);
   }
 }
 
 // The e^{-} DFT of Y, truncation to the nz kept rows, scaling, the columns'
-// output (G, or u_hat = eta_hat - G/L)
-template <typename T, int LOGK, bool C16, typename V>
+// output (G, or u_hat = eta_hat - G/L).  STASH: eta_hat comes from stash(v), the
+// eight samples forward's `loaded` was given, instead of memory.
+template <typename T, int LOGK, bool C16, bool STASH, typename V, typename Stash>
 __device__ __forceinline__ void ax_inverse(const AxArgs<T>& A, V* Y, const cplx<T>* tw,
-                                           int c1, int c2, bool two) {
+                                           int c1, int c2, bool two, Stash stash) {
   if constexpr (ax_col16<T, LOGK, C16>()) {
     // rows j + i K/16 of this thread's column; rows [K/4, 3K/4) are dropped
     constexpr int K = 1 << LOGK, nz = K / 2, K16 = K / 16;
@@ -765,13 +773,19 @@ __device__ __forceinline__ void ax_inverse(const AxArgs<T>& A, V* Y, const cplx<
     const int col = c ? c2 : c1;
     cplx<T>* o = A.out + size_t(col) * nz;
     const bool keep = c == 0 || two;
+    float2 v[8];
+    const bool u_hat = A.u_hat_scale != T(0);
     c16::inverse<LOGK>(reinterpret_cast<float2*>(Y), reinterpret_cast<const float4*>(tw),
+                       [&] { if (STASH) stash(v); },
                        [&](int i, const float2& y) {
                          if (!keep || (i >= 4 && i < 12)) return;
                          const int p = jb + i * K16;
                          const int n = i < 4 ? p + nz / 2 : p - (K - nz / 2);
-                         put_output1(A, o, col, n, reinterpret_cast<const cplx<T>&>(y),
-                                     __ldg(A.tab.scale + n));
+                         const float s = __ldg(A.tab.scale + n);
+                         if (STASH && u_hat)
+                           o[n] = csub(v[i < 4 ? i + 4 : i - 12], cscale(y, s * A.u_hat_scale));
+                         else
+                           put_output1(A, o, col, n, reinterpret_cast<const cplx<T>&>(y), s);
                        });
   } else {
     inverse_and_store<T, LOGK, V>(A, Y, tw, c1, c2, two);
@@ -801,7 +815,7 @@ __global__ void __launch_bounds__(512, ax_min_blocks<T>()) k_ax_fwd(const __grid
   // programmatic dependent launch (as k_ax_fused): twiddles before the wait
   const C* tw = ax_twiddles<T, LOGK, C16>(A, smem_raw);
   cudaGridDependencySynchronize();
-  ax_forward<T, LOGK, C16, V>(A, Y, tw, c1, c2, two);
+  ax_forward<T, LOGK, C16, V>(A, Y, tw, c1, c2, two, [](const float2*) {});
 
   cudaTriggerProgrammaticLaunchCompletion();   // as late as k_ax_fused, for its reason
   const Positions<T> pos(A, mx, my);
@@ -814,7 +828,8 @@ __global__ void __launch_bounds__(512, ax_min_blocks<T>()) k_ax_fwd(const __grid
   pos.quad(A, q, sm);
   cpair<T> ph;
   C a1, a2;
-  interp_quad<T, J, V>(A, Coefficients<T, J>(A, pos, q), Y, K, sm, [&](int rho, V s) {
+  interp_quad<T, J, V>(Coefficients<T, J>(A, pos, q), Y, K, sm, quad_fits<T, V>(A, sm),
+                       [](int, const T*) {}, [&](int rho, V s) {
     const int j = NRES * q + rho;
     if (rho % 2 == 0) {
       ph = pos.phases(A, q, rho / 2, sm);
@@ -879,10 +894,18 @@ __global__ void __launch_bounds__(512, ax_min_blocks<T>()) k_ax_adj(const __grid
     }
   }
   if (stopped) return;   // an earlier check stopped the solve: write nothing
-  scatter<T, J, V>(A, Coefficients<T, J>(A, pos, tid), Y, K, nt, nk, sm, &ch_lo, &ch_hi, &ch_tail,
-                   heads);
+  const Coefficients<T, J> co(A, pos, tid);
+  bool fits = A.sc.window != 0;
+  if (NRES * tid < nk) {
+    heads.mfl[tid] = sm[0].mfl;
+    fits = quad_fits<T, V>(A, sm);
+  }
+  scatter<T, J, false, V>(A, co, Y, K, nt, nk, sm, fits, &ch_lo, &ch_hi, &ch_tail, heads,
+                          [&](int rho, T* e) {
+                            window_taps<T, J>(co, rho, sm[rho].frac, window_offset(sm, rho) != 0, e);
+                          }, [] {});
   cudaTriggerProgrammaticLaunchCompletion();
-  ax_inverse<T, LOGK, C16, V>(A, Y, tw, c1, c2, two);
+  ax_inverse<T, LOGK, C16, false, V>(A, Y, tw, c1, c2, two, [](float2*) {});
 }
 
 // Forward model, data residual and adjoint of one column pair in one pass
@@ -904,6 +927,15 @@ __global__ void __launch_bounds__(512, ax_min_blocks<T>()) k_ax_fused(const __gr
   V* Y = reinterpret_cast<V*>(smem_raw);
   __shared__ int ch_lo, ch_hi, ch_tail;
   __shared__ WindowHeads heads;
+  // The column-split form keeps in tensor memory (tmem.cuh) what its 64 registers a
+  // thread do not hold from the forward half to the adjoint: the samples' taps,
+  // which it evaluated twice, and its eight samples of eta_hat, which it read twice
+  // (1024 x 2048 solve 10.34 -> 10.17 ms, 768 x 1024 2.65 -> 2.42 ms; of either alone
+  // the taps gain nothing and eta_hat half).
+  constexpr bool TM = ax_col16<T, LOGK, C16>();
+  constexpr int TAPS = tmem::kTapWords<J>, ETA = NRES * TAPS;
+  static_assert(ETA + 16 <= tmem::kWords, "a thread's words");
+  __shared__ uint32_t tm_slot;
   const int tid = threadIdx.x, nt = axial_threads<LOGK>();
   int c1, c2, mx, my;
   pair_columns(A, c1, c2, mx, my);
@@ -912,26 +944,50 @@ __global__ void __launch_bounds__(512, ax_min_blocks<T>()) k_ax_fused(const __gr
   // Programmatic dependent launch: this grid builds its twiddles, then waits for
   // the previous kernel before touching global data; the next kernel may start
   // once every block here is in its inverse transform (below).
-  const C* tw = ax_twiddles<T, LOGK, C16>(A, smem_raw);
+  if (TM && tid < 32) tmem::allocate(&tm_slot, nt);
+  const C* tw = ax_twiddles<T, LOGK, C16>(A, smem_raw);   // ends with a barrier
+  const uint32_t tm = TM ? tmem::base(tm_slot) : 0;
   cudaGridDependencySynchronize();
   // the solve's stop flag (written by an earlier kernel, so visible after the
   // wait): loaded here, tested after the forward transform (before the first
   // global write), so its latency overlaps the transform
   const bool stopped = A.stop != nullptr && __ldcg(A.stop) != 0;
   const C* d1 = A.sdh + size_t(c1) * nk;
-  ax_forward<T, LOGK, C16, V>(A, Y, tw, c1, c2, two);
-  if (stopped) return;   // an earlier check stopped the solve: write nothing
+  ax_forward<T, LOGK, C16, V>(A, Y, tw, c1, c2, two, [&](const float2* v) {
+    tmem::put16(tm + ETA, &v[0].x);
+  });
+  auto finish = [&] {                    // every warp's accesses to tensor memory done
+    if (TM) {
+      tmem::wait_stores();
+      tmem::before_barrier();
+      __syncthreads();
+      if (tid < 32) tmem::release(tm_slot, nt);
+    }
+  };
+  if (stopped) {         // an earlier check stopped the solve: write nothing
+    finish();
+    return;
+  }
   const Positions<T> pos(A, mx, my);
   Sample<T, V> sm[NRES];
 #pragma unroll
   for (int rho = 0; rho < NRES; ++rho) sm[rho].mfl = INT_MIN;
-  if (NRES * tid < nk) {
-    pos.quad(A, tid, sm);
+  bool fits = A.sc.window != 0;
+  // tensor memory takes whole warps: lanes without samples follow the last ones
+  const bool active = NRES * tid < nk;
+  if (TM ? NRES * (tid & ~31) < nk : active) {
+    const int q = TM ? min(tid, nk / NRES - 1) : tid;
+    pos.quad(A, q, sm);
+    fits = quad_fits<T, V>(A, sm);
+    if (TM) fits = __all_sync(0xffffffffu, fits);
+    if (active) heads.mfl[tid] = sm[0].mfl;
     V php, dq, w1, w2;                   // of two samples: phases, F s_d, model spectra
-    interp_quad<T, J, V>(A, Coefficients<T, J>(A, pos, tid), Y, K, sm, [&](int rho, V n) {
-      const int j = NRES * tid + rho;
+    interp_quad<T, J, V>(Coefficients<T, J>(A, pos, q), Y, K, sm, fits, [&](int rho, const T* e) {
+      if constexpr (TM) tmem::put_taps<J>(tm + rho * TAPS, e);
+    }, [&](int rho, V n) {
+      const int j = NRES * q + rho;
       if (rho % 2 == 0) {
-        php = pos.phases(A, tid, rho / 2, sm);
+        php = pos.phases(A, q, rho / 2, sm);
         dq = load_two<T>(d1 + j);
       }
       const C ph = rho % 2 == 0 ? php.a : php.b;
@@ -940,7 +996,7 @@ __global__ void __launch_bounds__(512, ax_min_blocks<T>()) k_ax_fused(const __gr
         if (rho % 2 == 0) {
           w1.a = s1;
           w2.a = s2;
-        } else {
+        } else if (active) {
           store_two<T>(A.s_out + size_t(c1) * nk + j - 1, w1.a, s1);
           if (two) store_two<T>(A.s_out + size_t(c2) * nk + j - 1, w2.a, s2);
         }
@@ -951,13 +1007,32 @@ __global__ void __launch_bounds__(512, ax_min_blocks<T>()) k_ax_fused(const __gr
       sm[rho].val.b = two ? cmulc(cconj(R), ph) : mk<T>(0, 0);
     });
   }
-  scatter<T, J, V>(A, Coefficients<T, J>(A, pos, tid), Y, K, nt, nk, sm, &ch_lo, &ch_hi, &ch_tail,
-                   heads);
+  if (TM) tmem::wait_stores();
+  const Coefficients<T, J> co(A, pos, tid);
+  scatter<T, J, TM, V>(A, co, Y, K, nt, nk, sm, fits, &ch_lo, &ch_hi, &ch_tail, heads,
+                       [&](int rho, T* e) {
+                         if constexpr (TM) tmem::get_taps<J>(tm + rho * TAPS, e);
+                         else window_taps<T, J>(co, rho, sm[rho].frac,
+                                                window_offset(sm, rho) != 0, e);
+                       }, [&] {
+                         // (positions are not kept in registers for this)
+                         if (!TM) return;
+                         Sample<T, V> again[NRES];
+                         if (active) pos.quad(A, tid, again);
+#pragma unroll
+                         for (int rho = 0; rho < NRES; ++rho) {
+                           sm[rho].mfl = active ? again[rho].mfl : INT_MIN;
+                           sm[rho].frac = again[rho].frac;
+                         }
+                       });
   // Not earlier: the next kernel's waiting blocks take the first slots that fall
   // free, several to a multiprocessor, and stay there (1024 x 2048 solve 11.4 ms
   // with the trigger at the start of this kernel and of the update, 10.9 ms so)
   cudaTriggerProgrammaticLaunchCompletion();
-  ax_inverse<T, LOGK, C16, V>(A, Y, tw, c1, c2, two);
+  ax_inverse<T, LOGK, C16, TM, V>(A, Y, tw, c1, c2, two, [&](float2* v) {
+    tmem::get16(tm + ETA, &v[0].x);
+  });
+  finish();
 }
 
 // One thread per (|q| class, quad): the same evaluation the kernels do on the fly.

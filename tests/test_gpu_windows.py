@@ -98,3 +98,28 @@ def test_integer_positions(torch, nk, nz, prec, table):
                                            (1024, 1024, 4, False), (2048, 2048, 6, True)])
 def test_steps_fp64(torch, nk, nz, J, table, step):
     check(torch, geometry(8, nk, nz, step), "fp64", J, table)
+
+
+@pytest.mark.parametrize("integer", [False, True], ids=["", "integer"])
+@pytest.mark.parametrize("step", [2.0, 2.299, 2.301, None], ids=str)
+@pytest.mark.parametrize("nk,nz,J", [(16, 512, 6), (64, 512, 4), (512, 512, 8), (32, 1024, 6),
+                                     (1024, 1024, 4), (1024, 1024, 6), (16, 2048, 8),
+                                     (2048, 2048, 6)])
+def test_gradient(torch, nk, nz, J, step, integer):
+    """The fused kernel where it keeps taps in tensor memory (K = 1024 to 4096), down to
+    a few lanes of one warp with samples, through two linear FISTA iterations
+    (lambda = 0; A and A^H twice each, so four times the bar, and at integer
+    positions four times the jump)."""
+    from paper_1905_06058_gb300.isam import Plan
+    if integer and J != 6:
+        pytest.skip("one J is enough")
+    g = geometry(4, nk, nz, step, integer)
+    ref = O.IsamOracle(g, "nufft", J=J)
+    s = np.random.default_rng(52).standard_normal(ref.spec_shape).astype(np.float32)
+    res = O.fista(ref.forward, ref.adjoint, s.astype(np.float64), 0.0, 4.0, max_iter=2,
+                  shape=ref.image_shape)
+    for table in (True, False):
+        plan = Plan(g, J=J, stolt_table=table)
+        out, _ = plan.solve(torch.from_numpy(s).cuda(), lambda_rel=0.0, L=4.0, max_iter=2)
+        plan.close()
+        assert rel(out.cpu().numpy(), res.eta) < 4e-5 + (4 * 2 * 5e-6 if integer else 0.0)
