@@ -80,6 +80,9 @@ enum LatMode : int {
   LAT_UPDATE = 5,    // FISTA step in image space between F^-1 and F
   LAT_GRAD_STEP = 6, // u = eta^k - g/L after F^-1 (no threshold, no F): other priors
   LAT_EXTRAP_FWD = 7,// X = F(z1 + mu (z1 - z2)): the momentum step, then F
+  LAT_R2C_HALF = 9,  // real input, X = F x, the rows 0 .. L/2 of the Hermitian spectrum:
+                     // [B][L/2+1][M] (lat_reg_takes only)
+  LAT_C2R_HALF = 10, // its inverse
   LAT_UPDATE_U = 8,  // as LAT_UPDATE from u_hat = eta_hat^k - G/L: u = F^-1 u_hat (no z2,
                      // no norm partials)
 };
@@ -127,6 +130,10 @@ template <typename T> struct AxArgs {
   // fused kernel only: lateral spectrum of the data, F s_d ([ny][nx][nk]; the
   // first column of each pair is read)
   const cplx<T>* sdh;
+  // standalone operators, FP32: the spectra are the half x <= nx/2 of the Hermitian
+  // spectrum of a real array, [ny][nx/2+1][nk]; k_ax_fwd forms it from the pair,
+  // (S(q) + conj S(-q)) / 2
+  int half;
   // fused kernel: 0 writes G; else writes u_hat = eta - u_hat_scale * G (the
   // lateral spectrum of eta^k - g/L, u_hat_scale = 1/L)
   T u_hat_scale;
@@ -152,10 +159,13 @@ template <typename F> void allow_smem(F* kern, size_t bytes) {
 // launchers (return cudaGetLastError())
 template <typename T> cudaError_t launch_lat(int mode, const LatArgs<T>& a, cudaStream_t s);
 // the passes with the tile in registers, for lengths L at TZ pair-columns that
-// lat_reg_takes
+// lat_reg_takes.  The half-spectrum modes (FP32) transform two real columns as one
+// complex one: lat_half_takes, for M real columns
+bool lat_half_takes(int L, int M);
 template <typename T> bool lat_reg_takes(int L, int TZ);
 template <> bool lat_reg_takes<float>(int L, int TZ);
 template <> bool lat_reg_takes<double>(int L, int TZ);
+cudaError_t launch_lat_half(int mode, const LatArgs<float>& a, cudaStream_t s);
 template <typename T> cudaError_t launch_lat_reg(int mode, const LatArgs<T>& a, cudaStream_t s);
 template <> cudaError_t launch_lat_reg<float>(int mode, const LatArgs<float>& a, cudaStream_t s);
 template <> cudaError_t launch_lat_reg<double>(int mode, const LatArgs<double>& a, cudaStream_t s);

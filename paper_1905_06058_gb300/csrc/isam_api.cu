@@ -406,9 +406,31 @@ template <typename T> isam_status lat_inverse(isam_plan* P, Impl<T>& im, cplx<T>
   return lat<T>(P, m1, lat_args<T>(P->ny, P->nx, W, in, out));
 }
 
+// The standalone operators' spectra belong to real arrays, so FP32 plans keep half of
+// them where the x passes can: nx of the register form, and real arrays s on 8 bytes
+// (two columns a load; the whole-spectrum form below reads one).  256 x 256 x 2048,
+// A + A^H: 4.40 -> 3.90 ms, 1.1 of 10 GB less; 1024 x 2048: 69 us either way.
+template <typename T> bool half_spectra(const isam_plan* P, const void* s) {
+  return sizeof(T) == 4 && P->tune_radix_lat == 16 && lat_half_takes(P->nx, P->nk) &&
+         reinterpret_cast<uintptr_t>(s) % 8 == 0;
+}
+template <typename T> LatArgs<T> half_x_args(isam_plan* P, const void* in, void* out) {
+  return lat_args<T>(P->ny, P->nx, P->nk, in, out);
+}
+template <typename T> LatArgs<T> half_y_args(isam_plan* P, cplx<T>* x) {
+  return lat_args<T>(1, P->ny, (P->nx / 2 + 1) * P->nk, x, x);
+}
+
 template <typename T> isam_status op_forward(isam_plan* P, const void* eta, void* s) {
   Impl<T>& im = impl_of<T>(P);
   ISAM_TRY(lat_forward<T>(P, im, eta, im.eta_hat, P->nz, false));
+  if (half_spectra<T>(P, s)) {
+    AxArgs<T> a = ax_args<T>(P, im, im.eta_hat, im.spec);
+    a.half = 1;
+    ISAM_TRY(launch(P, ISAM_KCLASS_AX_FWD, [&] { return launch_ax_fwd<T>(a, P->npairs, P->stream); }));
+    if (P->ny > 1) ISAM_TRY(lat<T>(P, LAT_C2C_INV, half_y_args<T>(P, im.spec)));
+    return lat<T>(P, LAT_C2R_HALF, half_x_args<T>(P, im.spec, s));
+  }
   ISAM_TRY(launch(P, ISAM_KCLASS_AX_FWD, [&] {
     return launch_ax_fwd<T>(ax_args<T>(P, im, im.eta_hat, im.spec), P->npairs, P->stream);
   }));
@@ -417,10 +439,15 @@ template <typename T> isam_status op_forward(isam_plan* P, const void* eta, void
 
 template <typename T> isam_status op_adjoint(isam_plan* P, const void* s, void* eta) {
   Impl<T>& im = impl_of<T>(P);
-  ISAM_TRY(lat_forward<T>(P, im, s, im.spec, P->nk, true));
-  ISAM_TRY(launch(P, ISAM_KCLASS_AX_ADJ, [&] {
-    return launch_ax_adj<T>(ax_args<T>(P, im, im.spec, im.grad), P->npairs, P->stream);
-  }));
+  AxArgs<T> a = ax_args<T>(P, im, im.spec, im.grad);
+  if (half_spectra<T>(P, s)) {
+    a.half = 1;
+    ISAM_TRY(lat<T>(P, LAT_R2C_HALF, half_x_args<T>(P, s, im.spec)));
+    if (P->ny > 1) ISAM_TRY(lat<T>(P, LAT_C2C_FWD, half_y_args<T>(P, im.spec)));
+  } else {
+    ISAM_TRY(lat_forward<T>(P, im, s, im.spec, P->nk, true));
+  }
+  ISAM_TRY(launch(P, ISAM_KCLASS_AX_ADJ, [&] { return launch_ax_adj<T>(a, P->npairs, P->stream); }));
   return lat_inverse<T>(P, im, im.grad, eta, P->nz, false);
 }
 
@@ -1035,14 +1062,15 @@ isam_status build_poly(isam_plan* P) {
   return ISAM_OK;
 }
 
-// Columns (ix, iy) and (-ix, -iy) mod (nx, ny) share |q|; list each pair once.
+// Columns (ix, iy) and (-ix, -iy) mod (nx, ny) share |q|; list each pair once, the one
+// of ix <= nx/2 first (where the half spectrum has it).
 isam_status build_pairs(isam_plan* P) {
   std::vector<int2> pr;
   for (int iy = 0; iy < P->ny; ++iy)
     for (int ix = 0; ix < P->nx; ++ix) {
       const int c = iy * P->nx + ix;
       const int d = ((P->ny - iy) % P->ny) * P->nx + (P->nx - ix) % P->nx;
-      if (c <= d) pr.push_back(make_int2(c, d));
+      if (c <= d) pr.push_back(2 * ix <= P->nx ? make_int2(c, d) : make_int2(d, c));
     }
   P->npairs = int(pr.size());
   ISAM_TRY(dalloc(&P->pairs, pr.size()));

@@ -269,6 +269,12 @@ __device__ __forceinline__ void pair_columns(const AxArgs<T>& A, int& c1, int& c
   my = signed_freq(c1 / A.sc.nx, A.sc.ny);
 }
 
+// Column c of the spectra arrays (of the half spectrum, for x <= nx/2)
+template <typename T>
+__device__ __forceinline__ int spectrum_column(const AxArgs<T>& A, int c, bool half) {
+  return half ? c - c / A.sc.nx * (A.sc.nx - A.sc.nx / 2 - 1) : c;
+}
+
 // Shared memory of the axial kernels: the FFT buffer Y (padded rows of
 // column pairs) followed by the K-point twiddle table.
 template <typename T>
@@ -819,8 +825,11 @@ __global__ void __launch_bounds__(512, ax_min_blocks<T>()) k_ax_fwd(const __grid
 
   cudaTriggerProgrammaticLaunchCompletion();   // as late as k_ax_fused, for its reason
   const Positions<T> pos(A, mx, my);
-  C* o1 = A.out + size_t(c1) * nk;
-  C* o2 = A.out + size_t(c2) * nk;
+  const bool half = !ONE && A.half;
+  C* o1 = A.out + size_t(spectrum_column(A, c1, half)) * nk;
+  C* o2 = A.out + size_t(spectrum_column(A, c2, half)) * nk;
+  // the half spectrum holds the pair's second column where both have x = 0 or nx/2
+  const bool second = two && (!half || c1 % sc.nx == 0 || 2 * (c1 % sc.nx) == sc.nx);
   // nk <= K/2 = NRES blockDim: a quad of samples per thread
   const int q = threadIdx.x;
   if (NRES * q >= nk) return;
@@ -831,14 +840,22 @@ __global__ void __launch_bounds__(512, ax_min_blocks<T>()) k_ax_fwd(const __grid
   interp_quad<T, J, V>(Coefficients<T, J>(A, pos, q), Y, K, sm, quad_fits<T, V>(A, sm),
                        [](int, const T*) {}, [&](int rho, V s) {
     const int j = NRES * q + rho;
+    if (rho % 2 == 0) ph = pos.phases(A, q, rho / 2, sm);
+    const C p = rho % 2 == 0 ? ph.a : ph.b;
+    C s1 = cmul(s.a, p), s2 = s1;
+    if constexpr (!ONE) {
+      if (two) s2 = cmul(s.b, p);
+      if (half) {
+        s1 = cscale(cadd(s1, cconj(s2)), T(0.5));
+        s2 = cconj(s1);
+      }
+    }
     if (rho % 2 == 0) {
-      ph = pos.phases(A, q, rho / 2, sm);
-      a1 = cmul(s.a, ph.a);
-      if constexpr (!ONE) a2 = cmul(s.b, ph.a);
+      a1 = s1;
+      a2 = s2;
     } else {
-      store_two<T>(o1 + j - 1, a1, cmul(s.a, ph.b));
-      if constexpr (!ONE)
-        if (two) store_two<T>(o2 + j - 1, a2, cmul(s.b, ph.b));
+      store_two<T>(o1 + j - 1, a1, s1);
+      if (second) store_two<T>(o2 + j - 1, a2, s2);
     }
   });
 }
@@ -867,7 +884,8 @@ __global__ void __launch_bounds__(512, ax_min_blocks<T>()) k_ax_adj(const __grid
   cudaGridDependencySynchronize();
   const bool stopped = RES && A.stop != nullptr && __ldcg(A.stop) != 0;
   const Positions<T> pos(A, mx, my);
-  const C* r1 = A.in + size_t(c1) * nk;
+  const bool half = !ONE && A.half;
+  const C* r1 = A.in + size_t(spectrum_column(A, c1, half)) * nk;
   const C* r2 = A.in + size_t(c2) * nk;
   Sample<T, V> sm[NRES];
 #pragma unroll
@@ -887,7 +905,8 @@ __global__ void __launch_bounds__(512, ax_min_blocks<T>()) k_ax_adj(const __grid
       sm[2 * h].val.a = cmulc(x.a, ph.a);
       sm[2 * h + 1].val.a = cmulc(x.b, ph.b);
       if constexpr (!ONE) {
-        const cpair<T> y = two ? load_two<T>(r2 + j) : cpair<T>{};
+        cpair<T> y{};
+        if (two) y = half ? cpair<T>{cconj(x.a), cconj(x.b)} : load_two<T>(r2 + j);
         sm[2 * h].val.b = cmulc(y.a, ph.a);
         sm[2 * h + 1].val.b = cmulc(y.b, ph.b);
       }

@@ -323,6 +323,9 @@ template <typename T> cudaError_t launch_lat(int mode, const LatArgs<T>& a, cuda
     case LAT_GRAD_STEP: return launch_lat_mode<T, LAT_GRAD_STEP>(a, s);
     case LAT_EXTRAP_FWD: return launch_lat_mode<T, LAT_EXTRAP_FWD>(a, s);
     case LAT_UPDATE_U: return launch_lat_mode<T, LAT_UPDATE_U>(a, s);
+    case LAT_R2C_HALF:
+    case LAT_C2R_HALF:
+      if constexpr (std::is_same<T, float>::value) return launch_lat_half(mode, a, s);
   }
   return cudaErrorInvalidValue;
 }

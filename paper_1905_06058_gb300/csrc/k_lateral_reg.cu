@@ -25,4 +25,22 @@ template <> cudaError_t launch_lat_reg<float>(int mode, const LatArgs<float>& a,
   return cudaErrorInvalidValue;
 }
 
+bool lat_half_takes(int L, int M) {
+  return lat_reg_takes<float>(L, L >= 768 ? 4 : 8) && M % (L >= 768 ? 16 : 32) == 0;
+}
+
+cudaError_t launch_lat_half(int mode, const LatArgs<float>& a, cudaStream_t s) {
+  switch (a.L) {
+    case 1024: return launch_lat_half_length<1024>(mode, a, s);
+    case 768: return launch_lat_half_length<768>(mode, a, s);
+    case 512: return launch_lat_half_length<512>(mode, a, s);
+    case 384: return launch_lat_half_length<384>(mode, a, s);
+    case 256: return launch_lat_half_length<256>(mode, a, s);
+    case 192: return launch_lat_half_length<192>(mode, a, s);
+    case 128: return launch_lat_half_length<128>(mode, a, s);
+    case 64: return launch_lat_half_length<64>(mode, a, s);
+  }
+  return cudaErrorInvalidValue;
+}
+
 }  // namespace isam

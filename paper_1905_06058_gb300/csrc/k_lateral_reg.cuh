@@ -198,6 +198,85 @@ static cudaError_t launch_lat_reg_mode(const LatArgs<T>& a, cudaStream_t s) {
   return cudaLaunchKernelEx(&cfg, kern, a);
 }
 
+// Real transforms of the half spectrum: a thread's complex column is two neighbouring
+// real ones, z = x_m + i x_{m+1}, so a real array takes half the transforms and its
+// spectrum half the memory.  FWD: H_m = (Z(q) + conj Z(-q)) / 2 and H_{m+1} = -i (Z(q) -
+// conj Z(-q)) / 2 of rows q <= L/2 after one more exchange; else Z(q) = H_m(q) + i
+// H_{m+1}(q), with H(-q) = conj H(q), as the rows are loaded.  M: real columns.
+template <bool FWD, int L>
+__global__ void __launch_bounds__(lat_reg_threads<float, L>(), lat_reg_min_blocks<float, L>())
+    k_lat_half(const __grid_constant__ LatArgs<float> a) {
+  constexpr int P = lreg::Plan<float, L>::P, TH = L / P, W = lreg::columns<float, L>();
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  float2* S = reinterpret_cast<float2*>(smem_raw);
+  const int tid = threadIdx.x, c = tid % W, b = tid / W;
+  // dependent launch as the plain passes of k_lat_reg
+  const unsigned blocks = gridDim.x * gridDim.y;
+  const bool early = blocks <= 32 || blocks > 152;
+  if (early) cudaTriggerProgrammaticLaunchCompletion();
+  const lreg::Twiddles<float, L> tw(b, nullptr);
+  cudaGridDependencySynchronize();
+  const size_t M = size_t(a.M), m = size_t(blockIdx.x) * (2 * W) + 2 * c;
+  const size_t real0 = size_t(blockIdx.y) * L * M + m, half0 = size_t(blockIdx.y) * (L / 2 + 1) * M + m;
+  float2 v[P];
+  if constexpr (FWD) {
+    const float* in = static_cast<const float*>(a.in) + real0;
+#pragma unroll
+    for (int i = 0; i < P; ++i) v[i] = *reinterpret_cast<const float2*>(in + (b + i * TH) * M);
+    lreg::transform<-1, L, W, 0, float>(v, S, tw, b, c, true, [] {});
+    __syncthreads();
+#pragma unroll
+    for (int i = 0; i < P; ++i) S[lreg::slot<float, L, W>(b + i * TH, c)] = v[i];
+    __syncthreads();
+    if (!early) cudaTriggerProgrammaticLaunchCompletion();
+    float2* out = static_cast<float2*>(a.out) + half0;
+    const float f = 0.5f * a.norm;
+#pragma unroll
+    for (int i = 0; i <= P / 2; ++i) {
+      const int q = b + i * TH;
+      if (q > L / 2) break;
+      const float2 z = v[i], y = S[lreg::slot<float, L, W>(q ? L - q : 0, c)];
+      const float4 h = make_float4(f * (z.x + y.x), f * (z.y - y.y), f * (z.y + y.y), f * (y.x - z.x));
+      *reinterpret_cast<float4*>(out + q * M) = h;
+    }
+  } else {
+    const float2* in = static_cast<const float2*>(a.in) + half0;
+#pragma unroll
+    for (int i = 0; i < P; ++i) {
+      const int q = b + i * TH;
+      const bool upper = q > L / 2;
+      const float4 h = *reinterpret_cast<const float4*>(in + (upper ? L - q : q) * M);
+      const float s = upper ? -1.0f : 1.0f;             // conj
+      v[i] = make_float2(h.x - s * h.w, s * h.y + h.z);
+    }
+    lreg::transform<+1, L, W, 0, float>(v, S, tw, b, c, true, [] {});
+    if (!early) cudaTriggerProgrammaticLaunchCompletion();
+    float* out = static_cast<float*>(a.out) + real0;
+#pragma unroll
+    for (int i = 0; i < P; ++i)
+      *reinterpret_cast<float2*>(out + (b + i * TH) * M) = cscale(v[i], a.norm);
+  }
+}
+
+template <int L> static cudaError_t launch_lat_half_length(int mode, const LatArgs<float>& a,
+                                                           cudaStream_t s) {
+  constexpr int W = lreg::columns<float, L>();
+  constexpr size_t sm = lreg::smem_elements<float, L, W>() * sizeof(float2);
+  auto* kern = mode == LAT_R2C_HALF ? k_lat_half<true, L> : k_lat_half<false, L>;
+  allow_smem(kern, sm);
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(a.M / (2 * W), a.B);
+  cfg.blockDim = dim3(lat_reg_threads<float, L>());
+  cfg.dynamicSmemBytes = sm;
+  cfg.stream = s;
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = at;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, kern, a);
+}
+
 template <typename T, int L>
 static cudaError_t launch_lat_reg_length(int mode, const LatArgs<T>& a, cudaStream_t s) {
   switch (mode) {

@@ -100,3 +100,34 @@ def test_fp64(torch, L, along_y):
         assert rel(got[0][0], got[1][0]) < 1e-10
         assert got[0][1] == pytest.approx(got[1][1], rel=1e-10)
     plan.close()
+
+
+@pytest.mark.parametrize("kw", [dict(nx=L, nk=nk, nz=64) for L in LENGTHS for nk in (32, 64)] +
+                         [dict(nx=64, ny=ny, nk=32, nz=32) for ny in (2, 4, 24, 64)] +
+                         [dict(nx=192, ny=2, nk=64, nz=64)],
+                         ids=lambda k: "x".join(str(v) for v in k.values()))
+def test_half_spectra(torch, kw):
+    """A and A^H of FP32 plans whose x passes keep half of the Hermitian spectra, with
+    columns paired across y at x = 0 and nx/2, against the oracle and the radix-8 form,
+    which keeps them whole."""
+    from paper_1905_06058_gb300.isam import Plan
+    g = I.small_bscan(seed=68, **kw).geom
+    ref = O.IsamOracle(g, "nufft")
+    eta = I.random_image(ref.image_shape, 69).astype(np.complex64)
+    y = I.random_spectra(ref.spec_shape, 70).astype(np.float32)
+    plan = Plan(g)
+    for r in (16, 8):
+        plan.set_tuning(lateral_radix=r)
+        a = plan.forward(torch.from_numpy(eta).cuda()).cpu().numpy()
+        b = plan.adjoint(torch.from_numpy(y).cuda()).cpu().numpy()
+        assert rel(a, ref.forward(eta.astype(np.complex128))) < 1e-5
+        assert rel(b, ref.adjoint(y.astype(np.float64))) < 1e-5
+    plan.set_tuning(lateral_radix=16)                    # real arrays off the 8-byte grid
+    buf = torch.zeros(2 * (y.size + 1), dtype=torch.float32, device="cuda")
+    odd = buf[1:1 + y.size].view(y.shape)
+    out = buf[y.size + 1 | 1:][:y.size].view(y.shape)
+    odd.copy_(torch.from_numpy(y))
+    assert rel(plan.adjoint(odd).cpu().numpy(), b) < 2e-5
+    plan.forward(torch.from_numpy(eta).cuda(), out=out)
+    assert rel(out.cpu().numpy(), a) < 2e-5
+    plan.close()
