@@ -28,6 +28,15 @@ template <typename T> struct alignas(2 * sizeof(cplx<T>)) cpair { cplx<T> a, b; 
 // one column where the axial kernels otherwise take a pair
 template <typename T> struct alignas(sizeof(cplx<T>)) cone { cplx<T> a; };
 
+// Two complex numbers next to each other in memory, one 16-byte (32-byte) load
+// or store; p is a multiple of that.
+template <typename T> __device__ __forceinline__ cpair<T> load_two(const cplx<T>* p) {
+  return *reinterpret_cast<const cpair<T>*>(p);
+}
+template <typename T> __device__ __forceinline__ void store_two(cplx<T>* p, cplx<T> a, cplx<T> b) {
+  *reinterpret_cast<cpair<T>*>(p) = {a, b};
+}
+
 // arithmetic on complex numbers and complex pairs
 template <typename C> __device__ __forceinline__ C eadd(C a, C b) { return cadd(a, b); }
 template <typename C> __device__ __forceinline__ C esub(C a, C b) { return csub(a, b); }

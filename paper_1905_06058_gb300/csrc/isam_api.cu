@@ -1448,7 +1448,7 @@ template <typename T> isam_status unrolled_impl(isam_plan* P, const T* s_d,
 //   ubar = J_T(u^k)^T zbar^k,  etabar = ubar - (1/L) A^H A ubar,
 //   theta_bar -= (1/L)(<dA ubar, A eta^k - s_d> + <A ubar, dA eta^k>),
 //   s_bar += (1/L) A ubar,  zbar^{k-1} += (1 + mu_{k-1}) etabar,
-//   zbar^{k-2} -= mu_{k-1} etabar.
+//   zbar^{k-2} = -mu_{k-1} etabar (its first term).
 template <typename T> isam_status unrolled_vjp_impl(isam_plan* P, const T* s_d,
                                                     const isam_solve_opts* o, int every,
                                                     const cplx<T>* ckpt, const cplx<T>* z_bar,
@@ -1473,7 +1473,7 @@ template <typename T> isam_status unrolled_vjp_impl(isam_plan* P, const T* s_d,
   CUDA_TRY(cudaMemsetAsync(P->flag, 0, sizeof(int), s));
   CUDA_TRY(cudaMemsetAsync(P->cpartial, 0, sizeof(double) * 5 * P->npairs, s));
   CUDA_TRY(cudaMemcpyAsync(zb[0], z_bar, bytes, cudaMemcpyDeviceToDevice, s));
-  CUDA_TRY(cudaMemsetAsync(zb[1], 0, 2 * bytes, s));
+  CUDA_TRY(cudaMemsetAsync(zb[1], 0, bytes, s));   // zbar^{k-2} is written before it is added to
   if (s_bar) CUDA_TRY(cudaMemsetAsync(s_bar, 0, sizeof(T) * P->n_spec, s));
   ISAM_TRY(lat_forward<T>(P, im, s_d, im.sdh, P->nk, true));
   int cur = 0;                          // zb[cur] = zbar^k, then zbar^{k-1}, zbar^{k-2}
@@ -1517,10 +1517,11 @@ template <typename T> isam_status unrolled_vjp_impl(isam_plan* P, const T* s_d,
         return launch_param_reduce<T>(param_args<T>(P, im.spec, seg_S + i * ns, im.sdh, T(-1), true),
                                       P->npairs, s);
       }));
-      // b = A^H A ubar
-      ISAM_TRY(launch(P, ISAM_KCLASS_AX_ADJ, [&] {
-        return launch_ax_adj<T>(ax_args<T>(P, im, im.spec, im.grad), P->npairs, s);
-      }));
+      // b = A^H A ubar, wanted by zbar^{k-1} and zbar^{k-2}
+      if (k > 1)
+        ISAM_TRY(launch(P, ISAM_KCLASS_AX_ADJ, [&] {
+          return launch_ax_adj<T>(ax_args<T>(P, im, im.spec, im.grad), P->npairs, s);
+        }));
       if (s_bar) {
         ISAM_TRY(lat_inverse<T>(P, im, im.spec, im.s_tmp, P->nk, true));
         ISAM_TRY(launch(P, ISAM_KCLASS_MISC, [&] {
@@ -1529,12 +1530,13 @@ template <typename T> isam_status unrolled_vjp_impl(isam_plan* P, const T* s_d,
                                  reinterpret_cast<cplx<T>*>(s_bar), P->n_spec / 2, s);
         }));
       }
-      ISAM_TRY(lat_inverse<T>(P, im, im.grad, bimg, P->nz, false));
-      ISAM_TRY(launch(P, ISAM_KCLASS_MISC, [&] {
-        return launch_bwd_combine<T>(ubar, bimg, T(1.0 / L), T(mu[k - 1]), k - 1 >= 1 ? zm1 : nullptr,
-                                     k - 2 >= 1 ? zm2 : nullptr, n, s);
-      }));
-      CUDA_TRY(cudaMemsetAsync(zcur, 0, bytes, s));   // becomes zbar^{k-3}
+      if (k > 1) {
+        ISAM_TRY(lat_inverse<T>(P, im, im.grad, bimg, P->nz, false));
+        ISAM_TRY(launch(P, ISAM_KCLASS_MISC, [&] {
+          return launch_bwd_combine<T>(ubar, bimg, T(1.0 / L), T(mu[k - 1]), zm1,
+                                       k > 2 ? zm2 : nullptr, n, s);
+        }));
+      }
       cur = (cur + 1) % 3;
     }
   }

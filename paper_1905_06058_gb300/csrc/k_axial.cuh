@@ -129,15 +129,6 @@ template <typename T, typename V> struct Sample {
                   // (evanescent, or past nk)
 };
 
-// Two complex numbers next to each other in memory, one 16-byte (32-byte) load
-// or store; p is a multiple of that.
-template <typename T> __device__ __forceinline__ cpair<T> load_two(const cplx<T>* p) {
-  return *reinterpret_cast<const cpair<T>*>(p);
-}
-template <typename T> __device__ __forceinline__ void store_two(cplx<T>* p, cplx<T> a, cplx<T> b) {
-  *reinterpret_cast<cpair<T>*>(p) = {a, b};
-}
-
 // Stolt positions and spectral phases of a quad of samples 4 q .. 4 q + 3 of one
 // column pair, from the plan's table when present, else evaluated (float-float /
 // double).
