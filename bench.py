@@ -228,22 +228,23 @@ def algorithmic_bytes(cls: str, n_img: int, n_spec: int, real_bytes=4) -> int:
 # Volume figures are per launch of the 256 x 256 x 2048 case, scaled from a
 # 128 x 128 x 2048 capture by the column pairs (32,770 / 8,194).
 KERNEL_SOURCES = {
-    "ax_fused": ["k_axial.cuh", "k_axial.cu", "fft_smem.cuh", "fft_col16.cuh", "internal.cuh",
-                 "common.cuh"],
-    "lat_update": ["k_lateral.cu", "fft_smem.cuh", "internal.cuh", "common.cuh"],
+    "ax_fused": ["k_axial.cuh", "k_axial.cu", "tmem.cuh", "fft_smem.cuh", "fft_col16.cuh",
+                 "internal.cuh", "common.cuh"],
+    "lat_update": ["k_lateral.cu", "k_lateral_reg.cuh", "k_lateral_reg.cu", "lat_reg.cuh",
+                   "lat_point.cuh", "fft_smem.cuh", "internal.cuh", "common.cuh"],
 }
 NCU_CAPTURES = {
     "bscan_1024x2048": {
-        "ax_fused": {"sha": "42f5dcc0e5acc4f1", "dram": 42414080, "table": 16809984,
-                     "smem_wavefronts": 6623241},
-        "lat_update": {"sha": "aa2e880b8cc2d1e4", "dram": 34312448, "table": 0,
-                       "smem_wavefronts": 2414784},
+        "ax_fused": {"sha": "e96a16716a1edf05", "dram": 42348800, "table": 16809984,
+                     "smem_wavefronts": 4433003},
+        "lat_update": {"sha": "d98e511182027fc8", "dram": 34208256, "table": 0,
+                       "smem_wavefronts": 537628},
     },
     "volume_256x256x2048": {
-        # 128 x 128 x 2048 capture with the plan's Stolt table: 781,895,936 B and
-        # 116,578,155 wavefronts over 8,194 pairs
-        "ax_fused": {"sha": "42f5dcc0e5acc4f1", "dram": 3127011206, "table": 545292288,
-                     "smem_wavefronts": 466227256},
+        # 128 x 128 x 2048 capture with the plan's Stolt table: 780,832,512 B and
+        # 75,660,361 wavefronts over 8,194 pairs
+        "ax_fused": {"sha": "e96a16716a1edf05", "dram": 3122758289, "table": 545292288,
+                     "smem_wavefronts": 302586042},
     },
 }
 

@@ -461,7 +461,9 @@ __device__ __forceinline__ void scatter_samples(const Coefficients<T, J>& co, V*
 // scatter took 56 shared-memory accesses a thread (8 to zero, 24 reads, 24
 // writes) in 8 barrier phases, the per-sample gather 24; the windows take 23
 // and 13 (J = 6).  k_ax_fused, 1024 x 2048 B-scan: 51.5 -> 47.6 us, 256 x 256 x
-// 2048 volume: 2,414 -> 2,117 us; k_ax_adj 36.8 -> 30.7 us and 1,598 -> 1,300 us.
+// 2048 volume: 2,414 -> 2,117 us; k_ax_adj 36.8 -> 30.7 us and 1,598 -> 1,300 us
+// (40.2, 1,817 and 1,096 us with what followed: the quad-major table, constant
+// shared-memory distances, tensor memory, half spectra).
 //
 // The bound of 2.3 bins keeps four samples and the next thread's first within
 // the offsets the kernels hold as constants (three steps below 7 bins, four
@@ -926,6 +928,12 @@ __global__ void __launch_bounds__(512, ax_min_blocks<T>()) k_ax_adj(const __grid
 // columns of the pair; then G = N'(conj(phase) R), written as is or, when
 // u_hat_scale = 1/L, as u_hat = eta_hat - G/L (put_output).  F s_d is
 // Hermitian, so only its c1 column is read.
+//
+// What bounds it: two blocks a multiprocessor (64 registers a thread) with some 2,300
+// instructions a warp between ten barriers.  On a 128 x 128 x 2048 volume (464 us, 27
+// waves) 53 % of the issue slots and 64 % of the load/store data path are taken, half
+// of the latter by the transforms' exchanges; DRAM 21 %.  A 1024 x 2048 B-scan (513
+// blocks, 40.2 us) leaves the second of its 1.7 waves two thirds full.
 // WS: also write the model spectra S to A.s_out.
 template <typename T, int J, int LOGK, bool WS, bool C16>
 __global__ void __launch_bounds__(512, ax_min_blocks<T>()) k_ax_fused(const __grid_constant__ AxArgs<T> A) {

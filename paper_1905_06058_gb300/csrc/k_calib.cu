@@ -55,9 +55,8 @@ __device__ __forceinline__ cplx<T> real_part_spectrum(cplx<T> a, cplx<T> b) {
 // of both columns a load and has two such groups in flight; TPB is a quarter of nk up
 // to 512, so that they cover nk = 2048.  FP32 plans keep the samples' arithmetic in
 // float, the cancelling 2 kappa - sqrt(a) from a two-float constant, and the threads'
-// sums are added in double by one warp a moment.  512 x 2048: 24.7 -> 16.5 us
-// at one block a multiprocessor (72 registers), and 7.15 -> 6.8 ms a calibration step's
-// passes at two (64) with dependent launches.
+// sums are added in double by one warp a moment.  512 x 2048: 24.7 -> 15.2 us (16.5 at
+// one block a multiprocessor, 72 registers).
 template <typename T> struct ParamSamples {
   cpair<T> S1, S2, E1, E2, f1, f2;
 };
@@ -206,8 +205,11 @@ __device__ __forceinline__ double2 st_vjp(double2 u, double2 zb, double tau) {
   return make_double2(zb.x - tau * (zb.x * inv - u.x * rz), zb.y - tau * (zb.y * inv - u.y * rz));
 }
 
-// The pointwise kernels move 24 and 48 bytes an element out of DRAM; a thread takes two
-// pairs of neighbours, half a grid apart, all of its loads in flight at once.
+// The pointwise kernels move 24 and 40 bytes an element (48, and 8 to clear zbar^{k-3},
+// when zbar^{k-2} was added to); a thread takes two pairs of neighbours, half a grid
+// apart, all of its loads in flight at once.  512 x 2048, cold caches: 7.3 -> 7.5 and
+// 10.0 -> 9.0 us; dependent launch hides their ramps (7.15 -> 6.8 ms a calibration
+// case of 120 such launches).
 constexpr int POINT_THREADS = 256;
 inline unsigned point_blocks(size_t n) {
   return unsigned((n + 4 * POINT_THREADS - 1) / (4 * POINT_THREADS));

@@ -5,7 +5,9 @@
 // eta_hat^{k+1} out), 67 MB at 1024 x 2048 out of the L2.  256 blocks of 256
 // threads, two on a multiprocessor (128 registers: 32 points of data, 8 of
 // z^{k-1} in flight).  The iterates are loaded in batches of eight, the first
-// before the last exchange's barrier so that its latency covers the exchange.
+// before the last exchange's barrier so that its latency covers the exchange
+// (one by one as the points are used up: 4 us a launch more).  LAT_UPDATE_U at 1024 x
+// 2048: 25.6 -> 16.5 us; along y of a 128 x 128 x 2048 volume 209 -> 158 us, 6.8 TB/s.
 #pragma once
 
 #include <type_traits>
