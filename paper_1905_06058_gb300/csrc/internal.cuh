@@ -197,6 +197,7 @@ template <typename T> cudaError_t launch_norm2(const cplx<T>* x, size_t n, doubl
 // written) leave everything as it is.  stop null: the plain sums only.
 struct StopRule {
   int* stop;       // [2] device: stopped flag, iteration of the stop
+  int* host;       // pinned copy of stop[0..1] for the host to read, or null
   double* rr;      // device: r_r of the latest evaluated check
   double tol, eps;
   int iter;

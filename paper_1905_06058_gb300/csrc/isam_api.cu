@@ -796,21 +796,29 @@ template <typename T> isam_status solve_impl(isam_plan* P, const T* s_d, const i
   double rr = -1.0;
   int done = 0;
   // The stop rule runs on the device (StopRule; only the l1 prior takes
-  // tol > 0).  The host reads a check's outcome kStopLag iterations after
-  // queuing it, so a check never drains the GPU; only the iterations queued
+  // tol > 0), whose check also writes its outcome to pinned memory.  The host reads
+  // it kStopLag iterations after queuing it, so a check never drains the GPU, after
+  // an event that is recorded behind the iteration after the check (a copy or an
+  // event right behind the check held the next kernel's launch back: a check every
+  // iteration 82 -> 68 us at 1024 x 2048); only the iterations queued
   // while an outcome is unread carry the stop flag (their kernels write nothing
   // once it is set), and the result is the iterate of the stopping check.
-  constexpr int kStopLag = 2;
+  constexpr int kStopLag = 3;
   const bool dev_stop = check;
-  if (dev_stop) CUDA_TRY(cudaMemsetAsync(P->dstop, 0, 2 * sizeof(int), s));
+  if (dev_stop) {
+    CUDA_TRY(cudaMemsetAsync(P->dstop, 0, 2 * sizeof(int), s));
+    P->hstop[0] = 0;
+  }
   bool pending = false;   // a check whose outcome the host has not read
   int since = 0;          // iterations queued after it
   for (int it = 1; it <= o->max_iter; ++it) {
     const int k = k0 + it;
-    const bool norms = check && (it % every == 0 || it == o->max_iter);
+    auto checks = [&](int i) { return check && (i % every == 0 || i == o->max_iter); };
+    const bool norms = checks(it);
     StopRule sr{};
     if (dev_stop) {
       sr.stop = P->dstop;
+      sr.host = P->hstop;
       sr.rr = P->dscal + 7;
       sr.tol = o->tol;
       sr.eps = eps;
@@ -824,15 +832,15 @@ template <typename T> isam_status solve_impl(isam_plan* P, const T* s_d, const i
     done = it;
     if (dev_stop) {
       // read the pending check once kStopLag iterations keep the GPU busy, or
-      // before this check's outcome takes the pinned slot
-      if (pending && (++since >= kStopLag || norms)) {
+      // at the next check
+      if (pending && ++since == 1 && !norms) CUDA_TRY(cudaEventRecord(P->ev_check, s));
+      if (pending && (since >= kStopLag || norms)) {
         CUDA_TRY(cudaEventSynchronize(P->ev_check));
         pending = false;
-        if (P->hstop[0]) break;
+        if (*static_cast<volatile int*>(P->hstop)) break;
       }
       if (norms) {
-        CUDA_TRY(cudaMemcpyAsync(P->hstop, P->dstop, 2 * sizeof(int), cudaMemcpyDeviceToHost, s));
-        CUDA_TRY(cudaEventRecord(P->ev_check, s));
+        if (checks(it + 1)) CUDA_TRY(cudaEventRecord(P->ev_check, s));
         pending = true;
         since = 0;
       }

@@ -210,10 +210,13 @@ template cudaError_t launch_wl1<float>(const float2*, size_t, const float*, int,
 template cudaError_t launch_wl1<double>(const double2*, size_t, const double*, int, double*, int,
                                         double*, cudaStream_t);
 
-// out[0..2] = column sums of partial[n][3]
+// out[0..2] = column sums of partial[n][3].  Dependent launch: the next kernel may
+// start its prologue once the partials' kernel is complete.
 __global__ void __launch_bounds__(256) k_sum3(const double* partial, int n, double* out,
                                               const StopRule sr) {
   __shared__ double red[3][8];
+  cudaGridDependencySynchronize();
+  cudaTriggerProgrammaticLaunchCompletion();
   // an earlier check stopped the solve: this iteration's kernels returned
   // without writing the partials
   if (sr.stop && *reinterpret_cast<const volatile int*>(sr.stop)) return;
@@ -231,14 +234,26 @@ __global__ void __launch_bounds__(256) k_sum3(const double* partial, int n, doub
       if (rr < sr.tol) {
         sr.stop[1] = sr.iter;
         sr.stop[0] = 1;
+        if (sr.host) {
+          sr.host[1] = sr.iter;
+          sr.host[0] = 1;
+        }
       }
     }
   }
 }
 cudaError_t launch_sum3(const double* partial, int n, double* out, const StopRule& sr,
                         cudaStream_t s) {
-  k_sum3<<<1, 256, 0, s>>>(partial, n, out, sr);
-  return cudaGetLastError();
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(1);
+  cfg.blockDim = dim3(256);
+  cfg.stream = s;
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = at;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, k_sum3, partial, n, out, sr);
 }
 
 template <typename T>
