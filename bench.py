@@ -235,16 +235,16 @@ KERNEL_SOURCES = {
 }
 NCU_CAPTURES = {
     "bscan_1024x2048": {
-        "ax_fused": {"sha": "e96a16716a1edf05", "dram": 42348800, "table": 16809984,
-                     "smem_wavefronts": 4433003},
-        "lat_update": {"sha": "d98e511182027fc8", "dram": 34208256, "table": 0,
-                       "smem_wavefronts": 537628},
+        "ax_fused": {"sha": "576d9684e6edeac1", "dram": 42535168, "table": 16809984,
+                     "smem_wavefronts": 4430443},
+        "lat_update": {"sha": "4497d26ea88790d5", "dram": 34221312, "table": 0,
+                       "smem_wavefronts": 536837},
     },
     "volume_256x256x2048": {
-        # 128 x 128 x 2048 capture with the plan's Stolt table: 780,832,512 B and
-        # 75,660,361 wavefronts over 8,194 pairs
-        "ax_fused": {"sha": "e96a16716a1edf05", "dram": 3122758289, "table": 545292288,
-                     "smem_wavefronts": 302586042},
+        # 128 x 128 x 2048 capture with the plan's Stolt table: 780,839,680 B and
+        # 75,660,736 wavefronts over 8,194 pairs
+        "ax_fused": {"sha": "576d9684e6edeac1", "dram": 3122786956, "table": 545292288,
+                     "smem_wavefronts": 302587542},
     },
 }
 
