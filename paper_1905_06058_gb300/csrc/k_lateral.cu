@@ -56,6 +56,22 @@ bool fft_length(int L, int* log2, int* r3) {
   return true;
 }
 
+// Two neighbours of a caller's array, in one access where the array starts on its size
+// (`aligned`), else in two: the operators take arrays at any element.
+template <typename V, typename E> __device__ __forceinline__ V load_pair(const E* p, bool aligned) {
+  if (aligned) return *reinterpret_cast<const V*>(p);
+  return {p[0], p[1]};
+}
+template <typename V, typename E>
+__device__ __forceinline__ void store_pair(E* p, E x, E y, bool aligned) {
+  if (aligned) {
+    *reinterpret_cast<V*>(p) = V{x, y};
+  } else {
+    p[0] = x;
+    p[1] = y;
+  }
+}
+
 template <typename T> struct rpair_t;
 template <> struct rpair_t<float> { using type = float2; };
 template <> struct rpair_t<double> { using type = double2; };
@@ -92,6 +108,11 @@ __global__ void __launch_bounds__(512, std::is_same<T, float>::value ? 2 : 1) k_
   // Every thread owns ept = n_el / blockDim elements (8 for L >= 8):
   // element i of a thread is e = tid + i * nt (row e / TP, pair-column e % TP).
   const int ept = n_el / nt;
+  constexpr bool REAL_IN = MODE == LAT_R2C_FWD, REAL_OUT = MODE == LAT_INV_REAL;
+  const bool in_aligned =
+      reinterpret_cast<uintptr_t>(a.in) % (REAL_IN ? sizeof(RP) : sizeof(V)) == 0;
+  const bool out_aligned =
+      reinterpret_cast<uintptr_t>(a.out) % (REAL_OUT ? sizeof(RP) : sizeof(V)) == 0;
   auto gidx = [&](int e) { return base + size_t(e >> logTP) * M + 2 * (e & (TP - 1)); };
   auto sidx = [&](int e) { return prow(e >> logTP) * TP + (e & (TP - 1)); };
   auto lat_fft = [&](auto sign) {
@@ -110,7 +131,7 @@ __global__ void __launch_bounds__(512, std::is_same<T, float>::value ? 2 : 1) k_
       if (i >= ept) break;
       const size_t gi = gidx(tid + i * nt);
       if (MODE == LAT_R2C_FWD) {
-        const RP r = *reinterpret_cast<const RP*>(static_cast<const T*>(a.in) + gi);
+        const RP r = load_pair<RP>(static_cast<const T*>(a.in) + gi, in_aligned);
         v[i].a = mk<T>(r.x, T(0));
         v[i].b = mk<T>(r.y, T(0));
       } else if (MODE == LAT_EXTRAP_FWD) {
@@ -118,7 +139,7 @@ __global__ void __launch_bounds__(512, std::is_same<T, float>::value ? 2 : 1) k_
         const V z2 = *reinterpret_cast<const V*>(a.z2 + gi);
         v[i] = eadd(z1, escale(esub(z1, z2), a.mu));
       } else {
-        v[i] = *reinterpret_cast<const V*>(static_cast<const C*>(a.in) + gi);
+        v[i] = load_pair<V>(static_cast<const C*>(a.in) + gi, in_aligned);
       }
     }
 #pragma unroll
@@ -141,7 +162,8 @@ __global__ void __launch_bounds__(512, std::is_same<T, float>::value ? 2 : 1) k_
     for (int i = 0; i < 8; ++i) {
       if (i >= ept) break;
       const int e = tid + i * nt;
-      *reinterpret_cast<V*>(out + gidx(e)) = escale(buf[sidx(e)], nrm);
+      const V v = escale(buf[sidx(e)], nrm);
+      store_pair<V>(out + gidx(e), v.a, v.b, out_aligned);
     }
     return;
   }
@@ -152,10 +174,7 @@ __global__ void __launch_bounds__(512, std::is_same<T, float>::value ? 2 : 1) k_
       if (i >= ept) break;
       const int e = tid + i * nt;
       const V v = buf[sidx(e)];
-      RP r;
-      r.x = v.a.x * nrm;
-      r.y = v.b.x * nrm;
-      *reinterpret_cast<RP*>(out + gidx(e)) = r;
+      store_pair<RP>(out + gidx(e), v.a.x * nrm, v.b.x * nrm, out_aligned);
     }
     return;
   }
