@@ -25,18 +25,19 @@ namespace c16 {
 
 enum { P8 = 8, P16 = 16 };
 
-// float2 index of (row, column c) in layout PAD
-template <int PAD> __device__ __forceinline__ int el(int row, int c) {
-  return 2 * (PAD == P8 ? row + (row >> 3) : row + (row >> 4)) + c;
+// float2 index of (row, column c) in layout PAD, W columns a row (2 for the axial
+// column pair, 2 TP for a lateral tile of TP column pairs)
+template <int PAD, int W = 2> __device__ __forceinline__ int el(int row, int c) {
+  return W * (PAD == P8 ? row + (row >> 3) : row + (row >> 4)) + c;
 }
 // ... of (row + STEP r, c), given e = el(row, c): a constant distance, which the
 // compiler does not find through the shift (left to it, the index arithmetic of the
 // passes was a tenth of k_ax_fused's instructions).  STEP is a multiple of the
 // padding period, or the rows row .. row + STEP r stay within one (row a multiple
 // of 16, STEP 1, r < 16 in P16).
-template <int PAD, int STEP> __device__ __forceinline__ constexpr int el_step(int r) {
+template <int PAD, int STEP, int W = 2> __device__ __forceinline__ constexpr int el_step(int r) {
   static_assert(STEP % PAD == 0 || (STEP == 1 && PAD == P16), "a constant distance in the layout");
-  return STEP % PAD == 0 ? 2 * r * (STEP + STEP / PAD) : 2 * r;
+  return STEP % PAD == 0 ? W * r * (STEP + STEP / PAD) : W * r;
 }
 
 // multiply by W16^1 = e^{SIGN 2 pi i / 16} and W16^3
@@ -152,15 +153,15 @@ template <int SIGN, int R> __device__ __forceinline__ void twiddle(float2* a, fl
 // buffer: this thread's 16 / R butterflies j = b + u L/16 read
 // rows j + r L/R (layout IN), barrier, write rows (j - k) R + k + r NS (layout
 // OUT), barrier.  tw: this pass's segment (unused for NS = 1).
-template <int SIGN, int R, int L, int NS, int IN, int OUT>
+template <int SIGN, int R, int L, int NS, int IN, int OUT, int W = 2>
 __device__ __forceinline__ void pass(float2* Y, int b, int c, const float4* tw) {
   constexpr int NB = 16 / R, LR = L / R, L16 = L / 16;
   float2 v[16];
 #pragma unroll
   for (int u = 0; u < NB; ++u) {
-    const float2* in = Y + el<IN>(b + u * L16, c);
+    const float2* in = Y + el<IN, W>(b + u * L16, c);
 #pragma unroll
-    for (int r = 0; r < R; ++r) v[u * R + r] = in[el_step<IN, LR>(r)];
+    for (int r = 0; r < R; ++r) v[u * R + r] = in[el_step<IN, LR, W>(r)];
   }
   __syncthreads();
 #pragma unroll
@@ -170,9 +171,9 @@ __device__ __forceinline__ void pass(float2* Y, int b, int c, const float4* tw) 
     float2* a = v + u * R;
     if (NS > 1) twiddle<SIGN, R>(a, tw[k]);
     dft_r<SIGN, R>(a);
-    float2* out = Y + el<OUT>((j - k) * R + k, c);
+    float2* out = Y + el<OUT, W>((j - k) * R + k, c);
 #pragma unroll
-    for (int r = 0; r < R; ++r) out[el_step<OUT, NS>(r)] = a[r];
+    for (int r = 0; r < R; ++r) out[el_step<OUT, NS, W>(r)] = a[r];
   }
   __syncthreads();
 }
@@ -227,6 +228,40 @@ __device__ __forceinline__ void inverse(float2* Y, const float4* tw, Before befo
     if (u == 0) before();
 #pragma unroll
     for (int r = 0; r < R; ++r) emit(u + r * NB, a[r]);   // row jj + 256 r = j + (u + r NB) K/16
+  }
+}
+
+// Lateral transforms of a tile of W = 2 TP columns (k_lat's instances of LAT_FIT), L =
+// 1024 = 16 * 4 * 16 or 256 = 16 * 16: thread t owns column c = t mod W of butterfly
+// j = t / W, the tile's rows in layout P8 before and after the transform, P16 between
+// its passes.  Twiddle segments as Passes', of the spans 16 and 64 (the radix-4 pass
+// sits at span 16, where a thread's four butterflies j = b + 64 u share one entry).
+template <int LOGL> __host__ __device__ constexpr int lat_entries() {
+  return LOGL == 10 ? 16 + 64 : 16;
+}
+template <int LOGL> __device__ __forceinline__ const float4* build_lat_twiddles(float4* tw) {
+  for (int e = threadIdx.x; e < lat_entries<LOGL>(); e += blockDim.x) {
+    const int ns = e < 16 ? 16 : 64, k = e < 16 ? e : e - 16;
+    const int R = e < 16 && LOGL == 10 ? 4 : 16;
+    float s1, c1, s4, c4;
+    sincospif(float(2 * k) / float(ns * R), &s1, &c1);
+    sincospif(float(8 * k) / float(ns * R), &s4, &c4);
+    tw[e] = make_float4(c1, -s1, c4, -s4);
+  }
+  __syncthreads();
+  return tw;
+}
+// unnormalised, in place (SIGN -1: e^{-}); ends with a barrier
+template <int SIGN, int LOGL, int W>
+__device__ __forceinline__ void lat_transform(float2* Y, const float4* tw) {
+  constexpr int L = 1 << LOGL;
+  const int c = threadIdx.x & (W - 1), j = threadIdx.x / W;
+  pass<SIGN, 16, L, 1, P8, P16, W>(Y, j, c, tw);
+  if constexpr (LOGL == 10) {
+    pass<SIGN, 4, L, 16, P16, P16, W>(Y, j, c, tw);
+    pass<SIGN, 16, L, 64, P16, P8, W>(Y, j, c, tw + 16);
+  } else {
+    pass<SIGN, 16, L, 16, P16, P8, W>(Y, j, c, tw);
   }
 }
 

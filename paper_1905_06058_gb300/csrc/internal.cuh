@@ -87,6 +87,10 @@ enum LatMode : int {
                      // no norm partials)
 };
 
+// LAT_REGS: the tile in registers where lat_reg_takes; LAT_RADIX8: radix-8 column-pair
+// transforms in shared memory; LAT_FIT: those of calibrations with nz > nk (FitOrder)
+enum LatForm : int { LAT_RADIX8 = 0, LAT_REGS = 1, LAT_FIT = 2 };
+
 template <typename T> struct LatArgs {
   const void* in;        // complex (or real for R2C)
   void* out;             // complex (or real for INV_REAL)
@@ -107,9 +111,8 @@ template <typename T> struct LatArgs {
   cplx<T>* uout;         // optional: u^k = eta^k - g^k before the threshold
   const double* lam_dev; // optional: lambda / L = lam_scale * (*lam_dev), read on the device
   double lam_scale;
-  // tiles that have a register form (lat_reg_takes): 1 runs it, 0 the
-  // radix-8 column-pair transforms in shared memory; ignored elsewhere
-  int radix16;
+  // which transforms (LatForm); ignored by tiles that have one form only
+  int form;
   // solve with the device-side stop rule (see StopRule): a nonzero *stop, read
   // after the wait for the previous kernel, makes the launch return at once;
   // null elsewhere
@@ -143,6 +146,7 @@ template <typename T> struct AxArgs {
   // FP32, K = 1024 to 4096: 1 runs the column-split radix-16 transforms, 0 the
   // radix-8 column-pair ones (the plan's tuned choice); ignored elsewhere
   int radix16;
+  int fit;                // the scatter by residue classes (FitOrder)
   unsigned past_offset;  // shared-memory offset of window_past's bins (set at launch)
   // fused kernel in a solve with the device-side stop rule: as LatArgs::stop
   const int* stop;
@@ -237,6 +241,7 @@ template <typename T> struct ParamArgs {
   StoltConst sc;
   double* partial;       // [npairs][5], accumulated
   int write_fa;
+  int fit;               // FP32: the sums in FitOrder
 };
 template <typename T> cudaError_t launch_param_reduce(const ParamArgs<T>& a, int npairs,
                                                       cudaStream_t s);

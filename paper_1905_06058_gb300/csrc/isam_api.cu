@@ -89,6 +89,7 @@ struct isam_plan {
   // in registers, the default) or 8 (radix-8 column-pair passes)
   int tune_radix_ax = 16;
   int tune_radix_lat = 16;
+  bool fit_order = false;       // see FitOrder
   int batch_refs = 0;           // batches whose graph records this plan's kernels
   // filter B of Eq. 3 per |q| class, interleaved (re, im); empty: B = 1
   std::vector<double> filt_host;
@@ -362,7 +363,7 @@ template <typename T> isam_status lat(isam_plan* P, int mode, const LatArgs<T>& 
   const int cls = mode == LAT_UPDATE || mode == LAT_UPDATE_U ? ISAM_KCLASS_LAT_UPDATE
                                                              : ISAM_KCLASS_LAT_FFT;
   LatArgs<T> b = a;
-  b.radix16 = P->tune_radix_lat == 16 ? 1 : 0;
+  b.form = P->tune_radix_lat != 16 ? LAT_RADIX8 : P->fit_order ? LAT_FIT : LAT_REGS;
   if constexpr (sizeof(T) == 8)
     b.roots = impl_of<T>(P).roots + P->K + (b.L == P->nx ? 0 : P->nx);
   return launch(P, cls, [&] { return launch_lat<T>(mode, b, P->stream); });
@@ -371,6 +372,29 @@ template <typename T> isam_status lat(isam_plan* P, int mode, const LatArgs<T>& 
 template <typename T> const Poly<T>& poly_of(const isam_plan* P);
 template <> const Poly<float>& poly_of<float>(const isam_plan* P) { return P->poly32; }
 template <> const Poly<double>& poly_of<double>(const isam_plan* P) { return P->poly64; }
+
+// FP32 plans whose image is finer than their spectra (nz > nk).  Such a model can form
+// any spectra: positions rise by two to 2.3 of the K = 2 nz bins a sample, so nk samples
+// cover a part of the bins and A A^H is close to a multiple of one.  A fit's residual
+// falls to 1e-3 or less of the spectra in 15 iterations, the loss (its square) and the
+// gradient are differences of nearly equal numbers, and both follow the order of every
+// sum before them, that of lambda = c max |A^H s| included: between this order and the
+// windows, register tiles and half spectra of the other calls gradients moved by 1 to
+// 47 %, losses by 1e-6 to 6e-3 (17 fits of 128 to 512 columns), with either 9 to 11 %
+// from 64 bits.  So that such fits give the values they always gave, the operators and
+// the calibration entries keep one order: the scatter by residue classes (the
+// window form of the gather is the same sum), transforms in shared memory, a parameter's sums over every 256th sample.  Solves,
+// whose image agrees to 1e-5 either way, do not.  With nz = nk the band covers all bins
+// and a fit leaves a residual.
+// A + A^H in this order and in the other: 128 x 256 -> 512 31 and 29 us (calls bound),
+// 1024 x 1024 -> 2048 84 and 59, 64 x 64 x 256 -> 512 94 and 58.
+struct FitOrder {
+  isam_plan* P;
+  explicit FitOrder(isam_plan* P_) : P(P_) {
+    P->fit_order = P->p.precision == ISAM_FP32 && P->nz > P->nk;
+  }
+  ~FitOrder() { P->fit_order = false; }
+};
 
 template <typename T> AxArgs<T> ax_args(isam_plan* P, const Impl<T>& im, const cplx<T>* in,
                                        cplx<T>* out) {
@@ -383,6 +407,10 @@ template <typename T> AxArgs<T> ax_args(isam_plan* P, const Impl<T>& im, const c
     a.tab.coef = nullptr;
   }
   a.radix16 = P->tune_radix_ax == 16 ? 1 : 0;
+  if (P->fit_order) {
+    a.fit = 1;
+    if (P->K < 2048) a.radix16 = 0;
+  }
   return a;
 }
 
@@ -411,8 +439,8 @@ template <typename T> isam_status lat_inverse(isam_plan* P, Impl<T>& im, cplx<T>
 // (two columns a load; the whole-spectrum form below reads one).  256 x 256 x 2048,
 // A + A^H: 4.40 -> 3.90 ms, 1.1 of 10 GB less; 1024 x 2048: 69 us either way.
 template <typename T> bool half_spectra(const isam_plan* P, const void* s) {
-  return sizeof(T) == 4 && P->tune_radix_lat == 16 && lat_half_takes(P->nx, P->nk) &&
-         reinterpret_cast<uintptr_t>(s) % 8 == 0;
+  return sizeof(T) == 4 && P->nz == P->nk && P->tune_radix_lat == 16 &&
+         lat_half_takes(P->nx, P->nk) && reinterpret_cast<uintptr_t>(s) % 8 == 0;
 }
 template <typename T> LatArgs<T> half_x_args(isam_plan* P, const void* in, void* out) {
   return lat_args<T>(P->ny, P->nx, P->nk, in, out);
@@ -1071,14 +1099,15 @@ isam_status build_poly(isam_plan* P) {
 }
 
 // Columns (ix, iy) and (-ix, -iy) mod (nx, ny) share |q|; list each pair once, the one
-// of ix <= nx/2 first (where the half spectrum has it).
+// of ix <= nx/2 first (where the half spectrum has it; with nz > nk, which takes no half
+// spectra, the one of the lower index, see FitOrder).
 isam_status build_pairs(isam_plan* P) {
   std::vector<int2> pr;
   for (int iy = 0; iy < P->ny; ++iy)
     for (int ix = 0; ix < P->nx; ++ix) {
       const int c = iy * P->nx + ix;
       const int d = ((P->ny - iy) % P->ny) * P->nx + (P->nx - ix) % P->nx;
-      if (c <= d) pr.push_back(2 * ix <= P->nx ? make_int2(c, d) : make_int2(d, c));
+      if (c <= d) pr.push_back(2 * ix <= P->nx || P->nz > P->nk ? make_int2(c, d) : make_int2(d, c));
     }
   P->npairs = int(pr.size());
   ISAM_TRY(dalloc(&P->pairs, pr.size()));
@@ -1194,6 +1223,7 @@ isam_status isam_set_stream(isam_plan* P, void* stream) {
 isam_status isam_forward(isam_plan* P, const void* eta, void* s) {
   if (!P || !eta || !s) return ISAM_ERR_INVALID;
   DeviceGuard g(P->device);
+  const FitOrder order(P);
   P->launches = 0;
   if (P->p.precision == ISAM_FP64) return op_forward<double>(P, eta, s);
   return op_forward<float>(P, eta, s);
@@ -1202,6 +1232,7 @@ isam_status isam_forward(isam_plan* P, const void* eta, void* s) {
 isam_status isam_adjoint(isam_plan* P, const void* s, void* eta) {
   if (!P || !eta || !s) return ISAM_ERR_INVALID;
   DeviceGuard g(P->device);
+  const FitOrder order(P);
   P->launches = 0;
   if (P->p.precision == ISAM_FP64) return op_adjoint<double>(P, s, eta);
   return op_adjoint<float>(P, s, eta);
@@ -1289,6 +1320,7 @@ isam_status isam_data_fidelity(isam_plan* P, const void* eta, const void* s_d, v
                                double* value) {
   if (!P || !eta || !s_d || !value) return ISAM_ERR_INVALID;
   DeviceGuard g(P->device);
+  const FitOrder order(P);
   P->launches = 0;
   if (P->p.precision == ISAM_FP64)
     return fidelity_impl<double>(P, eta, static_cast<const double*>(s_d),
@@ -1381,6 +1413,7 @@ template <typename T> ParamArgs<T> param_args(isam_plan* P, cplx<T>* su, const c
   ParamArgs<T> a{};
   a.su = su; a.se = se; a.fd = fd; a.fd_sign = fd_sign;
   a.pairs = P->pairs; a.sc = P->sc; a.partial = P->cpartial; a.write_fa = write_fa ? 1 : 0;
+  a.fit = P->fit_order;
   return a;
 }
 
@@ -1596,6 +1629,7 @@ isam_status isam_set_filter(isam_plan* P, const double* b) {
 isam_status isam_param_grad(isam_plan* P, const void* x, const void* y, double* grad) {
   if (!P || !x || !y || !grad) return ISAM_ERR_INVALID;
   DeviceGuard g(P->device);
+  const FitOrder order(P);
   P->launches = 0;
   if (P->p.precision == ISAM_FP64) return param_grad_impl<double>(P, x, y, grad);
   return param_grad_impl<float>(P, x, y, grad);
@@ -1611,6 +1645,7 @@ isam_status isam_fista_unrolled(isam_plan* P, const void* s_d, const isam_solve_
   if (!P || !s_d || !z_out) return ISAM_ERR_INVALID;
   ISAM_TRY(check_unrolled_opts(P, o, every));
   DeviceGuard g(P->device);
+  const FitOrder order(P);
   P->launches = 0;
   if (P->p.precision == ISAM_FP64)
     return unrolled_impl<double>(P, static_cast<const double*>(s_d), o, every,
@@ -1625,6 +1660,7 @@ isam_status isam_fista_unrolled_vjp(isam_plan* P, const void* s_d, const isam_so
   if (!P || !s_d || !ckpt || !z_bar || !grad) return ISAM_ERR_INVALID;
   ISAM_TRY(check_unrolled_opts(P, o, every));
   DeviceGuard g(P->device);
+  const FitOrder order(P);
   P->launches = 0;
   if (P->p.precision == ISAM_FP64)
     return unrolled_vjp_impl<double>(P, static_cast<const double*>(s_d), o, every,

@@ -581,16 +581,16 @@ __device__ __forceinline__ bool quad_fits(const AxArgs<T>& A, const Sample<T, V>
 }
 
 // Y = the scatter of the block's samples, in the window form where every thread's
-// samples fit one (fits; true where a thread has none).  heads holds every such
-// thread's first floor; taps gives the window's taps (see window_scatter), reload the
-// samples' positions again for the residue-class form.  Starts with a barrier (all
-// reads of Y are done) and ends with one.
+// samples fit one (fits; true where a thread has none) and the call is none of
+// FitOrder's.  heads holds every such thread's first floor; taps gives the window's
+// taps (see window_scatter), reload the samples' positions again for the residue-class
+// form.  Starts with a barrier (all reads of Y are done) and ends with one.
 template <typename T, int J, bool WARP, typename V, typename Taps, typename Reload>
 __device__ __forceinline__ void scatter(const AxArgs<T>& A, const Coefficients<T, J>& co, V* Y,
                                         int K, int nt, int nk, Sample<T, V>* sm, bool fits,
                                         int* lo, int* hi, int* ch_tail, WindowHeads& heads,
                                         Taps taps, Reload reload) {
-  if (__syncthreads_and(fits)) {
+  if (__syncthreads_and(fits && !A.fit)) {
     window_scatter<T, J, WARP, V>(Y, K, nt, nk, sm, window_past<T, V>(A, Y), heads, taps);
     return;
   }
@@ -811,7 +811,10 @@ __global__ void __launch_bounds__(512, ax_min_blocks<T>()) k_ax_fwd(const __grid
   int c1, c2, mx, my;
   pair_columns<T, ONE>(A, c1, c2, mx, my);
   const bool two = !ONE && c2 != c1;
-  // programmatic dependent launch (as k_ax_fused): twiddles before the wait
+  // programmatic dependent launch (as k_ax_fused): twiddles before the wait; FitOrder's
+  // calls let the next kernel start at once at K = 4096 (A + A^H at 512 x 1024 -> 2048:
+  // 53.3 us, 55.9 late; at 512 x 512 -> 1024 47.4, 38.5 late)
+  if (A.fit && K == 4096) cudaTriggerProgrammaticLaunchCompletion();
   const C* tw = ax_twiddles<T, LOGK, C16>(A, smem_raw);
   cudaGridDependencySynchronize();
   ax_forward<T, LOGK, C16, V>(A, Y, tw, c1, c2, two, [](const float2*) {});
@@ -872,7 +875,10 @@ __global__ void __launch_bounds__(512, ax_min_blocks<T>()) k_ax_adj(const __grid
   pair_columns<T, ONE>(A, c1, c2, mx, my);
   const bool two = !ONE && c2 != c1;
   if (tid == 0) { ch_lo = INT_MAX; ch_hi = INT_MIN; }
-  // programmatic dependent launch (as k_ax_fused): twiddles before the wait
+  // programmatic dependent launch (as k_ax_fused): twiddles before the wait; FitOrder's
+  // calls let the next kernel start at once at K = 4096 (A + A^H at 512 x 1024 -> 2048:
+  // 53.3 us, 55.9 late; at 512 x 512 -> 1024 47.4, 38.5 late)
+  if (A.fit && K == 4096) cudaTriggerProgrammaticLaunchCompletion();
   const C* tw = ax_twiddles<T, LOGK, C16>(A, smem_raw);
   cudaGridDependencySynchronize();
   const bool stopped = RES && A.stop != nullptr && __ldcg(A.stop) != 0;

@@ -57,11 +57,14 @@ __device__ __forceinline__ cplx<T> real_part_spectrum(cplx<T> a, cplx<T> b) {
 // float, the cancelling 2 kappa - sqrt(a) from a two-float constant, and the threads'
 // sums are added in double by one warp a moment.  512 x 2048: 24.7 -> 15.2 us (16.5 at
 // one block a multiprocessor, 72 registers).
+//
+// FIT (FP32 calibrations with nz > nk, see FitOrder): sample j belongs to thread j mod
+// TPB, whose terms are summed in that order, and 4 kappa^2 - a is formed in double.
 template <typename T> struct ParamSamples {
   cpair<T> S1, S2, E1, E2, f1, f2;
 };
 
-template <typename T, int TPB>
+template <typename T, int TPB, bool FIT = false>
 __global__ void __launch_bounds__(TPB, sizeof(T) == 4 && TPB == 512 ? 2 : 1)
     k_param_reduce(const __grid_constant__ ParamArgs<T> A) {
   using C = cplx<T>;
@@ -78,7 +81,7 @@ __global__ void __launch_bounds__(TPB, sizeof(T) == 4 && TPB == 512 ? 2 : 1)
   __shared__ float4 cut_s;
   __shared__ T part[5][TPB];
   float4 cut = {};
-  if constexpr (std::is_same<T, float>::value) {
+  if constexpr (std::is_same<T, float>::value && !FIT) {
     if (threadIdx.x == 0) {
       const double sa = sqrt(a), lo = 2.0 * A.sc.kap - sa;
       cut_s = make_float4(float(lo), float(lo - double(float(lo))), float(2.0 * A.sc.kap + sa),
@@ -131,6 +134,12 @@ __global__ void __launch_bounds__(TPB, sizeof(T) == 4 && TPB == 512 ? 2 : 1)
         m[i] = fmaf(tp, v, m[i]);
         tp *= t;
       }
+      if constexpr (FIT) {
+        const double kap = A.sc.kap + double(j), x = fma(4.0 * kap, kap, -a);
+        if (x > 0.0)
+          m[4] = fmaf(float(a) / (2.0f * float(kap) + sqrtf(float(x))), v, m[4]);
+        return;
+      }
       const float j2 = float(2 * j), dm = (cut.x + j2) + cut.y, dp = cut.z + j2;
       if (dm > 0.0f) m[4] = fmaf(cut.w / (0.5f * (dm + dp) + sqrtf(dm * dp)), v, m[4]);
     } else {
@@ -157,14 +166,27 @@ __global__ void __launch_bounds__(TPB, sizeof(T) == 4 && TPB == 512 ? 2 : 1)
       if (two) store_two<T>(s2 + j, a2.a, a2.b);
     }
   };
-  for (int j = 2 * threadIdx.x; j < nk || j == 2 * threadIdx.x; j += 4 * TPB) {
-    const ParamSamples<T> x = load(j), y = load(j + 2 * TPB);
-    if (j == 2 * threadIdx.x) {
-      __syncthreads();
-      cut = cut_s;
+  if constexpr (FIT) {
+    const C zero = mk<T>(0, 0);
+    for (int j = threadIdx.x; j < nk; j += TPB) {
+      C Fa1, Fa2;
+      point(j, s1[j], s2[j], e1 ? e1[j] : zero, e1 ? e2[j] : zero, f1 ? f1[j] : zero,
+            f1 ? f2[j] : zero, Fa1, Fa2);
+      if (A.write_fa) {
+        s1[j] = Fa1;
+        if (two) s2[j] = Fa2;
+      }
     }
-    use(j, x);
-    use(j + 2 * TPB, y);
+  } else {
+    for (int j = 2 * threadIdx.x; j < nk || j == 2 * threadIdx.x; j += 4 * TPB) {
+      const ParamSamples<T> x = load(j), y = load(j + 2 * TPB);
+      if (j == 2 * threadIdx.x) {
+        __syncthreads();
+        cut = cut_s;
+      }
+      use(j, x);
+      use(j + 2 * TPB, y);
+    }
   }
   cudaTriggerProgrammaticLaunchCompletion();
 #pragma unroll
@@ -180,6 +202,8 @@ __global__ void __launch_bounds__(TPB, sizeof(T) == 4 && TPB == 512 ? 2 : 1)
 
 template <typename T> cudaError_t launch_param_reduce(const ParamArgs<T>& a, int npairs,
                                                       cudaStream_t s) {
+  if constexpr (sizeof(T) == 4)
+    if (a.fit) return launch_dependent<T>(k_param_reduce<T, 256, true>, npairs, 256, s, a);
   if (a.sc.nk > 1024) return launch_dependent<T>(k_param_reduce<T, 512>, npairs, 512, s, a);
   if (a.sc.nk > 256) return launch_dependent<T>(k_param_reduce<T, 256>, npairs, 256, s, a);
   return launch_dependent<T>(k_param_reduce<T, 64>, npairs, 64, s, a);

@@ -17,6 +17,7 @@
 
 #include <type_traits>
 
+#include "fft_col16.cuh"
 #include "fft_smem.cuh"
 #include "internal.cuh"
 #include "lat_point.cuh"
@@ -78,8 +79,9 @@ template <> struct rpair_t<double> { using type = double2; };
 
 // LOGL > 0: the transforms are the compile-time-length ones for L = 2^LOGL at
 // the stride 2^LOGTP = TP (no radix-3 pass), with constant row offsets;
-// LOGL = 0: runtime-length transforms.  The tile indexing is the same.
-template <typename T, int MODE, int LOGL, int LOGTP>
+// LOGL = 0: runtime-length transforms.  The tile indexing is the same.  C16 (FP32,
+// L = 1024 or 256): column-split radix-16 transforms (fft_col16.cuh).
+template <typename T, int MODE, int LOGL, int LOGTP, bool C16>
 __global__ void __launch_bounds__(512, std::is_same<T, float>::value ? 2 : 1) k_lat(const __grid_constant__ LatArgs<T> a) {
   using C = cplx<T>;
   using V = cpair<T>;
@@ -92,8 +94,13 @@ __global__ void __launch_bounds__(512, std::is_same<T, float>::value ? 2 : 1) k_
   // programmatic dependent launch: let the next kernel start its prologue,
   // build the twiddles, then wait for the previous kernel's results
   cudaTriggerProgrammaticLaunchCompletion();
-  const C* tw = build_twiddles<T>(reinterpret_cast<C*>(buf + size_t(padded_rows(L)) * TP), a.roots,
-                                  L, CT ? LOGL : a.logL, CT ? 0 : a.r3);
+  C* table = reinterpret_cast<C*>(buf + size_t(padded_rows(L)) * TP);
+  const C* tw;
+  if constexpr (C16)
+    tw = reinterpret_cast<const C*>(
+        c16::build_lat_twiddles<LOGL>(reinterpret_cast<float4*>(table)));
+  else
+    tw = build_twiddles<T>(table, a.roots, L, CT ? LOGL : a.logL, CT ? 0 : a.r3);
   cudaGridDependencySynchronize();
   // the solve's stop flag (written by an earlier kernel, so visible after the
   // wait): loaded here, tested before the first global write (after the first
@@ -117,7 +124,10 @@ __global__ void __launch_bounds__(512, std::is_same<T, float>::value ? 2 : 1) k_
   auto sidx = [&](int e) { return prow(e >> logTP) * TP + (e & (TP - 1)); };
   auto lat_fft = [&](auto sign) {
     constexpr int SIGN = decltype(sign)::value;
-    if constexpr (CT) fft_cols_ct<SIGN, false, LOGL, (1 << LOGTP), T>(buf, col, b, tw);
+    if constexpr (C16)
+      c16::lat_transform<SIGN, LOGL, 2 * (1 << LOGTP)>(reinterpret_cast<float2*>(buf),
+                                                       reinterpret_cast<const float4*>(tw));
+    else if constexpr (CT) fft_cols_ct<SIGN, false, LOGL, (1 << LOGTP), T>(buf, col, b, tw);
     else fft_smem<SIGN, false, T>(buf, TP, col, b, L, a.logL, tw, true, a.r3);
   };
   using FWD = std::integral_constant<int, -1>;
@@ -294,11 +304,11 @@ template <typename T> size_t lat_smem_bytes(int L, int TP) {
          size_t(twiddle_entries<T>(L, lg, r3)) * sizeof(cplx<T>);
 }
 
-template <typename T, int MODE, int LOGL, int LOGTP>
+template <typename T, int MODE, int LOGL, int LOGTP, bool C16 = false>
 static cudaError_t launch_lat_tile(const LatArgs<T>& a, cudaStream_t s) {
   const int threads = (a.L >= 8 ? a.L / 8 : 1) * a.TZ;
   const size_t sm = lat_smem_bytes<T>(a.L, a.TZ);
-  auto* kern = k_lat<T, MODE, LOGL, LOGTP>;
+  auto* kern = k_lat<T, MODE, LOGL, LOGTP, C16>;
   allow_smem(kern, sm);
   dim3 grid(a.M / (2 * a.TZ), a.B);
   cudaLaunchConfig_t cfg = {};
@@ -315,15 +325,22 @@ static cudaError_t launch_lat_tile(const LatArgs<T>& a, cudaStream_t s) {
 }
 
 // Passes at the built-in tile of the lengths that have a register form take it
-// (k_lateral_reg.cuh) unless the plan chose radix 8 (a.radix16 = 0).  That form of
-// the FP32 solve's passes runs compile-time-length transforms at (L, pair-columns) =
+// (k_lateral_reg.cuh) unless the plan chose radix 8 (LAT_RADIX8).  That form of the
+// FP32 solve's passes runs compile-time-length transforms at (L, pair-columns) =
 // (1024, 4), (512, 8) and (256, 8); every other case the runtime-length ones.
+// LAT_FIT: radix 8 too, but the column-split form at (1024, 4) and (256, 8).
 template <typename T, int MODE>
 static cudaError_t launch_lat_mode(const LatArgs<T>& a, cudaStream_t s) {
   constexpr bool hot = std::is_same<T, float>::value &&
                        (MODE == LAT_UPDATE || MODE == LAT_UPDATE_U || MODE == LAT_C2C_FWD ||
                         MODE == LAT_C2C_INV);
-  if (a.radix16 && lat_reg_takes<T>(a.L, a.TZ)) return launch_lat_reg<T>(MODE, a, s);
+  if (a.form == LAT_REGS && lat_reg_takes<T>(a.L, a.TZ)) return launch_lat_reg<T>(MODE, a, s);
+  if constexpr (hot && MODE != LAT_UPDATE) {             // (a fit takes no norms)
+    if (a.form == LAT_FIT && a.L == 1024 && a.TZ == 4)
+      return launch_lat_tile<T, MODE, 10, 2, true>(a, s);
+    if (a.form == LAT_FIT && a.L == 256 && a.TZ == 8)
+      return launch_lat_tile<T, MODE, 8, 3, true>(a, s);
+  }
   if constexpr (hot) {
     if (!a.r3 && a.L == 1024 && a.TZ == 4) return launch_lat_tile<T, MODE, 10, 2>(a, s);
     if (!a.r3 && a.L == 512 && a.TZ == 8) return launch_lat_tile<T, MODE, 9, 3>(a, s);
