@@ -205,7 +205,9 @@ isam_status dalloc_bytes(void** p, size_t bytes) {
     alloc_owners()[*p] = g_alloc;
     return ISAM_OK;
   }
-  return from_cuda(cudaMalloc(p, bytes));
+  const cudaError_t e = cudaMalloc(p, bytes);
+  if (e != cudaSuccess) cudaGetLastError();   // reported here, not by the next launch
+  return from_cuda(e);
 }
 
 void dfree(void* p) {
@@ -230,6 +232,17 @@ template <typename T> isam_status dalloc(T** p, size_t n) {
   const isam_status st = dalloc_bytes(&v, n * sizeof(T));
   *p = static_cast<T*>(v);
   return st;
+}
+
+// An array of plan P.  The FP64 coefficient table, which the kernels can do without, gives
+// way to it where memory is short (no batch graph may hold the table's address then).
+template <typename T> isam_status plan_alloc(isam_plan* P, T** p, size_t n) {
+  const isam_status st = dalloc(p, n);
+  if (st != ISAM_ERR_OOM || !P->f64.tab.coef || P->batch_refs) return st;
+  CUDA_TRY(cudaDeviceSynchronize());
+  dfree(P->f64.tab.coef);
+  P->f64.tab.coef = nullptr;
+  return dalloc(p, n);
 }
 
 template <typename T> void impl_free(Impl<T>& im) {
@@ -269,7 +282,7 @@ template <typename T> isam_status phase_tables(isam_plan* P, Impl<T>& im) {
     std::vector<cplx<T>> h(rows * P->nk);
     for (size_t i = 0; i < h.size(); ++i)
       h[i] = mk<T>(T(P->filt_host[2 * i]), T(P->filt_host[2 * i + 1]));
-    if (!im.tab.filt) ISAM_TRY(dalloc(&im.tab.filt, h.size()));
+    if (!im.tab.filt) ISAM_TRY(plan_alloc(P, &im.tab.filt, h.size()));
     CUDA_TRY(cudaMemcpy(im.tab.filt, h.data(), sizeof(cplx<T>) * h.size(), cudaMemcpyHostToDevice));
   }
   {
@@ -282,24 +295,30 @@ template <typename T> isam_status phase_tables(isam_plan* P, Impl<T>& im) {
       for (int i = 0; i < p.n_disp; ++i) { pw *= d; phi += p.disp[i] * pw; }
       h[j] = mk<T>(T(cos(phi)), T(sin(phi)));
     }
-    if (!im.tab.disp) ISAM_TRY(dalloc(&im.tab.disp, P->nk));
+    if (!im.tab.disp) ISAM_TRY(plan_alloc(P, &im.tab.disp, P->nk));
     CUDA_TRY(cudaMemcpy(im.tab.disp, h.data(), sizeof(cplx<T>) * P->nk, cudaMemcpyHostToDevice));
   }
   {
     const size_t bytes = rows * P->nk * StoltTable<T>::sample_bytes;
     const size_t cap = std::max(kStoltTableMaxBytes, P->n_img * sizeof(cplx<T>));
     if (bytes <= cap && !(p.flags & ISAM_FLAG_NO_STOLT_TABLE)) {
-      if (!im.tab.stab) ISAM_TRY(dalloc(&im.tab.stab, bytes / sizeof(int4)));
+      if (!im.tab.stab) ISAM_TRY(plan_alloc(P, &im.tab.stab, bytes / sizeof(int4)));
       AxArgs<T> a{};
       a.sc = P->sc;
       a.tab = im.tab;
       CUDA_TRY(launch_stolt_table<T>(a, im.tab.stab, P->stream));
-      // FP64: the coefficients too, under the same cap (they depend on the
-      // positions only, so once)
+      // FP64: the coefficients too (they depend on the positions only, so once).  The
+      // kernels evaluate them without the table, so no call fails for it (plan_alloc);
+      // an FP32 plan, whose FP64 state serves its power iteration, keeps a small one
+      // only.  At most 3/2 images: J = 8 takes 64 B a class sample, an image of a volume
+      // with nz = nk about as much (128 x 128 x 1024 iteration 15.1 ms without the
+      // table, 11.5 with it).
       if constexpr (sizeof(T) == 8) {
         const size_t n = rows * P->nk * size_t(P->J) / 2;
-        if (!im.tab.coef && n * sizeof(double2) <= cap) {
-          ISAM_TRY(dalloc(&im.tab.coef, n));
+        const size_t most = p.precision == ISAM_FP64
+                                ? std::max(2 * kStoltTableMaxBytes, P->n_img * sizeof(cplx<T>) * 3 / 2)
+                                : kStoltTableMaxBytes;
+        if (!im.tab.coef && n * sizeof(double2) <= most && dalloc(&im.tab.coef, n) == ISAM_OK) {
           a.tab = im.tab;
           a.poly = P->poly64;
           CUDA_TRY(launch_coef_table(a, im.tab.coef, P->stream));
@@ -318,12 +337,12 @@ template <typename T> isam_status impl_init(isam_plan* P, Impl<T>& im) {
     std::vector<T> h(P->nz);
     for (int n = 0; n < P->nz; ++n)
       h[n] = T(host_kb_scale(n - P->nz / 2, P->K, P->J) / sqrt(double(P->nz)));
-    ISAM_TRY(dalloc(&im.tab.scale, P->nz));
+    ISAM_TRY(plan_alloc(P, &im.tab.scale, P->nz));
     CUDA_TRY(cudaMemcpy(im.tab.scale, h.data(), sizeof(T) * P->nz, cudaMemcpyHostToDevice));
   }
   if constexpr (sizeof(T) == 8) {
     const int len[4] = {P->K, P->nx, P->ny, P->nz};
-    ISAM_TRY(dalloc(&im.roots, size_t(len[0]) + len[1] + len[2] + len[3]));
+    ISAM_TRY(plan_alloc(P, &im.roots, size_t(len[0]) + len[1] + len[2] + len[3]));
     double2* r = im.roots;
     for (int n : len) {
       CUDA_TRY(launch_roots(r, n, P->stream));
@@ -332,9 +351,9 @@ template <typename T> isam_status impl_init(isam_plan* P, Impl<T>& im) {
     im.tab.roots = im.roots;
   }
   ISAM_TRY(phase_tables<T>(P, im));
-  ISAM_TRY(dalloc(&im.eta_hat, P->n_img));
-  ISAM_TRY(dalloc(&im.spec, P->n_spec));
-  ISAM_TRY(dalloc(&im.grad, P->n_img));
+  ISAM_TRY(plan_alloc(P, &im.eta_hat, P->n_img));
+  ISAM_TRY(plan_alloc(P, &im.spec, P->n_spec));
+  ISAM_TRY(plan_alloc(P, &im.grad, P->n_img));
   CUDA_TRY(cudaStreamSynchronize(P->stream));
   harvest_events(P);
   im.ready = true;
@@ -498,7 +517,7 @@ template <typename T> isam_status fidelity_impl(isam_plan* P, const void* eta, c
   Impl<T>& im = impl_of<T>(P);
   T* r = r_out;
   if (!r) {
-    if (!im.s_tmp) ISAM_TRY(dalloc(&im.s_tmp, P->n_spec));
+    if (!im.s_tmp) ISAM_TRY(plan_alloc(P, &im.s_tmp, P->n_spec));
     r = im.s_tmp;
   }
   ISAM_TRY(op_forward<T>(P, eta, r));
@@ -521,9 +540,9 @@ template <typename T> isam_status power_iteration(isam_plan* P, int iters, doubl
                                                   const void* v0, int v0_double, double* L_out) {
   Impl<T>& im = impl_of<T>(P);
   ISAM_TRY(impl_init<T>(P, im));
-  if (!im.zA) ISAM_TRY(dalloc(&im.zA, P->n_img));
-  if (!im.zB) ISAM_TRY(dalloc(&im.zB, P->n_img));
-  if (!im.s_tmp) ISAM_TRY(dalloc(&im.s_tmp, P->n_spec));
+  if (!im.zA) ISAM_TRY(plan_alloc(P, &im.zA, P->n_img));
+  if (!im.zB) ISAM_TRY(plan_alloc(P, &im.zB, P->n_img));
+  if (!im.s_tmp) ISAM_TRY(plan_alloc(P, &im.s_tmp, P->n_spec));
   cudaStream_t s = P->stream;
   if (v0) {
     const bool same = (sizeof(T) == 8) == (v0_double != 0);
@@ -765,8 +784,8 @@ template <typename T> isam_status solve_impl(isam_plan* P, const T* s_d, const i
                                              isam_solve_info* info) {
   Impl<T>& im = impl_of<T>(P);
   cudaStream_t s = P->stream;
-  if (!im.zA) ISAM_TRY(dalloc(&im.zA, P->n_img));
-  if (!im.zB) ISAM_TRY(dalloc(&im.zB, P->n_img));
+  if (!im.zA) ISAM_TRY(plan_alloc(P, &im.zA, P->n_img));
+  if (!im.zB) ISAM_TRY(plan_alloc(P, &im.zB, P->n_img));
   int64_t launches0 = P->launches;
   const bool resume = state && state->k > 0;
   // lambda = c ||A^H s_d||_inf unless given
@@ -811,12 +830,12 @@ template <typename T> isam_status solve_impl(isam_plan* P, const T* s_d, const i
     CUDA_TRY(cudaMemsetAsync(im.eta_hat, 0, sizeof(cplx<T>) * P->n_img, s));
   }
   if (o->prior == ISAM_PRIOR_TV) {                 // TV dual starts at 0 for every solve
-    if (!im.tv) ISAM_TRY(dalloc(&im.tv, tv_images<T>(P) * P->n_img));
+    if (!im.tv) ISAM_TRY(plan_alloc(P, &im.tv, tv_images<T>(P) * P->n_img));
     CUDA_TRY(cudaMemsetAsync(im.tv, 0, 2 * sizeof(cplx<T>) * P->n_img, s));
     im.tv_cur = 0;
   }
   // lateral spectrum of the data, used by every iteration's residual
-  if (!im.sdh) ISAM_TRY(dalloc(&im.sdh, P->n_spec));
+  if (!im.sdh) ISAM_TRY(plan_alloc(P, &im.sdh, P->n_spec));
   ISAM_TRY(lat_forward<T>(P, im, s_d, im.sdh, P->nk, true));
   const bool check = o->tol > 0;
   const int every = std::max(1, o->check_every);
@@ -890,7 +909,7 @@ template <typename T> isam_status solve_impl(isam_plan* P, const T* s_d, const i
   // objective of Eq. 12 at z^K
   double objective = -1.0;
   if (o->objective && o->prior == ISAM_PRIOR_L1) {
-    if (!im.s_tmp) ISAM_TRY(dalloc(&im.s_tmp, P->n_spec));
+    if (!im.s_tmp) ISAM_TRY(plan_alloc(P, &im.s_tmp, P->n_spec));
     ISAM_TRY(op_forward<T>(P, zP, im.s_tmp));
     ISAM_TRY(launch(P, ISAM_KCLASS_MISC, [&] {
       return launch_rsub<T>(im.s_tmp, s_d, im.s_tmp, P->n_spec, s);
@@ -912,7 +931,7 @@ template <typename T> isam_status solve_impl(isam_plan* P, const T* s_d, const i
   }
   // result: z^K, optionally with the residual added back (Alg. 1, last step)
   if (o->residual_addback) {
-    if (!im.s_tmp) ISAM_TRY(dalloc(&im.s_tmp, P->n_spec));
+    if (!im.s_tmp) ISAM_TRY(plan_alloc(P, &im.s_tmp, P->n_spec));
     ISAM_TRY(op_forward<T>(P, zP, im.s_tmp));
     ISAM_TRY(launch(P, ISAM_KCLASS_MISC, [&] {
       return launch_rsub<T>(s_d, im.s_tmp, im.s_tmp, P->n_spec, s);
@@ -1272,8 +1291,8 @@ template <typename T>
 static isam_status solve_host_impl(isam_plan* P, const void* s_h, const isam_solve_opts* o,
                                    void* eta_h, isam_solve_info* info) {
   Impl<T>& im = impl_of<T>(P);
-  if (!im.s_host_stage) ISAM_TRY(dalloc(&im.s_host_stage, P->n_spec));
-  if (!im.out_stage) ISAM_TRY(dalloc(&im.out_stage, P->n_img));
+  if (!im.s_host_stage) ISAM_TRY(plan_alloc(P, &im.s_host_stage, P->n_spec));
+  if (!im.out_stage) ISAM_TRY(plan_alloc(P, &im.out_stage, P->n_img));
   CUDA_TRY(cudaMemcpyAsync(im.s_host_stage, s_h, sizeof(T) * P->n_spec, cudaMemcpyHostToDevice,
                            P->stream));
   ISAM_TRY(solve_impl<T>(P, im.s_host_stage, o, im.out_stage, nullptr, info));
@@ -1369,21 +1388,21 @@ isam_status isam_profile_read(isam_plan* P, double* ms, int64_t* counts, int32_t
 namespace {
 
 template <typename T> isam_status calib_buffers(isam_plan* P, Impl<T>& im, int seg_cap) {
-  if (!im.spec2) ISAM_TRY(dalloc(&im.spec2, P->n_spec));
-  if (!im.cal) ISAM_TRY(dalloc(&im.cal, 5 * P->n_img));
-  if (!P->cpartial) ISAM_TRY(dalloc(&P->cpartial, size_t(P->npairs) * 5));
+  if (!im.spec2) ISAM_TRY(plan_alloc(P, &im.spec2, P->n_spec));
+  if (!im.cal) ISAM_TRY(plan_alloc(P, &im.cal, 5 * P->n_img));
+  if (!P->cpartial) ISAM_TRY(plan_alloc(P, &P->cpartial, size_t(P->npairs) * 5));
   if (seg_cap > im.seg_cap) {
     dfree(im.seg);
     im.seg = nullptr;
     im.seg_cap = 0;
     // [seg_cap] u^k, [seg_cap + 1] eta_hat^k, [seg_cap] model spectra S^k
-    ISAM_TRY(dalloc(&im.seg, size_t(2 * seg_cap + 1) * P->n_img + size_t(seg_cap) * P->n_spec));
+    ISAM_TRY(plan_alloc(P, &im.seg, size_t(2 * seg_cap + 1) * P->n_img + size_t(seg_cap) * P->n_spec));
     im.seg_cap = seg_cap;
   }
-  if (!im.zA) ISAM_TRY(dalloc(&im.zA, P->n_img));
-  if (!im.zB) ISAM_TRY(dalloc(&im.zB, P->n_img));
-  if (!im.sdh) ISAM_TRY(dalloc(&im.sdh, P->n_spec));
-  if (!im.s_tmp) ISAM_TRY(dalloc(&im.s_tmp, P->n_spec));
+  if (!im.zA) ISAM_TRY(plan_alloc(P, &im.zA, P->n_img));
+  if (!im.zB) ISAM_TRY(plan_alloc(P, &im.zB, P->n_img));
+  if (!im.sdh) ISAM_TRY(plan_alloc(P, &im.sdh, P->n_spec));
+  if (!im.s_tmp) ISAM_TRY(plan_alloc(P, &im.s_tmp, P->n_spec));
   return ISAM_OK;
 }
 
@@ -1694,7 +1713,7 @@ template <typename T> isam_status dc_ifft_impl(isam_plan* P, const T* s, cplx<T>
       const double ang = -2.0 * M_PI * (turn - floor(turn));
       h[n] = mk<T>(T(cos(ang) / sqrt(double(P->nz))), T(sin(ang) / sqrt(double(P->nz))));
     }
-    ISAM_TRY(dalloc(&im.dc_post, P->nz));
+    ISAM_TRY(plan_alloc(P, &im.dc_post, P->nz));
     CUDA_TRY(cudaMemcpy(im.dc_post, h.data(), sizeof(cplx<T>) * P->nz, cudaMemcpyHostToDevice));
   }
   return launch(P, ISAM_KCLASS_MISC, [&] {
@@ -1751,11 +1770,11 @@ namespace {
 template <typename T> isam_status batch_prepare(isam_plan* P, const isam_solve_opts* o,
                                                 double* L_out) {
   Impl<T>& im = impl_of<T>(P);
-  if (!im.zA) ISAM_TRY(dalloc(&im.zA, P->n_img));
-  if (!im.zB) ISAM_TRY(dalloc(&im.zB, P->n_img));
-  if (!im.sdh) ISAM_TRY(dalloc(&im.sdh, P->n_spec));
-  if (!im.s_tmp) ISAM_TRY(dalloc(&im.s_tmp, P->n_spec));
-  if (o->prior == ISAM_PRIOR_TV && !im.tv) ISAM_TRY(dalloc(&im.tv, tv_images<T>(P) * P->n_img));
+  if (!im.zA) ISAM_TRY(plan_alloc(P, &im.zA, P->n_img));
+  if (!im.zB) ISAM_TRY(plan_alloc(P, &im.zB, P->n_img));
+  if (!im.sdh) ISAM_TRY(plan_alloc(P, &im.sdh, P->n_spec));
+  if (!im.s_tmp) ISAM_TRY(plan_alloc(P, &im.s_tmp, P->n_spec));
+  if (o->prior == ISAM_PRIOR_TV && !im.tv) ISAM_TRY(plan_alloc(P, &im.tv, tv_images<T>(P) * P->n_img));
   double L = o->L;
   if (!(L > 0)) {
     if (!(P->L_cache > 0)) {
@@ -2155,9 +2174,9 @@ template <typename T> isam_status autotune_impl(isam_plan* P, isam_tuning* out) 
       return ISAM_OK;
     }
   }
-  if (!im.zA) ISAM_TRY(dalloc(&im.zA, P->n_img));
-  if (!im.zB) ISAM_TRY(dalloc(&im.zB, P->n_img));
-  if (!im.sdh) ISAM_TRY(dalloc(&im.sdh, P->n_spec));
+  if (!im.zA) ISAM_TRY(plan_alloc(P, &im.zA, P->n_img));
+  if (!im.zB) ISAM_TRY(plan_alloc(P, &im.zB, P->n_img));
+  if (!im.sdh) ISAM_TRY(plan_alloc(P, &im.sdh, P->n_spec));
   int L, M;
   update_geometry(P, &L, &M);
   const int threads_per_tp = L >= 8 ? L / 8 : 1;

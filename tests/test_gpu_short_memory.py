@@ -1,0 +1,93 @@
+"""Plans under an allocator with a budget: arrays that a call can do without (the FP64
+coefficient table) give way, and the results are those of plenty of memory (1e-13: the
+coefficients are the same polynomials, tabulated or evaluated)."""
+import numpy as np
+import pytest
+
+from paper_1905_06058_gb300 import inputs as I
+from test_gpu_calibration import torch   # noqa: F401
+
+pytestmark = pytest.mark.gpu
+
+
+class Pool:
+    """Device memory for plans: `budget` bytes at once, no block of a size in `refused`."""
+
+    def __init__(self, torch):   # noqa: F811
+        from paper_1905_06058_gb300 import isam as B
+        self.torch, self.B = torch, B
+        self.live, self.budget, self.refused = {}, 1 << 40, ()
+
+    def alloc(self, n):
+        if n in self.refused or sum(self.live.values()) + n > self.budget:
+            return 0
+        p = self.torch.cuda.caching_allocator_alloc(n)
+        self.live[p] = n
+        return p
+
+    def free(self, p):
+        self.live.pop(p)
+        self.torch.cuda.caching_allocator_delete(p)
+
+    def __enter__(self):
+        self.B.set_allocator(self.alloc, self.free)
+        return self
+
+    def __exit__(self, *_):
+        self.B.set_allocator()
+
+    def held(self):
+        return sum(self.live.values())
+
+
+NX, NK, J = 32, 64, 6
+COEF = (NX // 2 + 1) * NK * J // 2 * 16        # bytes of the table: 8 J a class sample
+
+
+def solve(plan, s):
+    return plan.solve(s, lambda_rel=0.01, L=4.0, max_iter=5)[0]
+
+
+def test_no_coefficient_table(torch):   # noqa: F811
+    from paper_1905_06058_gb300.isam import Plan
+    g = I.small_bscan(seed=73, nx=NX, nk=NK).geom
+    ref = Plan(g, precision="fp64", J=J)
+    s = torch.from_numpy(I.random_spectra(ref.spec_shape, 8)).cuda()
+    z = solve(ref, s)
+    L = Plan(g, J=J).lipschitz(20, 1e-30)
+    ref.close()
+    with Pool(torch) as pool:
+        whole = Plan(g, precision="fp64", J=J)
+        assert COEF in pool.live.values()
+        whole.close()
+        pool.refused = (COEF,)
+        plan = Plan(g, precision="fp64", J=J)
+        got = solve(plan, s)
+        fp32 = Plan(g, J=J)
+        L2 = fp32.lipschitz(20, 1e-30)
+        plan.close()
+        fp32.close()
+        assert not pool.live
+    assert float((got - z).norm()) <= 1e-13 * float(z.norm())
+    assert L2 == pytest.approx(L, rel=1e-13)
+
+
+def test_coefficient_table_gives_way(torch):   # noqa: F811
+    from paper_1905_06058_gb300.isam import Plan
+    g = I.small_bscan(seed=73, nx=NX, nk=NK).geom
+    with Pool(torch) as pool:
+        ref = Plan(g, precision="fp64", J=J)
+        s = torch.from_numpy(I.random_spectra(ref.spec_shape, 8)).cuda()
+        z = solve(ref, s)
+        most = pool.held()
+        ref.close()
+        plan = Plan(g, precision="fp64", J=J)
+        pool.budget = most - COEF
+        got = solve(plan, s)
+        assert COEF not in pool.live.values()
+        plan.set_model(g.disp, g.z0)            # rebuilds the tables, without room for it
+        again = solve(plan, s)
+        plan.close()
+        assert not pool.live
+    assert float((got - z).norm()) <= 1e-13 * float(z.norm())
+    assert float((again - z).norm()) <= 1e-13 * float(z.norm())
