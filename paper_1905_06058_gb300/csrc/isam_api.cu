@@ -47,10 +47,11 @@ template <typename T> struct Impl {
   cplx<T>* cal = nullptr;       // [5][n_img]: zbar x 3, ubar, b
   cplx<T>* roots = nullptr;     // FP64: roots of unity of K, nx, ny and nz, one after another
   cplx<T>* dc_post = nullptr;   // [nz] output phase of the Eq. 9 reconstruction
-  // [tv_images][n_img]; FP32: TV duals p (x, z) of two launches in turn and a
-  // momentum r; FP64: p_x, p_z, r_x, r_z and the primal w
+  // TV workspace, images; tv_tiles: duals p (x, z) of two launches in turn and a
+  // momentum r (tv_alloc); else p_x, p_z, r_x, r_z and the primal w
   cplx<T>* tv = nullptr;
-  int tv_cur = 0;               // FP32: which p the next prox starts from
+  bool tv_tiles = false;        // launches of several steps (FP32), else two a step
+  int tv_cur = 0;               // tv_tiles: which p the next prox starts from
   bool ready = false;
 };
 
@@ -584,12 +585,21 @@ template <typename T> isam_status power_iteration(isam_plan* P, int iters, doubl
 // ----------------------------------------------------------------------------
 // FISTA (Alg. 1)
 // ----------------------------------------------------------------------------
-// Images of the TV workspace.  FP32 launches read (p, r) and write the next ones,
-// so each exists twice; of the two r pairs one is lent by eta_hat and z^k, which
-// are free during the prox, and half of the other by the spectra when they are as
-// large as an image (nk = nz).
-template <typename T> int tv_images(const isam_plan* P) {
-  return sizeof(T) == 8 || P->n_spec == P->n_img ? 5 : 6;
+// The TV workspace.  FP32 launches of several steps read (p, r) and write the next ones,
+// so each exists twice; of the two r pairs one is lent by eta_hat and z^k, which are free
+// during the prox, and half of the other by the spectra when they are as large as an
+// image (nk = nz).  Else that takes a sixth image; where it cannot be had, five serve the
+// two launches a step that FP64 runs.
+template <typename T> isam_status tv_alloc(isam_plan* P, Impl<T>& im) {
+  if (im.tv) return ISAM_OK;
+  im.tv_tiles = sizeof(T) == 4;
+  const int images = im.tv_tiles && P->n_spec < P->n_img ? 6 : 5;
+  isam_status st = plan_alloc(P, &im.tv, images * P->n_img);
+  if (st == ISAM_ERR_OOM && images == 6) {
+    im.tv_tiles = false;
+    st = plan_alloc(P, &im.tv, 5 * P->n_img);
+  }
+  return st;
 }
 
 // TV prox of u = im.grad into zout: the dual p carries over from the previous
@@ -598,7 +608,7 @@ template <typename T> isam_status tv_prox(isam_plan* P, Impl<T>& im, cplx<T>* zo
                                           double L, const double* lam_dev, double lam_scale,
                                           int iters) {
   cudaStream_t s = P->stream;
-  if constexpr (sizeof(T) == 4) {
+  if constexpr (sizeof(T) == 4) if (im.tv_tiles) {
     // five steps a launch: 20 in four launches of tiles whose inner 54 x 54 pixels
     // are 71% of what they compute
     constexpr int kSteps = 5;
@@ -638,35 +648,34 @@ template <typename T> isam_status tv_prox(isam_plan* P, Impl<T>& im, cplx<T>* zo
       r_in = r_out;
     }
     return ISAM_OK;
-  } else {
-    const size_t n = P->n_img;
-    cplx<T>* px = im.tv;
-    cplx<T>* pz = im.tv + n;
-    cplx<T>* rx = im.tv + 2 * n;
-    cplx<T>* rz = im.tv + 3 * n;
-    cplx<T>* w = im.tv + 4 * n;
-    const T tau = T(lam / L);
-    CUDA_TRY(cudaMemcpyAsync(rx, px, 2 * n * sizeof(cplx<T>), cudaMemcpyDeviceToDevice, s));
-    double t = 1.0;
-    for (int i = 0; i < iters; ++i) {
-      const double t_next = 0.5 * (1.0 + sqrt(1.0 + 4.0 * t * t));
-      const T beta = T((t - 1.0) / t_next);
-      t = t_next;
-      ISAM_TRY(launch(P, ISAM_KCLASS_MISC, [&] {
-        return launch_tv_primal<T>(im.grad, rx, rz, tau, lam_dev, lam_scale, w, P->nx, P->nz, n,
-                                   s);
-      }));
-      ISAM_TRY(launch(P, ISAM_KCLASS_MISC, [&] {
-        return launch_tv_dual<T>(w, px, pz, rx, rz, tau, lam_dev, lam_scale, beta, P->nx, P->nz,
-                                 n, s);
-      }));
-    }
-    ISAM_TRY(launch(P, ISAM_KCLASS_MISC, [&] {
-      return launch_tv_primal<T>(im.grad, px, pz, tau, lam_dev, lam_scale, zout, P->nx, P->nz,
-                                 n, s);
-    }));
-    return ISAM_OK;
   }
+  const size_t n = P->n_img;
+  cplx<T>* px = im.tv;
+  cplx<T>* pz = im.tv + n;
+  cplx<T>* rx = im.tv + 2 * n;
+  cplx<T>* rz = im.tv + 3 * n;
+  cplx<T>* w = im.tv + 4 * n;
+  const T tau = T(lam / L);
+  CUDA_TRY(cudaMemcpyAsync(rx, px, 2 * n * sizeof(cplx<T>), cudaMemcpyDeviceToDevice, s));
+  double t = 1.0;
+  for (int i = 0; i < iters; ++i) {
+    const double t_next = 0.5 * (1.0 + sqrt(1.0 + 4.0 * t * t));
+    const T beta = T((t - 1.0) / t_next);
+    t = t_next;
+    ISAM_TRY(launch(P, ISAM_KCLASS_MISC, [&] {
+      return launch_tv_primal<T>(im.grad, rx, rz, tau, lam_dev, lam_scale, w, P->nx, P->nz, n,
+                                 s);
+    }));
+    ISAM_TRY(launch(P, ISAM_KCLASS_MISC, [&] {
+      return launch_tv_dual<T>(w, px, pz, rx, rz, tau, lam_dev, lam_scale, beta, P->nx, P->nz,
+                               n, s);
+    }));
+  }
+  ISAM_TRY(launch(P, ISAM_KCLASS_MISC, [&] {
+    return launch_tv_primal<T>(im.grad, px, pz, tau, lam_dev, lam_scale, zout, P->nx, P->nz,
+                               n, s);
+  }));
+  return ISAM_OK;
 }
 
 // One iteration of Alg. 1: the fused gradient kernel on eta_hat^k (ehat_in,
@@ -829,13 +838,14 @@ template <typename T> isam_status solve_impl(isam_plan* P, const T* s_d, const i
     CUDA_TRY(cudaMemsetAsync(zQ, 0, sizeof(cplx<T>) * P->n_img, s));
     CUDA_TRY(cudaMemsetAsync(im.eta_hat, 0, sizeof(cplx<T>) * P->n_img, s));
   }
+  if (!im.sdh) ISAM_TRY(plan_alloc(P, &im.sdh, P->n_spec));
+  if (o->residual_addback && !im.s_tmp) ISAM_TRY(plan_alloc(P, &im.s_tmp, P->n_spec));
   if (o->prior == ISAM_PRIOR_TV) {                 // TV dual starts at 0 for every solve
-    if (!im.tv) ISAM_TRY(plan_alloc(P, &im.tv, tv_images<T>(P) * P->n_img));
+    ISAM_TRY(tv_alloc<T>(P, im));                  // after the arrays it cannot do without
     CUDA_TRY(cudaMemsetAsync(im.tv, 0, 2 * sizeof(cplx<T>) * P->n_img, s));
     im.tv_cur = 0;
   }
   // lateral spectrum of the data, used by every iteration's residual
-  if (!im.sdh) ISAM_TRY(plan_alloc(P, &im.sdh, P->n_spec));
   ISAM_TRY(lat_forward<T>(P, im, s_d, im.sdh, P->nk, true));
   const bool check = o->tol > 0;
   const int every = std::max(1, o->check_every);
@@ -931,7 +941,6 @@ template <typename T> isam_status solve_impl(isam_plan* P, const T* s_d, const i
   }
   // result: z^K, optionally with the residual added back (Alg. 1, last step)
   if (o->residual_addback) {
-    if (!im.s_tmp) ISAM_TRY(plan_alloc(P, &im.s_tmp, P->n_spec));
     ISAM_TRY(op_forward<T>(P, zP, im.s_tmp));
     ISAM_TRY(launch(P, ISAM_KCLASS_MISC, [&] {
       return launch_rsub<T>(s_d, im.s_tmp, im.s_tmp, P->n_spec, s);
@@ -1774,7 +1783,6 @@ template <typename T> isam_status batch_prepare(isam_plan* P, const isam_solve_o
   if (!im.zB) ISAM_TRY(plan_alloc(P, &im.zB, P->n_img));
   if (!im.sdh) ISAM_TRY(plan_alloc(P, &im.sdh, P->n_spec));
   if (!im.s_tmp) ISAM_TRY(plan_alloc(P, &im.s_tmp, P->n_spec));
-  if (o->prior == ISAM_PRIOR_TV && !im.tv) ISAM_TRY(plan_alloc(P, &im.tv, tv_images<T>(P) * P->n_img));
   double L = o->L;
   if (!(L > 0)) {
     if (!(P->L_cache > 0)) {
@@ -1788,6 +1796,7 @@ template <typename T> isam_status batch_prepare(isam_plan* P, const isam_solve_o
     L = P->L_cache;
   }
   if (!(L > 0)) return ISAM_ERR_INVALID;
+  if (o->prior == ISAM_PRIOR_TV) ISAM_TRY(tv_alloc<T>(P, im));
   *L_out = L;
   return ISAM_OK;
 }

@@ -9,8 +9,9 @@
 // momentum beta_k from the host.
 //
 // FP32 runs several dual steps per launch on tiles in registers (k_tv_tile);
-// FP64, whose arithmetic the tiles' halos would repeat at the FP64 pipe's rate,
-// runs two kernels a step, each writing only its own pixel.
+// FP64, whose arithmetic the tiles' halos would repeat at the FP64 pipe's rate, and
+// FP32 plans without room for the tiles' images run two kernels a step, each writing
+// only its own pixel.
 #include <math.h>
 
 #include "internal.cuh"
@@ -247,9 +248,15 @@ template <typename T> cudaError_t launch_tv_dual(const cplx<T>* w, cplx<T>* px, 
   k_tv_dual<T><<<1024, 256, 0, s>>>(w, px, pz, rx, rz, tau, lam_dev, lam_scale, beta, nx, nz, n);
   return cudaGetLastError();
 }
+template cudaError_t launch_tv_primal<float>(const float2*, const float2*, const float2*,
+                                              float, const double*, double, float2*, int, int,
+                                              size_t, cudaStream_t);
 template cudaError_t launch_tv_primal<double>(const double2*, const double2*, const double2*,
                                               double, const double*, double, double2*, int, int,
                                               size_t, cudaStream_t);
+template cudaError_t launch_tv_dual<float>(const float2*, float2*, float2*, float2*, float2*,
+                                            float, const double*, double, float, int, int, size_t,
+                                            cudaStream_t);
 template cudaError_t launch_tv_dual<double>(const double2*, double2*, double2*, double2*, double2*,
                                             double, const double*, double, double, int, int, size_t,
                                             cudaStream_t);

@@ -91,3 +91,35 @@ def test_coefficient_table_gives_way(torch):   # noqa: F811
         assert not pool.live
     assert float((got - z).norm()) <= 1e-13 * float(z.norm())
     assert float((again - z).norm()) <= 1e-13 * float(z.norm())
+
+
+@pytest.mark.parametrize("addback", [False, True])
+def test_tv_without_its_sixth_image(torch, addback):   # noqa: F811
+    """FP32 with nk < nz: the two-launch steps in place of the tiles'.  Both round each
+    step's arithmetic to 32 bits; 60 steps of rounding 1.2e-7 at |p| <= 1: 1e-5."""
+    from paper_1905_06058_gb300.isam import Batch, Plan
+    g = I.small_bscan(seed=74, nx=NX, nk=NK, nz=2 * NK).geom
+    with Pool(torch) as pool:
+        ref = Plan(g)
+        s = torch.from_numpy(I.random_spectra(ref.spec_shape, 9).astype(np.float32)).cuda()
+        kw = dict(lambda_rel=0.05, L=4.0, max_iter=3, prior="tv", addback=addback)
+        z = ref.solve(s, **kw)[0]
+        most = pool.held()
+        ref.close()
+        plan = Plan(g)
+        pool.budget = most - z.numel() * z.element_size()
+        got = plan.solve(s, **kw)[0]
+        again = plan.solve(s, **kw)[0]
+        plan.close()
+        pool.budget = 1 << 40
+        plan = Plan(g)
+        pool.refused = (6 * z.numel() * z.element_size(),)
+        out = torch.empty_like(z)
+        batch = Batch([(plan, s, out, kw)])
+        batch.run()
+        batch.close()
+        plan.close()
+        assert not pool.live
+    assert float((got - z).norm()) <= 1e-5 * float(z.norm())
+    assert torch.equal(got, again)
+    assert torch.equal(got, out)
