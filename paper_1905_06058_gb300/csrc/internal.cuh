@@ -152,6 +152,8 @@ template <typename T> struct AxArgs {
   const int* stop;
 };
 
+constexpr int kMultiprocessors = 152;   // of a GB300
+
 // Lets a kernel take `bytes` of dynamic shared memory; up to 44 KB (48 with the
 // kernels' static arrays) it may without being told, which saves small plans' launches
 // the call.

@@ -24,6 +24,8 @@
 
 #include <limits.h>
 
+#include <algorithm>
+
 #include "fft_col16.cuh"
 #include "fft_smem.cuh"
 #include "internal.cuh"
@@ -492,9 +494,6 @@ __device__ __forceinline__ void window_taps(const Coefficients<T, J>& co, int rh
   e[J] = shift ? c[J - 1] : T(0);
 }
 
-// Per block: the first sample's floor of every thread that has samples.
-struct WindowHeads { int mfl[512]; };
-
 // One thread's window: sums its samples, of taps (rho, e), slot by slot and hands
 // each finished slot (l, value) to put.
 template <typename T, int J, typename V, typename Taps, typename Put>
@@ -526,15 +525,15 @@ __device__ __forceinline__ void window_sums(const Sample<T, V>* sm, Taps taps, P
 template <typename T, int J, bool WARP, typename V, typename Taps>
 __device__ __forceinline__ void window_scatter(V* Y, int K, int nt, int nk,
                                                const Sample<T, V>* sm, V* past,
-                                               const WindowHeads& heads, Taps taps) {
-  constexpr int WS = window_slots<J>(), W_MIN = 2 * NRES - 1, W_MAX = 2 * NRES + 2;
+                                               const int* heads, Taps taps) {
+  constexpr int WS = window_slots<J>(), W_MIN = 2 * NRES - 1;
   const int tid = threadIdx.x, nact = nk / NRES;
   const bool active = tid < nact;
   const int off = 1 - J / 2;                          // first bin of a window - its head
-  const int base = heads.mfl[0] + off, end = heads.mfl[nact - 1] + off + WS;
-  const int m0 = active ? heads.mfl[tid] + off : 0;
+  const int base = heads[0] + off, end = heads[nact - 1] + off + WS;
+  const int m0 = active ? heads[tid] + off : 0;
   // bins before the next thread's window (all of them for the last thread)
-  const int own = tid < nact - 1 ? heads.mfl[tid + 1] + off - m0 : WS;
+  const int own = tid < nact - 1 ? heads[tid + 1] + off - m0 : WS;
   const int limit = base + K - m0;                    // slots from here on lie past one period
   for (int i = end + tid; i < base + K; i += nt)
     Y[prow(i & (K - 1))] = V{};
@@ -565,10 +564,15 @@ __device__ __forceinline__ void window_scatter(V* Y, int K, int nt, int nk,
   }
 }
 
-// The bins past one period: A.sc.window_past elements after the twiddles.
+// The bins past one period: A.sc.past elements after the twiddles; then the heads, the
+// first sample's floor of every thread that has samples.
 template <typename T, typename V>
 __device__ __forceinline__ V* window_past(const AxArgs<T>& A, V* Y) {
   return reinterpret_cast<V*>(reinterpret_cast<unsigned char*>(Y) + A.past_offset);
+}
+template <typename T, typename V>
+__device__ __forceinline__ int* window_heads(const AxArgs<T>& A, V* Y) {
+  return reinterpret_cast<int*>(window_past<T, V>(A, Y) + A.sc.past);
 }
 
 // the thread's samples fit one window
@@ -588,7 +592,7 @@ __device__ __forceinline__ bool quad_fits(const AxArgs<T>& A, const Sample<T, V>
 template <typename T, int J, bool WARP, typename V, typename Taps, typename Reload>
 __device__ __forceinline__ void scatter(const AxArgs<T>& A, const Coefficients<T, J>& co, V* Y,
                                         int K, int nt, int nk, Sample<T, V>* sm, bool fits,
-                                        int* lo, int* hi, int* ch_tail, WindowHeads& heads,
+                                        int* lo, int* hi, int* ch_tail, const int* heads,
                                         Taps taps, Reload reload) {
   if (__syncthreads_and(fits && !A.fit)) {
     window_scatter<T, J, WARP, V>(Y, K, nt, nk, sm, window_past<T, V>(A, Y), heads, taps);
@@ -791,17 +795,26 @@ __device__ __forceinline__ void ax_inverse(const AxArgs<T>& A, V* Y, const cplx<
   }
 }
 
-// FP32: two blocks of 512 threads on an SM (64 registers).  FP64: the pair at
+// FP32: 64 registers a thread (two blocks of 512 threads on an SM).  FP64: the pair at
 // K = 4096 fills an SM's shared memory by itself, so one (128 registers; at 64
 // the adjoint half spilled 0.5 to 2 KB a thread).
-template <typename T> __host__ __device__ constexpr int ax_min_blocks() {
-  return std::is_same<T, float>::value ? 2 : 1;
+// WIDE: the FP32 runtime lengths (K <= 1024, 128 threads at most) at 96 registers, for
+// grids that one round of blocks holds at that width: latency is what they take, and the
+// spills of 64 registers (up to 52 B) and their later trigger lie in it.  An iteration
+// at 32 x 24 x 256 takes 25.8 us (29.2 with the residue-class scatter, 33.1 with windows
+// and 64 registers), at 24 x 24 x 128 27.5 (28.5, 32.0), at 64 x 64 x 128 20.8 (47.7,
+// 24.4).  Larger grids are quicker at 64: 128 x 128 x 256 93 us, 100 wide.
+template <typename T, bool WIDE> __host__ __device__ constexpr int ax_max_threads() {
+  return WIDE ? 128 : 512;
+}
+template <typename T, bool WIDE> __host__ __device__ constexpr int ax_min_blocks() {
+  return WIDE ? 5 : std::is_same<T, float>::value ? 2 : 1;
 }
 
 // ONE: a block per column instead of per pair (FP64, see
 // launch_ax_JKC).
-template <typename T, int J, int LOGK, bool C16, bool ONE>
-__global__ void __launch_bounds__(512, ax_min_blocks<T>()) k_ax_fwd(const __grid_constant__ AxArgs<T> A) {
+template <typename T, int J, int LOGK, bool C16, bool ONE, bool WIDE>
+__global__ void __launch_bounds__(ax_max_threads<T, WIDE>(), (ax_min_blocks<T, WIDE>())) k_ax_fwd(const __grid_constant__ AxArgs<T> A) {
   using C = cplx<T>;
   using V = column_t<T, ONE>;
   extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -859,8 +872,8 @@ __global__ void __launch_bounds__(512, ax_min_blocks<T>()) k_ax_fwd(const __grid
 // RES: the input holds the model spectra S and the kernel forms the residual
 // spectrum R(q) = (S(q) + conj S(-q)) / 2 - F s_d(q) on load (ONE only; see
 // k_ax_fused).
-template <typename T, int J, int LOGK, bool C16, bool ONE, bool RES>
-__global__ void __launch_bounds__(512, ax_min_blocks<T>()) k_ax_adj(const __grid_constant__ AxArgs<T> A) {
+template <typename T, int J, int LOGK, bool C16, bool ONE, bool RES, bool WIDE>
+__global__ void __launch_bounds__(ax_max_threads<T, WIDE>(), (ax_min_blocks<T, WIDE>())) k_ax_adj(const __grid_constant__ AxArgs<T> A) {
   static_assert(ONE || !RES, "the pair kernel with a residual is k_ax_fused");
   using C = cplx<T>;
   using V = column_t<T, ONE>;
@@ -869,7 +882,7 @@ __global__ void __launch_bounds__(512, ax_min_blocks<T>()) k_ax_adj(const __grid
   const int K = axial_K<LOGK>(sc), nk = sc.nk;
   V* Y = reinterpret_cast<V*>(smem_raw);
   __shared__ int ch_lo, ch_hi, ch_tail;
-  __shared__ WindowHeads heads;
+  int* heads = window_heads<T, V>(A, Y);
   const int tid = threadIdx.x, nt = axial_threads<LOGK>();
   int c1, c2, mx, my;
   pair_columns<T, ONE>(A, c1, c2, mx, my);
@@ -915,7 +928,7 @@ __global__ void __launch_bounds__(512, ax_min_blocks<T>()) k_ax_adj(const __grid
   const Coefficients<T, J> co(A, pos, tid);
   bool fits = A.sc.window != 0;
   if (NRES * tid < nk) {
-    heads.mfl[tid] = sm[0].mfl;
+    heads[tid] = sm[0].mfl;
     fits = quad_fits<T, V>(A, sm);
   }
   scatter<T, J, false, V>(A, co, Y, K, nt, nk, sm, fits, &ch_lo, &ch_hi, &ch_tail, heads,
@@ -941,8 +954,8 @@ __global__ void __launch_bounds__(512, ax_min_blocks<T>()) k_ax_adj(const __grid
 // of the latter by the transforms' exchanges; DRAM 21 %.  A 1024 x 2048 B-scan (513
 // blocks, 40.2 us) leaves the second of its 1.7 waves two thirds full.
 // WS: also write the model spectra S to A.s_out.
-template <typename T, int J, int LOGK, bool WS, bool C16>
-__global__ void __launch_bounds__(512, ax_min_blocks<T>()) k_ax_fused(const __grid_constant__ AxArgs<T> A) {
+template <typename T, int J, int LOGK, bool WS, bool C16, bool WIDE>
+__global__ void __launch_bounds__(ax_max_threads<T, WIDE>(), (ax_min_blocks<T, WIDE>())) k_ax_fused(const __grid_constant__ AxArgs<T> A) {
   using C = cplx<T>;
   using V = cpair<T>;
   extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -950,7 +963,7 @@ __global__ void __launch_bounds__(512, ax_min_blocks<T>()) k_ax_fused(const __gr
   const int K = axial_K<LOGK>(sc), nk = sc.nk;
   V* Y = reinterpret_cast<V*>(smem_raw);
   __shared__ int ch_lo, ch_hi, ch_tail;
-  __shared__ WindowHeads heads;
+  int* heads = window_heads<T, V>(A, Y);
   // The column-split form keeps in tensor memory (tmem.cuh) what its 64 registers a
   // thread do not hold from the forward half to the adjoint: the samples' taps,
   // which it evaluated twice, and its eight samples of eta_hat, which it read twice
@@ -1004,7 +1017,7 @@ __global__ void __launch_bounds__(512, ax_min_blocks<T>()) k_ax_fused(const __gr
     pos.quad(A, q, sm);
     fits = quad_fits<T, V>(A, sm);
     if (TM) fits = __all_sync(0xffffffffu, fits);
-    if (active) heads.mfl[tid] = sm[0].mfl;
+    if (active) heads[tid] = sm[0].mfl;
     V php, dq, w1, w2;                   // of two samples: phases, F s_d, model spectra
     interp_quad<T, J, V>(Coefficients<T, J>(A, pos, q), Y, K, sm, fits, [&](int rho, const T* e) {
       if constexpr (TM) tmem::put_taps<J>(tm + rho * TAPS, e);
@@ -1138,7 +1151,7 @@ enum { AX_FWD = 0, AX_ADJ = 1, AX_FUSED = 2, AX_ADJ_RES = 3 };
 // compiled for FP32 only
 template <typename T> constexpr bool ax_one() { return sizeof(T) == 8; }
 
-template <typename T, int J, int LOGK, bool C16>
+template <typename T, int J, int LOGK, bool C16, bool WIDE = false>
 static cudaError_t launch_ax_JKC(const AxArgs<T>& a, int npairs, cudaStream_t s, int kind) {
   constexpr bool ONE = ax_one<T>();
   using V = column_t<T, ONE>;
@@ -1147,12 +1160,12 @@ static cudaError_t launch_ax_JKC(const AxArgs<T>& a, int npairs, cudaStream_t s,
   size_t sm = ax_smem<T, ONE>(K);
   AxArgs<T> b = a;
   b.past_offset = unsigned(sm);
-  if (kind != AX_FWD) sm += size_t(a.sc.past) * sizeof(V);
+  if (kind != AX_FWD) sm += size_t(a.sc.past) * sizeof(V) + a.sc.nk / NRES * sizeof(int);
   void (*kern)(AxArgs<T>) = nullptr;
-  if (kind == AX_ADJ) kern = k_ax_adj<T, J, LOGK, C16, ONE, false>;
-  else if (kind == AX_FWD) kern = k_ax_fwd<T, J, LOGK, C16, ONE>;
-  else if constexpr (ONE) kern = k_ax_adj<T, J, LOGK, C16, ONE, true>;
-  else kern = a.s_out ? k_ax_fused<T, J, LOGK, true, C16> : k_ax_fused<T, J, LOGK, false, C16>;
+  if (kind == AX_ADJ) kern = k_ax_adj<T, J, LOGK, C16, ONE, false, WIDE>;
+  else if (kind == AX_FWD) kern = k_ax_fwd<T, J, LOGK, C16, ONE, WIDE>;
+  else if constexpr (ONE) kern = k_ax_adj<T, J, LOGK, C16, ONE, true, WIDE>;
+  else kern = a.s_out ? k_ax_fused<T, J, LOGK, true, C16, WIDE> : k_ax_fused<T, J, LOGK, false, C16, WIDE>;
   allow_smem(kern, sm);
   // programmatic dependent launch: each axial kernel builds its twiddles while
   // the previous kernel finishes, then waits for it (cudaGridDependencySynchronize)
@@ -1192,6 +1205,12 @@ cudaError_t launch_ax_J(const AxArgs<T>& a, int npairs, cudaStream_t s, int kind
   }
   if constexpr (sizeof(T) == 4) {
     if (a.radix16 && a.sc.K == 1024) return launch_ax_JKC<T, J, 10, true>(a, npairs, s, kind);
+  }
+  if constexpr (sizeof(T) == 4) {
+    // one round of blocks of whole warps at 96 registers
+    const int threads = std::max(32, a.sc.K / 8), resident = kMultiprocessors * (65536 / 96);
+    if (size_t(npairs) * threads <= size_t(resident))
+      return launch_ax_JKC<T, J, 0, false, true>(a, npairs, s, kind);
   }
   return launch_ax_JK<T, J, 0>(a, npairs, s, kind);
 }
