@@ -223,8 +223,9 @@ __device__ __forceinline__ float2 st_vjp(float2 u, float2 zb, float tau) {
 }
 __device__ __forceinline__ double2 st_vjp(double2 u, double2 zb, double tau) {
   const double m2 = fma(u.x, u.x, u.y * u.y);
-  const double inv = m2 > 0.0 ? rsqrt(m2) : 0.0;
-  if (!(m2 > 0.0) || !(1.0 - tau * inv > 0.0)) return make_double2(0.0, 0.0);
+  const double am = sqrt(m2);
+  if (!(m2 > 0.0) || !(1.0 - tau / am > 0.0)) return make_double2(0.0, 0.0);
+  const double inv = 1.0 / am;
   const double rz = fma(u.x, zb.x, u.y * zb.y) * inv * inv * inv;
   return make_double2(zb.x - tau * (zb.x * inv - u.x * rz), zb.y - tau * (zb.y * inv - u.y * rz));
 }

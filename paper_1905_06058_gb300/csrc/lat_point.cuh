@@ -15,7 +15,7 @@ __device__ __forceinline__ float2 soft_threshold(float2 u, float tau) {
 }
 __device__ __forceinline__ double2 soft_threshold(double2 u, double tau) {
   const double m2 = fma(u.x, u.x, u.y * u.y);
-  const double f = m2 > 0.0 ? fmax(1.0 - tau * rsqrt(m2), 0.0) : 0.0;
+  const double f = m2 > 0.0 ? fmax(1.0 - tau / sqrt(m2), 0.0) : 0.0;
   return cscale(u, f);
 }
 
