@@ -50,11 +50,17 @@ __device__ __forceinline__ cplx<T> real_part_spectrum(cplx<T> a, cplx<T> b) {
   return cscale(cadd(a, cconj(b)), T(0.5));   // F(Re v)(q) from F v(q), F v(-q)
 }
 
+// a + b for an exact b
+__device__ __forceinline__ ff plus(ff a, float b) {
+  const ff t = ff_two_sum(a.hi, b);
+  return ff_quick(t.hi, __fadd_rn(t.lo, a.lo));
+}
+
 // What bounds k_param_reduce: the latency of its loads and the FP64 pipe (2 lanes a
 // clock), for 40 bytes of each column sample.  A thread takes two neighbouring samples
 // of both columns a load and has two such groups in flight; TPB is a quarter of nk up
 // to 512, so that they cover nk = 2048.  FP32 plans keep the samples' arithmetic in
-// float, the cancelling 2 kappa - sqrt(a) from a two-float constant, and the threads'
+// float, the cancelling 4 kappa^2 - a from float pairs, and the threads'
 // sums are added in double by one warp a moment.  512 x 2048: 24.7 -> 15.2 us (16.5 at
 // one block a multiprocessor, 72 registers).
 //
@@ -77,15 +83,19 @@ __global__ void __launch_bounds__(TPB, sizeof(T) == 4 && TPB == 512 ? 2 : 1)
   const int my = iy <= (ny - 1) / 2 ? iy : iy - ny;
   const double a = A.sc.Qx * double(mx) * mx + A.sc.Qy * double(my) * my;
   const double tc = 0.5 * double(nk - 1);
-  // FP32: 2 kappa_j -+ sqrt(a) = (cut.x + 2 j) + cut.y and (cut.z + 2 j)
-  __shared__ float4 cut_s;
+  // FP32: 2 kappa_0 - sqrt(a), 2 kappa_0 + sqrt(a) and 2 kappa_0 as float pairs, and a
+  __shared__ float cut_s[7];
   __shared__ T part[5][TPB];
-  float4 cut = {};
+  ff lo = {}, hi = {}, mid = {};
+  float af = 0.0f;
   if constexpr (std::is_same<T, float>::value && !FIT) {
     if (threadIdx.x == 0) {
-      const double sa = sqrt(a), lo = 2.0 * A.sc.kap - sa;
-      cut_s = make_float4(float(lo), float(lo - double(float(lo))), float(2.0 * A.sc.kap + sa),
-                          float(a));
+      const double sa = sqrt(a), v[3] = {2.0 * A.sc.kap - sa, 2.0 * A.sc.kap + sa, 2.0 * A.sc.kap};
+      for (int i = 0; i < 3; ++i) {
+        cut_s[2 * i] = float(v[i]);
+        cut_s[2 * i + 1] = float(v[i] - double(float(v[i])));
+      }
+      cut_s[6] = float(a);
     }
   }
   C* s1 = A.su + size_t(c1) * nk;
@@ -140,8 +150,12 @@ __global__ void __launch_bounds__(TPB, sizeof(T) == 4 && TPB == 512 ? 2 : 1)
           m[4] = fmaf(float(a) / (2.0f * float(kap) + sqrtf(float(x))), v, m[4]);
         return;
       }
-      const float j2 = float(2 * j), dm = (cut.x + j2) + cut.y, dp = cut.z + j2;
-      if (dm > 0.0f) m[4] = fmaf(cut.w / (0.5f * (dm + dp) + sqrtf(dm * dp)), v, m[4]);
+      // 4 kappa^2 - a as the product of its factors, each a float pair (44 bits): as
+      // near as the difference in double, rounded to float
+      const float j2 = float(2 * j);
+      const ff dm = plus(lo, j2), dp = plus(hi, j2), k2 = plus(mid, j2);
+      const float x = fmaf(dm.hi, dp.hi, fmaf(dm.hi, dp.lo, dm.lo * dp.hi));
+      if (dm.hi > 0.0f) m[4] = fmaf(af / (k2.hi + sqrtf(x)), v, m[4]);
     } else {
       const double dv = double(v);
       const double t = double(j) - tc;
@@ -182,7 +196,10 @@ __global__ void __launch_bounds__(TPB, sizeof(T) == 4 && TPB == 512 ? 2 : 1)
       const ParamSamples<T> x = load(j), y = load(j + 2 * TPB);
       if (j == 2 * threadIdx.x) {
         __syncthreads();
-        cut = cut_s;
+        lo = {cut_s[0], cut_s[1]};
+        hi = {cut_s[2], cut_s[3]};
+        mid = {cut_s[4], cut_s[5]};
+        af = cut_s[6];
       }
       use(j, x);
       use(j + 2 * TPB, y);
