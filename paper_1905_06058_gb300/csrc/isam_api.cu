@@ -457,9 +457,11 @@ template <typename T> isam_status lat_inverse(isam_plan* P, Impl<T>& im, cplx<T>
 // The standalone operators' spectra belong to real arrays, so FP32 plans keep half of
 // them where the x passes can: nx of the register form, and real arrays s on 8 bytes
 // (two columns a load; the whole-spectrum form below reads one).  256 x 256 x 2048,
-// A + A^H: 4.40 -> 3.90 ms, 1.1 of 10 GB less; 1024 x 2048: 69 us either way.
+// A + A^H: 4.40 -> 3.90 ms, 1.1 of 10 GB less; 1024 x 2048: 69 us either way.  Two
+// neighbouring samples share a transform, so each is right to 32 bits of the larger of
+// them: not with a filter B, which may set one to zero and leave the other.
 template <typename T> bool half_spectra(const isam_plan* P, const void* s) {
-  return sizeof(T) == 4 && P->nz == P->nk && P->tune_radix_lat == 16 &&
+  return sizeof(T) == 4 && P->nz == P->nk && P->filt_host.empty() && P->tune_radix_lat == 16 &&
          lat_half_takes(P->nx, P->nk) && reinterpret_cast<uintptr_t>(s) % 8 == 0;
 }
 template <typename T> LatArgs<T> half_x_args(isam_plan* P, const void* in, void* out) {
