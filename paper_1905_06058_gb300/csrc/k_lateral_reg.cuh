@@ -118,9 +118,9 @@ __global__ void __launch_bounds__(lat_reg_threads<T, L>(), lat_reg_min_blocks<T,
   }
   if constexpr (UPDATE) {
     // the FISTA step of k_lat: LAT_UPDATE forms u = eta^k - g/L from the gradient,
-    // LAT_UPDATE_U transformed u itself; norm partials as there (a thread's points
-    // in the plan's precision, the block's threads in double)
-    T acc0 = T(0), acc1 = T(0), acc2 = T(0);
+    // LAT_UPDATE_U transformed u itself; norm partials as there (at most 16 points of a
+    // thread, so 32 squares, in the plan's precision, then in double)
+    T acc0 = T(0), acc1 = T(0), acc2 = T(0), first0 = T(0), first1 = T(0), first2 = T(0);
     bool bad = false;
     const T sg = nrm * a.inv_L;
     T tau = a.lam_dev ? T(a.lam_scale * *a.lam_dev) : a.lam_over_L;
@@ -128,6 +128,10 @@ __global__ void __launch_bounds__(lat_reg_threads<T, L>(), lat_reg_min_blocks<T,
 #pragma unroll
     for (int h = 0; h < P; h += BATCH) {
       if (h || !EARLY) load_iterates(h);
+      if (!FROM_U && P > 16 && h == P / 2) {
+        first0 = acc0; first1 = acc1; first2 = acc2;
+        acc0 = acc1 = acc2 = T(0);
+      }
 #pragma unroll
       for (int i = 0; i < BATCH; ++i) {
         const size_t g = g0 + (h + i) * step;
@@ -163,9 +167,9 @@ __global__ void __launch_bounds__(lat_reg_threads<T, L>(), lat_reg_min_blocks<T,
       if (a.partial != nullptr) {
         __shared__ double red[3][NT / 32];
         const int wid = tid >> 5, lane = tid & 31;
-        const double w0 = warp_sum_lanes(double(acc0), 32);
-        const double w1 = warp_sum_lanes(double(acc1), 32);
-        const double w2 = warp_sum_lanes(double(acc2), 32);
+        const double w0 = warp_sum_lanes(double(acc0) + double(first0), 32);
+        const double w1 = warp_sum_lanes(double(acc1) + double(first1), 32);
+        const double w2 = warp_sum_lanes(double(acc2) + double(first2), 32);
         if (lane == 0) { red[0][wid] = w0; red[1][wid] = w1; red[2][wid] = w2; }
         __syncthreads();
         if (tid < 3) {
