@@ -269,7 +269,11 @@ isam_status isam_param_grad(isam_plan* plan, const void* x, const void* y, doubl
  * to z_out and, if ckpt is not NULL, the pair (z^{c e}, z^{c e - 1}) before
  * iteration c e + 1 to images 2c, 2c+1 of ckpt, e = every; ckpt holds
  * isam_unrolled_checkpoint_images(K, every) images of the plan's type.
- * Synchronous; ISAM_ERR_NONFINITE if an iterate is not finite. */
+ * Synchronous; ISAM_ERR_NONFINITE if an iterate is not finite.
+ * FP32 plans with nz > nk, whose fits leave a residual at the size of rounding,
+ * keep one order of sums in these calls, isam_param_grad, isam_data_fidelity and
+ * the operators; their iterates agree with isam_solve's to rounding, those of
+ * other plans bit for bit. */
 int32_t isam_unrolled_checkpoint_images(int32_t K, int32_t every);
 isam_status isam_fista_unrolled(isam_plan* plan, const void* s_d, const isam_solve_opts* opts,
                                 int32_t every, void* ckpt, void* z_out);
@@ -340,10 +344,13 @@ void isam_batch_destroy(isam_batch* batch);
  *                  transforms at K = 1024 to 4096 (three shared-memory passes);
  *                  8: radix-8 passes on column pairs (four); other plans run
  *                  radix 8 whatever the value
- *   lateral_radix  16: FP32 lateral passes of lengths 64 to 1024 (2^p, 3 * 2^p
- *                  from 192) at the built-in tile keep it in registers; 8: radix-8
- *                  passes on column pairs in shared memory; other plans and
- *                  tiles run the latter whatever the value */
+ *   lateral_radix  16: lateral passes of lengths 64 to 1024 (2^p, 3 * 2^p from 192;
+ *                  FP64: 2^p, 64 to 512) at the built-in tile keep it in
+ *                  registers, and isam_forward / isam_adjoint of FP32 plans with
+ *                  nz = nk and no filter keep half of the Hermitian spectra; 8:
+ *                  radix-8 passes on column pairs in shared memory and whole
+ *                  spectra; other lengths and tiles run the latter whatever the
+ *                  value.  The autotuner times solve iterations only */
 typedef struct {
   int32_t lateral_tile;
   int32_t stolt_table;

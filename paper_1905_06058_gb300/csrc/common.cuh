@@ -57,11 +57,13 @@ __host__ __device__ __forceinline__ float2 cscale(float2 a, float s) {
   a.x *= s; a.y *= s; return a;
 #endif
 }
-// FP32: which product is rounded first is said here, not left to each kernel's
-// contraction (the adjoint's values depend on it, see FitOrder)
-__device__ __forceinline__ float2 cmulc(float2 a, float2 b) {
+// The same, where FP32 says which product is rounded first and does not leave it to the
+// kernel's contraction: the adjoint's values follow it (FitOrder).  (In k_ax_fused, which
+// contracts cmulc that way by itself, it cost 44 B of spills a thread with WS.)
+__device__ __forceinline__ float2 cmulc_ordered(float2 a, float2 b) {
   return make_float2(fmaf(a.x, b.x, a.y * b.y), fmaf(a.y, b.x, -(a.x * b.y)));
 }
+__device__ __forceinline__ double2 cmulc_ordered(double2 a, double2 b) { return cmulc(a, b); }
 template <typename C> __host__ __device__ __forceinline__ C cconj(C a) { a.y = -a.y; return a; }
 // acc + c y for a real c
 template <typename C, typename T> __device__ __forceinline__ C cfma_r(T c, C y, C acc) {

@@ -94,8 +94,7 @@ __device__ __forceinline__ void dft16(float2* a) {
 template <int SIGN, int R> __device__ __forceinline__ void dft_r(float2* a) {
   if constexpr (R == 16) dft16<SIGN, false>(a);
   else if constexpr (R == 8) dft8<SIGN>(a);
-  else if constexpr (R == 4) dft4<SIGN>(a[0], a[1], a[2], a[3]);
-  else dft2<SIGN>(a[0], a[1]);
+  else dft4<SIGN>(a[0], a[1], a[2], a[3]);
 }
 
 // Twiddle table: per pass with span NS > 1 (radix R), entry k < NS holds
@@ -121,13 +120,12 @@ template <int LOGK> __device__ __forceinline__ void build_twiddles(float4* tw) {
   __syncthreads();
 }
 
-// a[r] *= w^r, r = 1 .. R-1 (R = 2, 4, 8 or 16), from (w, w^4) (conjugated
+// a[r] *= w^r, r = 1 .. R-1 (R = 4, 8 or 16), from (w, w^4) (conjugated
 // for SIGN > 0)
 template <int SIGN, int R> __device__ __forceinline__ void twiddle(float2* a, float4 t) {
   float2 w1 = make_float2(t.x, t.y), w4 = make_float2(t.z, t.w);
   if (SIGN > 0) { w1.y = -w1.y; w4.y = -w4.y; }
   a[1] = cmul(a[1], w1);
-  if constexpr (R == 2) return;
   const float2 w2 = cmul(w1, w1), w3 = cmul(w2, w1);
   a[2] = cmul(a[2], w2);
   a[3] = cmul(a[3], w3);

@@ -175,9 +175,6 @@ __device__ __forceinline__ void dft8(E* a) {
 __host__ __device__ __forceinline__ int prow(int r) { return r + (r >> 3); }
 __host__ __device__ __forceinline__ int padded_rows(int L) { return L + (L >> 3); }
 
-__device__ __forceinline__ void sincospi_(float x, float* s, float* c) { sincospif(x, s, c); }
-__device__ __forceinline__ void sincospi_(double x, double* s, double* c) { sincospi(x, s, c); }
-
 // FP32 twiddle table of an L-point transform, in shared memory: for every pass
 // with span Ns > 1 and radix R, entry k of that pass's segment holds
 // w_k = e^{-2 pi i k / (Ns R)}, k < Ns.  A butterfly raises w_k to the powers
@@ -205,26 +202,29 @@ __host__ __device__ __forceinline__ int twiddle_entries(int L, int logL, int r3 
 template <typename T>
 __device__ __forceinline__ const cplx<T>* build_twiddles(cplx<T>* tab, const cplx<T>* roots, int L,
                                                          int logL, int r3 = 0) {
-  if constexpr (sizeof(T) == 8) return roots;
-  if (L >= 8) {
-    const int n8 = logL / 3, rem = logL - 3 * n8;
-    const int npass = n8 + (rem ? 1 : 0) + r3;
-    int off = 0, Ns = 1;
-    for (int p = 0; p < npass; ++p) {
-      const int R = p < n8 ? 8 : (p == n8 && rem ? (rem == 2 ? 4 : 2) : 3);
-      if (Ns > 1) {
-        for (int k = threadIdx.x; k < Ns; k += blockDim.x) {
-          T s, c;
-          sincospi_(T(2 * k) / T(Ns * R), &s, &c);
-          tab[off + k] = mk<T>(c, -s);
+  if constexpr (sizeof(T) == 8) {
+    return roots;
+  } else {
+    if (L >= 8) {
+      const int n8 = logL / 3, rem = logL - 3 * n8;
+      const int npass = n8 + (rem ? 1 : 0) + r3;
+      int off = 0, Ns = 1;
+      for (int p = 0; p < npass; ++p) {
+        const int R = p < n8 ? 8 : (p == n8 && rem ? (rem == 2 ? 4 : 2) : 3);
+        if (Ns > 1) {
+          for (int k = threadIdx.x; k < Ns; k += blockDim.x) {
+            float s, c;
+            sincospif(float(2 * k) / float(Ns * R), &s, &c);
+            tab[off + k] = make_float2(c, -s);
+          }
+          off += Ns;
         }
-        off += Ns;
+        Ns *= R;
       }
-      Ns *= R;
     }
+    __syncthreads();
+    return tab;
   }
-  __syncthreads();
-  return tab;
 }
 
 // the twiddles of the passes after one of span Ns

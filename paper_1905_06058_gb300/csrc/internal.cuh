@@ -178,7 +178,7 @@ template <> cudaError_t launch_lat_reg<double>(int mode, const LatArgs<double>& 
 template <typename T> cudaError_t launch_ax_fwd(const AxArgs<T>& a, int npairs, cudaStream_t s);
 template <typename T> cudaError_t launch_ax_adj(const AxArgs<T>& a, int npairs, cudaStream_t s);
 template <typename T> cudaError_t launch_ax_fused(const AxArgs<T>& a, int npairs, cudaStream_t s);
-template <typename T> size_t ax_smem_bytes(int K, int nk, bool adj);
+template <typename T> size_t ax_smem_bytes(int K);
 
 // Stolt table: class |my| (nx/2+1) + |mx| of every |q|
 template <typename T> cudaError_t launch_stolt_table(const AxArgs<T>& a, int4* out,

@@ -74,9 +74,9 @@ struct isam_plan {
   double* dscal = nullptr;      // device scalars [8]
   double* hscal = nullptr;      // pinned host mirror [8]
   int* flag = nullptr;          // device non-finite flag
-  // device-side stop rule of the solve: [stopped, iteration] on the device,
-  // pinned mirrors of the pending check's outcome [0, 2) and of the final one
-  // [2, 4), and an event after the pending check's copy
+  // device-side stop rule of the solve: [stopped, iteration] on the device, pinned:
+  // the pending check's outcome [0, 2), written by its reduction, and the final one
+  // [2, 4), and an event behind the pending check (see solve_impl)
   int* dstop = nullptr;
   int* hstop = nullptr;
   cudaEvent_t ev_check = nullptr;
@@ -265,8 +265,7 @@ double host_kb_scale(int n, int K, int J) {
 }
 
 template <typename T> bool precision_fits(const isam_plan* P) {
-  return ax_smem_bytes<T>(P->K, P->nk, true) <= 227u * 1024u &&
-         ax_smem_bytes<T>(P->K, P->nk, false) <= 227u * 1024u;
+  return ax_smem_bytes<T>(P->K) <= 227u * 1024u;
 }
 
 // Tables that depend on the dispersion coefficients and the focal depth:
@@ -612,7 +611,9 @@ template <typename T> isam_status tv_prox(isam_plan* P, Impl<T>& im, cplx<T>* zo
   cudaStream_t s = P->stream;
   if constexpr (sizeof(T) == 4) if (im.tv_tiles) {
     // five steps a launch: 20 in four launches of tiles whose inner 54 x 54 pixels
-    // are 71% of what they compute
+    // are 71% of what they compute.  (One block fills a multiprocessor, so a launch's
+    // time goes by whole rounds of blocks: at 384 x 1024 the first three launches are
+    // one round of 152 and the last, whose halo is six pixels, 160 in two.)
     constexpr int kSteps = 5;
     static_assert(kSteps <= TV_STEPS, "TvLaunch holds the momentum of a launch");
     const size_t n = P->n_img;

@@ -564,11 +564,15 @@ __device__ __forceinline__ void window_scatter(V* Y, int K, int nt, int nk,
   }
 }
 
-// The bins past one period: A.sc.past elements after the twiddles; then the heads, the
-// first sample's floor of every thread that has samples.
+// The bins past one period: A.sc.past elements after the twiddles.  The heads, the first
+// sample's floor of every thread that has samples: a static array where K is a constant,
+// else after the bins.
 template <typename T, typename V>
 __device__ __forceinline__ V* window_past(const AxArgs<T>& A, V* Y) {
   return reinterpret_cast<V*>(reinterpret_cast<unsigned char*>(Y) + A.past_offset);
+}
+template <int LOGK> __host__ __device__ constexpr int window_heads_fixed() {
+  return LOGK > 0 ? (1 << LOGK) / 8 : 1;
 }
 template <typename T, typename V>
 __device__ __forceinline__ int* window_heads(const AxArgs<T>& A, V* Y) {
@@ -882,7 +886,8 @@ __global__ void __launch_bounds__(ax_max_threads<T, WIDE>(), (ax_min_blocks<T, W
   const int K = axial_K<LOGK>(sc), nk = sc.nk;
   V* Y = reinterpret_cast<V*>(smem_raw);
   __shared__ int ch_lo, ch_hi, ch_tail;
-  int* heads = window_heads<T, V>(A, Y);
+  __shared__ int heads_fixed[window_heads_fixed<LOGK>()];
+  int* heads = LOGK > 0 ? heads_fixed : window_heads<T, V>(A, Y);
   const int tid = threadIdx.x, nt = axial_threads<LOGK>();
   int c1, c2, mx, my;
   pair_columns<T, ONE>(A, c1, c2, mx, my);
@@ -914,13 +919,13 @@ __global__ void __launch_bounds__(ax_max_threads<T, WIDE>(), (ax_min_blocks<T, W
         x.a = csub(cscale(cadd(x.a, cconj(y.a)), T(0.5)), d.a);
         x.b = csub(cscale(cadd(x.b, cconj(y.b)), T(0.5)), d.b);
       }
-      sm[2 * h].val.a = cmulc(x.a, ph.a);
-      sm[2 * h + 1].val.a = cmulc(x.b, ph.b);
+      sm[2 * h].val.a = cmulc_ordered(x.a, ph.a);
+      sm[2 * h + 1].val.a = cmulc_ordered(x.b, ph.b);
       if constexpr (!ONE) {
         cpair<T> y{};
         if (two) y = half ? cpair<T>{cconj(x.a), cconj(x.b)} : load_two<T>(r2 + j);
-        sm[2 * h].val.b = cmulc(y.a, ph.a);
-        sm[2 * h + 1].val.b = cmulc(y.b, ph.b);
+        sm[2 * h].val.b = cmulc_ordered(y.a, ph.a);
+        sm[2 * h + 1].val.b = cmulc_ordered(y.b, ph.b);
       }
     }
   }
@@ -953,6 +958,8 @@ __global__ void __launch_bounds__(ax_max_threads<T, WIDE>(), (ax_min_blocks<T, W
 // waves) 53 % of the issue slots and 64 % of the load/store data path are taken, half
 // of the latter by the transforms' exchanges; DRAM 21 %.  A 1024 x 2048 B-scan (513
 // blocks, 40.2 us) leaves the second of its 1.7 waves two thirds full.
+// At 64 registers the column-split form spills 16 to 44 bytes a thread at J = 6, 72 to
+// 112 at J = 8, whose four samples share 15 slots.
 // WS: also write the model spectra S to A.s_out.
 template <typename T, int J, int LOGK, bool WS, bool C16, bool WIDE>
 __global__ void __launch_bounds__(ax_max_threads<T, WIDE>(), (ax_min_blocks<T, WIDE>())) k_ax_fused(const __grid_constant__ AxArgs<T> A) {
@@ -963,7 +970,8 @@ __global__ void __launch_bounds__(ax_max_threads<T, WIDE>(), (ax_min_blocks<T, W
   const int K = axial_K<LOGK>(sc), nk = sc.nk;
   V* Y = reinterpret_cast<V*>(smem_raw);
   __shared__ int ch_lo, ch_hi, ch_tail;
-  int* heads = window_heads<T, V>(A, Y);
+  __shared__ int heads_fixed[window_heads_fixed<LOGK>()];
+  int* heads = LOGK > 0 ? heads_fixed : window_heads<T, V>(A, Y);
   // The column-split form keeps in tensor memory (tmem.cuh) what its 64 registers a
   // thread do not hold from the forward half to the adjoint: the samples' taps,
   // which it evaluated twice, and its eight samples of eta_hat, which it read twice
@@ -1138,11 +1146,7 @@ template <typename T, bool ONE> static size_t ax_smem(int K) {
                    size_t(twiddle_entries<T>(K, ilog2_dev(K))) * sizeof(cplx<T>);
   return (b + sizeof(V) - 1) / sizeof(V) * sizeof(V);
 }
-template <typename T> size_t ax_smem_bytes(int K, int nk, bool adj) {
-  (void)nk;
-  (void)adj;
-  return ax_smem<T, false>(K);
-}
+template <typename T> size_t ax_smem_bytes(int K) { return ax_smem<T, false>(K); }
 
 // AX_ADJ_RES: the adjoint of the residual of model spectra (one column a block)
 enum { AX_FWD = 0, AX_ADJ = 1, AX_FUSED = 2, AX_ADJ_RES = 3 };
@@ -1160,7 +1164,10 @@ static cudaError_t launch_ax_JKC(const AxArgs<T>& a, int npairs, cudaStream_t s,
   size_t sm = ax_smem<T, ONE>(K);
   AxArgs<T> b = a;
   b.past_offset = unsigned(sm);
-  if (kind != AX_FWD) sm += size_t(a.sc.past) * sizeof(V) + a.sc.nk / NRES * sizeof(int);
+  if (kind != AX_FWD) {
+    sm += size_t(a.sc.past) * sizeof(V);
+    if (LOGK == 0) sm += a.sc.nk / NRES * sizeof(int);
+  }
   void (*kern)(AxArgs<T>) = nullptr;
   if (kind == AX_ADJ) kern = k_ax_adj<T, J, LOGK, C16, ONE, false, WIDE>;
   else if (kind == AX_FWD) kern = k_ax_fwd<T, J, LOGK, C16, ONE, WIDE>;

@@ -5,7 +5,7 @@
 namespace isam {
 
 template cudaError_t launch_stolt_table<double>(const AxArgs<double>&, int4*, cudaStream_t);
-template size_t ax_smem_bytes<double>(int, int, bool);
+template size_t ax_smem_bytes<double>(int);
 template cudaError_t launch_ax_fwd<double>(const AxArgs<double>&, int, cudaStream_t);
 template cudaError_t launch_ax_adj<double>(const AxArgs<double>&, int, cudaStream_t);
 template cudaError_t launch_ax_fused<double>(const AxArgs<double>&, int, cudaStream_t);

@@ -27,6 +27,12 @@ template <typename T, int L> __host__ __device__ constexpr int lat_reg_min_block
   return n > 16 ? 16 : n;
 }
 
+// of a plain transform's grid (see k_lat_reg)
+__device__ __forceinline__ bool trigger_at_once() {
+  const unsigned blocks = gridDim.x * gridDim.y;
+  return blocks <= 32 || blocks > unsigned(kMultiprocessors);
+}
+
 template <typename T, int MODE, int L>
 __global__ void __launch_bounds__(lat_reg_threads<T, L>(), lat_reg_min_blocks<T, L>())
     k_lat_reg(const __grid_constant__ LatArgs<T> a) {
@@ -42,13 +48,16 @@ __global__ void __launch_bounds__(lat_reg_threads<T, L>(), lat_reg_min_blocks<T,
   // programmatic dependent launch: build the twiddles, then wait for the previous
   // kernel's results.  The next kernel may start its prologue before the last
   // transform or stores of a solve's pass (see k_ax_fused).  The plain transforms of
-  // 33 to 152 blocks, which leave multiprocessors free for the next grid's blocks to
-  // crowd, allow it before their stores (A^H at 512 x 1024: 15.1 us, 17.5 if at
-  // once), the others at once (A + A^H at 1024 x 2048: 69 us, 71 if late).
+  // 33 to kMultiprocessors blocks, which leave multiprocessors free for the next grid's
+  // blocks to crowd, allow it before their stores, the others at once: more blocks
+  // leave none free (1024 x 2048: 69 us, 71 if late), and up to 32 are over before the
+  // next launch comes, which is then what takes the time.  A + A^H, GPU time at once
+  // and late: 4 blocks (128 x 64) 13.4 and 16.2 us, 32 (128 x 512) 13.5 and 15.8, (512 x
+  // 512) 23.9 and 25.9, 64 (192 x 1024) 22.5 and 20.5, (256 x 1024) 22.2 and 20.5,
+  // 128 (1024 x 1024) 40.0 and 39.2.
   constexpr bool PLAIN = MODE == LAT_C2C_FWD || MODE == LAT_C2C_INV || MODE == LAT_R2C_FWD ||
                          MODE == LAT_INV_REAL;
-  const unsigned blocks = gridDim.x * gridDim.y;
-  const bool early = PLAIN && (blocks <= 32 || blocks > 152);
+  const bool early = PLAIN && trigger_at_once();
   if (early) cudaTriggerProgrammaticLaunchCompletion();
   const lreg::Twiddles<T, L> tw(b, a.roots);
   cudaGridDependencySynchronize();
@@ -217,8 +226,7 @@ __global__ void __launch_bounds__(lat_reg_threads<float, L>(), lat_reg_min_block
   float2* S = reinterpret_cast<float2*>(smem_raw);
   const int tid = threadIdx.x, c = tid % W, b = tid / W;
   // dependent launch as the plain passes of k_lat_reg
-  const unsigned blocks = gridDim.x * gridDim.y;
-  const bool early = blocks <= 32 || blocks > 152;
+  const bool early = trigger_at_once();
   if (early) cudaTriggerProgrammaticLaunchCompletion();
   const lreg::Twiddles<float, L> tw(b, nullptr);
   cudaGridDependencySynchronize();

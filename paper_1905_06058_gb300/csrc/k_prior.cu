@@ -84,7 +84,8 @@ __global__ void k_tv_dual(const cplx<T>* w, cplx<T>* px, cplx<T>* pz, cplx<T>* r
 // One step as two kernels moved 10 images through the L2; a launch of five steps
 // reads 5 images and writes 4, with 1.2 to 1.4 times the arithmetic, and its time
 // is the steps' arithmetic, barriers and shared-memory neighbours.  20 steps at
-// 384 x 1024: 41 launches in 250 us before, 4 in 70 us now.
+// 384 x 1024: 41 launches in 250 us before, 4 in 70 us now.  At 128 registers it spills 128
+// bytes a thread.
 constexpr int TV_TILE = 64, TV_ROWS = 8;
 
 struct TvTile {
