@@ -281,7 +281,8 @@ isam_status isam_fista_unrolled(isam_plan* plan, const void* s_d, const isam_sol
 /* Gradient of <z_bar, z^K> (real inner product) through the iterations of
  * isam_fista_unrolled (same s_d, opts, every and the ckpt it wrote, theta
  * unchanged since): grad (host double[5]) with respect to theta and, when
- * s_bar (device spectra) is not NULL, with respect to s_d.  Each segment of
+ * s_bar (device spectra, on 8 bytes, 16 for FP64: ISAM_ERR_INVALID otherwise)
+ * is not NULL, with respect to s_d.  Each segment of
  * `every` iterations is recomputed from its checkpoint, then reversed:
  *   ubar = J_T(u^k)^T zbar^k   (Jacobian of the soft threshold, Eq. 14),
  *   etabar = ubar - (1/L) A^H A ubar,

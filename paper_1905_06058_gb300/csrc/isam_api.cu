@@ -518,7 +518,8 @@ template <typename T> isam_status fidelity_impl(isam_plan* P, const void* eta, c
                                                 T* r_out, double* value) {
   Impl<T>& im = impl_of<T>(P);
   T* r = r_out;
-  if (!r) {
+  // (the norm reads the residual in pairs)
+  if (!r || reinterpret_cast<uintptr_t>(r) % sizeof(cplx<T>)) {
     if (!im.s_tmp) ISAM_TRY(plan_alloc(P, &im.s_tmp, P->n_spec));
     r = im.s_tmp;
   }
@@ -529,6 +530,8 @@ template <typename T> isam_status fidelity_impl(isam_plan* P, const void* eta, c
     return launch_norm2<T>(reinterpret_cast<const cplx<T>*>(r), P->n_spec / 2, P->partial,
                            RED_BLOCKS, P->dscal + 5, P->stream);
   }));
+  if (r_out && r != r_out)
+    CUDA_TRY(cudaMemcpyAsync(r_out, r, sizeof(T) * P->n_spec, cudaMemcpyDeviceToDevice, P->stream));
   CUDA_TRY(cudaMemcpyAsync(P->hscal + 5, P->dscal + 5, sizeof(double), cudaMemcpyDeviceToHost,
                            P->stream));
   CUDA_TRY(cudaStreamSynchronize(P->stream));
@@ -1690,6 +1693,9 @@ isam_status isam_fista_unrolled_vjp(isam_plan* P, const void* s_d, const isam_so
                                     void* s_bar, double* grad) {
   if (!P || !s_d || !ckpt || !z_bar || !grad) return ISAM_ERR_INVALID;
   ISAM_TRY(check_unrolled_opts(P, o, every));
+  // s_bar is added to in pairs
+  if (reinterpret_cast<uintptr_t>(s_bar) % (P->p.precision == ISAM_FP64 ? 16 : 8))
+    return ISAM_ERR_INVALID;
   DeviceGuard g(P->device);
   const FitOrder order(P);
   P->launches = 0;

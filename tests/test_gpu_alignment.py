@@ -40,3 +40,18 @@ def test_operators_at_any_element(torch, prec, tol, nx, ny, nk, nz):   # noqa: F
     plan.close()
     assert float((a1 - a).abs().max()) <= tol * float(a.abs().max())
     assert float((b1 - b).abs().max()) <= tol * float(b.abs().max())
+
+
+@pytest.mark.parametrize("prec,tol", [("fp32", 2e-6), ("fp64", 1e-14)])
+def test_residual_at_any_element(torch, prec, tol):   # noqa: F811
+    from paper_1905_06058_gb300.isam import Plan
+    plan = Plan(I.small_bscan(seed=78, nx=32, nk=64).geom, precision=prec)
+    x = torch.from_numpy(I.random_image(plan.image_shape, 5)).cuda().to(plan.cplx_dtype)
+    y = torch.from_numpy(I.random_spectra(plan.spec_shape, 6)).cuda().to(plan.real_dtype)
+    v, r = plan.data_fidelity(x, y)
+    y1, r1 = off_grid(torch, y.shape, y.dtype), off_grid(torch, y.shape, y.dtype)
+    y1.copy_(y)
+    v1, _ = plan.data_fidelity(x, y1, r_out=r1)
+    plan.close()
+    assert v1 == pytest.approx(v, rel=tol)
+    assert float((r1 - r).abs().max()) <= tol * float(r.abs().max())
