@@ -57,11 +57,11 @@ __host__ __device__ __forceinline__ float2 cscale(float2 a, float s) {
   a.x *= s; a.y *= s; return a;
 #endif
 }
-// The same, where FP32 says which product is rounded first and does not leave it to the
-// kernel's contraction: the adjoint's values follow it (FitOrder).  (In k_ax_fused, which
-// contracts cmulc that way by itself, it cost 44 B of spills a thread with WS.)
+// The same for FP32, packed, with the product with b.y rounded first (said, not left to
+// the kernel's contraction: the values of FitOrder's calls follow it)
 __device__ __forceinline__ float2 cmulc_ordered(float2 a, float2 b) {
-  return make_float2(fmaf(a.x, b.x, a.y * b.y), fmaf(a.y, b.x, -(a.x * b.y)));
+  const float2 p = __fmul2_rn(make_float2(a.y, -a.x), make_float2(b.y, b.y));
+  return __ffma2_rn(a, make_float2(b.x, b.x), p);
 }
 __device__ __forceinline__ double2 cmulc_ordered(double2 a, double2 b) { return cmulc(a, b); }
 template <typename C> __host__ __device__ __forceinline__ C cconj(C a) { a.y = -a.y; return a; }

@@ -589,16 +589,16 @@ __device__ __forceinline__ bool quad_fits(const AxArgs<T>& A, const Sample<T, V>
 }
 
 // Y = the scatter of the block's samples, in the window form where every thread's
-// samples fit one (fits; true where a thread has none) and the call is none of
-// FitOrder's.  heads holds every such thread's first floor; taps gives the window's
-// taps (see window_scatter), reload the samples' positions again for the residue-class
-// form.  Starts with a barrier (all reads of Y are done) and ends with one.
+// samples fit one (fits; true where a thread has none; false in FitOrder's calls).  heads
+// holds every such thread's first floor; taps gives the window's taps (see
+// window_scatter), reload the samples' positions again for the residue-class form.
+// Starts with a barrier (all reads of Y are done) and ends with one.
 template <typename T, int J, bool WARP, typename V, typename Taps, typename Reload>
 __device__ __forceinline__ void scatter(const AxArgs<T>& A, const Coefficients<T, J>& co, V* Y,
                                         int K, int nt, int nk, Sample<T, V>* sm, bool fits,
                                         int* lo, int* hi, int* ch_tail, const int* heads,
                                         Taps taps, Reload reload) {
-  if (__syncthreads_and(fits && !A.fit)) {
+  if (__syncthreads_and(fits)) {
     window_scatter<T, J, WARP, V>(Y, K, nt, nk, sm, window_past<T, V>(A, Y), heads, taps);
     return;
   }
@@ -808,17 +808,22 @@ __device__ __forceinline__ void ax_inverse(const AxArgs<T>& A, V* Y, const cplx<
 // at 32 x 24 x 256 takes 25.8 us (29.2 with the residue-class scatter, 33.1 with windows
 // and 64 registers), at 24 x 24 x 128 27.5 (28.5, 32.0), at 64 x 64 x 128 20.8 (47.7,
 // 24.4).  Larger grids are quicker at 64: 128 x 128 x 256 93 us, 100 wide.
-template <typename T, bool WIDE> __host__ __device__ constexpr int ax_max_threads() {
-  return WIDE ? 128 : 512;
+// FIT: FitOrder's operators (FP32): the scatter by residue classes, which product of the
+// spectra and the phase rounds first, and at K = 4096 a trigger at the start (A + A^H at
+// 512 x 1024 -> 2048: 53.3 us, 55.9 late; at 512 x 512 -> 1024 47.4, 38.5 late).  (As a
+// flag of the other instances that cost 1.3 % of k_ax_fwd and k_ax_adj.)
+enum AxVariant { PLAIN = 0, WIDE = 1, FIT = 2 };
+template <typename T, int VAR> __host__ __device__ constexpr int ax_max_threads() {
+  return VAR == WIDE ? 128 : 512;
 }
-template <typename T, bool WIDE> __host__ __device__ constexpr int ax_min_blocks() {
-  return WIDE ? 5 : std::is_same<T, float>::value ? 2 : 1;
+template <typename T, int VAR> __host__ __device__ constexpr int ax_min_blocks() {
+  return VAR == WIDE ? 5 : std::is_same<T, float>::value ? 2 : 1;
 }
 
 // ONE: a block per column instead of per pair (FP64, see
 // launch_ax_JKC).
-template <typename T, int J, int LOGK, bool C16, bool ONE, bool WIDE>
-__global__ void __launch_bounds__(ax_max_threads<T, WIDE>(), (ax_min_blocks<T, WIDE>())) k_ax_fwd(const __grid_constant__ AxArgs<T> A) {
+template <typename T, int J, int LOGK, bool C16, bool ONE, int VAR>
+__global__ void __launch_bounds__(ax_max_threads<T, VAR>(), (ax_min_blocks<T, VAR>())) k_ax_fwd(const __grid_constant__ AxArgs<T> A) {
   using C = cplx<T>;
   using V = column_t<T, ONE>;
   extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -828,10 +833,8 @@ __global__ void __launch_bounds__(ax_max_threads<T, WIDE>(), (ax_min_blocks<T, W
   int c1, c2, mx, my;
   pair_columns<T, ONE>(A, c1, c2, mx, my);
   const bool two = !ONE && c2 != c1;
-  // programmatic dependent launch (as k_ax_fused): twiddles before the wait; FitOrder's
-  // calls let the next kernel start at once at K = 4096 (A + A^H at 512 x 1024 -> 2048:
-  // 53.3 us, 55.9 late; at 512 x 512 -> 1024 47.4, 38.5 late)
-  if (A.fit && K == 4096) cudaTriggerProgrammaticLaunchCompletion();
+  // programmatic dependent launch (as k_ax_fused): twiddles before the wait
+  if (VAR == FIT && LOGK == 12) cudaTriggerProgrammaticLaunchCompletion();
   const C* tw = ax_twiddles<T, LOGK, C16>(A, smem_raw);
   cudaGridDependencySynchronize();
   ax_forward<T, LOGK, C16, V>(A, Y, tw, c1, c2, two, [](const float2*) {});
@@ -873,11 +876,17 @@ __global__ void __launch_bounds__(ax_max_threads<T, WIDE>(), (ax_min_blocks<T, W
   });
 }
 
+// a conj(b), by cmulc_ordered or as the kernel contracts it
+template <bool ORDERED, typename C> __device__ __forceinline__ C conj_product(C a, C b) {
+  if constexpr (ORDERED) return cmulc_ordered(a, b);
+  else return cmulc(a, b);
+}
+
 // RES: the input holds the model spectra S and the kernel forms the residual
 // spectrum R(q) = (S(q) + conj S(-q)) / 2 - F s_d(q) on load (ONE only; see
 // k_ax_fused).
-template <typename T, int J, int LOGK, bool C16, bool ONE, bool RES, bool WIDE>
-__global__ void __launch_bounds__(ax_max_threads<T, WIDE>(), (ax_min_blocks<T, WIDE>())) k_ax_adj(const __grid_constant__ AxArgs<T> A) {
+template <typename T, int J, int LOGK, bool C16, bool ONE, bool RES, int VAR>
+__global__ void __launch_bounds__(ax_max_threads<T, VAR>(), (ax_min_blocks<T, VAR>())) k_ax_adj(const __grid_constant__ AxArgs<T> A) {
   static_assert(ONE || !RES, "the pair kernel with a residual is k_ax_fused");
   using C = cplx<T>;
   using V = column_t<T, ONE>;
@@ -893,10 +902,8 @@ __global__ void __launch_bounds__(ax_max_threads<T, WIDE>(), (ax_min_blocks<T, W
   pair_columns<T, ONE>(A, c1, c2, mx, my);
   const bool two = !ONE && c2 != c1;
   if (tid == 0) { ch_lo = INT_MAX; ch_hi = INT_MIN; }
-  // programmatic dependent launch (as k_ax_fused): twiddles before the wait; FitOrder's
-  // calls let the next kernel start at once at K = 4096 (A + A^H at 512 x 1024 -> 2048:
-  // 53.3 us, 55.9 late; at 512 x 512 -> 1024 47.4, 38.5 late)
-  if (A.fit && K == 4096) cudaTriggerProgrammaticLaunchCompletion();
+  // programmatic dependent launch (as k_ax_fused): twiddles before the wait
+  if (VAR == FIT && LOGK == 12) cudaTriggerProgrammaticLaunchCompletion();
   const C* tw = ax_twiddles<T, LOGK, C16>(A, smem_raw);
   cudaGridDependencySynchronize();
   const bool stopped = RES && A.stop != nullptr && __ldcg(A.stop) != 0;
@@ -919,13 +926,13 @@ __global__ void __launch_bounds__(ax_max_threads<T, WIDE>(), (ax_min_blocks<T, W
         x.a = csub(cscale(cadd(x.a, cconj(y.a)), T(0.5)), d.a);
         x.b = csub(cscale(cadd(x.b, cconj(y.b)), T(0.5)), d.b);
       }
-      sm[2 * h].val.a = cmulc_ordered(x.a, ph.a);
-      sm[2 * h + 1].val.a = cmulc_ordered(x.b, ph.b);
+      sm[2 * h].val.a = conj_product<VAR == FIT>(x.a, ph.a);
+      sm[2 * h + 1].val.a = conj_product<VAR == FIT>(x.b, ph.b);
       if constexpr (!ONE) {
         cpair<T> y{};
         if (two) y = half ? cpair<T>{cconj(x.a), cconj(x.b)} : load_two<T>(r2 + j);
-        sm[2 * h].val.b = cmulc_ordered(y.a, ph.a);
-        sm[2 * h + 1].val.b = cmulc_ordered(y.b, ph.b);
+        sm[2 * h].val.b = conj_product<VAR == FIT>(y.a, ph.a);
+        sm[2 * h + 1].val.b = conj_product<VAR == FIT>(y.b, ph.b);
       }
     }
   }
@@ -936,7 +943,7 @@ __global__ void __launch_bounds__(ax_max_threads<T, WIDE>(), (ax_min_blocks<T, W
     heads[tid] = sm[0].mfl;
     fits = quad_fits<T, V>(A, sm);
   }
-  scatter<T, J, false, V>(A, co, Y, K, nt, nk, sm, fits, &ch_lo, &ch_hi, &ch_tail, heads,
+  scatter<T, J, false, V>(A, co, Y, K, nt, nk, sm, fits && VAR != FIT, &ch_lo, &ch_hi, &ch_tail, heads,
                           [&](int rho, T* e) {
                             window_taps<T, J>(co, rho, sm[rho].frac, window_offset(sm, rho) != 0, e);
                           }, [] {});
@@ -958,11 +965,13 @@ __global__ void __launch_bounds__(ax_max_threads<T, WIDE>(), (ax_min_blocks<T, W
 // waves) 53 % of the issue slots and 64 % of the load/store data path are taken, half
 // of the latter by the transforms' exchanges; DRAM 21 %.  A 1024 x 2048 B-scan (513
 // blocks, 40.2 us) leaves the second of its 1.7 waves two thirds full.
-// At 64 registers the column-split form spills 16 to 44 bytes a thread at J = 6, 72 to
-// 112 at J = 8, whose four samples share 15 slots.
+// At 64 registers the column-split form spills 8 bytes a thread at J = 6 (44 with WS), 60
+// (112) at J = 8, whose four samples share 15 slots.  conj(phase) R goes by the packed
+// ordered product (1024 x 2048 solve 9.99 -> 9.89 ms), with WS, where that spilled more,
+// by the compiler's, which rounds alike.
 // WS: also write the model spectra S to A.s_out.
-template <typename T, int J, int LOGK, bool WS, bool C16, bool WIDE>
-__global__ void __launch_bounds__(ax_max_threads<T, WIDE>(), (ax_min_blocks<T, WIDE>())) k_ax_fused(const __grid_constant__ AxArgs<T> A) {
+template <typename T, int J, int LOGK, bool WS, bool C16, int VAR>
+__global__ void __launch_bounds__(ax_max_threads<T, VAR>(), (ax_min_blocks<T, VAR>())) k_ax_fused(const __grid_constant__ AxArgs<T> A) {
   using C = cplx<T>;
   using V = cpair<T>;
   extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -1048,13 +1057,13 @@ __global__ void __launch_bounds__(ax_max_threads<T, WIDE>(), (ax_min_blocks<T, W
       }
       // R(-q) = conj R(q): the residual is real
       const C R = csub(cscale(cadd(s1, cconj(s2)), T(0.5)), rho % 2 == 0 ? dq.a : dq.b);
-      sm[rho].val.a = cmulc(R, ph);
-      sm[rho].val.b = two ? cmulc(cconj(R), ph) : mk<T>(0, 0);
+      sm[rho].val.a = conj_product<!WS>(R, ph);
+      sm[rho].val.b = two ? conj_product<!WS>(cconj(R), ph) : mk<T>(0, 0);
     });
   }
   if (TM) tmem::wait_stores();
   const Coefficients<T, J> co(A, pos, tid);
-  scatter<T, J, TM, V>(A, co, Y, K, nt, nk, sm, fits, &ch_lo, &ch_hi, &ch_tail, heads,
+  scatter<T, J, TM, V>(A, co, Y, K, nt, nk, sm, fits && !A.fit, &ch_lo, &ch_hi, &ch_tail, heads,
                        [&](int rho, T* e) {
                          if constexpr (TM) tmem::get_taps<J>(tm + rho * TAPS, e);
                          else window_taps<T, J>(co, rho, sm[rho].frac,
@@ -1155,7 +1164,7 @@ enum { AX_FWD = 0, AX_ADJ = 1, AX_FUSED = 2, AX_ADJ_RES = 3 };
 // compiled for FP32 only
 template <typename T> constexpr bool ax_one() { return sizeof(T) == 8; }
 
-template <typename T, int J, int LOGK, bool C16, bool WIDE = false>
+template <typename T, int J, int LOGK, bool C16, int VAR = PLAIN>
 static cudaError_t launch_ax_JKC(const AxArgs<T>& a, int npairs, cudaStream_t s, int kind) {
   constexpr bool ONE = ax_one<T>();
   using V = column_t<T, ONE>;
@@ -1169,10 +1178,11 @@ static cudaError_t launch_ax_JKC(const AxArgs<T>& a, int npairs, cudaStream_t s,
     if (LOGK == 0) sm += a.sc.nk / NRES * sizeof(int);
   }
   void (*kern)(AxArgs<T>) = nullptr;
-  if (kind == AX_ADJ) kern = k_ax_adj<T, J, LOGK, C16, ONE, false, WIDE>;
-  else if (kind == AX_FWD) kern = k_ax_fwd<T, J, LOGK, C16, ONE, WIDE>;
-  else if constexpr (ONE) kern = k_ax_adj<T, J, LOGK, C16, ONE, true, WIDE>;
-  else kern = a.s_out ? k_ax_fused<T, J, LOGK, true, C16, WIDE> : k_ax_fused<T, J, LOGK, false, C16, WIDE>;
+  if (kind == AX_ADJ) kern = k_ax_adj<T, J, LOGK, C16, ONE, false, VAR>;
+  else if (kind == AX_FWD) kern = k_ax_fwd<T, J, LOGK, C16, ONE, VAR>;
+  else if constexpr (ONE) kern = k_ax_adj<T, J, LOGK, C16, ONE, true, VAR>;
+  else if constexpr (VAR == FIT) return cudaErrorInvalidValue;
+  else kern = a.s_out ? k_ax_fused<T, J, LOGK, true, C16, VAR> : k_ax_fused<T, J, LOGK, false, C16, VAR>;
   allow_smem(kern, sm);
   // programmatic dependent launch: each axial kernel builds its twiddles while
   // the previous kernel finishes, then waits for it (cudaGridDependencySynchronize)
@@ -1206,6 +1216,13 @@ static cudaError_t launch_ax_JK(const AxArgs<T>& a, int npairs, cudaStream_t s, 
 // ahead: a 128 x 128 x 256 volume's iteration takes 98 us, 102 split)
 template <typename T, int J>
 cudaError_t launch_ax_J(const AxArgs<T>& a, int npairs, cudaStream_t s, int kind) {
+  if constexpr (sizeof(T) == 4) {
+    if (a.fit && kind != AX_FUSED) {
+      if (a.radix16 && a.sc.K == 4096) return launch_ax_JKC<T, J, 12, true, FIT>(a, npairs, s, kind);
+      if (a.radix16 && a.sc.K == 2048) return launch_ax_JKC<T, J, 11, true, FIT>(a, npairs, s, kind);
+      return launch_ax_JKC<T, J, 0, false, FIT>(a, npairs, s, kind);
+    }
+  }
   switch (a.sc.K) {
     case 4096: return launch_ax_JK<T, J, 12>(a, npairs, s, kind);
     case 2048: return launch_ax_JK<T, J, 11>(a, npairs, s, kind);
@@ -1217,7 +1234,7 @@ cudaError_t launch_ax_J(const AxArgs<T>& a, int npairs, cudaStream_t s, int kind
     // one round of blocks of whole warps at 96 registers
     const int threads = std::max(32, a.sc.K / 8), resident = kMultiprocessors * (65536 / 96);
     if (size_t(npairs) * threads <= size_t(resident))
-      return launch_ax_JKC<T, J, 0, false, true>(a, npairs, s, kind);
+      return launch_ax_JKC<T, J, 0, false, WIDE>(a, npairs, s, kind);
   }
   return launch_ax_JK<T, J, 0>(a, npairs, s, kind);
 }
