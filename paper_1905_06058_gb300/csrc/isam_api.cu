@@ -268,6 +268,24 @@ template <typename T> bool precision_fits(const isam_plan* P) {
   return ax_smem_bytes<T>(P->K) <= 227u * 1024u;
 }
 
+// The FP64 coefficient table, next to a Stolt table (it depends on the positions only, so
+// once).  The kernels evaluate the coefficients without it, so no call fails for it
+// (plan_alloc).  At most 3/2 images: J = 8 takes 64 B a class sample, an image of a volume
+// with nz = nk about as much (128 x 128 x 1024 iteration 15.1 ms without the table, 11.5
+// with it).
+isam_status coef_table(isam_plan* P, Impl<double>& im) {
+  const size_t n = size_t(P->ny / 2 + 1) * (P->nx / 2 + 1) * P->nk * size_t(P->J) / 2;
+  if (im.tab.coef || !im.tab.stab ||
+      n * sizeof(double2) > std::max(2 * kStoltTableMaxBytes, P->n_img * sizeof(double2) * 3 / 2) ||
+      dalloc(&im.tab.coef, n) != ISAM_OK)
+    return ISAM_OK;
+  AxArgs<double> a{};
+  a.sc = P->sc;
+  a.tab = im.tab;
+  a.poly = P->poly64;
+  return from_cuda(launch_coef_table(a, im.tab.coef, P->stream));
+}
+
 // Tables that depend on the dispersion coefficients and the focal depth:
 // e^{j phi(k_j)} (Eq. 7) and, when kept, the Stolt position/phase table.
 // Asynchronous on the plan's stream (the host vector is copied synchronously).
@@ -307,23 +325,8 @@ template <typename T> isam_status phase_tables(isam_plan* P, Impl<T>& im) {
       a.sc = P->sc;
       a.tab = im.tab;
       CUDA_TRY(launch_stolt_table<T>(a, im.tab.stab, P->stream));
-      // FP64: the coefficients too (they depend on the positions only, so once).  The
-      // kernels evaluate them without the table, so no call fails for it (plan_alloc);
-      // an FP32 plan, whose FP64 state serves its power iteration, keeps a small one
-      // only.  At most 3/2 images: J = 8 takes 64 B a class sample, an image of a volume
-      // with nz = nk about as much (128 x 128 x 1024 iteration 15.1 ms without the
-      // table, 11.5 with it).
-      if constexpr (sizeof(T) == 8) {
-        const size_t n = rows * P->nk * size_t(P->J) / 2;
-        const size_t most = p.precision == ISAM_FP64
-                                ? std::max(2 * kStoltTableMaxBytes, P->n_img * sizeof(cplx<T>) * 3 / 2)
-                                : kStoltTableMaxBytes;
-        if (!im.tab.coef && n * sizeof(double2) <= most && dalloc(&im.tab.coef, n) == ISAM_OK) {
-          a.tab = im.tab;
-          a.poly = P->poly64;
-          CUDA_TRY(launch_coef_table(a, im.tab.coef, P->stream));
-        }
-      }
+      if constexpr (sizeof(T) == 8)
+        if (p.precision == ISAM_FP64) ISAM_TRY(coef_table(P, im));
     }
   }
   return ISAM_OK;
@@ -548,6 +551,7 @@ template <typename T> isam_status power_iteration(isam_plan* P, int iters, doubl
   if (!im.zA) ISAM_TRY(plan_alloc(P, &im.zA, P->n_img));
   if (!im.zB) ISAM_TRY(plan_alloc(P, &im.zB, P->n_img));
   if (!im.s_tmp) ISAM_TRY(plan_alloc(P, &im.s_tmp, P->n_spec));
+  if constexpr (sizeof(T) == 8) ISAM_TRY(coef_table(P, im));
   cudaStream_t s = P->stream;
   if (v0) {
     const bool same = (sizeof(T) == 8) == (v0_double != 0);
@@ -581,6 +585,14 @@ template <typename T> isam_status power_iteration(isam_plan* P, int iters, doubl
     if (L == 0.0) break;
     if (fabs(L - L_prev) <= rtol * L) break;
     L_prev = L;
+  }
+  // an FP32 plan keeps a large table for the iteration only (the stream is idle here)
+  if constexpr (sizeof(T) == 8) {
+    const size_t bytes = size_t(P->ny / 2 + 1) * (P->nx / 2 + 1) * P->nk * size_t(P->J) * 8;
+    if (im.tab.coef && P->p.precision != ISAM_FP64 && bytes > kStoltTableMaxBytes) {
+      dfree(im.tab.coef);
+      im.tab.coef = nullptr;
+    }
   }
   *L_out = L;
   return ISAM_OK;

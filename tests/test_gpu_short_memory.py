@@ -123,3 +123,22 @@ def test_tv_without_its_sixth_image(torch, addback):   # noqa: F811
     assert float((got - z).norm()) <= 1e-5 * float(z.norm())
     assert torch.equal(got, again)
     assert torch.equal(got, out)
+
+
+def test_power_iteration_gives_a_large_table_back(torch):   # noqa: F811
+    """An FP32 plan holds a table of more than 64 MB while it iterates for L, not after."""
+    from paper_1905_06058_gb300.isam import Plan
+    g = I.small_bscan(seed=75, nx=64, ny=64, nk=1024).geom
+    coef = 33 * 33 * 1024 * 8 * 8
+    with Pool(torch) as pool:
+        plan = Plan(g, J=8)
+        plan.lipschitz(2, 1e-30)                 # FP64 state and its workspace
+        kept = pool.held()
+        assert coef not in pool.live.values()
+        seen = []
+        alloc = pool.alloc
+        pool.B.set_allocator(lambda n: (seen.append(n), alloc(n))[1], pool.free)
+        plan.lipschitz(2, 1e-30)
+        assert seen == [coef] and pool.held() == kept
+        plan.close()
+        assert not pool.live
