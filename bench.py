@@ -235,16 +235,16 @@ KERNEL_SOURCES = {
 }
 NCU_CAPTURES = {
     "bscan_1024x2048": {
-        "ax_fused": {"sha": "576d9684e6edeac1", "dram": 42535168, "table": 16809984,
-                     "smem_wavefronts": 4430443},
-        "lat_update": {"sha": "4497d26ea88790d5", "dram": 34221312, "table": 0,
-                       "smem_wavefronts": 536837},
+        "ax_fused": {"sha": "8b3a43f533b27a36", "dram": 42423040, "table": 16809984,
+                     "smem_wavefronts": 4431661},
+        "lat_update": {"sha": "4fef39ffcf46e894", "dram": 34220032, "table": 0,
+                       "smem_wavefronts": 536861},
     },
     "volume_256x256x2048": {
-        # 128 x 128 x 2048 capture with the plan's Stolt table: 780,839,680 B and
-        # 75,660,736 wavefronts over 8,194 pairs
-        "ax_fused": {"sha": "576d9684e6edeac1", "dram": 3122786956, "table": 545292288,
-                     "smem_wavefronts": 302587542},
+        # 128 x 128 x 2048 capture with the plan's Stolt table: 780,375,808 B and
+        # 75,628,593 wavefronts over 8,194 pairs
+        "ax_fused": {"sha": "8b3a43f533b27a36", "dram": 3120931807, "table": 545292288,
+                     "smem_wavefronts": 302458993},
     },
 }
 
