@@ -169,6 +169,10 @@ isam_status isam_set_stream(isam_plan* plan, void* stream);
 /* s = A eta (Eq. 12-13, 16).  eta: device image, s: device spectra. */
 isam_status isam_forward(isam_plan* plan, const void* eta, void* s);
 
+/* The same in the order of sums of the calibration entries (see
+ * isam_fista_unrolled): A z of a fitted z, bit for bit isam_data_fidelity's. */
+isam_status isam_calib_forward(isam_plan* plan, const void* eta, void* s);
+
 /* eta = A^H s (Eq. 17), exact adjoint of isam_forward under <a,b> = Re(a^H b). */
 isam_status isam_adjoint(isam_plan* plan, const void* s, void* eta);
 
@@ -271,9 +275,9 @@ isam_status isam_param_grad(isam_plan* plan, const void* x, const void* y, doubl
  * isam_unrolled_checkpoint_images(K, every) images of the plan's type.
  * Synchronous; ISAM_ERR_NONFINITE if an iterate is not finite.
  * FP32 plans with nz > nk, whose fits leave a residual at the size of rounding,
- * keep one order of sums in these calls, isam_param_grad, isam_data_fidelity and
- * the operators; their iterates agree with isam_solve's to rounding, those of
- * other plans bit for bit. */
+ * keep one order of sums in these calls, isam_param_grad, isam_data_fidelity,
+ * isam_calib_forward and isam_adjoint; their iterates agree with isam_solve's to
+ * rounding, those of other plans bit for bit. */
 int32_t isam_unrolled_checkpoint_images(int32_t K, int32_t every);
 isam_status isam_fista_unrolled(isam_plan* plan, const void* s_d, const isam_solve_opts* opts,
                                 int32_t every, void* ckpt, void* z_out);
@@ -347,11 +351,12 @@ void isam_batch_destroy(isam_batch* batch);
  *                  radix 8 whatever the value
  *   lateral_radix  16: lateral passes of lengths 64 to 1024 (2^p, 3 * 2^p from 192;
  *                  FP64: 2^p, 64 to 512) at the built-in tile keep it in
- *                  registers, and isam_forward / isam_adjoint of FP32 plans with
- *                  nz = nk and no filter keep half of the Hermitian spectra; 8:
- *                  radix-8 passes on column pairs in shared memory and whole
- *                  spectra; other lengths and tiles run the latter whatever the
- *                  value.  The autotuner times solve iterations only */
+ *                  registers, and isam_forward / isam_adjoint of FP32 plans
+ *                  without a filter (isam_adjoint: with nz = nk) keep half of
+ *                  the Hermitian spectra; 8: radix-8 passes on column pairs in
+ *                  shared memory and whole spectra; other lengths and tiles run
+ *                  the latter whatever the value.  The autotuner times solve
+ *                  iterations only */
 typedef struct {
   int32_t lateral_tile;
   int32_t stolt_table;

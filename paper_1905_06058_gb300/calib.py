@@ -38,7 +38,7 @@ class IsamA(torch.autograd.Function):
         _apply_theta(plan, theta)
         ctx.plan = plan
         ctx.save_for_backward(eta, theta)
-        return plan.forward(eta.contiguous())
+        return plan.calib_forward(eta.contiguous())
 
     @staticmethod
     def backward(ctx, g):
@@ -69,7 +69,7 @@ class IsamAH(torch.autograd.Function):
         plan = ctx.plan
         _apply_theta(plan, theta)
         xb = xb.contiguous()
-        d_y = plan.forward(xb) if ctx.needs_input_grad[0] else None
+        d_y = plan.calib_forward(xb) if ctx.needs_input_grad[0] else None
         d_theta = None
         if ctx.needs_input_grad[1]:
             d_theta = torch.from_numpy(plan.param_grad(xb, y.contiguous()))

@@ -68,6 +68,7 @@ struct isam_plan {
   Poly<float> poly32{};
   Poly<double> poly64{};
   int2* pairs = nullptr;        // (q, -q) column pairs of the axial kernels
+  int2* pairs_fit = nullptr;    // the same by lower index, or null (build_pairs)
   int npairs = 0;
   double* partial = nullptr;    // reduction partials
   int n_partial = 0;
@@ -403,13 +404,14 @@ template <> const Poly<double>& poly_of<double>(const isam_plan* P) { return P->
 // sum before them, that of lambda = c max |A^H s| included: between this order and the
 // windows, register tiles and half spectra of the other calls gradients moved by 1 to
 // 47 %, losses by 1e-6 to 6e-3 (17 fits of 128 to 512 columns), with either 9 to 11 %
-// from 64 bits.  So that such fits give the values they always gave, the operators and
-// the calibration entries keep one order: the scatter by residue classes (the
-// window form of the gather is the same sum), transforms in shared memory, a parameter's sums over every 256th sample.  Solves,
-// whose image agrees to 1e-5 either way, do not.  With nz = nk the band covers all bins
-// and a fit leaves a residual.
-// A + A^H in this order and in the other: 128 x 256 -> 512 31 and 29 us (calls bound),
-// 1024 x 1024 -> 2048 84 and 59, 64 x 64 x 256 -> 512 94 and 58.
+// from 64 bits.  So that such fits give the values they always gave, isam_adjoint and
+// the calibration entries keep one order: the scatter by residue classes (the window
+// form of the gather is the same sum), transforms in shared memory, whole spectra, a
+// parameter's sums over every 256th sample.  isam_forward and the solves, whose outputs
+// agree to 3e-7 and 1e-5 either way, do not.  With nz = nk the band covers all bins and
+// a fit leaves a residual.
+// A^H in this order and in the other: 128 x 256 -> 512 15 us (calls bound) either way,
+// 1024 x 1024 -> 2048 42 and 31, 64 x 64 x 256 -> 512 48 and 29.
 struct FitOrder {
   isam_plan* P;
   explicit FitOrder(isam_plan* P_) : P(P_) {
@@ -423,7 +425,7 @@ template <typename T> AxArgs<T> ax_args(isam_plan* P, const Impl<T>& im, const c
   AxArgs<T> a{};
   a.in = in; a.out = out; a.sc = P->sc; a.tab = im.tab;
   a.poly = poly_of<T>(P);
-  a.pairs = P->pairs;
+  a.pairs = P->fit_order && P->pairs_fit ? P->pairs_fit : P->pairs;
   if (P->tune_table == 2) {
     a.tab.stab = nullptr;
     a.tab.coef = nullptr;
@@ -463,7 +465,7 @@ template <typename T> isam_status lat_inverse(isam_plan* P, Impl<T>& im, cplx<T>
 // neighbouring samples share a transform, so each is right to 32 bits of the larger of
 // them: not with a filter B, which may set one to zero and leave the other.
 template <typename T> bool half_spectra(const isam_plan* P, const void* s) {
-  return sizeof(T) == 4 && P->nz == P->nk && P->filt_host.empty() && P->tune_radix_lat == 16 &&
+  return sizeof(T) == 4 && !P->fit_order && P->filt_host.empty() && P->tune_radix_lat == 16 &&
          lat_half_takes(P->nx, P->nk) && reinterpret_cast<uintptr_t>(s) % 8 == 0;
 }
 template <typename T> LatArgs<T> half_x_args(isam_plan* P, const void* in, void* out) {
@@ -1145,19 +1147,24 @@ isam_status build_poly(isam_plan* P) {
 }
 
 // Columns (ix, iy) and (-ix, -iy) mod (nx, ny) share |q|; list each pair once, the one
-// of ix <= nx/2 first (where the half spectrum has it; with nz > nk, which takes no half
-// spectra, the one of the lower index, see FitOrder).
+// of ix <= nx/2 first (where the half spectrum has it), and for FitOrder's calls on
+// volumes the one of the lower index.
 isam_status build_pairs(isam_plan* P) {
-  std::vector<int2> pr;
+  std::vector<int2> pr, by_index;
   for (int iy = 0; iy < P->ny; ++iy)
     for (int ix = 0; ix < P->nx; ++ix) {
       const int c = iy * P->nx + ix;
       const int d = ((P->ny - iy) % P->ny) * P->nx + (P->nx - ix) % P->nx;
-      if (c <= d) pr.push_back(2 * ix <= P->nx || P->nz > P->nk ? make_int2(c, d) : make_int2(d, c));
+      if (c > d) continue;
+      pr.push_back(2 * ix <= P->nx ? make_int2(c, d) : make_int2(d, c));
+      by_index.push_back(make_int2(c, d));
     }
   P->npairs = int(pr.size());
   ISAM_TRY(dalloc(&P->pairs, pr.size()));
-  return from_cuda(cudaMemcpy(P->pairs, pr.data(), sizeof(int2) * pr.size(),
+  CUDA_TRY(cudaMemcpy(P->pairs, pr.data(), sizeof(int2) * pr.size(), cudaMemcpyHostToDevice));
+  if (P->ny == 1 || P->nz == P->nk || P->p.precision != ISAM_FP32) return ISAM_OK;
+  ISAM_TRY(dalloc(&P->pairs_fit, pr.size()));
+  return from_cuda(cudaMemcpy(P->pairs_fit, by_index.data(), sizeof(int2) * pr.size(),
                               cudaMemcpyHostToDevice));
 }
 
@@ -1248,7 +1255,7 @@ void isam_plan_destroy(isam_plan* P) {
   impl_free(P->f64);
   dfree(P->partial);
   dfree(P->cpartial);
-  dfree(P->pairs);
+  dfree(P->pairs); dfree(P->pairs_fit);
   dfree(P->dscal);
   dfree(P->flag);
   dfree(P->dstop);
@@ -1269,10 +1276,15 @@ isam_status isam_set_stream(isam_plan* P, void* stream) {
 isam_status isam_forward(isam_plan* P, const void* eta, void* s) {
   if (!P || !eta || !s) return ISAM_ERR_INVALID;
   DeviceGuard g(P->device);
-  const FitOrder order(P);
   P->launches = 0;
   if (P->p.precision == ISAM_FP64) return op_forward<double>(P, eta, s);
   return op_forward<float>(P, eta, s);
+}
+
+isam_status isam_calib_forward(isam_plan* P, const void* eta, void* s) {
+  if (!P) return ISAM_ERR_INVALID;
+  const FitOrder order(P);
+  return isam_forward(P, eta, s);
 }
 
 isam_status isam_adjoint(isam_plan* P, const void* s, void* eta) {
@@ -1458,7 +1470,8 @@ template <typename T> ParamArgs<T> param_args(isam_plan* P, cplx<T>* su, const c
                                               const cplx<T>* fd, T fd_sign, bool write_fa) {
   ParamArgs<T> a{};
   a.su = su; a.se = se; a.fd = fd; a.fd_sign = fd_sign;
-  a.pairs = P->pairs; a.sc = P->sc; a.partial = P->cpartial; a.write_fa = write_fa ? 1 : 0;
+  a.pairs = P->fit_order && P->pairs_fit ? P->pairs_fit : P->pairs;
+  a.sc = P->sc; a.partial = P->cpartial; a.write_fa = write_fa ? 1 : 0;
   a.fit = P->fit_order;
   return a;
 }

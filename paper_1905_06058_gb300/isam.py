@@ -74,6 +74,7 @@ _SIGS = {
     "isam_plan_destroy": (None, [_P]),
     "isam_set_stream": (ctypes.c_int, [_P, _P]),
     "isam_forward": (ctypes.c_int, [_P, _P, _P]),
+    "isam_calib_forward": (ctypes.c_int, [_P, _P, _P]),
     "isam_adjoint": (ctypes.c_int, [_P, _P, _P]),
     "isam_solve": (ctypes.c_int, [_P, _P, ctypes.POINTER(SolveOpts), _P,
                                   ctypes.POINTER(SolveState), ctypes.POINTER(SolveInfo)]),
@@ -270,6 +271,17 @@ class Plan:
         _check(_lib.isam_forward(self._h, self._dev(eta, self.cplx_dtype, self.image_shape, "eta"),
                                  self._dev(out, self.real_dtype, self.spec_shape, "out")),
                "isam_forward")
+        return out
+
+    def calib_forward(self, eta):
+        """isam_calib_forward: A eta as the calibration entries sum it."""
+        import torch
+        self._sync_stream()
+        out = torch.empty(self.spec_shape, dtype=self.real_dtype, device=eta.device)
+        _check(_lib.isam_calib_forward(self._h,
+                                       self._dev(eta, self.cplx_dtype, self.image_shape, "eta"),
+                                       self._dev(out, self.real_dtype, self.spec_shape, "out")),
+               "isam_calib_forward")
         return out
 
     def data_fidelity(self, eta, s_d, r_out=None):

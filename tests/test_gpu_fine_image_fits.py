@@ -61,3 +61,24 @@ def test_fit_keeps_its_values(torch, case):   # noqa: F811
     got, ref = np.array(fit(torch, *case)), np.array(golden()[case])
     assert abs(got[0] - ref[0]) <= 1e-7 * abs(ref[0])
     assert np.linalg.norm(got[1:] - ref[1:]) <= 1e-7 * np.linalg.norm(ref[1:])
+
+
+@pytest.mark.parametrize("case", CASES, ids=lambda c: "x".join(map(str, c)))
+def test_model_is_the_fits_operator(torch, case):   # noqa: F811
+    """A z of calib.model is the one whose residual the data term is of, bit for bit, and
+    isam_forward's to rounding (1e-6 of its norm)."""
+    from paper_1905_06058_gb300 import calib
+    from paper_1905_06058_gb300.isam import Plan
+    nx, ny, nk, nz, J = case
+    g = I.Geometry(nx, ny, nk, nz, 4.65e6, 5.03e6, 2.0e-6, 2.0e-6 if ny > 1 else 0.0, 0.1, 4.0e-4,
+                   (0.0, 5e-10, -8e-16, 0.0))
+    plan = Plan(g, J=J)
+    s = torch.from_numpy(spectra(plan.spec_shape)).cuda()
+    z = plan.adjoint(s)
+    theta = torch.tensor(list(g.disp) + [g.z0], dtype=torch.float64)
+    a = calib.model(z, theta, plan)
+    _, r = plan.data_fidelity(z, s)
+    f = plan.forward(z)
+    plan.close()
+    assert torch.equal(a - s, r)
+    assert float((a - f).norm()) <= 1e-6 * float(f.norm())
